@@ -123,7 +123,67 @@ __device__ __forceinline__ float wall_term(int i, const float uw[3]) {
     return 6.0f * (Codec<ST>::scaled ? Codec<ST>::K : Wq(i)) * xu;
 }
 
+// The boundary form of pull27: sources (sx, sy, szp) and flags per velocity
+// index, at least one of them set.  The address of every population is
+// selected first (the opposite population of the own cell for a bounce-back,
+// else the source, which is a valid cell whatever its flag) and all 27 loads
+// are issued together; the flags then select the value.  A form that branched
+// per population waited for 27 loads one after another: 24 steps of a
+// 75x101x143 window between walls took 1533 us with it and 1423 us with this.
 template <int ST>
+__device__ __forceinline__ void pull27_edge(const Geom &g, const typename Codec<ST>::T *__restrict__ f, int x, int y,
+                                            int zl, int ring, int reseed, const float *__restrict__ utop,
+                                            const int sx[3], const int sy[3], const int szp[3], const int bxf[3],
+                                            const int byf[3], const int bzf[3], const int mvf[3], float q[27]) {
+    const int nx = g.nx, plane = (int)g.plane, ncell = (int)g.ncell;
+    const int zo = zphys(zl, ring, g.nz);
+    const int own = zo * plane + y * nx + x;
+    const bool own_rest = (zo == reseed);
+    // (bounce-back: W_{26-i} = W_i, so the opposite population's stored value
+    // is this one's in every storage domain)
+#pragma unroll
+    for (int ez = 0; ez < 3; ++ez)
+#pragma unroll
+        for (int ey = 0; ey < 3; ++ey)
+#pragma unroll
+            for (int ex = 0; ex < 3; ++ex) {
+                const int i = ex + 3 * ey + 9 * ez;
+                const bool bb = bxf[ex] == 1 || byf[ey] == 1 || bzf[ez] == 1;
+                q[i] = Codec<ST>::load(f + (bb ? (26 - i) * ncell + own : i * ncell + szp[ez] * plane + sy[ey] * nx + sx[ex]));
+            }
+#pragma unroll
+    for (int ez = 0; ez < 3; ++ez)
+#pragma unroll
+        for (int ey = 0; ey < 3; ++ey)
+#pragma unroll
+            for (int ex = 0; ex < 3; ++ex) {
+                const int i = ex + 3 * ey + 9 * ez;
+                const bool bb = bxf[ex] == 1 || byf[ey] == 1 || bzf[ez] == 1;
+                // a source on the entering plane holds stale data: rest
+                if (bb ? own_rest : bzf[ez] == 3) q[i] = 0.0f;
+                if (mvf[ez]) q[i] += wall_term<ST>(i, mvf[ez] == 1 ? g.uw_bottom : g.uw_top);
+            }
+    if (bzf[0] == 2) {  // sources above the pressure top (xi_z = -1): the ghost equilibrium
+        float ux[9], uy[9], uz[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int c = sy[k / 3] * nx + sx[k % 3];
+            ux[k] = __ldg(utop + c);
+            uy[k] = __ldg(utop + plane + c);
+            uz[k] = __ldg(utop + 2 * plane + c);
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k)
+            if (!(bxf[k % 3] == 1 || byf[k / 3] == 1)) q[k] = ghost_dev<ST>(k, ux[k], uy[k], uz[k]);
+    }
+}
+
+// EDGE: boundary cells load all 27 sources together (pull27_edge); false: one
+// branch per population, fewer registers.  True in the cell-pair kernels that
+// sweep the window, false where boundary cells are few and the registers shape
+// the kernel: the x-pair kernels' one-cell fallback (192x192x384 FP16, 16 steps:
+// 6030 us with it, 5895 us without), the near region, the support moments.
+template <int ST, bool EDGE = false>
 __device__ __forceinline__ void pull27(const Geom &g, const typename Codec<ST>::T *__restrict__ f, int x, int y,
                                        int zl, int ring, int reseed, const float *__restrict__ utop, float q[27]) {
     int sx[3], sy[3], szp[3], bxf[3], byf[3], bzf[3], mvf[3];
@@ -164,6 +224,10 @@ __device__ __forceinline__ void pull27(const Geom &g, const typename Codec<ST>::
                     const int i = ex + 3 * ey + 9 * ez;
                     q[i] = Codec<ST>::load(P[ey][ex] + (i * ncell + szp[ez] * plane));
                 }
+        return;
+    }
+    if (EDGE) {
+        pull27_edge<ST>(g, f, x, y, zl, ring, reseed, utop, sx, sy, szp, bxf, byf, bzf, mvf, q);
         return;
     }
     const int zo = zphys(zl, ring, g.nz);
@@ -651,10 +715,10 @@ __device__ __forceinline__ void pull27x2(const Geom &g, const typename Codec<ST>
         return;
     }
     float qa[27];
-    pull27<ST>(g, f, x, y, za, ring, reseed, utop, qa);
+    pull27<ST, true>(g, f, x, y, za, ring, reseed, utop, qa);
 #pragma unroll
     for (int i = 0; i < 27; ++i) q[i].x = qa[i];
-    pull27<ST>(g, f, x, y, zb, ring, reseed, utop, qa);
+    pull27<ST, true>(g, f, x, y, zb, ring, reseed, utop, qa);
 #pragma unroll
     for (int i = 0; i < 27; ++i) q[i].y = qa[i];
 }
