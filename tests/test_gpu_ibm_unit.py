@@ -54,3 +54,26 @@ def test_spread_rejects_marker_outside_grid():
     with pytest.raises(T.TurretError) as e:
         _gpu_spread(X, h, dS, shape)
     assert e.value.status == 7
+
+
+@pytest.mark.parametrize("shape,n,radius,copies", [((4, 4, 4), 4, 0.0, 1), ((9, 7, 5), 4, 0.3, 1), ((40, 61, 35), 9, 8.0, 1),
+                                                   ((18, 22, 20), 5, 3.0, 8)])
+def test_spread_lists_at_grid_and_list_edges(shape, n, radius, copies):
+    """One tile; grids no multiple of a tile; many empty tiles; lists of more
+    candidates than one staged chunk (a surface repeated at the same place)."""
+    nz, ny, nx = shape
+    V, T = I.icosphere(n, 1.0)
+    rng = np.random.default_rng(7)
+    centre = np.array([nx, ny, nz]) / 2.0 - 0.5
+    X = np.concatenate([radius * V + centre + 0.05 * rng.standard_normal(3) for _ in range(copies)])
+    X = X.astype(np.float32).astype(np.float64)  # the positions the GPU sees
+    h = 1e-3 * rng.uniform(0.2, 1.0, (X.shape[0], 3))
+    dS = rng.uniform(0.5, 1.0, X.shape[0])
+    got = np.moveaxis(_gpu_spread(X, h, dS, shape), 0, -1).astype(np.float64)
+    want = O.spread(h, X, dS, shape, (False, False, False))
+    # a cell sums at most m non-negative terms: FP32 weights (a few ulp) and m
+    # additions give a relative error below (m + 16) 2^-24; the oracle's
+    # stencil skips the same cells (m <= all markers, a loose bound)
+    tol = (X.shape[0] + 16) * 2.0 ** -24
+    assert np.abs(got - want).max() <= tol * np.abs(want).max()
+    assert np.array_equal(got == 0.0, want == 0.0) or np.abs(want[got == 0.0]).max() <= tol * np.abs(want).max()
