@@ -5,24 +5,24 @@
 // predictor-corrector of Sec. 2.3; it predicts F(t+1), T(t+1) for the marker
 // velocities of the immersed-boundary step, Sec. 2.2.)
 //
-// Kernels:
-//   k_gemm        C = A B with either operand transposed, BF16 tensor-core
-//                 mma.sync m16n8k16 with FP32 accumulation (or an FP32
-//                 CUDA-core check mode), fused epilogues: bias + GELU
-//                 (forward), GELU' product (backward), plain store (weight
-//                 gradients).  64x64 tiles, 32-deep K chunks staged in shared
-//                 memory; no split-K, no atomics: deterministic.
-//   k_mlp_infer   the whole forward pass of up to 16 samples per block, with
-//                 activations in shared memory (the predictor's inference).
-//   k_loss, k_colsum, k_adamw, k_standardise: loss and its gradient, bias
-//                 gradients, AdamW (decoupled weight decay), normalisation.
+// Kernels (precision 0, BF16 tensor cores, mma.sync m16n8k16 with FP32
+// accumulation; the products are at most 4096x128x128, where the rate of the
+// matrix unit does not show):
+//   k_rows        32 rows per block: the four layers with the BF16 weights and
+//                 all activations in shared memory; with training also the
+//                 loss, and the backward pass down to the first layer
+//   k_wgrad       weight and bias gradients of one 256-row slice per block row
+//   k_update      sum of the slices in order, AdamW and the BF16 copy
+//   k_mlp_infer   up to 16 samples per block (the predictor's inference and
+//                 small batches)
+// Precision 1 (an FP32 check mode): k_gemm and the layer-by-layer passes.
+// Fixed summation orders, no atomics on data: deterministic.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
 
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include "../../include/turret.h"
@@ -48,7 +48,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
 
 // ---------------------------------------------------------------------------
-// GEMM.  A(m, k) = ta ? A[k * lda + m] : A[m * lda + k];
+// GEMM of the FP32 check mode.  A(m, k) = ta ? A[k * lda + m] : A[m * lda + k];
 //        B(k, n) = tb ? B[k * ldb + n] : B[n * ldb + k]   (tb = 0: weights [N][K]).
 struct GemmArgs {
     const float *A;
@@ -81,25 +81,13 @@ __device__ __forceinline__ void epilogue(const GemmArgs &g, int epi, int m, int 
     if (epi == EPI_GELU) g.Aout[(size_t)m * g.ldo + n] = gelu_f(v);
 }
 
-template <bool TC>
 __global__ void __launch_bounds__(GTHREADS) k_gemm(GemmArgs g, int epi) {
-    constexpr int PAD = TC ? 8 : 1;
-    using E = typename std::conditional<TC, __nv_bfloat16, float>::type;
-    __shared__ __align__(16) E As[GBM][GBK + PAD];
-    __shared__ __align__(16) E Bs[GBN][GBK + PAD];
+    __shared__ float As[GBM][GBK + 1];
+    __shared__ float Bs[GBN][GBK + 1];
     const int tid = threadIdx.x;
     const int m0 = blockIdx.x * GBM, n0 = blockIdx.y * GBN;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;  // warp tile origin (TC)
-    const int grp = lane >> 2, tig = lane & 3;
-    float acc[2][4][4];
+    const int tr = tid >> 3, tc = tid & 7;  // rows 4 tr + i, columns tc + 8 j
     float sacc[4][8];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0f;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -115,7 +103,7 @@ __global__ void __launch_bounds__(GTHREADS) k_gemm(GemmArgs g, int epi) {
             const int gm = m0 + m, gk = k0 + k;
             float v = 0.0f;
             if (gm < g.M && gk < kend) v = g.ta ? g.A[(size_t)gk * g.lda + gm] : g.A[(size_t)gm * g.lda + gk];
-            if constexpr (TC) As[m][k] = __float2bfloat16_rn(v); else As[m][k] = v;
+            As[m][k] = v;
         }
 #pragma unroll 4
         for (int e = tid; e < GBN * GBK; e += GTHREADS) {
@@ -124,61 +112,21 @@ __global__ void __launch_bounds__(GTHREADS) k_gemm(GemmArgs g, int epi) {
             const int gn = n0 + n, gk = k0 + k;
             float v = 0.0f;
             if (gn < g.N && gk < kend) v = g.tb ? g.B[(size_t)gk * g.ldb + gn] : g.B[(size_t)gn * g.ldb + gk];
-            if constexpr (TC) Bs[n][k] = __float2bfloat16_rn(v); else Bs[n][k] = v;
+            Bs[n][k] = v;
         }
         __syncthreads();
-        if constexpr (TC) {
-#pragma unroll
-            for (int kk = 0; kk < GBK; kk += 16) {
-                uint32_t a[2][4], b[4][2];
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int r = wm + 16 * i + grp;
-                    a[i][0] = ld_pair(&As[r][kk + 2 * tig]);
-                    a[i][1] = ld_pair(&As[r + 8][kk + 2 * tig]);
-                    a[i][2] = ld_pair(&As[r][kk + 8 + 2 * tig]);
-                    a[i][3] = ld_pair(&As[r + 8][kk + 8 + 2 * tig]);
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int c = wn + 8 * j + grp;
-                    b[j][0] = ld_pair(&Bs[c][kk + 2 * tig]);
-                    b[j][1] = ld_pair(&Bs[c][kk + 8 + 2 * tig]);
-                }
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j]);
-            }
-        } else {
-            const int tr = tid >> 3, tc = tid & 7;  // rows 4 tr + i, columns tc + 8 j
 #pragma unroll 4
-            for (int k = 0; k < GBK; ++k)
+        for (int k = 0; k < GBK; ++k)
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) sacc[i][j] = fmaf(As[4 * tr + i][k], Bs[tc + 8 * j][k], sacc[i][j]);
-        }
+                for (int j = 0; j < 8; ++j) sacc[i][j] = fmaf(As[4 * tr + i][k], Bs[tc + 8 * j][k], sacc[i][j]);
         __syncthreads();
     }
-    if constexpr (TC) {
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int r = m0 + wm + 16 * i + grp, c = n0 + wn + 8 * j + 2 * tig;
-                epilogue(g, epi, r, c, acc[i][j][0]);
-                epilogue(g, epi, r, c + 1, acc[i][j][1]);
-                epilogue(g, epi, r + 8, c, acc[i][j][2]);
-                epilogue(g, epi, r + 8, c + 1, acc[i][j][3]);
-            }
-    } else {
-        const int tr = tid >> 3, tc = tid & 7;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) epilogue(g, epi, m0 + 4 * tr + i, n0 + tc + 8 * j, sacc[i][j]);
-    }
+        for (int j = 0; j < 8; ++j) epilogue(g, epi, m0 + 4 * tr + i, n0 + tc + 8 * j, sacc[i][j]);
 }
 
 // ---------------------------------------------------------------------------
@@ -278,19 +226,411 @@ __global__ void k_refresh_bf16(const float *__restrict__ P, __nv_bfloat16 *__res
 
 // AdamW (Loshchilov & Hutter): moments, bias correction, decoupled decay of
 // the weight matrices.
+__device__ __forceinline__ float adamw_value(float p, float g, float &m, float &v, bool weight, float lr, float b1,
+                                             float b2, float eps, float wd, float bc1, float bc2) {
+    m = b1 * m + (1.0f - b1) * g;
+    v = b2 * v + (1.0f - b2) * g * g;
+    const float upd = (m / bc1) / (sqrtf(v / bc2) + eps) + (weight ? wd * p : 0.0f);
+    return p - lr * upd;
+}
+
 __global__ void k_adamw(float *__restrict__ P, const float *__restrict__ G, float *__restrict__ Mm,
                         float *__restrict__ Vv, float lr, float b1, float b2, float eps, float wd, float bc1,
                         float bc2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MLP_NPARAM) return;
-    const float g = G[i];
-    const float m = b1 * Mm[i] + (1.0f - b1) * g;
-    const float v = b2 * Vv[i] + (1.0f - b2) * g * g;
+    float m = Mm[i], v = Vv[i];
+    const float p = adamw_value(P[i], G[i], m, v, is_weight(i), lr, b1, b2, eps, wd, bc1, bc2);
     Mm[i] = m;
     Vv[i] = v;
-    const float p = P[i];
-    const float upd = (m / bc1) / (sqrtf(v / bc2) + eps) + (is_weight(i) ? wd * p : 0.0f);
-    P[i] = p - lr * upd;
+    P[i] = p;
+}
+
+// ---------------------------------------------------------------------------
+// The BF16 network on 32 rows per block of 256 threads.  Every layer is a
+// 32 x 128 x 128 product (67 MFLOP over a batch of 4096): what it costs is
+// passes over memory and launches, not the products.  So a block keeps the
+// whole network in shared memory (78 KB of BF16 weights), its rows' operands
+// beside it and the pre-activations z in the registers of the threads that
+// need them again for GELU'(z) (the backward product's accumulator tile is the
+// forward one's), and a training step is three launches instead of 28: batch
+// 4096 took 367 us per step with a launch per product, sum and pass, and
+// 42 us with k_rows, k_wgrad and k_update.  32 rows: 128 blocks at batch 4096,
+// one per SM.  Operands are rounded to BF16 where the
+// products take them, sums run in the k order of a 16-wide mma chain and
+// weight gradients over 256-row slices in order.
+constexpr int RT_ROWS = 32, RT_THREADS = 256;
+constexpr int LDK = MLP_H + 8, LDX = MLP_INP + 8, LDY = 24;  // row strides (BF16) free of bank conflicts for ldmatrix
+
+struct RowsSmem {
+    __nv_bfloat16 w1[MLP_H][LDX], w2[MLP_H][LDK], w3[MLP_H][LDK], w4[MLP_OUTP][LDK];
+    __nv_bfloat16 x[RT_ROWS][LDX];
+    __nv_bfloat16 a[2][RT_ROWS][LDK];  // the operand of the current layer and the one being formed
+    __nv_bfloat16 dy[RT_ROWS][LDY];
+    double loss[RT_THREADS / 32];
+};
+
+// What a training pass leaves for k_wgrad: the operands of the weight
+// gradients, activations rounded to BF16 as the products take them, and the
+// layer gradients in FP32.
+struct TrainOut {
+    __nv_bfloat16 *x;     // [n][48] standardised inputs
+    __nv_bfloat16 *a[3];  // [n][128]
+    float *dz[3];         // [n][128]
+    float *dy;            // [n][6]
+    double *loss;         // per block: sum of squared errors
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// acc (16 rows at m0 x 32 columns at n0) = A [.][K] W^T with W [n][K], K in 16-wide steps
+template <int LDA, int LDW>
+__device__ __forceinline__ void rows_product(const __nv_bfloat16 (*A)[LDA], const __nv_bfloat16 (*W)[LDW], int K, int m0,
+                                             int n0, float (&acc)[4][4]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; k += 16) {
+        uint32_t a[4], b[2][4];
+        ldsm4(a, &A[m0 + (lane & 15)][k + (lane >> 4) * 8]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) ldsm4(b[h], &W[n0 + 16 * h + (lane & 7) + (lane >> 4) * 8][k + ((lane >> 3) & 1) * 8]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t bj[2] = {b[j >> 1][2 * (j & 1)], b[j >> 1][2 * (j & 1) + 1]};
+            mma_bf16(acc[j], a, bj);
+        }
+    }
+}
+
+// acc = A [.][K] W with W [K][n]: the backward product, W read transposed
+template <int LDA, int LDW>
+__device__ __forceinline__ void rows_product_t(const __nv_bfloat16 (*A)[LDA], const __nv_bfloat16 (*W)[LDW], int K,
+                                               int m0, int n0, float (&acc)[4][4]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; k += 16) {
+        uint32_t a[4], b[2][4];
+        ldsm4(a, &A[m0 + (lane & 15)][k + (lane >> 4) * 8]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) ldsm4t(b[h], &W[k + (lane & 7) + ((lane >> 3) & 1) * 8][n0 + 16 * h + (lane >> 4) * 8]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t bj[2] = {b[j >> 1][2 * (j & 1)], b[j >> 1][2 * (j & 1) + 1]};
+            mma_bf16(acc[j], a, bj);
+        }
+    }
+}
+
+// bias + GELU of an accumulator tile: z kept in acc, the activation to smem
+__device__ __forceinline__ void rows_gelu(const float *__restrict__ bias, float (&acc)[4][4], __nv_bfloat16 (*out)[LDK],
+                                          int m0, int n0) {
+    const int lane = threadIdx.x & 31, grp = lane >> 2, tig = lane & 3;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int c = n0 + 8 * j + 2 * tig;
+        const float b0 = __ldg(bias + c), b1 = __ldg(bias + c + 1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            acc[j][2 * h] += b0;
+            acc[j][2 * h + 1] += b1;
+            *reinterpret_cast<uint32_t *>(&out[m0 + grp + 8 * h][c]) = pack_bf16(gelu_f(acc[j][2 * h]), gelu_f(acc[j][2 * h + 1]));
+        }
+    }
+}
+
+// gradient tile times GELU'(z): FP32 to global, BF16 operand to smem
+__device__ __forceinline__ void rows_dgelu(const float (&z)[4][4], float (&acc)[4][4], __nv_bfloat16 (*out)[LDK],
+                                           float *__restrict__ dz, int row0, int n, int m0, int n0) {
+    const int lane = threadIdx.x & 31, grp = lane >> 2, tig = lane & 3;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int c = n0 + 8 * j + 2 * tig;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float v0 = acc[j][2 * h] * gelu_prime_f(z[j][2 * h]), v1 = acc[j][2 * h + 1] * gelu_prime_f(z[j][2 * h + 1]);
+            const int r = m0 + grp + 8 * h;
+            *reinterpret_cast<uint32_t *>(&out[r][c]) = pack_bf16(v0, v1);
+            if (row0 + r < n) *reinterpret_cast<float2 *>(dz + (size_t)(row0 + r) * MLP_H + c) = make_float2(v0, v1);
+        }
+    }
+}
+
+// 16-byte copies of `rows` rows of `cols` BF16 values between global (row stride cols) and padded shared rows
+template <int LD>
+__device__ __forceinline__ void load_rows16(__nv_bfloat16 (*s)[LD], const __nv_bfloat16 *__restrict__ g, int rows, int cols) {
+    const int per = cols / 8;
+    for (int e = threadIdx.x; e < rows * per; e += RT_THREADS)
+        *reinterpret_cast<uint4 *>(&s[e / per][(e % per) * 8]) = __ldg(reinterpret_cast<const uint4 *>(g) + e);
+}
+template <int LD>
+__device__ __forceinline__ void store_rows16(__nv_bfloat16 *__restrict__ g, const __nv_bfloat16 (*s)[LD], int rows, int cols) {
+    const int per = cols / 8;
+    for (int e = threadIdx.x; e < rows * per; e += RT_THREADS)
+        reinterpret_cast<uint4 *>(g)[e] = *reinterpret_cast<const uint4 *>(&s[e / per][(e % per) * 8]);
+}
+
+// TRAIN: forward, loss and backward of rows 32 b .. (b = blockIdx.x), raw
+// inputs x and raw targets t.  Otherwise the outputs y, blocks striding over
+// the row groups so that the weights are staged once per block.
+template <bool TRAIN>
+__global__ void __launch_bounds__(RT_THREADS) k_rows(MlpDev w, const float *__restrict__ x, const float *__restrict__ t,
+                                                     int n, float *__restrict__ y, TrainOut o) {
+    extern __shared__ __align__(16) unsigned char rows_raw[];
+    RowsSmem &S = *reinterpret_cast<RowsSmem *>(rows_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = lane >> 2, tig = lane & 3;
+    const int m0 = 16 * (warp & 1), n0 = 32 * (warp >> 1);
+    load_rows16(S.w1, w.Wb + WB1, MLP_H, MLP_INP);
+    load_rows16(S.w2, w.Wb + WB2, MLP_H, MLP_H);
+    load_rows16(S.w3, w.Wb + WB3, MLP_H, MLP_H);
+    load_rows16(S.w4, w.Wb + WB4, MLP_OUTP, MLP_H);
+    for (int row0 = blockIdx.x * RT_ROWS; row0 < n; row0 += gridDim.x * RT_ROWS) {
+        const int nrows = min(RT_ROWS, n - row0);
+        for (int e = tid; e < RT_ROWS * MLP_INP; e += RT_THREADS) {
+            const int r = e / MLP_INP, c = e % MLP_INP;
+            float v = 0.0f;
+            if (r < nrows && c < MLP_IN) v = (x[(size_t)(row0 + r) * MLP_IN + c] - w.mean_x[c]) / w.std_x[c];
+            S.x[r][c] = __float2bfloat16_rn(v);
+        }
+        if (TRAIN)
+            for (int e = tid; e < RT_ROWS * 16; e += RT_THREADS) S.dy[e / 16][e % 16] = __float2bfloat16_rn(0.0f);
+        __syncthreads();
+        float z[3][4][4];
+        rows_product(S.x, S.w1, MLP_INP, m0, n0, z[0]);
+        rows_gelu(w.P + OFF_B1, z[0], S.a[0], m0, n0);
+        __syncthreads();
+        if (TRAIN) {
+            store_rows16(o.x + (size_t)row0 * MLP_INP, S.x, nrows, MLP_INP);
+            store_rows16(o.a[0] + (size_t)row0 * MLP_H, S.a[0], nrows, MLP_H);
+        }
+        rows_product(S.a[0], S.w2, MLP_H, m0, n0, z[1]);
+        rows_gelu(w.P + OFF_B2, z[1], S.a[1], m0, n0);
+        __syncthreads();
+        if (TRAIN) store_rows16(o.a[1] + (size_t)row0 * MLP_H, S.a[1], nrows, MLP_H);
+        rows_product(S.a[1], S.w3, MLP_H, m0, n0, z[2]);
+        rows_gelu(w.P + OFF_B3, z[2], S.a[0], m0, n0);
+        __syncthreads();
+        if (TRAIN) store_rows16(o.a[2] + (size_t)row0 * MLP_H, S.a[0], nrows, MLP_H);
+        double sq = 0.0;
+        if (warp < 2) {  // the six outputs: one 16 x 8 tile per warp
+            float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int k = 0; k < MLP_H; k += 16) {
+                uint32_t a[4], b[2];
+                ldsm4(a, &S.a[0][m0 + (lane & 15)][k + (lane >> 4) * 8]);
+                b[0] = ld_pair(&S.w4[grp][k + 2 * tig]);
+                b[1] = ld_pair(&S.w4[grp][k + 8 + 2 * tig]);
+                mma_bf16(acc, a, b);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int r = m0 + grp + (q >= 2 ? 8 : 0), c = 2 * tig + (q & 1);
+                if (c >= MLP_OUT || r >= nrows) continue;
+                const float out = acc[q] + __ldg(w.P + OFF_B4 + c);
+                const size_t at = (size_t)(row0 + r) * MLP_OUT + c;
+                if (TRAIN) {
+                    const float sc = 2.0f / (float)(n * MLP_OUT);  // dL/dy = 2 (y - t) / (6 n)
+                    const float e = out - (t[at] - w.mean_y[c]) / w.std_y[c];
+                    sq += (double)e * (double)e;
+                    const float d = sc * e;
+                    o.dy[at] = d;
+                    S.dy[r][c] = __float2bfloat16_rn(d);
+                } else {
+                    y[at] = fmaf(out, w.std_y[c], w.mean_y[c]);
+                }
+            }
+        }
+        if constexpr (TRAIN) {
+#pragma unroll
+            for (int q = 16; q > 0; q >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, q);
+            if (lane == 0) S.loss[warp] = sq;
+            __syncthreads();
+            if (tid == 0) o.loss[blockIdx.x] = S.loss[0] + S.loss[1];
+            // backward: (dy W4), (dz W3), (dz W2), each times GELU' of the layer below
+            float acc[4][4];
+            {
+                uint32_t a[4], b[4];
+                ldsm4(a, &S.dy[m0 + (lane & 15)][(lane >> 4) * 8]);
+                ldsm4t(b, &S.w4[lane & 7][n0 + (lane >> 3) * 8]);  // k 0..7; rows 8..15 are zero
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t bj[2] = {b[j], 0u};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
+                    mma_bf16(acc[j], a, bj);
+                }
+            }
+            rows_dgelu(z[2], acc, S.a[1], o.dz[2], row0, n, m0, n0);
+            __syncthreads();
+            rows_product_t(S.a[1], S.w3, MLP_H, m0, n0, acc);
+            rows_dgelu(z[1], acc, S.a[0], o.dz[1], row0, n, m0, n0);
+            __syncthreads();
+            rows_product_t(S.a[0], S.w2, MLP_H, m0, n0, acc);
+            rows_dgelu(z[0], acc, S.a[1], o.dz[0], row0, n, m0, n0);
+        }
+        __syncthreads();  // the buffers are free for the next rows
+    }
+}
+
+// Weight and bias gradients of the rows of slice blockIdx.y (KSLICE rows) into
+// part[slice][MLP_NPARAM].  blockIdx.x < WG_TILES: one 64 x 64 tile of one
+// layer's dz^T a, the whole slice of both operands staged once (ldmatrix
+// transposes them), 16 k-steps in row order; otherwise 128 columns of the
+// bias gradients, summed in row order.
+constexpr int WG_THREADS = 128, WG_TILES = 12, WG_COLS = 4, WG_LD = 64 + 8;
+struct WgradSmem {
+    __nv_bfloat16 dz[KSLICE][WG_LD], a[KSLICE][WG_LD];
+};
+
+__global__ void __launch_bounds__(WG_THREADS) k_wgrad(TrainOut o, int n, float *__restrict__ part) {
+    extern __shared__ __align__(16) unsigned char wg_raw[];
+    WgradSmem &S = *reinterpret_cast<WgradSmem *>(wg_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = lane >> 2, tig = lane & 3;
+    const int r0 = blockIdx.y * KSLICE, nr = min(KSLICE, n - r0);
+    float *out = part + (size_t)blockIdx.y * MLP_NPARAM;
+    if (blockIdx.x >= WG_TILES) {
+        const int c = (blockIdx.x - WG_TILES) * WG_THREADS + tid;
+        const int l = c / MLP_H;  // 0 .. 2: hidden layers, 3: the outputs
+        if (l > 3 || (l == 3 && c - 3 * MLP_H >= MLP_OUT)) return;
+        const int ld = l == 3 ? MLP_OUT : MLP_H, cc = c - l * MLP_H;
+        const float *d = (l == 3 ? o.dy : l == 2 ? o.dz[2] : l == 1 ? o.dz[1] : o.dz[0]) + (size_t)r0 * ld + cc;
+        float s = 0.0f;
+#pragma unroll 32
+        for (int r = 0; r < nr; ++r) s += __ldg(d + (size_t)r * ld);
+        out[(l == 3 ? OFF_B4 : l == 2 ? OFF_B3 : l == 1 ? OFF_B2 : OFF_B1) + cc] = s;
+        return;
+    }
+    // tiles: 0, 1 the first layer (128 x 34), 2..5 the second, 6..9 the third, 10, 11 the outputs (6 x 128)
+    const int b = blockIdx.x, l = b < 2 ? 0 : b < 6 ? 1 : b < 10 ? 2 : 3;
+    const int tm = l == 0 ? b : l == 3 ? 0 : ((b - 2) >> 1) & 1, tn = l == 0 ? 0 : b & 1;
+    const int M = l == 3 ? MLP_OUT : MLP_H, N = l == 0 ? MLP_IN : MLP_H, lda = l == 0 ? MLP_INP : MLP_H;
+    const float *dz = l == 3 ? o.dy : l == 2 ? o.dz[2] : l == 1 ? o.dz[1] : o.dz[0];
+    const __nv_bfloat16 *act = l == 0 ? o.x : l == 1 ? o.a[0] : l == 2 ? o.a[1] : o.a[2];
+    if (l == 3) {
+        for (int e = tid; e < KSLICE * 8; e += WG_THREADS) {  // eight values per row of the 64: six outputs, then zeros
+            const int r = e / 8, c = e % 8;
+            const float v = r < nr && c < MLP_OUT ? __ldg(dz + (size_t)(r0 + r) * MLP_OUT + c) : 0.0f;
+            S.dz[r][c] = __float2bfloat16_rn(v);
+#pragma unroll
+            for (int q = 1; q < 8; ++q) S.dz[r][8 * q + c] = __float2bfloat16_rn(0.0f);
+        }
+    } else {
+#pragma unroll 8
+        for (int e = tid; e < KSLICE * 16; e += WG_THREADS) {
+            const int r = e / 16, c = (e % 16) * 4;
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (r < nr) v = __ldg(reinterpret_cast<const float4 *>(dz + (size_t)(r0 + r) * MLP_H + 64 * tm + c));
+            *reinterpret_cast<uint2 *>(&S.dz[r][c]) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+        }
+    }
+    const int groups = l == 0 ? MLP_INP / 8 : 8;  // 16-byte groups of an activation row present in this tile
+#pragma unroll 8
+    for (int e = tid; e < KSLICE * 8; e += WG_THREADS) {
+        const int r = e / 8, c = e % 8;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (r < nr && c < groups) v = __ldg(reinterpret_cast<const uint4 *>(act + (size_t)(r0 + r) * lda + 64 * tn + 8 * c));
+        *reinterpret_cast<uint4 *>(&S.a[r][8 * c]) = v;
+    }
+    __syncthreads();
+    const int wm = 32 * (warp >> 1), wn = 32 * (warp & 1);
+    float acc[2][4][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0f;
+    for (int k = 0; k < KSLICE; k += 16) {
+        uint32_t a[2][4], bq[2][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            ldsm4t(a[i], &S.dz[k + (lane & 7) + (lane >> 4) * 8][wm + 16 * i + ((lane >> 3) & 1) * 8]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            ldsm4t(bq[h], &S.a[k + (lane & 7) + ((lane >> 3) & 1) * 8][wn + 16 * h + (lane >> 4) * 8]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t bj[2] = {bq[j >> 1][2 * (j & 1)], bq[j >> 1][2 * (j & 1) + 1]};
+                mma_bf16(acc[i][j], a[i], bj);
+            }
+    }
+    out += l == 0 ? OFF_W1 : l == 1 ? OFF_W2 : l == 2 ? OFF_W3 : OFF_W4;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int m = 64 * tm + wm + 16 * i + grp + (q >= 2 ? 8 : 0), c = 64 * tn + wn + 8 * j + 2 * tig + (q & 1);
+                if (m < M && c < N) out[(size_t)m * N + c] = acc[i][j][q];
+            }
+}
+
+// The place of parameter i in the padded BF16 weights, or -1 for a bias.
+__device__ __forceinline__ int wb_index(int i) {
+    if (i < OFF_B1) return WB1 + (i / MLP_IN) * MLP_INP + i % MLP_IN;
+    if (i >= OFF_W2 && i < OFF_B2) return WB2 + (i - OFF_W2);
+    if (i >= OFF_W3 && i < OFF_B3) return WB3 + (i - OFF_W3);
+    if (i >= OFF_W4 && i < OFF_B4) return WB4 + (i - OFF_W4);
+    return -1;
+}
+
+// Gradient of every parameter as the slice sums in slice order, and (step)
+// its AdamW update with the BF16 copy.  Block 0 also adds the blocks' losses
+// in block order: to *loss and, when given, to host-visible memory.
+__global__ void __launch_bounds__(256) k_update(const float *__restrict__ part, int nsl, float *__restrict__ G, int step,
+                                                float *__restrict__ P, float *__restrict__ Mm, float *__restrict__ Vv,
+                                                __nv_bfloat16 *__restrict__ wb, float lr, float b1, float b2, float eps,
+                                                float wd, float bc1, float bc2, const double *__restrict__ lpart,
+                                                int nloss, int total, double *loss, double *host_loss) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < MLP_NPARAM) {
+        float s = part[i];
+#pragma unroll 16
+        for (int z = 1; z < nsl; ++z) s += part[(size_t)z * MLP_NPARAM + i];
+        G[i] = s;
+        if (step) {
+            float m = Mm[i], v = Vv[i];
+            const float p = adamw_value(P[i], s, m, v, is_weight(i), lr, b1, b2, eps, wd, bc1, bc2);
+            Mm[i] = m;
+            Vv[i] = v;
+            P[i] = p;
+            const int at = wb_index(i);
+            if (at >= 0) wb[at] = __float2bfloat16_rn(p);
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        double s = 0.0;
+        for (int k = threadIdx.x; k < nloss; k += 32) s += lpart[k];
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+        if (threadIdx.x == 0) {
+            s /= (double)total;
+            *loss = s;
+            if (host_loss) *host_loss = s;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -400,11 +740,10 @@ __device__ __forceinline__ void mlp_infer_rows(const MlpDev &w, const float *__r
     }
 }
 
-template <bool TC>
 __global__ void __launch_bounds__(INF_THREADS) k_mlp_infer(MlpDev w, const float *__restrict__ x, int n,
                                                            float *__restrict__ y) {
     __shared__ InferSmem sm;
-    mlp_infer_rows<TC>(w, x, n, blockIdx.x * INF_ROWS, y, sm);
+    mlp_infer_rows<false>(w, x, n, blockIdx.x * INF_ROWS, y, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -582,11 +921,18 @@ __global__ void k_build_samples(const double *__restrict__ log, long long nsamp,
     }
 }
 
+// BF16 outputs of n rows: two blocks per SM at most, each striding over the row groups
+static cudaError_t launch_rows(const MlpDev &w, const float *x, int n, float *y, cudaStream_t s) {
+    const int groups = (n + RT_ROWS - 1) / RT_ROWS;
+    k_rows<false><<<groups < 304 ? groups : 304, RT_THREADS, sizeof(RowsSmem), s>>>(w, x, nullptr, n, y, TrainOut{});
+    return cudaGetLastError();
+}
+
 cudaError_t launch_mlp_infer(const MlpDev &w, const float *x, int n, float *y, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int nb = (n + INF_ROWS - 1) / INF_ROWS;
-    if (w.precision == 0) k_mlp_infer<true><<<nb, INF_THREADS, 0, s>>>(w, x, n, y);
-    else k_mlp_infer<false><<<nb, INF_THREADS, 0, s>>>(w, x, n, y);
+    if (w.precision == 0) return launch_rows(w, x, n, y, s);
+    k_mlp_infer<<<nb, INF_THREADS, 0, s>>>(w, x, n, y);
     return cudaGetLastError();
 }
 
@@ -604,8 +950,9 @@ struct turret_mlp {
     float *X0, *T, *Y, *dY, *Z[3], *A[3], *D[2];
     float *part;  // split-K partial sums [MAX_SLICES][128][128]
     double *loss;
+    double *host_loss;  // page-locked copy written by the update kernel, or null (the loss is then copied)
     long long adam_step;
-    // the training step (standardise, forward, backward, AdamW, BF16 copy) as
+    // the FP32 training step (standardise, forward, backward, AdamW, BF16 copy) as
     // one CUDA graph per batch size; between replays only the input pointers
     // and the optimiser's scalars change, in the three nodes that take them
     cudaGraph_t train_graph;  // kept: its nodes address the instantiated graph's nodes
@@ -651,6 +998,9 @@ void carve_mlp(MCarver &cv, int cap, turret_mlp *m) {
     M.loss = (double *)cv.take(8);
     M.part = (float *)cv.take((size_t)MAX_SLICES * MLP_H * MLP_H * 4);
 }
+// a batch of more slices than part holds has them in D: 1 KB a row against 598 B a row and one slice
+static_assert((size_t)MAX_SLICES * MLP_H * MLP_H / MLP_NPARAM * KSLICE * (2 * MLP_H * 4 - MLP_NPARAM * 4 / KSLICE - 1) >=
+                  (size_t)MLP_NPARAM * 4, "D holds the partial gradients of large batches");
 
 turret_status mfail(turret_mlp *m, turret_status s, const std::string &msg) {
     if (m) m->err = msg; else g_mlp_err = msg;
@@ -667,8 +1017,7 @@ turret_status mfail(turret_mlp *m, turret_status s, const std::string &msg) {
 cudaError_t gemm(const turret_mlp *m, const GemmArgs &g, int epi) {
     const dim3 grid((g.M + GBM - 1) / GBM, (g.N + GBN - 1) / GBN,
                     g.kslice > 0 ? (g.K + g.kslice - 1) / g.kslice : 1);
-    if (m->precision == 0) k_gemm<true><<<grid, GTHREADS, 0, m->stream>>>(g, epi);
-    else k_gemm<false><<<grid, GTHREADS, 0, m->stream>>>(g, epi);
+    k_gemm<<<grid, GTHREADS, 0, m->stream>>>(g, epi);
     return cudaGetLastError();
 }
 
@@ -683,7 +1032,7 @@ GemmArgs gargs(const float *A, int lda, int ta, const float *B, int ldb, int tb,
     return g;
 }
 
-// Forward pass of n standardised rows in X0 -> Y (keeps Z, A for backprop).
+// The FP32 check mode: forward pass of n standardised rows in X0 -> Y (keeps Z, A for backprop).
 cudaError_t forward(turret_mlp *m, int n) {
     const float *W[4] = {m->P + OFF_W1, m->P + OFF_W2, m->P + OFF_W3, m->P + OFF_W4};
     const float *b[4] = {m->P + OFF_B1, m->P + OFF_B2, m->P + OFF_B3, m->P + OFF_B4};
@@ -750,6 +1099,45 @@ cudaError_t prepare(turret_mlp *m, const float *x, const float *y, int n) {
     return cudaGetLastError();
 }
 
+// Gradients (and, with opt, one AdamW step) of raw rows x, targets y in BF16:
+// forward and backward by rows, weight gradients by slices, update.  The
+// buffers of the FP32 mode hold this mode's operands: X0, A the BF16 inputs
+// and activations, Z the layer gradients, T the losses per block; the slices'
+// partial gradients go to part, or to D where it is the larger (batches of
+// more than 27 slices).
+cudaError_t train_bf16(turret_mlp *m, const float *x, const float *y, int n, const turret_adamw *opt, float bc1,
+                       float bc2) {
+    const int groups = (n + RT_ROWS - 1) / RT_ROWS, nsl = (n + KSLICE - 1) / KSLICE;
+    TrainOut o;
+    o.x = (__nv_bfloat16 *)m->X0;
+    for (int l = 0; l < 3; ++l) {
+        o.a[l] = (__nv_bfloat16 *)m->A[l];
+        o.dz[l] = m->Z[l];
+    }
+    o.dy = m->dY;
+    o.loss = (double *)m->T;
+    const size_t need = (size_t)nsl * MLP_NPARAM, have = (size_t)MAX_SLICES * MLP_H * MLP_H;
+    float *part = need <= have ? m->part : m->D[0];
+    k_rows<true><<<groups, RT_THREADS, sizeof(RowsSmem), m->stream>>>(m->dev, x, y, n, nullptr, o);
+    k_wgrad<<<dim3(WG_TILES + WG_COLS, nsl), WG_THREADS, sizeof(WgradSmem), m->stream>>>(o, n, part);
+    const turret_adamw a = opt ? *opt : turret_adamw{0.0f, 0.0f, 0.0f, 1.0f, 0.0f};
+    k_update<<<(MLP_NPARAM + 255) / 256, 256, 0, m->stream>>>(part, nsl, m->G, opt != nullptr, m->P, m->Mm, m->Vv, m->Wb,
+                                                              a.lr, a.beta1, a.beta2, a.eps, a.weight_decay, bc1, bc2,
+                                                              o.loss, groups, n * MLP_OUT, m->loss, m->host_loss);
+    return cudaGetLastError();
+}
+
+// The loss of the last pass (waits for the stream).
+cudaError_t read_loss(turret_mlp *m, float *loss) {
+    double L = 0.0;
+    cudaError_t e = cudaSuccess;
+    const bool mapped = m->precision == 0 && m->host_loss;
+    if (!mapped) e = cudaMemcpyAsync(&L, m->loss, 8, cudaMemcpyDeviceToHost, m->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+    if (e == cudaSuccess) *loss = (float)(mapped ? *static_cast<volatile double *>(m->host_loss) : L);
+    return e;
+}
+
 cudaError_t refresh(turret_mlp *m) {
     k_refresh_bf16<<<(WB_END + 255) / 256, 256, 0, m->stream>>>(m->P, m->Wb);
     return cudaGetLastError();
@@ -783,6 +1171,7 @@ extern "C" turret_status mlp_init(turret_mlp **out, int32_t batch_cap, int32_t p
     m->train_exec = nullptr;
     m->train_graph = nullptr;
     m->train_n = 0;
+    m->host_loss = nullptr;
     MCarver cv{(char *)ws, 0};
     carve_mlp(cv, batch_cap, m);
     std::vector<float> norm(2 * (MLP_IN + MLP_OUT));
@@ -793,8 +1182,20 @@ extern "C" turret_status mlp_init(turret_mlp **out, int32_t batch_cap, int32_t p
     if (e == cudaSuccess) e = cudaMemsetAsync(m->Vv, 0, MLP_NPARAM * 4, m->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->norm, norm.data(), norm.size() * 4, cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess) e = refresh(m);
+    if (e == cudaSuccess && precision == 0) {
+        e = cudaFuncSetAttribute(k_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RowsSmem));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RowsSmem));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradSmem));
+        if (cudaHostAlloc((void **)&m->host_loss, sizeof(double), cudaHostAllocDefault) != cudaSuccess) {
+            m->host_loss = nullptr;  // the loss is then copied from the device
+            cudaGetLastError();
+        }
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) {
+        if (m->host_loss) cudaFreeHost(m->host_loss);
         delete m;
         return mfail(nullptr, TURRET_ECUDA, std::string("mlp_init: ") + cudaGetErrorString(e));
     }
@@ -846,6 +1247,10 @@ extern "C" turret_status mlp_set_norm(turret_mlp *m, const float *mean_x, const 
 extern "C" turret_status mlp_forward(turret_mlp *m, const float *x, int32_t n, float *y) {
     if (!m || !x || !y) return mfail(m, TURRET_EINVAL, "NULL argument");
     if (n < 1 || n > m->cap) return mfail(m, TURRET_EINVAL, "batch outside 1..capacity");
+    if (m->precision == 0) {
+        MK(launch_rows(m->dev, x, n, y, m->stream), "forward");
+        return TURRET_OK;
+    }
     MK(prepare(m, x, nullptr, n), "standardise");
     MK(forward(m, n), "forward");
     k_unstandardise<<<(n * MLP_OUT + 255) / 256, 256, 0, m->stream>>>(m->Y, n, m->dev.mean_y, m->dev.std_y, y);
@@ -864,14 +1269,15 @@ extern "C" turret_status mlp_loss_grad(turret_mlp *m, const float *x, const floa
                                        float *grad) {
     if (!m || !x || !y || !loss) return mfail(m, TURRET_EINVAL, "NULL argument");
     if (n < 1 || n > m->cap) return mfail(m, TURRET_EINVAL, "batch outside 1..capacity");
-    MK(prepare(m, x, y, n), "standardise");
-    MK(forward(m, n), "forward");
-    MK(backward(m, n), "backward");
-    double L = 0.0;
-    MK(cudaMemcpyAsync(&L, m->loss, 8, cudaMemcpyDeviceToHost, m->stream), "loss");
+    if (m->precision == 0) {
+        MK(train_bf16(m, x, y, n, nullptr, 1.0f, 1.0f), "loss and gradient");
+    } else {
+        MK(prepare(m, x, y, n), "standardise");
+        MK(forward(m, n), "forward");
+        MK(backward(m, n), "backward");
+    }
     if (grad) MK(cudaMemcpyAsync(grad, m->G, MLP_NPARAM * 4, cudaMemcpyDeviceToDevice, m->stream), "grad");
-    MK(cudaStreamSynchronize(m->stream), "loss sync");
-    *loss = (float)L;
+    MK(read_loss(m, loss), "loss");
     return TURRET_OK;
 }
 
@@ -978,29 +1384,32 @@ extern "C" turret_status mlp_train_step(turret_mlp *m, const float *x, const flo
     if (!(opt->lr >= 0.0f) || !(opt->beta1 >= 0.0f && opt->beta1 < 1.0f) || !(opt->beta2 >= 0.0f && opt->beta2 < 1.0f) ||
         !(opt->eps > 0.0f) || !(opt->weight_decay >= 0.0f))
         return mfail(m, TURRET_EINVAL, "invalid optimiser settings");
+    if (m->stream) {  // the step count is part of the update: not for replay in a caller's graph
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        MK(cudaStreamIsCapturing(m->stream, &cs), "training step");
+        if (cs != cudaStreamCaptureStatusNone) return mfail(m, TURRET_ECUDA, "training step on a capturing stream");
+    }
     m->adam_step += 1;
     const float bc1 = (float)(1.0 - pow((double)opt->beta1, (double)m->adam_step));
     const float bc2 = (float)(1.0 - pow((double)opt->beta2, (double)m->adam_step));
-    if (m->stream) {
-        // a graph replay per step (the captured step has ~25 kernels)
+    if (m->precision == 0) {
+        MK(train_bf16(m, x, y, n, opt, bc1, bc2), "training step");
+    } else if (m->stream) {
+        // FP32: a graph replay per step (the captured step has 28 kernels)
         if (m->train_n != n) MK(capture_train(m, x, y, n, opt), "training graph capture");
         MK(replay_train(m, x, y, n, opt, bc1, bc2), "training graph launch");
     } else {
         MK(enqueue_train(m, x, y, n, opt, bc1, bc2), "training step");
     }
-    if (loss) {
-        double L = 0.0;
-        MK(cudaMemcpyAsync(&L, m->loss, 8, cudaMemcpyDeviceToHost, m->stream), "loss");
-        MK(cudaStreamSynchronize(m->stream), "loss sync");
-        *loss = (float)L;
-    }
+    if (loss) MK(read_loss(m, loss), "loss");
     return TURRET_OK;
 }
 
 extern "C" turret_status mlp_destroy(turret_mlp *m) {
     if (!m) return TURRET_EINVAL;
-    if (m->stream) cudaStreamSynchronize(m->stream);
+    if (m->stream || m->host_loss) cudaStreamSynchronize(m->stream);
     drop_train_graph(m);
+    if (m->host_loss) cudaFreeHost(m->host_loss);
     delete m;
     return TURRET_OK;
 }

@@ -502,8 +502,11 @@ class MLP:
         return float(L.value), g
 
     def train_step(self, x, y, lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, want_loss=True):
-        """One AdamW step; x, y float32 CUDA tensors [n][34], [n][6] (n <= batch_cap)."""
+        """One AdamW step; x, y float32 CUDA tensors [n][34], [n][6] (n <= batch_cap).
+
+        Ordered after the work enqueued on the current stream (x and y may still be in the making)."""
         n = x.shape[0]
+        self.stream.wait_stream(self.torch.cuda.current_stream(self.device))
         opt = AdamW(lr, beta1, beta2, eps, weight_decay)
         L = C.c_float()
         self._check(self._L.mlp_train_step(self.m, C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()), n,

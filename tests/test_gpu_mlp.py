@@ -118,3 +118,21 @@ def test_training_loss_is_monotone_on_a_fixed_batch(precision):
     assert all(b < a for a, b in zip(losses, losses[1:])), losses
     assert losses[-1] < 0.5 * losses[0]
     net.close()
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 257, 7000])
+def test_bf16_gradients_at_block_and_slice_edges(n):
+    # 32-row blocks, 256-row gradient slices, and more slices than the first
+    # partial-sum buffer holds; the BF16 bar of the gradient test above
+    x, y = _data(max(n, 64), 9)  # the standardisation needs some spread
+    norm = _norm(x, y)
+    x, y = x[:n], y[:n]
+    p = I.mlp_init_params(10)
+    net = _net("bf16", p, norm, cap=n)
+    want_y, want_L, want_g = _oracle(p, x, y, norm)
+    got_y = net.forward(x).cpu().numpy().astype(np.float64)
+    assert np.abs(got_y - want_y).max() / np.abs(want_y).max() < 2e-2
+    L, g = net.loss_grad(x, y)
+    assert abs(L - want_L) / want_L < 2e-2
+    assert _per_tensor_err(g.cpu().numpy().astype(np.float64), want_g) < 2e-2
+    net.close()
