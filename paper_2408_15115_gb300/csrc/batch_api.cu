@@ -205,15 +205,14 @@ extern "C" turret_status turret_batch_init(turret_batch **out, turret_ctx *const
         R.g = c->geom;
         R.bc = c->body;
         R.box = c->box;
-        R.m = c->mk;
+        R.m[0] = c->mk[0];
+        R.m[1] = c->mk[1];
         R.ba = c->ba;
         for (int k = 0; k < 2; ++k) {
             R.f[k] = c->f[k];
             R.utop[k] = c->utop[k];
         }
         R.st = c->dstate;
-        R.tile_list = c->tile_list;
-        R.tile_count = c->tile_count;
         R.storage = c->storage;
         R.cap = c->cap;
         R.nm = c->nm;
@@ -292,7 +291,7 @@ static cudaError_t batch_enqueue(turret_batch *b, int p) {
     CE(launch_batch_collide(PHASE_NEAR, b->d_cdesc, tab(T_NEAR), n, p, b->total[T_NEAR], b->threads, 1, b->side));
     CE(cudaStreamWaitEvent(b->side, b->ev_pred, 0));
     CE(launch_batch_box_moments_bin(R, tab(T_MB), n, p, b->total[T_MB], b->side));
-    CE(launch_batch_interp0(R, tab(T_IP), n, b->total[T_IP], b->warm, b->side));
+    CE(launch_batch_interp0(R, tab(T_IP), n, p, b->total[T_IP], b->warm, b->side));
     CE(cudaEventRecord(b->ev_red, b->side));
     CE(cudaStreamWaitEvent(b->aux, b->ev_red, 0));
     CE(launch_batch_reduce_ft(R, n, p ^ 1, b->aux));
@@ -303,7 +302,7 @@ static cudaError_t batch_enqueue(turret_batch *b, int p) {
         int src = HSEL_R0;
         for (int cyc = 1; cyc <= C; ++cyc) {
             const int dst = ((C - cyc) % 2 == 0) ? HSEL_HL : HSEL_HB;
-            CE(launch_batch_cycle(R, tab(T_CYC), n, b->total[T_CYC], src, dst, -1, cyc == C, cyc - 1, 0, b->side));
+            CE(launch_batch_cycle(R, tab(T_CYC), n, p, b->total[T_CYC], src, dst, -1, cyc == C, cyc - 1, 0, b->side));
             src = dst;
         }
     } else {
@@ -313,11 +312,11 @@ static cudaError_t batch_enqueue(turret_batch *b, int p) {
         for (int cyc = 1; cyc <= C; ++cyc) {
             const int dst = (cyc % 2 == 1) ? HSEL_HB : HSEL_HL;
             const int fin = (cyc == C && dst != HSEL_HL) ? HSEL_HL : -1;
-            CE(launch_batch_cycle(R, tab(T_CYC), n, b->total[T_CYC], src, dst, fin, cyc == C, cyc - 1, 1, b->side));
+            CE(launch_batch_cycle(R, tab(T_CYC), n, p, b->total[T_CYC], src, dst, fin, cyc == C, cyc - 1, 1, b->side));
             src = dst;
         }
     }
-    CE(launch_batch_spread(R, tab(T_SP), n, b->total[T_SP], b->side));
+    CE(launch_batch_spread(R, tab(T_SP), n, p, b->total[T_SP], b->side));
     CE(cudaStreamWaitEvent(b->side, b->ev_red_done, 0));
     CE(cudaEventRecord(b->ev_join, b->side));
     CE(cudaStreamWaitEvent(b->stream, b->ev_join, 0));

@@ -9,11 +9,13 @@
 //                X_k = C_m + M^T Xb_k, n_k = M^T nb_k, U_k = v + w x (X_k - C_m)
 //                and each marker's 4x4x4 Peskin stencil (Sec. 2.2) in
 //                support-box coordinates.
-//   k_interp0_rows : I[u](X_k) = sum_x u(x) W(x - X_k) for u* and sigma, one
-//                warp per marker, two stencil cells per lane, xor-shuffle sums
-//                (deterministic); forms dS sigma.n and its moment about C_m
-//                for the surface force (Sec. 2.2 end) and row k of the
-//                interaction matrix A of the IBM cycles; one block per marker.
+//   k_rows     : row k of the interaction matrix A of the IBM cycles, one block
+//                per marker (k_interp0_tiles: rows and interpolation by tiles,
+//                for batches).
+//   k_interp   : I[u](X_k) = sum_x u(x) W(x - X_k) for u* and sigma, one warp per
+//                marker, two stencil cells per lane, xor-shuffle sums
+//                (deterministic); forms dS sigma.n and its moment about C_m for
+//                the surface force (Sec. 2.2 end).
 //   k_cycle    : one IBM cycle as h <- h + r0 - A h (a sparse product, one
 //                warp per marker), equal to spreading h and interpolating
 //                u* + S h without touching the grid.
@@ -47,11 +49,21 @@ constexpr int PM_THREADS = MARKER_SEG;
 __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, const BoxGeom &box, DevState *st,
                                          int slot, int advance, const MarkerArrays &m, int blk) {
     __shared__ BodySlot S;  // the body at the markers' time level
-    __shared__ double s_F[3], s_T[3], s_src[3], s_sb[3], s_wb[3], s_mid[9], s_dn[9];
+    __shared__ double s_F[3], s_T[3], s_src[3], s_sb[3], s_wb[3], s_mid[9];
     __shared__ float f_d[9], f_v[3], f_w[3], f_cf[3];
     __shared__ int i_ci[3], i_lo[3];
     const int tid = threadIdx.x;
     const int so = advance ? (slot ^ 1) : slot;  // slot of the markers' time level
+    // the body-frame marker is fetched beside the rigid-body update
+    const int nm = bc.nm;
+    const int k = blk * PM_THREADS + tid;
+    float xb[3] = {0.0f, 0.0f, 0.0f}, nbv[3] = {0.0f, 0.0f, 0.0f};
+    if (k < nm)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            xb[a] = __ldg(m.Xb + a * nm + k);
+            nbv[a] = __ldg(m.nb + a * nm + k);
+        }
     if (tid < 32) {
         const int lane = tid;
         {
@@ -94,10 +106,9 @@ __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, con
             const int i = lane / 3, a = lane % 3, a1 = (a + 1) % 3, a2 = (a + 2) % 3;
             if (lane < 9) s_mid[lane] = S.d[lane] + 0.5 * (S.w[a1] * S.d[3 * i + a2] - S.w[a2] * S.d[3 * i + a1]);
             __syncwarp();
-            if (lane < 9) s_dn[lane] = S.d[lane] + (S.w[a1] * s_mid[3 * i + a2] - S.w[a2] * s_mid[3 * i + a1]);
+            if (lane < 9) S.d[lane] += S.w[a1] * s_mid[3 * i + a2] - S.w[a2] * s_mid[3 * i + a1];
             __syncwarp();
             if (lane == 0) {
-                for (int k = 0; k < 9; ++k) S.d[k] = s_dn[k];
                 if (bc.renorm) {  // modified Gram-Schmidt of d_0, d_1, d_2
                     for (int q = 0; q < 3; ++q) {
                         for (int j = 0; j < q; ++j) {
@@ -125,27 +136,27 @@ __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, con
                         reseed = (ring == 0) ? g.nz - 1 : ring - 1;  // new logical top plane
                     }
                 }
-                const int nn[3] = {g.nx, g.ny, g.nz};
-                const bool pp[3] = {g.bc_x == BC_PERIODIC, g.bc_y == BC_PERIODIC, g.bc_bottom == BC_PERIODIC};
-                for (int c = 0; c < 3; ++c) {
-                    const double C = S.r[c] - (double)S.origin[c];
-                    const double fl = floor(C);
-                    S.Ci[c] = (int)fl;
-                    S.Cf[c] = C - fl;
-                    S.box_lo[c] = (int)fl - bc.rc - 2;
-                    int lw = S.box_lo[c];
-                    if (pp[c]) {
-                        lw %= nn[c];
-                        if (lw < 0) lw += nn[c];
-                    }
-                    S.box_lo_w[c] = lw;
-                }
                 S.ring = ring;
                 S.reseed = reseed;
                 S.step += 1;
             }
             __syncwarp();
-            if (blk == 0 && lane < 8) st->pr.slip[lane] = 0u;
+            if (lane < 3) {
+                const int nn = lane == 0 ? g.nx : (lane == 1 ? g.ny : g.nz);
+                const bool pp = (lane == 0 ? g.bc_x : (lane == 1 ? g.bc_y : g.bc_bottom)) == BC_PERIODIC;
+                const double C = S.r[lane] - (double)S.origin[lane];
+                const double fl = floor(C);
+                S.Ci[lane] = (int)fl;
+                S.Cf[lane] = C - fl;
+                int lw = (int)fl - bc.rc - 2;
+                S.box_lo[lane] = lw;
+                if (pp) {
+                    lw %= nn;
+                    if (lw < 0) lw += nn;
+                }
+                S.box_lo_w[lane] = lw;
+            }
+            __syncwarp();
             if (blk == 0) {
                 int *gdst = reinterpret_cast<int *>(&st->s[so]);
                 const int *ssrc = reinterpret_cast<const int *>(&S);
@@ -191,17 +202,13 @@ __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, con
     }
     __syncthreads();
     // ---- markers ---------------------------------------------------------------
-    const int nm = bc.nm;
     const int n[3] = {g.nx, g.ny, g.nz};
     const bool per[3] = {g.bc_x == BC_PERIODIC, g.bc_y == BC_PERIODIC, g.bc_bottom == BC_PERIODIC};
     const int B[3] = {box.Bx, box.By, box.Bz};
-    const int k = blk * PM_THREADS + tid;
     int bbv[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff};  // no marker: neutral for the minimum
     int bbmax[3] = {-1, -1, -1};
     if (k < nm) {
         bool bad = false;
-        const float xb[3] = {m.Xb[k], m.Xb[nm + k], m.Xb[2 * nm + k]};
-        const float nbv[3] = {m.nb[k], m.nb[nm + k], m.nb[2 * nm + k]};
         float arm[3], nn[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -364,6 +371,16 @@ __device__ __forceinline__ void interp_marker_warp(const BoxGeom &box, int nm, c
         d0 = c0, d1 = c1, v0 = w0, v1 = w1;
     }
     const size_t N = box.nbox;
+    // what the sums are combined with, fetched beside the stencil (the same
+    // address in every lane)
+    const float dS = m.dS[k], dA = fe == 0 ? m.dSo[k] : dS;  // dA: area of the surface the stress is taken on
+    float Uk[3], nk[3], rk3[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        Uk[c] = m.U[c * nm + k];
+        nk[c] = m.n[c * nm + k];
+        rk3[c] = m.arm[c * nm + k];
+    }
     float acc[10];
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[c] = w0 * ba.u[c * N + c0] + w1 * ba.u[c * N + c1];
@@ -376,9 +393,8 @@ __device__ __forceinline__ void interp_marker_warp(const BoxGeom &box, int nm, c
         for (int q = 16; q > 0; q >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], q);
     if (lane == 0) {
         // l = 0: h_k = U_k - I[u*](X_k); traction dS sigma(X_k) n_k and its moment
-        const float dS = m.dS[k];
         for (int c = 0; c < 3; ++c) {
-            const float h = m.U[c * nm + k] - acc[c];
+            const float h = Uk[c] - acc[c];
             m.r0[c * nm + k] = h;
             if (!warm) {
                 m.hl[c * nm + k] = h;
@@ -386,13 +402,12 @@ __device__ __forceinline__ void interp_marker_warp(const BoxGeom &box, int nm, c
             }
         }
         const float sxx = acc[3], syy = acc[4], szz = acc[5], sxy = acc[6], sxz = acc[7], syz = acc[8];
-        const float nx = m.n[k], ny = m.n[nm + k], nz = m.n[2 * nm + k];
-        const float dA = fe == 0 ? m.dSo[k] : dS;  // area of the surface the stress is taken on
+        const float nx = nk[0], ny = nk[1], nz = nk[2];
         const float f0 = dA * (sxx * nx + sxy * ny + sxz * nz);
         const float f1 = dA * (sxy * nx + syy * ny + syz * nz);
         const float f2 = dA * (sxz * nx + syz * ny + szz * nz);
         const float off = fe == 0 ? F_OFFSET : 0.0f;
-        const float r0 = m.arm[k] + off * nx, r1 = m.arm[nm + k] + off * ny, r2 = m.arm[2 * nm + k] + off * nz;
+        const float r0 = rk3[0] + off * nx, r1 = rk3[1] + off * ny, r2 = rk3[2] + off * nz;
         m.ft[k] = f0;
         m.ft[nm + k] = f1;
         m.ft[2 * nm + k] = f2;
@@ -409,17 +424,14 @@ __device__ __forceinline__ void interp_marker_warp(const BoxGeom &box, int nm, c
 
 
 template <int NT>
-__device__ __forceinline__ void interp0_block(const BoxGeom &box, int nm, const MarkerArrays &m, const BoxArrays &ba,
-                                              const int *__restrict__ wlist, const int *__restrict__ wcount,
-                                              int cap, DevState *st, int k, int warm) {
+__device__ __forceinline__ void rows_block(const BoxGeom &box, const MarkerArrays &m, const int *__restrict__ wlist,
+                                           const int *__restrict__ wcount, int cap, DevState *st, int k) {
     constexpr int NW = NT / 32;
     constexpr int CU = 4;
     __shared__ int wc[CU][NW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const MRec rk = m.rec[k];
     const int bx = rk.base & 1023, by = (rk.base >> 10) & 1023, bz = (rk.base >> 20) & 1023;
-    if (warp == 0) interp_marker_warp(box, nm, m, ba, k, rk, lane, warm);
-    // ---- row k of A -----------------------------------------------------------
     const int tile = (bx / TILE) + box.tx * ((by / TILE) + box.ty * (bz / TILE));
     const int cnt = wcount[tile];
     const int *list = wlist + (size_t)tile * cap;
@@ -488,11 +500,24 @@ __device__ __forceinline__ void interp0_block(const BoxGeom &box, int nm, const 
 // collide+stream for the latency of their loads, so idle threads are costly.
 constexpr int ROWS_MARKER_THREADS = 64;
 
-__global__ void __launch_bounds__(ROWS_MARKER_THREADS) k_interp0_rows(BoxGeom box, int nm, MarkerArrays m,
-                                                                      BoxArrays ba, const int *__restrict__ wlist,
-                                                                      const int *__restrict__ wcount, int cap,
-                                                                      DevState *st, int warm) {
-    interp0_block<ROWS_MARKER_THREADS>(box, nm, m, ba, wlist, wcount, cap, st, blockIdx.x, warm);
+__global__ void __launch_bounds__(ROWS_MARKER_THREADS) k_rows(BoxGeom box, MarkerArrays m, const int *__restrict__ wlist,
+                                                              const int *__restrict__ wcount, int cap, DevState *st) {
+    rows_block<ROWS_MARKER_THREADS>(box, m, wlist, wcount, cap, st, blockIdx.x);
+}
+
+// One warp per marker, small blocks (as above).  It used to share a launch
+// with the rows of A: 10 us of a 41 us step of a 32x32x64 window, where the
+// rows now are built beside the near region's launch and the moments.
+constexpr int INTERP_THREADS = 64;
+
+__global__ void __launch_bounds__(INTERP_THREADS) k_interp(BoxGeom box, int nm, MarkerArrays m, BoxArrays ba,
+                                                           DevState *st, int warm) {
+    // the previous step's cycles have read their slips; this step's follow
+    if (blockIdx.x == 0 && threadIdx.x < 8) st->pr.slip[threadIdx.x] = 0u;
+    const int k = blockIdx.x * (INTERP_THREADS / 32) + (threadIdx.x >> 5);
+    if (k >= nm) return;
+    const MRec rk = m.rec[k];
+    interp_marker_warp(box, nm, m, ba, k, rk, threadIdx.x & 31, warm);
 }
 
 // The same step l = 0 and rows of A with one block per TILE^3 tile of the
@@ -509,6 +534,7 @@ __device__ __forceinline__ void interp0_tile_block(const BoxGeom &box, int nm, c
                                                    const BoxArrays &ba, const int *__restrict__ tile_list,
                                                    const int *__restrict__ tile_count, int cap, DevState *st,
                                                    int tile, int warm) {
+    if (tile == 0 && threadIdx.x < 8) st->pr.slip[threadIdx.x] = 0u;  // as k_interp
     __shared__ int kb[IT_MAXB], klen[IT_MAXB];
     __shared__ int wc[ROWS_WARPS];
     __shared__ int nbased;
@@ -626,13 +652,6 @@ __device__ __forceinline__ void interp0_tile_block(const BoxGeom &box, int nm, c
         m.alen[kb[q]] = len < ROWCAP ? len : ROWCAP;
         if (len > ROWCAP) atomicCAS(&st->status, 0, STAT_OVERFLOW);
     }
-}
-
-__global__ void __launch_bounds__(ROWS_THREADS) k_interp0_tiles(BoxGeom box, int nm, MarkerArrays m, BoxArrays ba,
-                                                                 const int *__restrict__ tile_list,
-                                                                 const int *__restrict__ tile_count, int cap,
-                                                                 DevState *st, int warm) {
-    interp0_tile_block(box, nm, m, ba, tile_list, tile_count, cap, st, blockIdx.x, warm);
 }
 
 // One cycle of steps l = 1..4 (Sec. 2.2) in matrix form:
@@ -930,15 +949,16 @@ __global__ void __launch_bounds__(PM_THREADS) k_batch_particle_markers(const Run
                                                                         int p) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
-    pm_block(R.g, R.bc, R.box, R.st, p, 1, R.m, lb);
+    pm_block(R.g, R.bc, R.box, R.st, p, 1, R.m[p ^ 1], lb);
 }
 
 __global__ void __launch_bounds__(ROWS_THREADS) k_batch_interp0_tiles(const RunDesc *__restrict__ runs,
                                                                       const int *__restrict__ prefix, int nruns,
-                                                                      int warm) {
+                                                                      int p, int warm) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
-    interp0_tile_block(R.box, R.nm, R.m, R.ba, R.tile_list, R.tile_count, R.cap, R.st, lb, warm);
+    const MarkerArrays &m = R.m[p ^ 1];
+    interp0_tile_block(R.box, R.nm, m, R.ba, m.tile_list, m.tile_count, R.cap, R.st, lb, warm);
 }
 
 __device__ __forceinline__ float *hsel(const MarkerArrays &m, int sel) {
@@ -946,25 +966,27 @@ __device__ __forceinline__ float *hsel(const MarkerArrays &m, int sel) {
 }
 
 __global__ void __launch_bounds__(32 * INTERP_WARPS) k_batch_cycle(const RunDesc *__restrict__ runs,
-                                                                   const int *__restrict__ prefix, int nruns,
+                                                                   const int *__restrict__ prefix, int nruns, int p,
                                                                    int sel_in, int sel_out, int sel_final, int last,
                                                                    int cyc, int adaptive) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
-    cycle_block(R.nm, R.m, hsel(R.m, sel_in), hsel(R.m, sel_out), sel_final >= 0 ? hsel(R.m, sel_final) : nullptr,
-                last, lb, R.st, cyc, adaptive, R.bc.slip_eps);
+    const MarkerArrays &m = R.m[p ^ 1];
+    cycle_block(R.nm, m, hsel(m, sel_in), hsel(m, sel_out), sel_final >= 0 ? hsel(m, sel_final) : nullptr, last, lb, R.st,
+                cyc, adaptive, R.bc.slip_eps);
 }
 
 __global__ void __launch_bounds__(288) k_batch_reduce_ft(const RunDesc *__restrict__ runs, int slot) {
     const RunDesc &R = runs[blockIdx.x];
-    reduce_block(R.nm, R.m.ft, R.st, slot, R.bc.predictor, R.bc.pred_opts, R.bc.resid_theta, R.bc.log, R.bc.log_cap);
+    reduce_block(R.nm, R.m[slot].ft, R.st, slot, R.bc.predictor, R.bc.pred_opts, R.bc.resid_theta, R.bc.log, R.bc.log_cap);
 }
 
 __global__ void __launch_bounds__(SPREAD_THREADS) k_batch_spread(const RunDesc *__restrict__ runs,
-                                                                 const int *__restrict__ prefix, int nruns) {
+                                                                 const int *__restrict__ prefix, int nruns, int p) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
-    spread_block(R.box, R.m.rec, R.ba, R.tile_list, R.tile_count, R.cap, lb);
+    const MarkerArrays &m = R.m[p ^ 1];
+    spread_block(R.box, m.rec, R.ba, m.tile_list, m.tile_count, R.cap, lb);
 }
 
 // ---------------------------------------------------------------------------
@@ -974,22 +996,49 @@ cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const Bo
     return cudaGetLastError();
 }
 
-cudaError_t launch_interp0(const BoxGeom &box, int nm, MarkerArrays m, BoxArrays ba, const int *tile_list,
-                           const int *tile_count, int cap, DevState *st, int warm, cudaStream_t s, bool by_tile) {
+cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, cudaStream_t s) {
     const int ntiles = box.tx * box.ty * box.tz;  // list 1 (rows of A) follows list 0
-    if (by_tile)
-        k_interp0_tiles<<<ntiles, ROWS_THREADS, 0, s>>>(box, nm, m, ba, tile_list, tile_count, cap, st, warm);
-    else
-        k_interp0_rows<<<nm, ROWS_MARKER_THREADS, 0, s>>>(box, nm, m, ba, tile_list + (size_t)ntiles * cap,
-                                                   tile_count + ntiles, cap, st, warm);
+    k_rows<<<nm, ROWS_MARKER_THREADS, 0, s>>>(box, m, m.tile_list + (size_t)ntiles * cap, m.tile_count + ntiles, cap, st);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cycle(int nm, MarkerArrays m, const float *h_in, float *h_out, float *h_final, int last,
-                         DevState *st, int cyc, int adaptive, float eps, cudaStream_t s) {
+cudaError_t launch_interp0(const BoxGeom &box, int nm, const MarkerArrays &m, const BoxArrays &ba, DevState *st, int warm,
+                           cudaStream_t s) {
+    constexpr int per = INTERP_THREADS / 32;
+    k_interp<<<(nm + per - 1) / per, INTERP_THREADS, 0, s>>>(box, nm, m, ba, st, warm);
+    return cudaGetLastError();
+}
+
+static cudaError_t launch_cycle(int nm, const MarkerArrays &m, const float *h_in, float *h_out, float *h_final, int last,
+                                DevState *st, int cyc, int adaptive, float eps, cudaStream_t s) {
     k_cycle<<<(nm + INTERP_WARPS - 1) / INTERP_WARPS, 32 * INTERP_WARPS, 0, s>>>(nm, m, h_in, h_out, h_final, last,
                                                                                  st, cyc, adaptive, eps);
     return cudaGetLastError();
+}
+
+cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (!warm) {
+        // the paper's cycles: h^0 = r0, then cycles 1 .. n-1 alternating so
+        // that the last one writes hl
+        const float *src = m.r0;
+        for (int cyc = 1; cyc <= C && e == cudaSuccess; ++cyc) {
+            float *dst = ((C - cyc) % 2 == 0) ? m.hl : m.hb;
+            e = launch_cycle(nm, m, src, dst, nullptr, cyc == C, st, cyc - 1, 0, 0.0f, s);
+            src = dst;
+        }
+    } else {
+        // predictor modes: up to n cycles from the previous h (in hl), each
+        // skipped once the slip is below the tolerance; hl ends with the result
+        const float *src = m.hl;
+        for (int cyc = 1; cyc <= C && e == cudaSuccess; ++cyc) {
+            float *dst = (cyc % 2 == 1) ? m.hb : m.hl;
+            float *fin = (cyc == C && dst != m.hl) ? m.hl : nullptr;
+            e = launch_cycle(nm, m, src, dst, fin, cyc == C, st, cyc - 1, 1, eps, s);
+            src = dst;
+        }
+    }
+    return e;
 }
 
 cudaError_t launch_reduce_ft(int nm, MarkerArrays m, DevState *st, int slot, const BodyConst &bc, cudaStream_t s) {
@@ -997,10 +1046,8 @@ cudaError_t launch_reduce_ft(int nm, MarkerArrays m, DevState *st, int slot, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_spread(const BoxGeom &box, int nm, MarkerArrays m, BoxArrays ba, const int *tile_list,
-                          const int *tile_count, int cap, cudaStream_t s) {
-    (void)nm;
-    k_spread<<<box.tx * box.ty * box.tz, SPREAD_THREADS, 0, s>>>(box, m.rec, ba, tile_list, tile_count, cap);
+cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxArrays &ba, int cap, cudaStream_t s) {
+    k_spread<<<box.tx * box.ty * box.tz, SPREAD_THREADS, 0, s>>>(box, m.rec, ba, m.tile_list, m.tile_count, cap);
     return cudaGetLastError();
 }
 
@@ -1015,15 +1062,15 @@ cudaError_t launch_batch_particle_markers(const RunDesc *runs, const int *prefix
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nruns, int nblocks, int warm,
+cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int warm,
                                  cudaStream_t s) {
-    k_batch_interp0_tiles<<<nblocks, ROWS_THREADS, 0, s>>>(runs, prefix, nruns, warm);
+    k_batch_interp0_tiles<<<nblocks, ROWS_THREADS, 0, s>>>(runs, prefix, nruns, p, warm);
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns, int nblocks, int sel_in,
+cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int sel_in,
                                int sel_out, int sel_final, int last, int cyc, int adaptive, cudaStream_t s) {
-    k_batch_cycle<<<nblocks, 32 * INTERP_WARPS, 0, s>>>(runs, prefix, nruns, sel_in, sel_out, sel_final, last, cyc,
+    k_batch_cycle<<<nblocks, 32 * INTERP_WARPS, 0, s>>>(runs, prefix, nruns, p, sel_in, sel_out, sel_final, last, cyc,
                                                         adaptive);
     return cudaGetLastError();
 }
@@ -1033,8 +1080,8 @@ cudaError_t launch_batch_reduce_ft(const RunDesc *runs, int nruns, int slot, cud
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_spread(const RunDesc *runs, const int *prefix, int nruns, int nblocks, cudaStream_t s) {
-    k_batch_spread<<<nblocks, SPREAD_THREADS, 0, s>>>(runs, prefix, nruns);
+cudaError_t launch_batch_spread(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s) {
+    k_batch_spread<<<nblocks, SPREAD_THREADS, 0, s>>>(runs, prefix, nruns, p);
     return cudaGetLastError();
 }
 

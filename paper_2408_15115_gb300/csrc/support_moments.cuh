@@ -1,139 +1,138 @@
 // support_moments.cuh -- block code of the support-box moments and of the
-// marker binning that feeds the immersed-boundary transfers (one launch in the
-// single-run and the batched steps); the pull and moment code is the
+// marker binning that feeds the immersed-boundary transfers (two launches on
+// two streams in the single-run step, one launch in the batched step); the pull and moment code is the
 // collide+stream's (lbm_cell.cuh), so both see identical populations.
 #pragma once
 #include "lbm_cell.cuh"
 
 namespace turret {
 
-// K2 + binning, one launch.  Blocks [0, nmom): u* and the stress of Eq. 10,
-// sigma = -p I + (1/(2 tau) - 1) P1 with p = c_s^2 (rho - 1), at every
-// support-box cell, from f(t+1) pulled from the post-collision buffer (box
-// cells outside a closed face get zeros; cells no stencil reads, the outer
-// layer among them, are skipped).  Blocks [nmom, nmom + ntiles): for
-// one TILE^3 tile of the box, two lists in marker order (ordered compaction
-// with warp ballots; no atomics): list 0, the markers whose 4x4x4 stencil
-// overlaps the tile (spreading); list 1, those whose stencil overlaps the
-// stencil of any marker based in the tile (rows of A).
 constexpr int MB_THREADS = 128;
 
-template <int ST>
-__device__ __forceinline__ void mb_block(const Geom &g, const typename Codec<ST>::T *__restrict__ src,
-                                         const float *__restrict__ utop_in, const DevState *__restrict__ st, int slot,
-                                         const BoxGeom &box, const BoxArrays &ba, int nmom, int nm,
-                                         const int *__restrict__ mbase, const int *__restrict__ mseg,
-                                         int *__restrict__ tile_list, int *__restrict__ tile_count, int cap,
-                                         DevState *stw, float rmin,
-                                         float rmax, int blk) {
-    if (blk >= nmom) {
-        constexpr int NW = MB_THREADS / 32;
-        const int tile = blk - nmom;
-        const int tx = tile % box.tx, ty = (tile / box.tx) % box.ty, tz = tile / (box.tx * box.ty);
-        const int t0[3] = {TILE * tx, TILE * ty, TILE * tz};
-        {
-            // Both lists hold markers whose stencil base b lies in [t0 - 3, t0 + 6]
-            // per axis, i.e. whose position X lies in [t0 - 2, t0 + 8).  Markers
-            // sit at rmin <= |X - C| <= rmax (body-frame radii, up to rounding):
-            // a region outside that shell has no candidates.
-            const BodySlot &S = st->s[slot];
-            float dmin2 = 0.0f, dmax2 = 0.0f;
+// Tile lists.  For one TILE^3 tile of the support box, two lists in marker
+// order (ordered compaction with warp ballots; no atomics): list 0, the
+// markers whose 4x4x4 stencil overlaps the tile (spreading); list 1, those
+// whose stencil overlaps the stencil of any marker based in the tile (rows of
+// A).  Reads the markers and the window slot only.
+__device__ __forceinline__ void bin_block(const DevState *__restrict__ st, int slot, const BoxGeom &box, int nm,
+                                          const int *__restrict__ mbase, const int *__restrict__ mseg,
+                                          int *__restrict__ tile_list, int *__restrict__ tile_count, int cap,
+                                          DevState *stw, float rmin, float rmax, int tile) {
+    constexpr int NW = MB_THREADS / 32;
+    const int tx = tile % box.tx, ty = (tile / box.tx) % box.ty, tz = tile / (box.tx * box.ty);
+    const int t0[3] = {TILE * tx, TILE * ty, TILE * tz};
+    {
+        // Both lists hold markers whose stencil base b lies in [t0 - 3, t0 + 6]
+        // per axis, i.e. whose position X lies in [t0 - 2, t0 + 8).  Markers
+        // sit at rmin <= |X - C| <= rmax (body-frame radii, up to rounding):
+        // a region outside that shell has no candidates.
+        const BodySlot &S = st->s[slot];
+        float dmin2 = 0.0f, dmax2 = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float c = (float)(S.Ci[a] - S.box_lo[a]) + (float)S.Cf[a];
+            const float lo = (float)(t0[a] - 2), hi = (float)(t0[a] + 8);
+            const float dn = fmaxf(fmaxf(lo - c, c - hi), 0.0f);
+            const float dx = fmaxf(fabsf(c - lo), fabsf(c - hi));
+            dmin2 += dn * dn;
+            dmax2 += dx * dx;
+        }
+        const float margin = 0.25f;
+        if (dmin2 > (rmax + margin) * (rmax + margin) ||
+            (rmin > margin && dmax2 < (rmin - margin) * (rmin - margin))) {
+            if (threadIdx.x < 2) tile_count[threadIdx.x * (box.tx * box.ty * box.tz) + tile] = 0;
+            return;
+        }
+    }
+    // CU chunks of MB_THREADS markers per pass: their loads are issued
+    // together and their hits compacted chunk after chunk (marker order);
+    // one barrier per pass, the warp counts alternating between two buffers
+    constexpr int CU = 4;
+    __shared__ int wcount[2][CU][2][NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nseg = (nm + MARKER_SEG - 1) / MARKER_SEG;
+    int tot[2] = {0, 0};  // identical in every thread
+    int par = 0;
+    for (int group = 0; group < nm; group += CU * MB_THREADS) {
+        // skip chunks whose segments' stencil bases all miss [t0 - 3, t0 + 6];
+        // the test is the same in every thread, so a group with no chunk
+        // left is skipped whole, barrier included
+        bool reach[CU], any = false;
+#pragma unroll
+        for (int u = 0; u < CU; ++u) {
+            const int chunk = group + u * MB_THREADS;
+            reach[u] = false;
+            for (int sg = chunk / MARKER_SEG; sg < nseg && sg * MARKER_SEG < chunk + MB_THREADS; ++sg) {
+                const int *bb = mseg + 6 * sg;
+                bool in = true;
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    in = in && __ldg(bb + 3 + a) + 3 >= t0[a] && __ldg(bb + a) <= t0[a] + TILE + 2;
+                reach[u] = reach[u] || in;
+            }
+            any = any || reach[u];
+        }
+        if (!any) continue;
+        int pb[CU];
+#pragma unroll
+        for (int u = 0; u < CU; ++u) {
+            const int k = group + u * MB_THREADS + tid;
+            pb[u] = (reach[u] && k < nm) ? __ldg(mbase + k) : -1;  // culled chunks load nothing
+        }
+        unsigned bal[CU][2];
+        bool hit[CU][2];
+#pragma unroll
+        for (int u = 0; u < CU; ++u) {
+            hit[u][0] = hit[u][1] = pb[u] >= 0;
+            const int b[3] = {pb[u] & 1023, (pb[u] >> 10) & 1023, (pb[u] >> 20) & 1023};
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const float c = (float)(S.Ci[a] - S.box_lo[a]) + (float)S.Cf[a];
-                const float lo = (float)(t0[a] - 2), hi = (float)(t0[a] + 8);
-                const float dn = fmaxf(fmaxf(lo - c, c - hi), 0.0f);
-                const float dx = fmaxf(fabsf(c - lo), fabsf(c - hi));
-                dmin2 += dn * dn;
-                dmax2 += dx * dx;
+                const bool lo = b[a] + 3 >= t0[a];
+                hit[u][0] = hit[u][0] && lo && (b[a] <= t0[a] + TILE - 1);  // stencil overlaps the tile
+                hit[u][1] = hit[u][1] && lo && (b[a] <= t0[a] + TILE + 2);  // ... or a stencil based in it
             }
-            const float margin = 0.25f;
-            if (dmin2 > (rmax + margin) * (rmax + margin) ||
-                (rmin > margin && dmax2 < (rmin - margin) * (rmin - margin))) {
-                if (threadIdx.x < 2) tile_count[threadIdx.x * (box.tx * box.ty * box.tz) + tile] = 0;
-                return;
+#pragma unroll
+            for (int l = 0; l < 2; ++l) {
+                bal[u][l] = __ballot_sync(0xffffffffu, hit[u][l]);
+                if (lane == 0) wcount[par][u][l][warp] = __popc(bal[u][l]);
             }
         }
-        // CU chunks of MB_THREADS markers per pass: their loads are issued
-        // together and their hits compacted chunk after chunk (marker order);
-        // one barrier per pass, the warp counts alternating between two buffers
-        constexpr int CU = 4;
-        __shared__ int wcount[2][CU][2][NW];
-        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-        const int nseg = (nm + MARKER_SEG - 1) / MARKER_SEG;
-        int tot[2] = {0, 0};  // identical in every thread
-        int par = 0;
-        for (int group = 0; group < nm; group += CU * MB_THREADS) {
-            // skip chunks whose segments' stencil bases all miss [t0 - 3, t0 + 6];
-            // the test is the same in every thread, so a group with no chunk
-            // left is skipped whole, barrier included
-            bool reach[CU], any = false;
+        __syncthreads();
 #pragma unroll
-            for (int u = 0; u < CU; ++u) {
-                const int chunk = group + u * MB_THREADS;
-                reach[u] = false;
-                for (int sg = chunk / MARKER_SEG; sg < nseg && sg * MARKER_SEG < chunk + MB_THREADS; ++sg) {
-                    const int *bb = mseg + 6 * sg;
-                    bool in = true;
+        for (int u = 0; u < CU; ++u)
 #pragma unroll
-                    for (int a = 0; a < 3; ++a)
-                        in = in && __ldg(bb + 3 + a) + 3 >= t0[a] && __ldg(bb + a) <= t0[a] + TILE + 2;
-                    reach[u] = reach[u] || in;
+            for (int l = 0; l < 2; ++l) {
+                int off = tot[l], sum = 0;
+                for (int w = 0; w < NW; ++w) {
+                    const int c = wcount[par][u][l][w];
+                    off += (w < warp) ? c : 0;
+                    sum += c;
                 }
-                any = any || reach[u];
+                if (hit[u][l]) {
+                    const int pos = off + __popc(bal[u][l] & ((1u << lane) - 1u));
+                    if (pos < cap)
+                        tile_list[((size_t)l * (box.tx * box.ty * box.tz) + tile) * cap + pos] =
+                            group + u * MB_THREADS + tid;
+                }
+                tot[l] += sum;
             }
-            if (!any) continue;
-            int pb[CU];
-#pragma unroll
-            for (int u = 0; u < CU; ++u) {
-                const int k = group + u * MB_THREADS + tid;
-                pb[u] = (reach[u] && k < nm) ? __ldg(mbase + k) : -1;  // culled chunks load nothing
-            }
-            unsigned bal[CU][2];
-            bool hit[CU][2];
-#pragma unroll
-            for (int u = 0; u < CU; ++u) {
-                hit[u][0] = hit[u][1] = pb[u] >= 0;
-                const int b[3] = {pb[u] & 1023, (pb[u] >> 10) & 1023, (pb[u] >> 20) & 1023};
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const bool lo = b[a] + 3 >= t0[a];
-                    hit[u][0] = hit[u][0] && lo && (b[a] <= t0[a] + TILE - 1);  // stencil overlaps the tile
-                    hit[u][1] = hit[u][1] && lo && (b[a] <= t0[a] + TILE + 2);  // ... or a stencil based in it
-                }
-#pragma unroll
-                for (int l = 0; l < 2; ++l) {
-                    bal[u][l] = __ballot_sync(0xffffffffu, hit[u][l]);
-                    if (lane == 0) wcount[par][u][l][warp] = __popc(bal[u][l]);
-                }
-            }
-            __syncthreads();
-#pragma unroll
-            for (int u = 0; u < CU; ++u)
-#pragma unroll
-                for (int l = 0; l < 2; ++l) {
-                    int off = tot[l], sum = 0;
-                    for (int w = 0; w < NW; ++w) {
-                        const int c = wcount[par][u][l][w];
-                        off += (w < warp) ? c : 0;
-                        sum += c;
-                    }
-                    if (hit[u][l]) {
-                        const int pos = off + __popc(bal[u][l] & ((1u << lane) - 1u));
-                        if (pos < cap)
-                            tile_list[((size_t)l * (box.tx * box.ty * box.tz) + tile) * cap + pos] =
-                                group + u * MB_THREADS + tid;
-                    }
-                    tot[l] += sum;
-                }
-            par ^= 1;
-        }
-        if (tid < 2) {
-            tile_count[tid * (box.tx * box.ty * box.tz) + tile] = tot[tid] < cap ? tot[tid] : cap;
-            if (tot[tid] > cap) atomicCAS(&stw->status, 0, STAT_OVERFLOW);
-        }
-        return;
+        par ^= 1;
     }
+    if (tid < 2) {
+        tile_count[tid * (box.tx * box.ty * box.tz) + tile] = tot[tid] < cap ? tot[tid] : cap;
+        if (tot[tid] > cap) atomicCAS(&stw->status, 0, STAT_OVERFLOW);
+    }
+}
+
+// K2: u* and the stress of Eq. 10, sigma = -p I + (1/(2 tau) - 1) P1 with p =
+// c_s^2 (rho - 1), at every support-box cell, from f(t+1) pulled from the
+// post-collision buffer (box cells outside a closed face get zeros; cells no
+// stencil reads, the outer layer among them, are skipped).
+template <int ST>
+__device__ __forceinline__ void moments_block(const Geom &g, const typename Codec<ST>::T *__restrict__ src,
+                                              const float *__restrict__ utop_in, const DevState *__restrict__ st,
+                                              int slot, const BoxGeom &box, const BoxArrays &ba, float rmin, float rmax,
+                                              int blk) {
     const long long b = (long long)blk * blockDim.x + threadIdx.x;
     if (b >= box.nbox) return;
     const int bx = (int)(b % box.Bx);

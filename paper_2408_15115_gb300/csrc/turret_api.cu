@@ -6,17 +6,18 @@
 // Step graph (time t -> t+1, parity p = t % 2), when the particle's near
 // region fits the window:
 //
-//   caller stream: --fork--> collide+stream, far cells ------------------> join
-//   side stream  :       \-> collide+stream, near cells -+-> support moments
-//                           + tile lists -> interpolation + rows of A
-//                           -> (h <- h + r0 - A h) x (n-1) -> spread h_imm(t+1) --^
-//   aux stream   :       \-> [prediction] -> particle update + markers -/
-//                                                    ... -> F, T (FP64) ----^
+//   caller stream: --fork--> collide+stream, far cells --------------------> join
+//   aux stream   :       \-> [prediction] -> particle update + markers -> tile
+//                           lists -> rows of A              ... -> F, T (FP64) ^
+//   side stream  :       \-> collide+stream, near cells -> support moments
+//                           -> interpolation -> (h <- h + r0 - A h) x (n-1)
+//                           -> spread h_imm(t+1) -------------------------------^
 //
-// The near region (support box grown by two cells) contains every cell the
-// next support-box pull reads, so the immersed-boundary chain only waits for
-// the small near launch and runs concurrently with the bulk of the window
-// (the side stream has the highest priority).
+// The near region (the support box) contains every cell the next support-box
+// pull reads, so the immersed-boundary chain only waits for the small near
+// launch and runs concurrently with the bulk of the window (the side stream
+// has the highest priority).  Groups of steps are captured as one graph in
+// which the chain also overlaps the next step (enqueue_steps_pipelined).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -116,10 +117,7 @@ static void release(turret_ctx *c) {
     if (c->aux) cudaStreamDestroy(c->aux);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
-    if (c->ev_red) cudaEventDestroy(c->ev_red);
-    if (c->ev_red_done) cudaEventDestroy(c->ev_red_done);
-    if (c->ev_pred) cudaEventDestroy(c->ev_pred);
-    cudaEvent_t *xs[6] = {c->ev_far, c->ev_near, c->ev_pm, c->ev_ired, c->ev_redd, c->ev_spread};
+    cudaEvent_t *xs[7] = {c->ev_far, c->ev_near, c->ev_pm, c->ev_ired, c->ev_redd, c->ev_spread, c->ev_rowd};
     for (cudaEvent_t *x : xs)
         for (int k = 0; k < 2; ++k)
             if (x[k]) cudaEventDestroy(x[k]);
@@ -146,9 +144,9 @@ extern "C" turret_status lbm_init(turret_ctx **out, const turret_window *win, tu
 
     c = new turret_ctx();
     c->side = c->aux = nullptr;
-    c->ev_fork = c->ev_join = c->ev_red = c->ev_red_done = c->ev_pred = nullptr;
+    c->ev_fork = c->ev_join = nullptr;
     for (int k = 0; k < 2; ++k) {
-        c->ev_far[k] = c->ev_near[k] = c->ev_pm[k] = c->ev_ired[k] = c->ev_redd[k] = c->ev_spread[k] = nullptr;
+        c->ev_far[k] = c->ev_near[k] = c->ev_pm[k] = c->ev_ired[k] = c->ev_redd[k] = c->ev_spread[k] = c->ev_rowd[k] = nullptr;
         c->multi_ready[k] = false;
     }
     c->pred_mode = 0;
@@ -214,11 +212,8 @@ extern "C" turret_status lbm_init(turret_ctx **out, const turret_window *win, tu
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->aux, cudaStreamNonBlocking, hi_prio);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_red, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_red_done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_pred, cudaEventDisableTiming);
     {
-        cudaEvent_t *xs[6] = {c->ev_far, c->ev_near, c->ev_pm, c->ev_ired, c->ev_redd, c->ev_spread};
+        cudaEvent_t *xs[7] = {c->ev_far, c->ev_near, c->ev_pm, c->ev_ired, c->ev_redd, c->ev_spread, c->ev_rowd};
         for (cudaEvent_t *x : xs)
             for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&x[k], cudaEventDisableTiming);
     }
@@ -427,41 +422,56 @@ static bool ibm_layout(const MeshProps &mp, const double *V, int64_t nv, IbmLayo
     return B <= 1024;
 }
 
+// Two sets of the level's own marker arrays while the second costs at most
+// this much; a surface beyond it (some 200,000 markers) shares one set, and a
+// step's particle update then waits for the previous spreading.
+constexpr size_t SECOND_SET_MAX = (size_t)1 << 30;
+
+// The arrays a time level owns (see MarkerArrays).
+static void carve_level(Carver &cv, const IbmLayout &L, MarkerArrays &m) {
+    const size_t nm = (size_t)L.nm, ntiles = (size_t)L.box.tx * L.box.ty * L.box.tz;
+    m.rec = (MRec *)cv.take(nm * sizeof(MRec));
+    m.reco = (MRec *)cv.take(nm * sizeof(MRec));
+    m.base = (int *)cv.take(nm * 4);
+    m.U = (float *)cv.take(3 * nm * 4);
+    m.n = (float *)cv.take(3 * nm * 4);
+    m.arm = (float *)cv.take(3 * nm * 4);
+    m.aval = (float *)cv.take(nm * (size_t)ROWCAP * 4);
+    m.aidx = (int *)cv.take(nm * (size_t)ROWCAP * 4);
+    m.alen = (int *)cv.take(nm * 4);
+    m.seg = (int *)cv.take(6 * ((nm + MARKER_SEG - 1) / MARKER_SEG) * 4);
+    m.tile_list = (int *)cv.take(2 * ntiles * (size_t)L.cap * 4);  // spreading list, rows-of-A list
+    m.tile_count = (int *)cv.take(2 * ntiles * 4);
+}
+
 static size_t carve_ibm(Carver &cv, const IbmLayout &L, turret_ctx *c) {
     const size_t nm = (size_t)L.nm, nb = (size_t)L.box.nbox;
-    const size_t ntiles = (size_t)L.box.tx * L.box.ty * L.box.tz;
     MarkerArrays m;
     m.Xb = (const float *)cv.take(3 * nm * 4);
     m.nb = (const float *)cv.take(3 * nm * 4);
     m.dS = (const float *)cv.take(nm * 4);
     m.dSo = (const float *)cv.take(nm * 4);
-    m.rec = (MRec *)cv.take(nm * sizeof(MRec));
-    m.reco = (MRec *)cv.take(nm * sizeof(MRec));
-    m.base = (int *)cv.take(nm * 4);
     m.ft = (float *)cv.take(9 * nm * 4);
-    m.U = (float *)cv.take(3 * nm * 4);
-    m.n = (float *)cv.take(3 * nm * 4);
-    m.arm = (float *)cv.take(3 * nm * 4);
     m.hl = (float *)cv.take(3 * nm * 4);
     m.r0 = (float *)cv.take(3 * nm * 4);
     m.hb = (float *)cv.take(3 * nm * 4);
-    m.aval = (float *)cv.take(nm * (size_t)ROWCAP * 4);
-    m.aidx = (int *)cv.take(nm * (size_t)ROWCAP * 4);
-    m.alen = (int *)cv.take(nm * 4);
-    m.seg = (int *)cv.take(6 * ((nm + MARKER_SEG - 1) / MARKER_SEG) * 4);
     m.force_eval = c ? c->flags.force_eval : 0;
     BoxArrays ba;
     ba.u = (float *)cv.take(3 * nb * 4);
     ba.s = (float *)cv.take(6 * nb * 4);
     ba.p = (float *)cv.take(nb * 4);
     ba.h = (float *)cv.take(3 * nb * 4);
-    int *tl = (int *)cv.take(2 * ntiles * (size_t)L.cap * 4);  // spreading list, rows-of-A list
-    int *tc = (int *)cv.take(2 * ntiles * 4);
+    MarkerArrays m2 = m;
+    const size_t before = cv.off;
+    carve_level(cv, L, m);
+    const bool two = cv.off - before <= SECOND_SET_MAX;
+    if (two) carve_level(cv, L, m2);
+    else m2 = m;
     if (c) {
-        c->mk = m;
+        c->mk[0] = m;
+        c->mk[1] = m2;
+        c->two_sets = two;
         c->ba = ba;
-        c->tile_list = tl;
-        c->tile_count = tc;
     }
     return cv.off + 256;
 }
@@ -477,66 +487,38 @@ extern "C" size_t ibm_workspace_bytes(const turret_ctx *c, const double *V, int6
     return carve_ibm(cv, L, nullptr);
 }
 
-// Events (2)-(4) of Table 1.  advance = 1: particle update t -> t+1 from
-// window slot `slot` (markers land in slot^1), then u* and sigma on the
-// support box from f(t+1) = pull(f*(t)) together with the tile candidate
-// lists, the surface force and torque, and n IBM cycles -> h_imm(t+1).
-// advance = 0: the same at the current time level (slot `slot`) without
-// moving the particle (set-up of t = 0).
-// The IBM cycles of one step (the paper's n - 1 cycles from r0, or the
-// warm-started adaptive ones) on stream s.
-static cudaError_t enqueue_cycles(turret_ctx *c, int warm, cudaStream_t s) {
-    const int nm = c->nm;
-    if (!warm) {
-        // the paper's cycles: h^0 = r0, then cycles 1 .. n-1 alternating so
-        // that the last one writes hl
-        const int C = c->flags.ibm_cycles - 1;
-        const float *src = c->mk.r0;
-        for (int cyc = 1; cyc <= C; ++cyc) {
-            float *dst = ((C - cyc) % 2 == 0) ? c->mk.hl : c->mk.hb;
-            CE(launch_cycle(nm, c->mk, src, dst, nullptr, cyc == C, c->dstate, cyc - 1, 0, 0.0f, s));
-            src = dst;
-        }
-    } else {
-        // predictor modes: up to n cycles from the previous h (in hl), each
-        // skipped once the slip is below the tolerance; hl ends with the result
-        const int C = c->flags.ibm_cycles;
-        const float *src = c->mk.hl;
-        for (int cyc = 1; cyc <= C; ++cyc) {
-            float *dst = (cyc % 2 == 1) ? c->mk.hb : c->mk.hl;
-            float *fin = (cyc == C && dst != c->mk.hl) ? c->mk.hl : nullptr;
-            CE(launch_cycle(nm, c->mk, src, dst, fin, cyc == C, c->dstate, cyc - 1, 1, c->body.slip_eps, s));
-            src = dst;
-        }
-    }
-    return cudaSuccess;
+// Events (2)-(4) of Table 1 in two parts.  The markers' part: particle update
+// t -> t+1 from window slot `slot` (advance = 1; the markers land in slot^1,
+// and in that level's marker set) or the markers of the current level (advance
+// = 0, set-up of t = 0); then the tile lists and the rows of A, which depend
+// on the markers alone.
+static cudaError_t enqueue_lists(turret_ctx *c, int so, cudaStream_t s) {
+    CE(launch_bin(c->dstate, so, c->box, c->nm, c->mk[so], c->cap, c->body.rmin, c->body.rmax, s));
+    return launch_rows(c->box, c->nm, c->mk[so], c->cap, c->dstate, s);
 }
 
-// pm_done: when non-null, the particle/marker update was already enqueued
-// (on the aux stream, beside the near collide+stream) and this event marks it.
-static cudaError_t enqueue_coupling(turret_ctx *c, const void *fsrc, const float *utop_in, int slot, int advance,
-                                    cudaStream_t s, cudaEvent_t pm_done = nullptr) {
-    const int nm = c->nm;
-    const int so = advance ? (slot ^ 1) : slot;
-    const bool branch = (s == c->side);  // reduce F, T on the aux branch
-    if (pm_done) CE(cudaStreamWaitEvent(s, pm_done, 0));
-    else CE(launch_particle_markers(c->geom, c->body, c->box, c->dstate, slot, advance, c->mk, s));
-    CE(launch_box_moments_bin(c->geom, c->storage, fsrc, utop_in, c->dstate, so, c->box, c->ba, nm, c->mk.base, c->mk.seg,
-                              c->tile_list, c->tile_count, c->cap, c->dstate, c->body.rmin, c->body.rmax, s));
-    const int warm = (advance && c->body.predictor != 0 && (c->body.pred_opts & PRED_WARM)) ? 1 : 0;
-    CE(launch_interp0(c->box, nm, c->mk, c->ba, c->tile_list, c->tile_count, c->cap, c->dstate, warm, s));
-    if (branch) {
-        CE(cudaEventRecord(c->ev_red, s));
-        CE(cudaStreamWaitEvent(c->aux, c->ev_red, 0));
-        CE(launch_reduce_ft(nm, c->mk, c->dstate, so, c->body, c->aux));
-        CE(cudaEventRecord(c->ev_red_done, c->aux));
-    } else {
-        CE(launch_reduce_ft(nm, c->mk, c->dstate, so, c->body, s));
-    }
-    CE(enqueue_cycles(c, warm, s));
-    CE(launch_spread(c->box, nm, c->mk, c->ba, c->tile_list, c->tile_count, c->cap, s));
-    if (branch) CE(cudaStreamWaitEvent(s, c->ev_red_done, 0));
-    return cudaSuccess;
+// The IBM cycles of one step (the paper's n - 1 cycles from r0, or the
+// warm-started adaptive ones: up to n) on stream s.
+static cudaError_t enqueue_cycles(turret_ctx *c, int so, int warm, cudaStream_t s) {
+    return launch_cycles(c->nm, c->mk[so], c->flags.ibm_cycles - (warm ? 0 : 1), warm, c->dstate, c->body.slip_eps, s);
+}
+
+static int warm_cycles(const turret_ctx *c) {
+    return (c->body.predictor != 0 && (c->body.pred_opts & PRED_WARM)) ? 1 : 0;
+}
+
+// The fluid's part, with the markers of level `so` in place: u* and sigma on
+// the support box from f(t+1) = pull(f*(t)), the surface force and torque,
+// and the IBM cycles -> h_imm(t+1).  On one stream; the split step spreads the
+// same launches over three (enqueue_step, enqueue_steps_pipelined).
+static cudaError_t enqueue_coupling(turret_ctx *c, const void *fsrc, const float *utop_in, int so, int advance,
+                                    cudaStream_t s) {
+    const int nm = c->nm, warm = advance ? warm_cycles(c) : 0;
+    CE(launch_box_moments(c->geom, c->storage, fsrc, utop_in, c->dstate, so, c->box, c->ba, c->body.rmin, c->body.rmax, s));
+    CE(launch_interp0(c->box, nm, c->mk[so], c->ba, c->dstate, warm, s));
+    CE(launch_reduce_ft(nm, c->mk[so], c->dstate, so, c->body, s));
+    CE(enqueue_cycles(c, so, warm, s));
+    return launch_spread(c->box, c->mk[so], c->ba, c->cap, s);
 }
 
 // Tensor maps of the staged 16-bit collide+stream from f[p] into f[1 - p]
@@ -563,6 +545,8 @@ static cudaError_t collide_window(const turret_ctx *c, int p, cudaStream_t s) {
                                  1 - p, nullptr, c->box, false, REGION_ALL, s);
 }
 
+static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K);
+
 // One step from parity p: f[p] holds f*(t-1), f[1-p] receives f*(t).
 static cudaError_t enqueue_step(turret_ctx *c, int p) {
     const Geom &G = c->geom;
@@ -576,56 +560,46 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
                               c->body.predictor, c->stream));
         CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p, -1,
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
-        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk, c->stream));
+        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], c->stream));
         CE(launch_reinject(G, c->storage, c->f[1 - p], c->f[p], c->dstate, 1 - p, c->reinject, c->stream));
-        CE(cudaEventRecord(c->ev_pred, c->stream));
-        return enqueue_coupling(c, c->f[1 - p], c->utop[p], p, 1, c->stream, c->ev_pred);
+        CE(enqueue_lists(c, 1 - p, c->stream));
+        return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
-    cudaStream_t chain = c->split ? c->side : c->stream;
     const bool predict = c->body.predictor != 0;
     const MlpDev *net = (c->body.predictor == 2) ? mlp_device_view(c->net) : nullptr;
-    if (c->split) {
-        // the prediction and the particle/marker update (which reads only the
-        // body state) run on the aux stream beside the near collide+stream
-        CE(cudaEventRecord(c->ev_fork, c->stream));
-        CE(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-        CE(cudaStreamWaitEvent(c->aux, c->ev_fork, 0));
-        if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->aux));
-        CE(launch_particle_markers(c->geom, c->body, c->box, c->dstate, p, 1, c->mk, c->aux));
-        CE(cudaEventRecord(c->ev_pred, c->aux));
-        CE(launch_collide_far(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p, c->ba.h,
-                              c->box, c->stream, src_map(c, p), dst_map(c, p)));
-        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p, -1,
-                                 c->ba.h, c->box, true, REGION_NEAR, c->side));
-    } else {
+    if (!c->split) {
         if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->stream));
         CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p, -1,
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
+        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], c->stream));
+        CE(enqueue_lists(c, 1 - p, c->stream));
+        return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
-    CE(enqueue_coupling(c, c->f[1 - p], c->utop[p], p, 1, chain, c->split ? c->ev_pred : nullptr));
-    if (c->split) {
-        CE(cudaEventRecord(c->ev_join, c->side));
-        CE(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
-    }
-    return cudaSuccess;
+    // one step of the pipeline below
+    return enqueue_steps_pipelined(c, p, 1);
 }
 
-// Steps t .. t+K-1 (parity p0 first) as one capture with the exact cross-step
-// dependencies (split windows only), so the immersed-boundary chain of step
-// t overlaps the far-cell collide+stream of step t+1:
-//   far(t)    after near(t-1) [its near-region cells of f*(t-1)] and pm(t-1)
-//             [the window slot of t];
-//   pm(t)     (prediction + particle/marker update, aux) after far(t-1) and
-//             near(t-1) [they read the slot pm(t) writes] and spread(t-1)
-//             [the marker arrays pm(t) rewrites], and reduce(t-1) [F, T];
-//   near(t)   after far(t-1) [its far-cell sources and the buffer it writes];
-//   moments(t) after near(t) and pm(t); the chain then as in one step;
-//   reduce(t) (aux) after interpolation(t).
+// Steps t .. t+K-1 (parity p0 first) of a split window over three streams with
+// the exact dependencies, so the immersed-boundary chain of step t overlaps
+// the far-cell collide+stream of step t+1 and the markers, tile lists and rows
+// of A of t+1 are prepared beside the cycles and the spreading of t:
+//   caller  far(t)     after near(t-1) [its near-region cells of f*(t-1)] and
+//                      pm(t-1) [the window slot of t];
+//   aux     pm(t)      (prediction, particle update, markers of t+1) after
+//                      far(t-1) and near(t-1) [they read the slot pm(t) writes;
+//                      near(t-1) also follows the spreading of t-2, the last
+//                      reader of the marker set pm(t) writes] and reduce(t-1)
+//                      [F, T]; with a single marker set after spread(t-1);
+//           bin(t), rows(t)  tile lists and rows of A of those markers;
+//           reduce(t)  after interp(t);
+//   side    near(t)    after far(t-1) [its far-cell sources, the buffer it writes];
+//           moments(t) after near(t) and pm(t); interp(t);
+//           cycles(t)  after rows(t); spread(t).
 // Each event is recorded once per step parity; a wait always refers to the
-// step the dependency names.  Per-step results equal those of one-step graphs.
+// step the dependency names.  Results equal those of one-step graphs.
 static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K) {
     const Geom &G = c->geom;
-    const int nm = c->nm;
+    const int nm = c->nm, warm = warm_cycles(c);
     const bool predict = c->body.predictor != 0;
     const MlpDev *net = (c->body.predictor == 2) ? mlp_device_view(c->net) : nullptr;
     CE(cudaEventRecord(c->ev_fork, c->stream));
@@ -643,31 +617,32 @@ static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K) {
         CE(launch_collide_far(G, c->storage, c->f[p], c->f[q], c->utop[q], c->utop[p], c->dstate, p, c->ba.h, c->box,
                               c->stream, src_map(c, p), dst_map(c, p)));
         CE(cudaEventRecord(c->ev_far[p], c->stream));
-        // aux: prediction and particle/marker update
+        // aux: prediction, particle/marker update, tile lists, rows of A
         if (!first) {
             CE(cudaStreamWaitEvent(c->aux, c->ev_far[q], 0));
-            CE(cudaStreamWaitEvent(c->aux, c->ev_spread[q], 0));
+            CE(cudaStreamWaitEvent(c->aux, c->two_sets ? c->ev_near[q] : c->ev_spread[q], 0));
         }
         if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->aux));
-        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk, c->aux));
+        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[q], c->aux));
         CE(cudaEventRecord(c->ev_pm[p], c->aux));
+        CE(enqueue_lists(c, q, c->aux));
+        CE(cudaEventRecord(c->ev_rowd[p], c->aux));
         // side: the near cells, then the immersed-boundary chain
         if (!first) CE(cudaStreamWaitEvent(c->side, c->ev_far[q], 0));
         CE(launch_collide_stream(G, c->storage, c->f[p], c->f[q], c->utop[q], c->utop[p], c->dstate, p, -1, c->ba.h,
                                  c->box, true, REGION_NEAR, c->side));
         CE(cudaEventRecord(c->ev_near[p], c->side));
         CE(cudaStreamWaitEvent(c->side, c->ev_pm[p], 0));
-        CE(launch_box_moments_bin(G, c->storage, c->f[q], c->utop[p], c->dstate, q, c->box, c->ba, nm, c->mk.base,
-                                  c->mk.seg, c->tile_list, c->tile_count, c->cap, c->dstate, c->body.rmin,
-                                  c->body.rmax, c->side));
-        const int warm = (c->body.predictor != 0 && (c->body.pred_opts & PRED_WARM)) ? 1 : 0;
-        CE(launch_interp0(c->box, nm, c->mk, c->ba, c->tile_list, c->tile_count, c->cap, c->dstate, warm, c->side));
+        CE(launch_box_moments(G, c->storage, c->f[q], c->utop[p], c->dstate, q, c->box, c->ba, c->body.rmin, c->body.rmax,
+                              c->side));
+        CE(launch_interp0(c->box, nm, c->mk[q], c->ba, c->dstate, warm, c->side));
         CE(cudaEventRecord(c->ev_ired[p], c->side));
         CE(cudaStreamWaitEvent(c->aux, c->ev_ired[p], 0));
-        CE(launch_reduce_ft(nm, c->mk, c->dstate, q, c->body, c->aux));
+        CE(launch_reduce_ft(nm, c->mk[q], c->dstate, q, c->body, c->aux));
         CE(cudaEventRecord(c->ev_redd[p], c->aux));
-        CE(enqueue_cycles(c, warm, c->side));
-        CE(launch_spread(c->box, nm, c->mk, c->ba, c->tile_list, c->tile_count, c->cap, c->side));
+        CE(cudaStreamWaitEvent(c->side, c->ev_rowd[p], 0));
+        CE(enqueue_cycles(c, q, warm, c->side));
+        CE(launch_spread(c->box, c->mk[q], c->ba, c->cap, c->side));
         CE(cudaEventRecord(c->ev_spread[p], c->side));
     }
     const int last = p ^ 1;
@@ -766,11 +741,11 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
         const double ar = 0.5 * sqrt(cr[0] * cr[0] + cr[1] * cr[1] + cr[2] * cr[2]);
         for (int e = 0; e < 3; ++e) c->staging[7 * nm + T[3 * t + e]] += (float)(ar / 3.0);
     }
-    CK(cudaMemcpyAsync((void *)c->mk.Xb, c->staging.data(), 3 * nm * 4, cudaMemcpyHostToDevice, c->stream), "Xb");
-    CK(cudaMemcpyAsync((void *)c->mk.nb, c->staging.data() + 3 * nm, 3 * nm * 4, cudaMemcpyHostToDevice, c->stream),
+    CK(cudaMemcpyAsync((void *)c->mk[0].Xb, c->staging.data(), 3 * nm * 4, cudaMemcpyHostToDevice, c->stream), "Xb");
+    CK(cudaMemcpyAsync((void *)c->mk[0].nb, c->staging.data() + 3 * nm, 3 * nm * 4, cudaMemcpyHostToDevice, c->stream),
        "nb");
-    CK(cudaMemcpyAsync((void *)c->mk.dS, c->staging.data() + 6 * nm, nm * 4, cudaMemcpyHostToDevice, c->stream), "dS");
-    CK(cudaMemcpyAsync((void *)c->mk.dSo, c->staging.data() + 7 * nm, nm * 4, cudaMemcpyHostToDevice, c->stream),
+    CK(cudaMemcpyAsync((void *)c->mk[0].dS, c->staging.data() + 6 * nm, nm * 4, cudaMemcpyHostToDevice, c->stream), "dS");
+    CK(cudaMemcpyAsync((void *)c->mk[0].dSo, c->staging.data() + 7 * nm, nm * 4, cudaMemcpyHostToDevice, c->stream),
        "dSo");
     CK(cudaMemsetAsync(c->ba.h, 0, 3 * (size_t)L.box.nbox * 4, c->stream), "h");
     // the moments kernel skips the box cells no stencil reads: they keep
@@ -808,6 +783,8 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     CK(cudaMemcpyAsync(c->dstate, &D, sizeof(DevState), cudaMemcpyHostToDevice, c->stream), "state upload");
     c->has_particle = true;
     drop_graphs(c);
+    CK(launch_particle_markers(c->geom, c->body, c->box, c->dstate, t, 0, c->mk[t], c->stream), "initial markers");
+    CK(enqueue_lists(c, t, c->stream), "initial lists");
     CK(enqueue_coupling(c, c->f[t], c->utop[1 - t], t, 0, c->stream), "initial coupling");
     CK(cudaStreamSynchronize(c->stream), "initial coupling sync");
     return TURRET_OK;
@@ -1022,12 +999,12 @@ extern "C" turret_status query_particle_state(turret_ctx *c, turret_particle_sta
     out->n_markers = c->has_particle ? c->nm : 0;
     out->volume = c->has_particle ? c->vol : 0.0;
     out->area = c->has_particle ? c->area : 0.0;
-    // collide+stream (1, or far + near), particle + markers, moments + tile
-    // lists, interpolation + rows of A, F/T reduction, one product per extra
-    // cycle, spread of h_imm
-    out->kernels_per_step = c->has_particle ? (c->split ? 2 : 1) + 5 + (c->flags.ibm_cycles - 1) +
-                                                  (c->pred_mode != 0 ? 1 : 0) +  // prediction
-                                                  ((c->pred_mode != 0 && (c->pred_opts & PRED_WARM)) ? 1 : 0)
+    // collide+stream (1, or far + near), particle + markers, tile lists, rows
+    // of A, moments, interpolation, F/T reduction, cycles, spread of h_imm
+    const bool warm = c->pred_mode != 0 && (c->pred_opts & PRED_WARM);
+    out->kernels_per_step = c->has_particle ? (c->split ? 2 : 1) + 7 +
+                                                  c->flags.ibm_cycles - (warm ? 0 : 1) +
+                                                  (c->pred_mode != 0 ? 1 : 0)  // prediction
                                             : 1;
     if (D.status == STAT_DOMAIN) return fail(c, TURRET_EDOMAIN, "a marker stencil left the window");
     if (D.status == STAT_DIVERGED) return fail(c, TURRET_EDIVERGED, "non-finite force or torque");
@@ -1116,7 +1093,7 @@ extern "C" turret_status turret_save(turret_ctx *c, const char *path) {
                   {c->utop[1 - p], h.bytes_utop},
                   {c->dstate, h.bytes_state},
                   {c->has_particle ? c->ba.h : nullptr, h.bytes_h},
-                  {c->has_particle ? c->mk.hl : nullptr, h.bytes_hl}};
+                  {c->has_particle ? c->mk[0].hl : nullptr, h.bytes_hl}};
     CK(cudaStreamSynchronize(c->stream), "save sync");
     FILE *fp = fopen(path, "wb");
     if (!fp) return fail(c, TURRET_EINVAL, std::string("cannot open ") + path);
@@ -1157,7 +1134,7 @@ extern "C" turret_status turret_load(turret_ctx *c, const char *path) {
     CK(cudaStreamSynchronize(c->stream), "load sync");
     const int p = (int)(h.step & 1);
     void *dst[5] = {c->f[p], c->utop[1 - p], c->dstate, c->has_particle ? c->ba.h : nullptr,
-                    c->has_particle ? c->mk.hl : nullptr};
+                    c->has_particle ? c->mk[0].hl : nullptr};
     const int64_t bytes[5] = {h.bytes_pop, h.bytes_utop, h.bytes_state, h.bytes_h, h.bytes_hl};
     std::vector<char> buf;
     for (int k = 0; k < 5; ++k) {

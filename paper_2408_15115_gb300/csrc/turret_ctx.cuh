@@ -18,9 +18,9 @@ struct turret_ctx {
     cudaStream_t stream;  // caller's stream
     cudaStream_t side;    // internal high-priority stream of the immersed-boundary chain
     cudaStream_t aux;     // internal stream of the FP64 force/torque reduction
-    cudaEvent_t ev_fork, ev_join, ev_red, ev_red_done, ev_pred;
+    cudaEvent_t ev_fork, ev_join;
     // cross-step events of multi-step graphs, by step parity
-    cudaEvent_t ev_far[2], ev_near[2], ev_pm[2], ev_ired[2], ev_redd[2], ev_spread[2];
+    cudaEvent_t ev_far[2], ev_near[2], ev_pm[2], ev_ired[2], ev_redd[2], ev_spread[2], ev_rowd[2];
     turret::Geom geom;
     // fluid workspace
     void *f[2];
@@ -37,9 +37,9 @@ struct turret_ctx {
     int nm;
     turret::BodyConst body;
     turret::BoxGeom box;
-    turret::MarkerArrays mk;
+    turret::MarkerArrays mk[2];  // by time-level parity (the same set twice unless two_sets)
+    bool two_sets;
     turret::BoxArrays ba;
-    int *tile_list, *tile_count;
     int cap;
     double vol, area;
     turret::DevState host_state;

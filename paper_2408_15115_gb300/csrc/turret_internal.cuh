@@ -153,6 +153,10 @@ struct __align__(16) MRec {
     float hdS[3];
 };
 
+// Markers of one time level.  A context has two sets, by the level's parity:
+// Xb, nb, dS, dSo, ft, hl, r0 and hb are shared, the others (what the particle
+// update, the tile lists and the rows of A write) are the level's own, so those
+// of t + 1 are prepared while the cycles and the spreading of t still run.
 struct MarkerArrays {
     const float *Xb;   // [3][nm] body-frame offsets from C_m
     const float *nb;   // [3][nm] body-frame normals
@@ -173,6 +177,8 @@ struct MarkerArrays {
     int *alen;         // [nm] entries per row
     int *seg;          // [ceil(nm / MARKER_SEG)][6] per segment of MARKER_SEG consecutive
                        // markers: min x, y, z then max x, y, z of the stencil bases
+    int *tile_list;    // [2][tiles][cap] marker lists of the support tiles (spreading, rows of A)
+    int *tile_count;   // [2][tiles]
     int force_eval;    // 0: stress on the offset surface (reco, dSo), 1: at the markers
 };
 
@@ -199,12 +205,11 @@ struct RunDesc {
     Geom g;
     BodyConst bc;
     BoxGeom box;
-    MarkerArrays m;
+    MarkerArrays m[2];   // by time-level parity
     BoxArrays ba;
     void *f[2];          // ping-pong population buffers
     float *utop[2];      // top-plane velocity buffers
     DevState *st;
-    int *tile_list, *tile_count;
     int storage, cap, nm;
     int split;           // 1: far / near collide+stream, 0: the whole window in the near phase
     int tx;              // collide+stream tile width (threads along x)
@@ -385,13 +390,13 @@ cudaError_t launch_batch_collide(int phase, const CollideDesc *runs, const int *
 bool is_batch_bulk_kernel(const void *fn);
 cudaError_t launch_batch_box_moments_bin(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
                                          cudaStream_t s);
-// Support-box moments (u*, sigma) and the tile candidate lists, one launch.
-// Tiles that no marker can reach (outside the shell rmin <= |X - C_m| <= rmax
-// grown by the stencil reach) get empty lists without a scan.
-cudaError_t launch_box_moments_bin(const Geom &g, int storage, const void *src, const float *utop_in,
-                                   const DevState *st, int slot, const BoxGeom &box, BoxArrays ba, int nm,
-                                   const int *mbase, const int *mseg, int *tile_list, int *tile_count, int cap,
-                                   DevState *stw, float rmin, float rmax, cudaStream_t s);
+// Support-box moments (u*, sigma), and the tile candidate lists.  Tiles that
+// no marker can reach (outside the shell rmin <= |X - C_m| <= rmax grown by
+// the stencil reach) get empty lists without a scan.
+cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
+                               int slot, const BoxGeom &box, BoxArrays ba, float rmin, float rmax, cudaStream_t s);
+cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const MarkerArrays &m, int cap, float rmin,
+                       float rmax, cudaStream_t s);
 
 // Launchers (ibm_kernels.cu).
 // Rigid-body update t -> t+1 (advance = 1; reads window slot `slot`, writes
@@ -399,29 +404,30 @@ cudaError_t launch_box_moments_bin(const Geom &g, int storage, const void *src, 
 // advance = 0 only the markers of the current state (window slot `slot`).
 cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const BoxGeom &box, DevState *st, int slot,
                                     int advance, MarkerArrays m, cudaStream_t s);
-// l = 0 interpolation of u* and sigma, the surface traction per marker, and
-// the row k of the interaction matrix A (one warp per marker).
-cudaError_t launch_interp0(const BoxGeom &box, int nm, MarkerArrays m, BoxArrays ba, const int *tile_list,
-                           const int *tile_count, int cap, DevState *st, int warm, cudaStream_t s,
-                           bool by_tile = false);
-// One IBM cycle in matrix form: h_out = h_in + r0 - A h_in (= steps l = 1..4).
-cudaError_t launch_cycle(int nm, MarkerArrays m, const float *h_in, float *h_out, float *h_final, int last,
-                         DevState *st, int cyc, int adaptive, float eps, cudaStream_t s);
+// Rows of the interaction matrix A from the tile lists (one block per marker).
+cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, cudaStream_t s);
+// l = 0 interpolation of u* and sigma and the surface traction (one warp per
+// marker); warm 0 also starts h there.  Clears the slips of the last step.
+cudaError_t launch_interp0(const BoxGeom &box, int nm, const MarkerArrays &m, const BoxArrays &ba, DevState *st, int warm,
+                           cudaStream_t s);
+// The C IBM cycles of a step, one launch each, h <- h + r0 - A h (= steps l =
+// 1..4), from r0 (warm 0) or from the previous h, adaptively (warm 1); the
+// result in m.hl.
+cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, cudaStream_t s);
 // F = sum_k f_k, T = sum_k t_k in FP64, fixed order, into the device state.
 cudaError_t launch_reduce_ft(int nm, MarkerArrays m, DevState *st, int slot, const BodyConst &bc, cudaStream_t s);
-cudaError_t launch_spread(const BoxGeom &box, int nm, MarkerArrays m, BoxArrays ba, const int *tile_list,
-                          const int *tile_count, int cap, cudaStream_t s);
+cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxArrays &ba, int cap, cudaStream_t s);
 // Batched forms of the launches above, one launch over all runs of a batch
 // (time level p -> p ^ 1; blocks per run from the per-phase prefix table).
 cudaError_t launch_batch_particle_markers(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
                                           cudaStream_t s);
-cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nruns, int nblocks, int warm,
+cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int warm,
                                  cudaStream_t s);
-cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns, int nblocks, int sel_in,
+cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int sel_in,
                                int sel_out, int sel_final, int last, int cyc, int adaptive, cudaStream_t s);
 cudaError_t launch_batch_reduce_ft(const RunDesc *runs, int nruns, int slot, cudaStream_t s);
 cudaError_t launch_batch_predict(const RunDesc *runs, int nruns, int slot, cudaStream_t s);
-cudaError_t launch_batch_spread(const RunDesc *runs, const int *prefix, int nruns, int nblocks, cudaStream_t s);
+cudaError_t launch_batch_spread(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s);
 // Blocks of one run in each batched phase (host side, same formulas as the kernels).
 int blocks_bulk(const RunDesc &r, int threads);
 bool bulk16_run(const RunDesc &r);  // far cells in the 16-bit x-pair bulk launch
