@@ -307,6 +307,7 @@ __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, con
 
 __global__ void __launch_bounds__(PM_THREADS) k_particle_markers(Geom g, BodyConst bc, BoxGeom box, DevState *st,
                                                                   int slot, int advance, MarkerArrays m) {
+    pdl_trigger();
     pm_block(g, bc, box, st, slot, advance, m, blockIdx.x);
 }
 
@@ -502,6 +503,7 @@ constexpr int ROWS_MARKER_THREADS = 64;
 
 __global__ void __launch_bounds__(ROWS_MARKER_THREADS) k_rows(BoxGeom box, MarkerArrays m, const int *__restrict__ wlist,
                                                               const int *__restrict__ wcount, int cap, DevState *st) {
+    pdl_wait();
     rows_block<ROWS_MARKER_THREADS>(box, m, wlist, wcount, cap, st, blockIdx.x);
 }
 
@@ -512,11 +514,13 @@ constexpr int INTERP_THREADS = 64;
 
 __global__ void __launch_bounds__(INTERP_THREADS) k_interp(BoxGeom box, int nm, MarkerArrays m, BoxArrays ba,
                                                            DevState *st, int warm) {
+    const int k = blockIdx.x * (INTERP_THREADS / 32) + (threadIdx.x >> 5);
+    MRec rk;
+    if (k < nm) rk = m.rec[k];  // the markers precede the moments this launch may overlap
+    pdl_wait();
     // the previous step's cycles have read their slips; this step's follow
     if (blockIdx.x == 0 && threadIdx.x < 8) st->pr.slip[threadIdx.x] = 0u;
-    const int k = blockIdx.x * (INTERP_THREADS / 32) + (threadIdx.x >> 5);
     if (k >= nm) return;
-    const MRec rk = m.rec[k];
     interp_marker_warp(box, nm, m, ba, k, rk, threadIdx.x & 31, warm);
 }
 
@@ -663,16 +667,41 @@ __device__ __forceinline__ void interp0_tile_block(const BoxGeom &box, int nm, c
 // by cycle cyc - 1 is below eps; each executed cycle records its slip (an
 // atomic maximum of non-negative float bits: exact, order-independent).
 // h_final: also receives the last cycle's h when that is not h_out.
-__device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const float *__restrict__ h_in,
-                                            float *__restrict__ h_out, float *__restrict__ h_final, int last,
+__device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const float *h_in, float *h_out,
+                                            float *h_final, int last,
                                             int blk, DevState *st, int cyc, int adaptive, float eps) {
     __shared__ float smax[INTERP_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k = blk * INTERP_WARPS + warp;
+    // lane l adds entries l, l + 32, l + 64, ... in that order; the loads of
+    // four of them are issued together (two memory round trips per 128 entries
+    // instead of two per 32), the first four beside the row length and, in a
+    // launch that overlaps the cycle before it, before that cycle's h
+    constexpr int U = 4;
+    int len = 0;
+    float dS = 0.0f;
+    const float *arow = m.aval + (size_t)k * ROWCAP;
+    const int *irow = m.aidx + (size_t)k * ROWCAP;
+    float a[U];
+    int j[U];
+    auto load_entries = [&](int e0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + 32 * u + lane;
+            a[u] = e < ROWCAP ? arow[e] : 0.0f;
+            const int jj = e < ROWCAP ? irow[e] : k;
+            j[u] = (unsigned)jj < (unsigned)nm ? jj : k;  // entries past the row: any valid index
+        }
+    };
+    if (k < nm) {
+        len = m.alen[k];
+        dS = m.dS[k];
+        load_entries(0);
+    }
+    pdl_wait();
     const bool skip = adaptive && cyc > 0 && __uint_as_float(st->pr.slip[cyc - 1]) < eps;
     float res_max = 0.0f;
     if (k < nm) {
-        const float dS = m.dS[k];
         if (skip) {
             if (lane == 0)
                 for (int c = 0; c < 3; ++c) {
@@ -682,24 +711,10 @@ __device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const
                     if (last && h_final) h_final[c * nm + k] = h;
                 }
         } else {
-            const int len = m.alen[k];
-            const float *arow = m.aval + (size_t)k * ROWCAP;
-            const int *irow = m.aidx + (size_t)k * ROWCAP;
             float ax = 0.0f, ay = 0.0f, az = 0.0f;
-            // lane l adds entries l, l + 32, l + 64, ... in that order; the loads of
-            // four of them are issued together (two memory round trips per 128
-            // entries instead of two per 32), the first four beside the row length
-            constexpr int U = 4;
             for (int e0 = 0; e0 == 0 || e0 < len; e0 += 32 * U) {
-                float a[U], hx[U], hy[U], hz[U];
-                int j[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int e = e0 + 32 * u + lane;
-                    a[u] = e < ROWCAP ? arow[e] : 0.0f;
-                    const int jj = e < ROWCAP ? irow[e] : k;
-                    j[u] = (unsigned)jj < (unsigned)nm ? jj : k;  // entries past the row: any valid index
-                }
+                if (e0 > 0) load_entries(e0);
+                float hx[U], hy[U], hz[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     hx[u] = h_in[j[u]];
@@ -744,10 +759,10 @@ __device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const
     }
 }
 
-__global__ void __launch_bounds__(32 * INTERP_WARPS) k_cycle(int nm, MarkerArrays m, const float *__restrict__ h_in,
-                                                             float *__restrict__ h_out, float *__restrict__ h_final,
-                                                             int last, DevState *st, int cyc, int adaptive,
-                                                             float eps) {
+__global__ void __launch_bounds__(32 * INTERP_WARPS) k_cycle(int nm, MarkerArrays m, const float *h_in, float *h_out,
+                                                             float *h_final, int last, DevState *st, int cyc,
+                                                             int adaptive, float eps) {
+    pdl_trigger();
     cycle_block(nm, m, h_in, h_out, h_final, last, blockIdx.x, st, cyc, adaptive, eps);
 }
 
@@ -869,7 +884,7 @@ constexpr int SPREAD_STAGE = 256;
 // per 4^3 tile: the tile's candidate records are staged in shared memory as
 // structure of arrays; thread (cell c, slice q) sums slice q of each staged
 // chunk for cell c; the 8 slice sums are added in slice order (reproducible).
-__device__ __forceinline__ void spread_block(const BoxGeom &box, const MRec *__restrict__ rec, const BoxArrays &ba,
+__device__ __forceinline__ void spread_block(const BoxGeom &box, const MRec *rec, const BoxArrays &ba,
                                              const int *__restrict__ tile_list, const int *__restrict__ tile_count,
                                              int cap, int tile) {
     constexpr int TC = TILE * TILE * TILE;
@@ -883,10 +898,13 @@ __device__ __forceinline__ void spread_block(const BoxGeom &box, const MRec *__r
     const int cx = TILE * tx + c % TILE, cy = TILE * ty + (c / TILE) % TILE, cz = TILE * tz + c / (TILE * TILE);
     const int *list = tile_list + (size_t)tile * cap;
     float ax = 0.0f, ay = 0.0f, az = 0.0f;
+    int k = tid < min(SPREAD_STAGE, cnt) ? __ldg(list + tid) : 0;
+    pdl_wait();  // the records' h dS come from the last cycle
     for (int base = 0; base < cnt; base += SPREAD_STAGE) {
         const int n = min(SPREAD_STAGE, cnt - base);
         if (tid < n) {
-            const MRec r = rec[__ldg(list + base + tid)];
+            if (base > 0) k = __ldg(list + base + tid);
+            const MRec r = rec[k];
             sbase[tid] = r.base;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -933,9 +951,10 @@ __device__ __forceinline__ void spread_block(const BoxGeom &box, const MRec *__r
     }
 }
 
-__global__ void __launch_bounds__(SPREAD_THREADS) k_spread(BoxGeom box, const MRec *__restrict__ rec, BoxArrays ba,
+__global__ void __launch_bounds__(SPREAD_THREADS) k_spread(BoxGeom box, const MRec *rec, BoxArrays ba,
                                                            const int *__restrict__ tile_list,
                                                            const int *__restrict__ tile_count, int cap) {
+    pdl_trigger();
     spread_block(box, rec, ba, tile_list, tile_count, cap, blockIdx.x);
 }
 
@@ -996,27 +1015,37 @@ cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const Bo
     return cudaGetLastError();
 }
 
-cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, cudaStream_t s) {
+cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, bool overlap,
+                        cudaStream_t s) {
     const int ntiles = box.tx * box.ty * box.tz;  // list 1 (rows of A) follows list 0
+    if (overlap)
+        return launch_pdl(k_rows, nm, ROWS_MARKER_THREADS, s, box, m, m.tile_list + (size_t)ntiles * cap,
+                          m.tile_count + ntiles, cap, st);
     k_rows<<<nm, ROWS_MARKER_THREADS, 0, s>>>(box, m, m.tile_list + (size_t)ntiles * cap, m.tile_count + ntiles, cap, st);
     return cudaGetLastError();
 }
 
 cudaError_t launch_interp0(const BoxGeom &box, int nm, const MarkerArrays &m, const BoxArrays &ba, DevState *st, int warm,
-                           cudaStream_t s) {
+                           bool overlap, cudaStream_t s) {
     constexpr int per = INTERP_THREADS / 32;
+    if (overlap) return launch_pdl(k_interp, (nm + per - 1) / per, INTERP_THREADS, s, box, nm, m, ba, st, warm);
     k_interp<<<(nm + per - 1) / per, INTERP_THREADS, 0, s>>>(box, nm, m, ba, st, warm);
     return cudaGetLastError();
 }
 
+// overlap: the second and later cycles start beside the one before.
 static cudaError_t launch_cycle(int nm, const MarkerArrays &m, const float *h_in, float *h_out, float *h_final, int last,
-                                DevState *st, int cyc, int adaptive, float eps, cudaStream_t s) {
+                                DevState *st, int cyc, int adaptive, float eps, bool overlap, cudaStream_t s) {
+    if (cyc > 0 && overlap)
+        return launch_pdl(k_cycle, (nm + INTERP_WARPS - 1) / INTERP_WARPS, 32 * INTERP_WARPS, s, nm, m, h_in, h_out, h_final,
+                          last, st, cyc, adaptive, eps);
     k_cycle<<<(nm + INTERP_WARPS - 1) / INTERP_WARPS, 32 * INTERP_WARPS, 0, s>>>(nm, m, h_in, h_out, h_final, last,
                                                                                  st, cyc, adaptive, eps);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, cudaStream_t s) {
+cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, bool overlap,
+                          cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     if (!warm) {
         // the paper's cycles: h^0 = r0, then cycles 1 .. n-1 alternating so
@@ -1024,7 +1053,7 @@ cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevSta
         const float *src = m.r0;
         for (int cyc = 1; cyc <= C && e == cudaSuccess; ++cyc) {
             float *dst = ((C - cyc) % 2 == 0) ? m.hl : m.hb;
-            e = launch_cycle(nm, m, src, dst, nullptr, cyc == C, st, cyc - 1, 0, 0.0f, s);
+            e = launch_cycle(nm, m, src, dst, nullptr, cyc == C, st, cyc - 1, 0, 0.0f, overlap, s);
             src = dst;
         }
     } else {
@@ -1034,7 +1063,7 @@ cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevSta
         for (int cyc = 1; cyc <= C && e == cudaSuccess; ++cyc) {
             float *dst = (cyc % 2 == 1) ? m.hb : m.hl;
             float *fin = (cyc == C && dst != m.hl) ? m.hl : nullptr;
-            e = launch_cycle(nm, m, src, dst, fin, cyc == C, st, cyc - 1, 1, eps, s);
+            e = launch_cycle(nm, m, src, dst, fin, cyc == C, st, cyc - 1, 1, eps, overlap, s);
             src = dst;
         }
     }
@@ -1046,7 +1075,11 @@ cudaError_t launch_reduce_ft(int nm, MarkerArrays m, DevState *st, int slot, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxArrays &ba, int cap, cudaStream_t s) {
+cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxArrays &ba, int cap, bool overlap,
+                          cudaStream_t s) {
+    if (overlap)
+        return launch_pdl(k_spread, box.tx * box.ty * box.tz, SPREAD_THREADS, s, box, m.rec, ba, m.tile_list, m.tile_count,
+                          cap);
     k_spread<<<box.tx * box.ty * box.tz, SPREAD_THREADS, 0, s>>>(box, m.rec, ba, m.tile_list, m.tile_count, cap);
     return cudaGetLastError();
 }

@@ -614,15 +614,25 @@ __device__ __forceinline__ void k1_cell(const Geom &g, const typename Codec<ST>:
     const float omega = omega_of(g, zl);
     bool forced = false;
     float hx = 0.0f, hy = 0.0f, hz = 0.0f;
+    // the near launch may start beside the spreading that writes h: the pull
+    // is its own, h and every store follow
+    if (MODE == K1_NEAR) pdl_wait();
     if (MODE == K1_ALLF || MODE == K1_NEAR) {
         const int rx = rel_axis(x, S.box_lo[0], S.box_lo_w[0], 0, g.nx, perx);
         const int ry = rel_axis(y, S.box_lo[1], S.box_lo_w[1], 0, g.ny, pery);
         const int rz = rel_axis(zl, S.box_lo[2], S.box_lo_w[2], 0, g.nz, perz);
         if ((unsigned)rx < (unsigned)box.Bx && (unsigned)ry < (unsigned)box.By && (unsigned)rz < (unsigned)box.Bz) {
             const size_t b = ((size_t)rz * box.By + ry) * box.Bx + rx;
-            hx = __ldg(hbox + b);
-            hy = __ldg(hbox + box.nbox + b);
-            hz = __ldg(hbox + 2 * box.nbox + b);
+            if (MODE == K1_NEAR) {  // (not through the read-only path: see above)
+                const volatile float *hv = hbox;
+                hx = hv[b];
+                hy = hv[box.nbox + b];
+                hz = hv[2 * box.nbox + b];
+            } else {
+                hx = __ldg(hbox + b);
+                hy = __ldg(hbox + box.nbox + b);
+                hz = __ldg(hbox + 2 * box.nbox + b);
+            }
             forced = true;
         }
     }

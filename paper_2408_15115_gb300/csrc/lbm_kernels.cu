@@ -96,11 +96,14 @@ static dim3 near_grid(const BoxGeom &b) {
 template <int ST>
 static cudaError_t collide_t(const Geom &g, const void *src, void *dst, const float *utop_in, float *utop_out,
                              DevState *st, int slot, int slot_out, const float *hbox, const BoxGeom &box,
-                             bool has_box, int region, cudaStream_t s) {
+                             bool has_box, int region, cudaStream_t s, bool after_spread) {
     using T = typename Codec<ST>::T;
     const dim3 blk(32, 4);
     const T *fs = (const T *)src;
     T *fd = (T *)dst;
+    if (region == REGION_NEAR && after_spread)
+        return launch_pdl(k_collide_stream<ST, K1_NEAR>, near_grid(box), blk, s, g, fs, fd, utop_in, utop_out, st, slot,
+                          slot_out, hbox, box);
     if (region == REGION_NEAR)
         k_collide_stream<ST, K1_NEAR><<<near_grid(box), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box);
     else if (region == REGION_FAR)
@@ -114,11 +117,11 @@ static cudaError_t collide_t(const Geom &g, const void *src, void *dst, const fl
 
 cudaError_t launch_collide_stream(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
                                   float *utop_out, DevState *st, int slot, int slot_out, const float *hbox,
-                                  const BoxGeom &box, bool has_box, int region, cudaStream_t s) {
+                                  const BoxGeom &box, bool has_box, int region, cudaStream_t s, bool after_spread) {
     switch (storage) {
-        case ST_F32: return collide_t<ST_F32>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s);
-        case ST_F16: return collide_t<ST_F16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s);
-        default: return collide_t<ST_BF16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s);
+        case ST_F32: return collide_t<ST_F32>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
+        case ST_F16: return collide_t<ST_F16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
+        default: return collide_t<ST_BF16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
     }
 }
 

@@ -11,6 +11,7 @@ __global__ void __launch_bounds__(MB_THREADS) k_box_moments(Geom g, const typena
                                                             const float *__restrict__ utop_in,
                                                             const DevState *__restrict__ st, int slot, BoxGeom box,
                                                             BoxArrays ba, float rmin, float rmax) {
+    pdl_trigger();
     moments_block<ST>(g, src, utop_in, st, slot, box, ba, rmin, rmax, blockIdx.x);
 }
 
@@ -18,6 +19,8 @@ __global__ void __launch_bounds__(MB_THREADS) k_bin(const DevState *__restrict__
                                                     const int *__restrict__ mbase, const int *__restrict__ mseg,
                                                     int *__restrict__ tile_list, int *__restrict__ tile_count, int cap,
                                                     DevState *stw, float rmin, float rmax) {
+    pdl_trigger();
+    pdl_wait();
     bin_block(st, slot, box, nm, mbase, mseg, tile_list, tile_count, cap, stw, rmin, rmax, blockIdx.x);
 }
 
@@ -33,7 +36,10 @@ cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, cons
 }
 
 cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const MarkerArrays &m, int cap, float rmin,
-                       float rmax, cudaStream_t s) {
+                       float rmax, bool overlap, cudaStream_t s) {
+    if (overlap)
+        return launch_pdl(k_bin, box.tx * box.ty * box.tz, MB_THREADS, s, st, slot, box, nm, m.base, m.seg, m.tile_list,
+                          m.tile_count, cap, st, rmin, rmax);
     k_bin<<<box.tx * box.ty * box.tz, MB_THREADS, 0, s>>>(st, slot, box, nm, m.base, m.seg, m.tile_list, m.tile_count, cap,
                                                           st, rmin, rmax);
     return cudaGetLastError();

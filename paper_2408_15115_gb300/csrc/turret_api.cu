@@ -487,20 +487,33 @@ extern "C" size_t ibm_workspace_bytes(const turret_ctx *c, const double *V, int6
     return carve_ibm(cv, L, nullptr);
 }
 
+// Whether the launches of the chain start beside the ones before them
+// (programmatic dependent launch): windows whose far cells take no longer than
+// the launches before the cycles (64^3: 9 of 12 us), with a cycle of at most
+// one block per SM.  There the chain is the step: 32x32x64, 362 markers, 100
+// steps 4797 us without, 4420 us with it.  On a larger window the bulk
+// collide+stream fills the SMs and blocks that wait take its slots: 96x96x192
+// (1212 markers, 24 steps) 2148 us without, 2489 us with it.
+constexpr long long OVERLAP_CELLS = 1 << 18;
+constexpr int OVERLAP_MARKERS = 152 * INTERP_WARPS;
+static bool overlap_chain(const turret_ctx *c) { return c->geom.ncell <= OVERLAP_CELLS && c->nm <= OVERLAP_MARKERS; }
+
 // Events (2)-(4) of Table 1 in two parts.  The markers' part: particle update
 // t -> t+1 from window slot `slot` (advance = 1; the markers land in slot^1,
 // and in that level's marker set) or the markers of the current level (advance
 // = 0, set-up of t = 0); then the tile lists and the rows of A, which depend
 // on the markers alone.
-static cudaError_t enqueue_lists(turret_ctx *c, int so, cudaStream_t s) {
-    CE(launch_bin(c->dstate, so, c->box, c->nm, c->mk[so], c->cap, c->body.rmin, c->body.rmax, s));
-    return launch_rows(c->box, c->nm, c->mk[so], c->cap, c->dstate, s);
+// after_pm: the marker launch is the one just before on the stream.
+static cudaError_t enqueue_lists(turret_ctx *c, int so, bool after_pm, cudaStream_t s) {
+    CE(launch_bin(c->dstate, so, c->box, c->nm, c->mk[so], c->cap, c->body.rmin, c->body.rmax, after_pm && overlap_chain(c), s));
+    return launch_rows(c->box, c->nm, c->mk[so], c->cap, c->dstate, overlap_chain(c), s);
 }
 
 // The IBM cycles of one step (the paper's n - 1 cycles from r0, or the
 // warm-started adaptive ones: up to n) on stream s.
+static int cycle_count(const turret_ctx *c, int warm) { return c->flags.ibm_cycles - (warm ? 0 : 1); }
 static cudaError_t enqueue_cycles(turret_ctx *c, int so, int warm, cudaStream_t s) {
-    return launch_cycles(c->nm, c->mk[so], c->flags.ibm_cycles - (warm ? 0 : 1), warm, c->dstate, c->body.slip_eps, s);
+    return launch_cycles(c->nm, c->mk[so], cycle_count(c, warm), warm, c->dstate, c->body.slip_eps, overlap_chain(c), s);
 }
 
 static int warm_cycles(const turret_ctx *c) {
@@ -515,10 +528,10 @@ static cudaError_t enqueue_coupling(turret_ctx *c, const void *fsrc, const float
                                     cudaStream_t s) {
     const int nm = c->nm, warm = advance ? warm_cycles(c) : 0;
     CE(launch_box_moments(c->geom, c->storage, fsrc, utop_in, c->dstate, so, c->box, c->ba, c->body.rmin, c->body.rmax, s));
-    CE(launch_interp0(c->box, nm, c->mk[so], c->ba, c->dstate, warm, s));
+    CE(launch_interp0(c->box, nm, c->mk[so], c->ba, c->dstate, warm, overlap_chain(c), s));
     CE(launch_reduce_ft(nm, c->mk[so], c->dstate, so, c->body, s));
     CE(enqueue_cycles(c, so, warm, s));
-    return launch_spread(c->box, c->mk[so], c->ba, c->cap, s);
+    return launch_spread(c->box, c->mk[so], c->ba, c->cap, overlap_chain(c) && cycle_count(c, warm) > 0, s);
 }
 
 // Tensor maps of the staged 16-bit collide+stream from f[p] into f[1 - p]
@@ -562,7 +575,7 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
         CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], c->stream));
         CE(launch_reinject(G, c->storage, c->f[1 - p], c->f[p], c->dstate, 1 - p, c->reinject, c->stream));
-        CE(enqueue_lists(c, 1 - p, c->stream));
+        CE(enqueue_lists(c, 1 - p, false, c->stream));
         return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
     const bool predict = c->body.predictor != 0;
@@ -572,7 +585,7 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
         CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p, -1,
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
         CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], c->stream));
-        CE(enqueue_lists(c, 1 - p, c->stream));
+        CE(enqueue_lists(c, 1 - p, true, c->stream));
         return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
     // one step of the pipeline below
@@ -592,7 +605,8 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
 //                      [F, T]; with a single marker set after spread(t-1);
 //           bin(t), rows(t)  tile lists and rows of A of those markers;
 //           reduce(t)  after interp(t);
-//   side    near(t)    after far(t-1) [its far-cell sources, the buffer it writes];
+//   side    near(t)    after far(t-1) [its far-cell sources, the buffer it writes;
+//                      on small windows cycles(t-1) wait for it already];
 //           moments(t) after near(t) and pm(t); interp(t);
 //           cycles(t)  after rows(t); spread(t).
 // Each event is recorded once per step parity; a wait always refers to the
@@ -602,6 +616,10 @@ static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K) {
     const int nm = c->nm, warm = warm_cycles(c);
     const bool predict = c->body.predictor != 0;
     const MlpDev *net = (c->body.predictor == 2) ? mlp_device_view(c->net) : nullptr;
+    // on a small window the cycles also wait for the far cells (which are done
+    // by then), so that the next near launch follows the spreading alone and
+    // can start beside it
+    const bool overlap = overlap_chain(c), far_first = K > 1 && overlap && cycle_count(c, warm) > 0;
     CE(cudaEventRecord(c->ev_fork, c->stream));
     CE(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
     CE(cudaStreamWaitEvent(c->aux, c->ev_fork, 0));
@@ -625,24 +643,25 @@ static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K) {
         if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->aux));
         CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[q], c->aux));
         CE(cudaEventRecord(c->ev_pm[p], c->aux));
-        CE(enqueue_lists(c, q, c->aux));
+        CE(enqueue_lists(c, q, true, c->aux));
         CE(cudaEventRecord(c->ev_rowd[p], c->aux));
         // side: the near cells, then the immersed-boundary chain
-        if (!first) CE(cudaStreamWaitEvent(c->side, c->ev_far[q], 0));
+        if (!first && !far_first) CE(cudaStreamWaitEvent(c->side, c->ev_far[q], 0));
         CE(launch_collide_stream(G, c->storage, c->f[p], c->f[q], c->utop[q], c->utop[p], c->dstate, p, -1, c->ba.h,
-                                 c->box, true, REGION_NEAR, c->side));
+                                 c->box, true, REGION_NEAR, c->side, !first && far_first));
         CE(cudaEventRecord(c->ev_near[p], c->side));
         CE(cudaStreamWaitEvent(c->side, c->ev_pm[p], 0));
         CE(launch_box_moments(G, c->storage, c->f[q], c->utop[p], c->dstate, q, c->box, c->ba, c->body.rmin, c->body.rmax,
                               c->side));
-        CE(launch_interp0(c->box, nm, c->mk[q], c->ba, c->dstate, warm, c->side));
+        CE(launch_interp0(c->box, nm, c->mk[q], c->ba, c->dstate, warm, overlap, c->side));
         CE(cudaEventRecord(c->ev_ired[p], c->side));
         CE(cudaStreamWaitEvent(c->aux, c->ev_ired[p], 0));
         CE(launch_reduce_ft(nm, c->mk[q], c->dstate, q, c->body, c->aux));
         CE(cudaEventRecord(c->ev_redd[p], c->aux));
         CE(cudaStreamWaitEvent(c->side, c->ev_rowd[p], 0));
+        if (far_first) CE(cudaStreamWaitEvent(c->side, c->ev_far[p], 0));
         CE(enqueue_cycles(c, q, warm, c->side));
-        CE(launch_spread(c->box, c->mk[q], c->ba, c->cap, c->side));
+        CE(launch_spread(c->box, c->mk[q], c->ba, c->cap, overlap && cycle_count(c, warm) > 0, c->side));
         CE(cudaEventRecord(c->ev_spread[p], c->side));
     }
     const int last = p ^ 1;
@@ -784,7 +803,7 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     c->has_particle = true;
     drop_graphs(c);
     CK(launch_particle_markers(c->geom, c->body, c->box, c->dstate, t, 0, c->mk[t], c->stream), "initial markers");
-    CK(enqueue_lists(c, t, c->stream), "initial lists");
+    CK(enqueue_lists(c, t, true, c->stream), "initial lists");
     CK(enqueue_coupling(c, c->f[t], c->utop[1 - t], t, 0, c->stream), "initial coupling");
     CK(cudaStreamSynchronize(c->stream), "initial coupling sync");
     return TURRET_OK;

@@ -315,6 +315,32 @@ template <> struct Codec<ST_BF16> {
 inline size_t storage_bytes(int st) { return st == ST_F32 ? 4 : 2; }
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch between consecutive kernels of one stream: the
+// second starts once every block of the first has called pdl_trigger, does
+// what does not depend on the first, and calls pdl_wait before the rest (which
+// returns when the first has finished and its writes are visible; at once in
+// a kernel launched without the attribute).  Every kernel of such a chain
+// waits, so a kernel that has passed pdl_wait follows all before it.  What a
+// kernel reads before pdl_wait was complete before the chain's first kernel
+// started.  A launch that also waits for an event of another stream is an
+// ordinary one.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Launchers (lbm_kernels.cu).
 // Collide+stream region: all cells, the cells outside the near region around
 // the particle, or the near region only.  The near region is the region of
@@ -328,11 +354,14 @@ enum { REGION_ALL = 0, REGION_FAR = 1, REGION_NEAR = 2 };
 constexpr int NEAR_MARGIN = 2;
 constexpr int NEAR_GROW = NEAR_MARGIN - 2;
 static_assert(F_OFFSET == 2.0f, "the support box grows by F_OFFSET cells per side");
+// after_spread (REGION_NEAR): start beside the spreading launched just before on
+// the same stream, with everything else the pull needs complete.
 // slot_out >= 0: the kernel also copies the window slot to slot_out (with no
 // entering plane) for a following step that has no particle update.
 cudaError_t launch_collide_stream(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
                                   float *utop_out, DevState *st, int slot, int slot_out, const float *hbox,
-                                  const BoxGeom &box, bool has_box, int region, cudaStream_t s);
+                                  const BoxGeom &box, bool has_box, int region, cudaStream_t s,
+                                  bool after_spread = false);
 // The far cells of a coupled step (lbm_far.cu): FP32 storage under a register
 // cap that leaves room for the immersed-boundary chain's small blocks; 16-bit
 // storages staged in shared memory when the tensor maps lmap / smap of src and
@@ -396,7 +425,7 @@ cudaError_t launch_batch_box_moments_bin(const RunDesc *runs, const int *prefix,
 cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
                                int slot, const BoxGeom &box, BoxArrays ba, float rmin, float rmax, cudaStream_t s);
 cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const MarkerArrays &m, int cap, float rmin,
-                       float rmax, cudaStream_t s);
+                       float rmax, bool overlap, cudaStream_t s);
 
 // Launchers (ibm_kernels.cu).
 // Rigid-body update t -> t+1 (advance = 1; reads window slot `slot`, writes
@@ -404,19 +433,24 @@ cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const
 // advance = 0 only the markers of the current state (window slot `slot`).
 cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const BoxGeom &box, DevState *st, int slot,
                                     int advance, MarkerArrays m, cudaStream_t s);
+// (overlap, here and below: start beside the launch just before on the stream.)
 // Rows of the interaction matrix A from the tile lists (one block per marker).
-cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, cudaStream_t s);
+cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, bool overlap,
+                        cudaStream_t s);
 // l = 0 interpolation of u* and sigma and the surface traction (one warp per
 // marker); warm 0 also starts h there.  Clears the slips of the last step.
 cudaError_t launch_interp0(const BoxGeom &box, int nm, const MarkerArrays &m, const BoxArrays &ba, DevState *st, int warm,
-                           cudaStream_t s);
+                           bool overlap, cudaStream_t s);
 // The C IBM cycles of a step, one launch each, h <- h + r0 - A h (= steps l =
 // 1..4), from r0 (warm 0) or from the previous h, adaptively (warm 1); the
 // result in m.hl.
-cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, cudaStream_t s);
+cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, bool overlap,
+                          cudaStream_t s);
 // F = sum_k f_k, T = sum_k t_k in FP64, fixed order, into the device state.
 cudaError_t launch_reduce_ft(int nm, MarkerArrays m, DevState *st, int slot, const BodyConst &bc, cudaStream_t s);
-cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxArrays &ba, int cap, cudaStream_t s);
+// h_imm on the support box (overlap only directly after a cycle).
+cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxArrays &ba, int cap, bool overlap,
+                          cudaStream_t s);
 // Batched forms of the launches above, one launch over all runs of a batch
 // (time level p -> p ^ 1; blocks per run from the per-phase prefix table).
 cudaError_t launch_batch_particle_markers(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
