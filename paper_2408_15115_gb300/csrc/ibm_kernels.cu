@@ -424,11 +424,10 @@ __device__ __forceinline__ void interp_marker_warp(const BoxGeom &box, int nm, c
 }
 
 
-template <int NT>
-__device__ __forceinline__ void rows_block(const BoxGeom &box, const MarkerArrays &m, const int *__restrict__ wlist,
-                                           const int *__restrict__ wcount, int cap, DevState *st, int k) {
+template <int NT, int CU>
+__device__ __forceinline__ void rows_block(const BoxGeom &box, const MarkerArrays &m, const int *wlist,
+                                           const int *wcount, int cap, DevState *st, int k) {
     constexpr int NW = NT / 32;
-    constexpr int CU = 4;
     __shared__ int wc[CU][NW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const MRec rk = m.rec[k];
@@ -448,7 +447,7 @@ __device__ __forceinline__ void rows_block(const BoxGeom &box, const MarkerArray
 #pragma unroll
         for (int u = 0; u < CU; ++u) {
             const int ii = base + u * NT + tid;
-            j[u] = ii < cnt ? __ldg(list + ii) : -1;
+            j[u] = ii < cnt ? list[ii] : -1;
         }
 #pragma unroll
         for (int u = 0; u < CU; ++u) {
@@ -497,14 +496,17 @@ __device__ __forceinline__ void rows_block(const BoxGeom &box, const MarkerArray
     }
 }
 
-// 64 threads per marker: the blocks sit on the SMs beside the bulk
-// collide+stream for the latency of their loads, so idle threads are costly.
-constexpr int ROWS_MARKER_THREADS = 64;
+// 64 threads per marker where the blocks sit on the SMs beside the bulk
+// collide+stream for the latency of their loads (idle threads are costly
+// there); 256 on small windows, where the rows are the longest launch of a
+// single step and the SMs are idle: one candidate a thread.
+constexpr int ROWS_MARKER_THREADS = 64, ROWS_MARKER_THREADS_SMALL = 256;
 
-__global__ void __launch_bounds__(ROWS_MARKER_THREADS) k_rows(BoxGeom box, MarkerArrays m, const int *__restrict__ wlist,
-                                                              const int *__restrict__ wcount, int cap, DevState *st) {
+template <int NT, int CU>
+__global__ void __launch_bounds__(NT) k_rows(BoxGeom box, MarkerArrays m, const int *wlist, const int *wcount, int cap,
+                                             DevState *st) {
     pdl_wait();
-    rows_block<ROWS_MARKER_THREADS>(box, m, wlist, wcount, cap, st, blockIdx.x);
+    rows_block<NT, CU>(box, m, wlist, wcount, cap, st, blockIdx.x);
 }
 
 // One warp per marker, small blocks (as above).  It used to share a launch
@@ -1019,9 +1021,9 @@ cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int c
                         cudaStream_t s) {
     const int ntiles = box.tx * box.ty * box.tz;  // list 1 (rows of A) follows list 0
     if (overlap)
-        return launch_pdl(k_rows, nm, ROWS_MARKER_THREADS, s, box, m, m.tile_list + (size_t)ntiles * cap,
+        return launch_pdl(k_rows<ROWS_MARKER_THREADS_SMALL, 1>, nm, ROWS_MARKER_THREADS_SMALL, s, box, m, m.tile_list + (size_t)ntiles * cap,
                           m.tile_count + ntiles, cap, st);
-    k_rows<<<nm, ROWS_MARKER_THREADS, 0, s>>>(box, m, m.tile_list + (size_t)ntiles * cap, m.tile_count + ntiles, cap, st);
+    k_rows<ROWS_MARKER_THREADS, 4><<<nm, ROWS_MARKER_THREADS, 0, s>>>(box, m, m.tile_list + (size_t)ntiles * cap, m.tile_count + ntiles, cap, st);
     return cudaGetLastError();
 }
 

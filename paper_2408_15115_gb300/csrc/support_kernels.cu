@@ -15,9 +15,8 @@ __global__ void __launch_bounds__(MB_THREADS) k_box_moments(Geom g, const typena
     moments_block<ST>(g, src, utop_in, st, slot, box, ba, rmin, rmax, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(MB_THREADS) k_bin(const DevState *__restrict__ st, int slot, BoxGeom box, int nm,
-                                                    const int *__restrict__ mbase, const int *__restrict__ mseg,
-                                                    int *__restrict__ tile_list, int *__restrict__ tile_count, int cap,
+__global__ void __launch_bounds__(MB_THREADS) k_bin(const DevState *st, int slot, BoxGeom box, int nm, const int *mbase,
+                                                    const int *mseg, int *tile_list, int *tile_count, int cap,
                                                     DevState *stw, float rmin, float rmax) {
     pdl_trigger();
     pdl_wait();

@@ -13,10 +13,12 @@ constexpr int MB_THREADS = 128;
 // order (ordered compaction with warp ballots; no atomics): list 0, the
 // markers whose 4x4x4 stencil overlaps the tile (spreading); list 1, those
 // whose stencil overlaps the stencil of any marker based in the tile (rows of
-// A).  Reads the markers and the window slot only.
-__device__ __forceinline__ void bin_block(const DevState *__restrict__ st, int slot, const BoxGeom &box, int nm,
-                                          const int *__restrict__ mbase, const int *__restrict__ mseg,
-                                          int *__restrict__ tile_list, int *__restrict__ tile_count, int cap,
+// A).  Reads the markers and the window slot only, with ordinary loads: a
+// launch may start beside the particle update that writes them (pdl_wait), and
+// read-only loads could be moved ahead of that wait.
+__device__ __forceinline__ void bin_block(const DevState *st, int slot, const BoxGeom &box, int nm,
+                                          const int *mbase, const int *mseg,
+                                          int *tile_list, int *tile_count, int cap,
                                           DevState *stw, float rmin, float rmax, int tile) {
     constexpr int NW = MB_THREADS / 32;
     const int tx = tile % box.tx, ty = (tile / box.tx) % box.ty, tz = tile / (box.tx * box.ty);
@@ -67,7 +69,7 @@ __device__ __forceinline__ void bin_block(const DevState *__restrict__ st, int s
                 bool in = true;
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
-                    in = in && __ldg(bb + 3 + a) + 3 >= t0[a] && __ldg(bb + a) <= t0[a] + TILE + 2;
+                    in = in && bb[3 + a] + 3 >= t0[a] && bb[a] <= t0[a] + TILE + 2;
                 reach[u] = reach[u] || in;
             }
             any = any || reach[u];
@@ -77,7 +79,7 @@ __device__ __forceinline__ void bin_block(const DevState *__restrict__ st, int s
 #pragma unroll
         for (int u = 0; u < CU; ++u) {
             const int k = group + u * MB_THREADS + tid;
-            pb[u] = (reach[u] && k < nm) ? __ldg(mbase + k) : -1;  // culled chunks load nothing
+            pb[u] = (reach[u] && k < nm) ? mbase[k] : -1;  // culled chunks load nothing
         }
         unsigned bal[CU][2];
         bool hit[CU][2];
