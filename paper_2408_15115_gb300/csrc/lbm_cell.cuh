@@ -878,6 +878,30 @@ __device__ __forceinline__ void k1_pair_collide_store(const Geom &g, typename Co
     }
 }
 
+// The cells of a window block of 32 x 4 threads: tiles of 32 x 4 cells, or
+// (flat) 128 consecutive cells of the plane.  Flat blocks leave no lane idle at
+// the end of a row (22 % of them at nx = 75) and touch fewer sectors twice
+// (128 + 2 cells of a row for 128, not 32 + 2 for 32): one step of the fluid
+// alone, us, tiles -> flat: FP32 75x101x143 58.9 -> 49.3, 36x40x150 16.5 ->
+// 12.4, 200x120x300 244 -> 233, 256x256x512 1078 -> 1071; FP16 (cell pairs)
+// 93x70x151 39.1 -> 32.8.  16-bit rows that are whole tiles keep them (96x96x192
+// 48.9, flat 50.1).
+__device__ __forceinline__ void window_cell(const Geom &g, int flat, int &cx, int &cy) {
+    if (flat) {
+        const int c = blockIdx.x * 128 + threadIdx.y * 32 + threadIdx.x;
+        cy = c / g.nx;  // beyond the plane: cy >= ny, no cell
+        cx = c - cy * g.nx;
+    } else {
+        cx = blockIdx.x * 32 + threadIdx.x;
+        cy = blockIdx.y * 4 + threadIdx.y;
+    }
+}
+inline int window_flat(const Geom &g, int storage) { return storage == ST_F32 || g.nx % 32 != 0; }
+// its grid over `layers` planes (or pairs of planes)
+inline dim3 window_grid(const Geom &g, int storage, int layers) {
+    return window_flat(g, storage) ? dim3((unsigned)((g.plane + 127) / 128), 1, layers) : dim3((g.nx + 31) / 32, (g.ny + 3) / 4, layers);
+}
+
 // Tile of a 1-D block of blockDim.x threads over (x, y): tx threads along x,
 // blockDim.x / tx rows along y, one plane (pz = 1) or pair of planes (pz = 2);
 // block b of a region ex x ey x ez (ceil(ez / pz) plane groups), x fastest.

@@ -16,9 +16,10 @@ namespace turret {
 __global__ void __maxnreg__(120) k_collide_stream_far_f32(Geom g, const float *__restrict__ src,
                                                           float *__restrict__ dst, const float *__restrict__ utop_in,
                                                           float *__restrict__ utop_out, DevState *st, int slot,
-                                                          const float *__restrict__ hbox, BoxGeom box) {
-    k1_pair<ST_F32, K1_FAR>(g, src, dst, utop_in, utop_out, st->s[slot], hbox, box, blockIdx.x * 32 + threadIdx.x,
-                            blockIdx.y * 4 + threadIdx.y, 2 * blockIdx.z);
+                                                          const float *__restrict__ hbox, BoxGeom box, int flat) {
+    int cx, cy;
+    window_cell(g, flat, cx, cy);
+    k1_pair<ST_F32, K1_FAR>(g, src, dst, utop_in, utop_out, st->s[slot], hbox, box, cx, cy, 2 * blockIdx.z);
 }
 
 cudaError_t launch_collide_far(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
@@ -32,10 +33,11 @@ cudaError_t launch_collide_far(const Geom &g, int storage, const void *src, void
     if (storage != ST_F32)
         return launch_collide_stream(g, storage, src, dst, utop_in, utop_out, st, slot, -1, hbox, box, true,
                                      REGION_FAR, s);
-    const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, (g.nz + 1) / 2);  // one thread per pair of planes
-    k_collide_stream_far_f32<<<grid, dim3(32, 4), 0, s>>>(g, (const float *)src, (float *)dst, utop_in, utop_out, st,
-                                                          slot, hbox, box);
+    k_collide_stream_far_f32<<<window_grid(g, ST_F32, (g.nz + 1) / 2), dim3(32, 4), 0, s>>>(  // one thread per pair of planes
+        g, (const float *)src, (float *)dst, utop_in, utop_out, st, slot, hbox, box, window_flat(g, ST_F32));
     return cudaGetLastError();
 }
+
+bool is_far_kernel(const void *fn) { return fn == (const void *)k_collide_stream_far_f32; }
 
 }  // namespace turret

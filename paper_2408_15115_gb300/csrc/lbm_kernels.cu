@@ -12,7 +12,8 @@ __global__ void __launch_bounds__(128, MODE == K1_NEAR ? 1 : (ST == ST_F32 ? 4 :
                                                         typename Codec<ST>::T *__restrict__ dst,
                                                         const float *__restrict__ utop_in,
                                                         float *__restrict__ utop_out, DevState *st, int slot,
-                                                        int slot_out, const float *__restrict__ hbox, BoxGeom box) {
+                                                        int slot_out, const float *__restrict__ hbox, BoxGeom box,
+                                                        int flat) {
     if (slot_out >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 &&
         threadIdx.y == 0) {
         // carry the body and window to the next time level (no entering plane there)
@@ -23,9 +24,11 @@ __global__ void __launch_bounds__(128, MODE == K1_NEAR ? 1 : (ST == ST_F32 ? 4 :
     if (MODE == K1_NEAR)  // small, on the critical path: one cell per thread
         k1_cell<ST, MODE>(g, src, dst, utop_in, utop_out, st->s[slot], hbox, box, blockIdx.x * 32 + threadIdx.x,
                           blockIdx.y * 4 + threadIdx.y, blockIdx.z);
-    else  // the window: a pair of planes per thread
-        k1_pair<ST, MODE>(g, src, dst, utop_in, utop_out, st->s[slot], hbox, box, blockIdx.x * 32 + threadIdx.x,
-                          blockIdx.y * 4 + threadIdx.y, 2 * blockIdx.z);
+    else {  // the window: a pair of planes per thread
+        int cx, cy;
+        window_cell(g, flat, cx, cy);
+        k1_pair<ST, MODE>(g, src, dst, utop_in, utop_out, st->s[slot], hbox, box, cx, cy, 2 * blockIdx.z);
+    }
 }
 
 
@@ -61,9 +64,9 @@ __global__ void k_init_equilibrium(Geom g, typename Codec<ST>::T *__restrict__ d
 template <int ST>
 __global__ void __launch_bounds__(128) k_macro(Geom g, const typename Codec<ST>::T *__restrict__ src,
                                                const float *__restrict__ utop_in, const DevState *__restrict__ st,
-                                               int slot, float *__restrict__ out, int pops) {
-    const int x = blockIdx.x * 32 + threadIdx.x;
-    const int y = blockIdx.y * 4 + threadIdx.y;
+                                               int slot, float *__restrict__ out, int pops, int flat) {
+    int x, y;
+    window_cell(g, flat, x, y);
     const int zl = blockIdx.z;
     if (x >= g.nx || y >= g.ny) return;
     float q[27];
@@ -85,9 +88,6 @@ __global__ void __launch_bounds__(128) k_macro(Geom g, const typename Codec<ST>:
 
 // ---------------------------------------------------------------------------
 // Launchers.
-static dim3 cell_grid(const Geom &g) { return dim3((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz); }
-// collide+stream over the window: one thread per pair of planes
-static dim3 pair_grid(const Geom &g) { return dim3((g.nx + 31) / 32, (g.ny + 3) / 4, (g.nz + 1) / 2); }
 static dim3 near_grid(const BoxGeom &b) {
     const int ex = b.Bx + 2 * NEAR_GROW, ey = b.By + 2 * NEAR_GROW, ez = b.Bz + 2 * NEAR_GROW;
     return dim3((ex + 31) / 32, (ey + 3) / 4, ez);
@@ -103,15 +103,15 @@ static cudaError_t collide_t(const Geom &g, const void *src, void *dst, const fl
     T *fd = (T *)dst;
     if (region == REGION_NEAR && after_spread)
         return launch_pdl(k_collide_stream<ST, K1_NEAR>, near_grid(box), blk, s, g, fs, fd, utop_in, utop_out, st, slot,
-                          slot_out, hbox, box);
+                          slot_out, hbox, box, 0);
     if (region == REGION_NEAR)
-        k_collide_stream<ST, K1_NEAR><<<near_grid(box), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box);
+        k_collide_stream<ST, K1_NEAR><<<near_grid(box), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
     else if (region == REGION_FAR)
-        k_collide_stream<ST, K1_FAR><<<pair_grid(g), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box);
+        k_collide_stream<ST, K1_FAR><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
     else if (has_box)
-        k_collide_stream<ST, K1_ALLF><<<pair_grid(g), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box);
+        k_collide_stream<ST, K1_ALLF><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
     else
-        k_collide_stream<ST, K1_ALL><<<pair_grid(g), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box);
+        k_collide_stream<ST, K1_ALL><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
     return cudaGetLastError();
 }
 
@@ -123,6 +123,14 @@ cudaError_t launch_collide_stream(const Geom &g, int storage, const void *src, v
         case ST_F16: return collide_t<ST_F16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
         default: return collide_t<ST_BF16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
     }
+}
+
+bool is_window_kernel(const void *fn) {
+    return fn == (const void *)k_collide_stream<ST_F32, K1_ALL> || fn == (const void *)k_collide_stream<ST_F32, K1_ALLF> ||
+           fn == (const void *)k_collide_stream<ST_F32, K1_FAR> || fn == (const void *)k_collide_stream<ST_F16, K1_ALL> ||
+           fn == (const void *)k_collide_stream<ST_F16, K1_ALLF> || fn == (const void *)k_collide_stream<ST_F16, K1_FAR> ||
+           fn == (const void *)k_collide_stream<ST_BF16, K1_ALL> || fn == (const void *)k_collide_stream<ST_BF16, K1_ALLF> ||
+           fn == (const void *)k_collide_stream<ST_BF16, K1_FAR>;
 }
 
 cudaError_t launch_init_equilibrium(const Geom &g, int storage, void *dst, const double *drho, const double *u,
@@ -139,9 +147,9 @@ cudaError_t launch_init_equilibrium(const Geom &g, int storage, void *dst, const
 cudaError_t launch_macro(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
                          int slot, float *out, bool pops, cudaStream_t s) {
     switch (storage) {
-        case ST_F32: k_macro<ST_F32><<<cell_grid(g), dim3(32, 4), 0, s>>>(g, (const float *)src, utop_in, st, slot, out, pops); break;
-        case ST_F16: k_macro<ST_F16><<<cell_grid(g), dim3(32, 4), 0, s>>>(g, (const __half *)src, utop_in, st, slot, out, pops); break;
-        default: k_macro<ST_BF16><<<cell_grid(g), dim3(32, 4), 0, s>>>(g, (const __nv_bfloat16 *)src, utop_in, st, slot, out, pops); break;
+        case ST_F32: k_macro<ST_F32><<<window_grid(g, storage, g.nz), dim3(32, 4), 0, s>>>(g, (const float *)src, utop_in, st, slot, out, pops, window_flat(g, storage)); break;
+        case ST_F16: k_macro<ST_F16><<<window_grid(g, storage, g.nz), dim3(32, 4), 0, s>>>(g, (const __half *)src, utop_in, st, slot, out, pops, window_flat(g, storage)); break;
+        default: k_macro<ST_BF16><<<window_grid(g, storage, g.nz), dim3(32, 4), 0, s>>>(g, (const __nv_bfloat16 *)src, utop_in, st, slot, out, pops, window_flat(g, storage)); break;
     }
     return cudaGetLastError();
 }

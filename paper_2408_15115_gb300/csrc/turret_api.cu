@@ -813,22 +813,20 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
 // collide+stream node low and every other kernel node (the immersed-boundary
 // chain on the critical path) high, so the chain's blocks are dispatched
 // first whenever an SM frees up.
-static void set_node_priorities(const turret_ctx *c, cudaGraph_t gr) {
+static void set_node_priorities(cudaGraph_t gr) {
     int lo = 0, hi = 0;
     if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess) return;
     size_t n = 0;
     if (cudaGraphGetNodes(gr, nullptr, &n) != cudaSuccess || n == 0) return;
     std::vector<cudaGraphNode_t> nodes(n);
     if (cudaGraphGetNodes(gr, nodes.data(), &n) != cudaSuccess) return;
-    const dim3 bulk((c->geom.nx + 31) / 32, (c->geom.ny + 3) / 4, (c->geom.nz + 1) / 2);  // plane pairs
     for (cudaGraphNode_t nd : nodes) {
         cudaGraphNodeType t;
         if (cudaGraphNodeGetType(nd, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
         cudaKernelNodeParams kp;
         if (cudaGraphKernelNodeGetParams(nd, &kp) != cudaSuccess) continue;
-        const bool is_bulk = (kp.gridDim.x == bulk.x && kp.gridDim.y == bulk.y && kp.gridDim.z == bulk.z &&
-                              kp.blockDim.x == 32 && kp.blockDim.y == 4) ||
-                             is_staged_kernel(kp.func) || is_xpair_kernel(kp.func);
+        const bool is_bulk = is_far_kernel(kp.func) || is_window_kernel(kp.func) || is_staged_kernel(kp.func) ||
+                             is_xpair_kernel(kp.func);
         cudaLaunchAttributeValue v;
         memset(&v, 0, sizeof v);
         v.priority = is_bulk ? lo : hi;
@@ -851,7 +849,7 @@ static cudaError_t capture(turret_ctx *c, int p, int K, cudaGraphExec_t *out) {
         return e;
     }
     CE(e2);
-    set_node_priorities(c, gr);
+    set_node_priorities(gr);
     e = cudaGraphInstantiateWithFlags(out, gr, cudaGraphInstantiateFlagUseNodePriority);
     cudaGraphDestroy(gr);
     return e;

@@ -384,6 +384,9 @@ bool is_staged_kernel(const void *fn);
 // FP16 or round-to-nearest BF16 on a window the 64 x 2 x 2 tiles cover.
 bool xpair_eligible(const Geom &g, int storage);
 bool is_xpair_kernel(const void *fn);
+// The other kernels that sweep the window (bulk nodes of a step graph).
+bool is_window_kernel(const void *fn);
+bool is_far_kernel(const void *fn);
 cudaError_t launch_collide_xpair(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
                                  float *utop_out, DevState *st, int slot, int slot_out, const float *hbox,
                                  const BoxGeom &box, int region, cudaStream_t s);
