@@ -87,13 +87,13 @@ def train(x, y, epochs=30, batch=4096, lr=1e-3, weight_decay=1e-4, seed=0, preci
     history = []
     best = (validation_loss(net, *val), net.params()) if val is not None else None
     for _ in range(epochs):
-        perm = torch.as_tensor(rng.permutation(n), device=x.device)
+        # the epoch's minibatches in order, gathered once (a gather and its
+        # launches per minibatch cost as much as the training step)
+        perm = torch.as_tensor(rng.permutation(n)[:n - n % bsz], device=x.device)
+        xe, ye = x.index_select(0, perm), y.index_select(0, perm)
         tot, cnt = 0.0, 0
         for s in range(0, n - bsz + 1, bsz):
-            idx = perm[s:s + bsz]
-            xb = x.index_select(0, idx).contiguous()
-            yb = y.index_select(0, idx).contiguous()
-            tot += net.train_step(xb, yb, lr=lr, weight_decay=weight_decay)
+            tot += net.train_step(xe[s:s + bsz], ye[s:s + bsz], lr=lr, weight_decay=weight_decay)
             cnt += 1
         if val is None:
             history.append(tot / max(cnt, 1))

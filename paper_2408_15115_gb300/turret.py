@@ -449,6 +449,7 @@ class MLP:
             raise TurretError(rc, self._L.mlp_last_error(None).decode())
         self.m = m
         self.precision = precision
+        self._inputs = torch.cuda.Event()  # orders a training step after its inputs' stream
 
     def _check(self, rc):
         if rc != 0:
@@ -506,7 +507,10 @@ class MLP:
 
         Ordered after the work enqueued on the current stream (x and y may still be in the making)."""
         n = x.shape[0]
-        self.stream.wait_stream(self.torch.cuda.current_stream(self.device))
+        cur = self.torch.cuda.current_stream(self.device)
+        if cur != self.stream:
+            self._inputs.record(cur)
+            self.stream.wait_event(self._inputs)
         opt = AdamW(lr, beta1, beta2, eps, weight_decay)
         L = C.c_float()
         self._check(self._L.mlp_train_step(self.m, C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()), n,
