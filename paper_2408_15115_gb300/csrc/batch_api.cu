@@ -296,25 +296,13 @@ static cudaError_t batch_enqueue(turret_batch *b, int p) {
     CE(cudaStreamWaitEvent(b->aux, b->ev_red, 0));
     CE(launch_batch_reduce_ft(R, n, p ^ 1, b->aux));
     CE(cudaEventRecord(b->ev_red_done, b->aux));
-    if (!b->warm) {
-        // the paper's cycles: h^0 = r0, then 1 .. n-1 alternating so that the last writes hl
-        const int C = b->cycles - 1;
-        int src = HSEL_R0;
-        for (int cyc = 1; cyc <= C; ++cyc) {
-            const int dst = ((C - cyc) % 2 == 0) ? HSEL_HL : HSEL_HB;
-            CE(launch_batch_cycle(R, tab(T_CYC), n, p, b->total[T_CYC], src, dst, -1, cyc == C, cyc - 1, 0, b->side));
-            src = dst;
-        }
-    } else {
-        // predictor modes: up to n adaptive cycles from the previous h
-        const int C = b->cycles;
-        int src = HSEL_HL;
-        for (int cyc = 1; cyc <= C; ++cyc) {
-            const int dst = (cyc % 2 == 1) ? HSEL_HB : HSEL_HL;
-            const int fin = (cyc == C && dst != HSEL_HL) ? HSEL_HL : -1;
-            CE(launch_batch_cycle(R, tab(T_CYC), n, p, b->total[T_CYC], src, dst, fin, cyc == C, cyc - 1, 1, b->side));
-            src = dst;
-        }
+    // the cycles as in a single run (launch_cycles)
+    const int C = b->cycles - (b->warm ? 0 : 1);
+    int src = b->warm ? HSEL_HA : HSEL_R0;
+    for (int cyc = 1; cyc <= C; ++cyc) {
+        const int dst = src == HSEL_HA ? HSEL_HB : HSEL_HA;
+        CE(launch_batch_cycle(R, tab(T_CYC), n, p, b->total[T_CYC], src, dst, cyc == C, cyc - 1, b->warm, b->side));
+        src = dst;
     }
     CE(launch_batch_spread(R, tab(T_SP), n, p, b->total[T_SP], b->side));
     CE(cudaStreamWaitEvent(b->side, b->ev_red_done, 0));

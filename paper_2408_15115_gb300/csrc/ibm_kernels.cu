@@ -371,7 +371,6 @@ __device__ __forceinline__ void interp_marker_warp(const BoxGeom &box, int nm, c
     } else {
         d0 = c0, d1 = c1, v0 = w0, v1 = w1;
     }
-    const size_t N = box.nbox;
     // what the sums are combined with, fetched beside the stencil (the same
     // address in every lane)
     const float dS = m.dS[k], dA = fe == 0 ? m.dSo[k] : dS;  // dA: area of the surface the stress is taken on
@@ -383,23 +382,32 @@ __device__ __forceinline__ void interp_marker_warp(const BoxGeom &box, int nm, c
         rk3[c] = m.arm[c * nm + k];
     }
     float acc[10];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) acc[c] = w0 * ba.u[c * N + c0] + w1 * ba.u[c * N + c1];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) acc[3 + c] = v0 * ba.s[c * N + d0] + v1 * ba.s[c * N + d1];
-    acc[9] = v0 * ba.p[d0] + v1 * ba.p[d1];
+    const float4 ua = ba.u[c0], ub = ba.u[c1];
+    const float4 sa = ba.s[2 * d0], sb = ba.s[2 * d1], ta = ba.s[2 * d0 + 1], tb = ba.s[2 * d1 + 1];
+    acc[0] = w0 * ua.x + w1 * ub.x;
+    acc[1] = w0 * ua.y + w1 * ub.y;
+    acc[2] = w0 * ua.z + w1 * ub.z;
+    acc[3] = v0 * sa.x + v1 * sb.x;
+    acc[4] = v0 * sa.y + v1 * sb.y;
+    acc[5] = v0 * sa.z + v1 * sb.z;
+    acc[6] = v0 * sa.w + v1 * sb.w;
+    acc[7] = v0 * ta.x + v1 * tb.x;
+    acc[8] = v0 * ta.y + v1 * tb.y;
+    acc[9] = v0 * ta.z + v1 * tb.z;
 #pragma unroll
     for (int c = 0; c < 10; ++c)
 #pragma unroll
         for (int q = 16; q > 0; q >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], q);
     if (lane == 0) {
         // l = 0: h_k = U_k - I[u*](X_k); traction dS sigma(X_k) n_k and its moment
-        for (int c = 0; c < 3; ++c) {
-            const float h = Uk[c] - acc[c];
-            m.r0[c * nm + k] = h;
-            if (!warm) {
-                m.hl[c * nm + k] = h;
-                m.rec[k].hdS[c] = h * dS;
+        const float h[3] = {Uk[0] - acc[0], Uk[1] - acc[1], Uk[2] - acc[2]};
+        m.r0[k] = make_float4(h[0], h[1], h[2], 0.0f);
+        if (warm) {
+            m.ha[k] = make_float4(m.hl[k], m.hl[nm + k], m.hl[2 * nm + k], 0.0f);
+        } else {
+            for (int c = 0; c < 3; ++c) {
+                m.hl[c * nm + k] = h[c];
+                m.rec[k].hdS[c] = h[c] * dS;
             }
         }
         const float sxx = acc[3], syy = acc[4], szz = acc[5], sxy = acc[6], sxz = acc[7], syz = acc[8];
@@ -663,14 +671,14 @@ __device__ __forceinline__ void interp0_tile_block(const BoxGeom &box, int nm, c
 // One cycle of steps l = 1..4 (Sec. 2.2) in matrix form:
 //   h_out_k = h_in_k + U_k - I[u* + S h_in](X_k) = h_in_k + r0_k - sum_j A_kj h_in_j.
 // One warp per marker, entries of the row in order per lane, xor-shuffle sum.
-// The last cycle also stores h dS for the spreading of h_imm.
+// The last cycle stores h in m.hl, and h dS for the spreading of h_imm.  h is
+// gathered by column as one 16-byte load (three 4-byte gathers, one per
+// component, took 66 us a cycle of 69,000 markers in a batch, this 45).
 // adaptive (predictor modes): cycle `cyc` (0-based) is skipped -- h_out = h_in
 // -- once the slip max_k |U_k - I[u* + S h_in](X_k)| = max |r0 - A h_in| seen
 // by cycle cyc - 1 is below eps; each executed cycle records its slip (an
 // atomic maximum of non-negative float bits: exact, order-independent).
-// h_final: also receives the last cycle's h when that is not h_out.
-__device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const float *h_in, float *h_out,
-                                            float *h_final, int last,
+__device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const float4 *h_in, float4 *h_out, int last,
                                             int blk, DevState *st, int cyc, int adaptive, float eps) {
     __shared__ float smax[INTERP_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -700,35 +708,38 @@ __device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const
         dS = m.dS[k];
         load_entries(0);
     }
+    // the last cycle's result: the step's Lagrangian force, and h dS for the spreading
+    auto finish = [&](const float4 &h) {
+        m.hl[k] = h.x;
+        m.hl[nm + k] = h.y;
+        m.hl[2 * nm + k] = h.z;
+        m.rec[k].hdS[0] = h.x * dS;
+        m.rec[k].hdS[1] = h.y * dS;
+        m.rec[k].hdS[2] = h.z * dS;
+    };
     pdl_wait();
     const bool skip = adaptive && cyc > 0 && __uint_as_float(st->pr.slip[cyc - 1]) < eps;
     float res_max = 0.0f;
     if (k < nm) {
         if (skip) {
-            if (lane == 0)
-                for (int c = 0; c < 3; ++c) {
-                    const float h = h_in[c * nm + k];
-                    h_out[c * nm + k] = h;
-                    if (last) m.rec[k].hdS[c] = h * dS;
-                    if (last && h_final) h_final[c * nm + k] = h;
-                }
+            if (lane == 0) {
+                const float4 h = h_in[k];
+                if (last) finish(h);
+                else h_out[k] = h;
+            }
         } else {
             float ax = 0.0f, ay = 0.0f, az = 0.0f;
             for (int e0 = 0; e0 == 0 || e0 < len; e0 += 32 * U) {
                 if (e0 > 0) load_entries(e0);
-                float hx[U], hy[U], hz[U];
+                float4 h[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    hx[u] = h_in[j[u]];
-                    hy[u] = h_in[nm + j[u]];
-                    hz[u] = h_in[2 * nm + j[u]];
-                }
+                for (int u = 0; u < U; ++u) h[u] = h_in[j[u]];
 #pragma unroll
                 for (int u = 0; u < U; ++u)
                     if (e0 + 32 * u + lane < len) {
-                        ax = fmaf(a[u], hx[u], ax);
-                        ay = fmaf(a[u], hy[u], ay);
-                        az = fmaf(a[u], hz[u], az);
+                        ax = fmaf(a[u], h[u].x, ax);
+                        ay = fmaf(a[u], h[u].y, ay);
+                        az = fmaf(a[u], h[u].z, az);
                     }
             }
 #pragma unroll
@@ -738,15 +749,12 @@ __device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const
                 az += __shfl_xor_sync(0xffffffffu, az, o);
             }
             if (lane == 0) {
-                const float acc[3] = {ax, ay, az};
-                for (int c = 0; c < 3; ++c) {
-                    const float res = m.r0[c * nm + k] - acc[c];
-                    const float h = h_in[c * nm + k] + res;
-                    h_out[c * nm + k] = h;
-                    if (last) m.rec[k].hdS[c] = h * dS;
-                    if (last && h_final) h_final[c * nm + k] = h;
-                    res_max = fmaxf(res_max, fabsf(res));
-                }
+                const float4 r = m.r0[k], hk = h_in[k];
+                const float res[3] = {r.x - ax, r.y - ay, r.z - az};
+                const float4 h = make_float4(hk.x + res[0], hk.y + res[1], hk.z + res[2], 0.0f);
+                if (last) finish(h);
+                else h_out[k] = h;
+                for (int c = 0; c < 3; ++c) res_max = fmaxf(res_max, fabsf(res[c]));
             }
         }
     }
@@ -761,11 +769,11 @@ __device__ __forceinline__ void cycle_block(int nm, const MarkerArrays &m, const
     }
 }
 
-__global__ void __launch_bounds__(32 * INTERP_WARPS) k_cycle(int nm, MarkerArrays m, const float *h_in, float *h_out,
-                                                             float *h_final, int last, DevState *st, int cyc,
+__global__ void __launch_bounds__(32 * INTERP_WARPS) k_cycle(int nm, MarkerArrays m, const float4 *h_in,
+                                                             float4 *h_out, int last, DevState *st, int cyc,
                                                              int adaptive, float eps) {
     pdl_trigger();
-    cycle_block(nm, m, h_in, h_out, h_final, last, blockIdx.x, st, cyc, adaptive, eps);
+    cycle_block(nm, m, h_in, h_out, last, blockIdx.x, st, cyc, adaptive, eps);
 }
 
 // F = sum_k dS sigma.n, T = sum_k arm x (dS sigma.n) and the pressure part
@@ -982,19 +990,18 @@ __global__ void __launch_bounds__(ROWS_THREADS) k_batch_interp0_tiles(const RunD
     interp0_tile_block(R.box, R.nm, m, R.ba, m.tile_list, m.tile_count, R.cap, R.st, lb, warm);
 }
 
-__device__ __forceinline__ float *hsel(const MarkerArrays &m, int sel) {
-    return sel == HSEL_R0 ? m.r0 : (sel == HSEL_HL ? m.hl : m.hb);
+__device__ __forceinline__ float4 *hsel(const MarkerArrays &m, int sel) {
+    return sel == HSEL_R0 ? m.r0 : (sel == HSEL_HA ? m.ha : m.hb);
 }
 
 __global__ void __launch_bounds__(32 * INTERP_WARPS) k_batch_cycle(const RunDesc *__restrict__ runs,
                                                                    const int *__restrict__ prefix, int nruns, int p,
-                                                                   int sel_in, int sel_out, int sel_final, int last,
-                                                                   int cyc, int adaptive) {
+                                                                   int sel_in, int sel_out, int last, int cyc,
+                                                                   int adaptive) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
     const MarkerArrays &m = R.m[p ^ 1];
-    cycle_block(R.nm, m, hsel(m, sel_in), hsel(m, sel_out), sel_final >= 0 ? hsel(m, sel_final) : nullptr, last, lb, R.st,
-                cyc, adaptive, R.bc.slip_eps);
+    cycle_block(R.nm, m, hsel(m, sel_in), hsel(m, sel_out), last, lb, R.st, cyc, adaptive, R.bc.slip_eps);
 }
 
 __global__ void __launch_bounds__(288) k_batch_reduce_ft(const RunDesc *__restrict__ runs, int slot) {
@@ -1036,12 +1043,12 @@ cudaError_t launch_interp0(const BoxGeom &box, int nm, const MarkerArrays &m, co
 }
 
 // overlap: the second and later cycles start beside the one before.
-static cudaError_t launch_cycle(int nm, const MarkerArrays &m, const float *h_in, float *h_out, float *h_final, int last,
-                                DevState *st, int cyc, int adaptive, float eps, bool overlap, cudaStream_t s) {
+static cudaError_t launch_cycle(int nm, const MarkerArrays &m, const float4 *h_in, float4 *h_out, int last, DevState *st,
+                                int cyc, int adaptive, float eps, bool overlap, cudaStream_t s) {
     if (cyc > 0 && overlap)
-        return launch_pdl(k_cycle, (nm + INTERP_WARPS - 1) / INTERP_WARPS, 32 * INTERP_WARPS, s, nm, m, h_in, h_out, h_final,
-                          last, st, cyc, adaptive, eps);
-    k_cycle<<<(nm + INTERP_WARPS - 1) / INTERP_WARPS, 32 * INTERP_WARPS, 0, s>>>(nm, m, h_in, h_out, h_final, last,
+        return launch_pdl(k_cycle, (nm + INTERP_WARPS - 1) / INTERP_WARPS, 32 * INTERP_WARPS, s, nm, m, h_in, h_out, last, st,
+                          cyc, adaptive, eps);
+    k_cycle<<<(nm + INTERP_WARPS - 1) / INTERP_WARPS, 32 * INTERP_WARPS, 0, s>>>(nm, m, h_in, h_out, last,
                                                                                  st, cyc, adaptive, eps);
     return cudaGetLastError();
 }
@@ -1049,25 +1056,14 @@ static cudaError_t launch_cycle(int nm, const MarkerArrays &m, const float *h_in
 cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, bool overlap,
                           cudaStream_t s) {
     cudaError_t e = cudaSuccess;
-    if (!warm) {
-        // the paper's cycles: h^0 = r0, then cycles 1 .. n-1 alternating so
-        // that the last one writes hl
-        const float *src = m.r0;
-        for (int cyc = 1; cyc <= C && e == cudaSuccess; ++cyc) {
-            float *dst = ((C - cyc) % 2 == 0) ? m.hl : m.hb;
-            e = launch_cycle(nm, m, src, dst, nullptr, cyc == C, st, cyc - 1, 0, 0.0f, overlap, s);
-            src = dst;
-        }
-    } else {
-        // predictor modes: up to n cycles from the previous h (in hl), each
-        // skipped once the slip is below the tolerance; hl ends with the result
-        const float *src = m.hl;
-        for (int cyc = 1; cyc <= C && e == cudaSuccess; ++cyc) {
-            float *dst = (cyc % 2 == 1) ? m.hb : m.hl;
-            float *fin = (cyc == C && dst != m.hl) ? m.hl : nullptr;
-            e = launch_cycle(nm, m, src, dst, fin, cyc == C, st, cyc - 1, 1, eps, overlap, s);
-            src = dst;
-        }
+    // h alternates between ha and hb, starting from r0 or (warm) from the
+    // previous h in ha, each adaptive cycle skipped once the slip is below the
+    // tolerance; the last cycle writes hl
+    const float4 *src = warm ? m.ha : m.r0;
+    for (int cyc = 1; cyc <= C && e == cudaSuccess; ++cyc) {
+        float4 *dst = src == m.ha ? m.hb : m.ha;
+        e = launch_cycle(nm, m, src, dst, cyc == C, st, cyc - 1, warm, eps, overlap, s);
+        src = dst;
     }
     return e;
 }
@@ -1104,8 +1100,8 @@ cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nru
 }
 
 cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int sel_in,
-                               int sel_out, int sel_final, int last, int cyc, int adaptive, cudaStream_t s) {
-    k_batch_cycle<<<nblocks, 32 * INTERP_WARPS, 0, s>>>(runs, prefix, nruns, p, sel_in, sel_out, sel_final, last, cyc,
+                               int sel_out, int last, int cyc, int adaptive, cudaStream_t s) {
+    k_batch_cycle<<<nblocks, 32 * INTERP_WARPS, 0, s>>>(runs, prefix, nruns, p, sel_in, sel_out, last, cyc,
                                                         adaptive);
     return cudaGetLastError();
 }

@@ -179,11 +179,7 @@ __device__ __forceinline__ void moments_block(const Geom &g, const typename Code
         }
     }
     if (!inside) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) ba.u[k * box.nbox + b] = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) ba.s[k * box.nbox + b] = 0.0f;
-        ba.p[b] = 0.0f;
+        ba.u[b] = ba.s[2 * b] = ba.s[2 * b + 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         return;
     }
     float q[27];
@@ -193,16 +189,9 @@ __device__ __forceinline__ void moments_block(const Geom &g, const typename Code
     // (1/(2 tau) - 1) P1 with P1 = P1~ / 216 = P / (216 K)
     const float k2 = (0.5f / tau - 1.0f) * (INV_SCALE / Codec<ST>::K);
     const float p = M.drho * (1.0f / 3.0f);
-    ba.u[b] = M.ux;
-    ba.u[box.nbox + b] = M.uy;
-    ba.u[2 * box.nbox + b] = M.uz;
-    ba.s[b] = -p + k2 * M.Pxx;
-    ba.s[box.nbox + b] = -p + k2 * M.Pyy;
-    ba.s[2 * box.nbox + b] = -p + k2 * M.Pzz;
-    ba.s[3 * box.nbox + b] = k2 * M.Pxy;
-    ba.s[4 * box.nbox + b] = k2 * M.Pxz;
-    ba.s[5 * box.nbox + b] = k2 * M.Pyz;
-    ba.p[b] = p;
+    ba.u[b] = make_float4(M.ux, M.uy, M.uz, 0.0f);
+    ba.s[2 * b] = make_float4(-p + k2 * M.Pxx, -p + k2 * M.Pyy, -p + k2 * M.Pzz, k2 * M.Pxy);
+    ba.s[2 * b + 1] = make_float4(k2 * M.Pxz, k2 * M.Pyz, p, 0.0f);
 }
 
 }  // namespace turret

@@ -453,13 +453,13 @@ static size_t carve_ibm(Carver &cv, const IbmLayout &L, turret_ctx *c) {
     m.dSo = (const float *)cv.take(nm * 4);
     m.ft = (float *)cv.take(9 * nm * 4);
     m.hl = (float *)cv.take(3 * nm * 4);
-    m.r0 = (float *)cv.take(3 * nm * 4);
-    m.hb = (float *)cv.take(3 * nm * 4);
+    m.r0 = (float4 *)cv.take(nm * 16);
+    m.ha = (float4 *)cv.take(nm * 16);
+    m.hb = (float4 *)cv.take(nm * 16);
     m.force_eval = c ? c->flags.force_eval : 0;
     BoxArrays ba;
-    ba.u = (float *)cv.take(3 * nb * 4);
-    ba.s = (float *)cv.take(6 * nb * 4);
-    ba.p = (float *)cv.take(nb * 4);
+    ba.u = (float4 *)cv.take(nb * 16);
+    ba.s = (float4 *)cv.take(nb * 32);
     ba.h = (float *)cv.take(3 * nb * 4);
     MarkerArrays m2 = m;
     const size_t before = cv.off;
@@ -769,9 +769,8 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     CK(cudaMemsetAsync(c->ba.h, 0, 3 * (size_t)L.box.nbox * 4, c->stream), "h");
     // the moments kernel skips the box cells no stencil reads: they keep
     // finite values (zeros, or an earlier step's moments)
-    CK(cudaMemsetAsync(c->ba.u, 0, 3 * (size_t)L.box.nbox * 4, c->stream), "u");
-    CK(cudaMemsetAsync(c->ba.s, 0, 6 * (size_t)L.box.nbox * 4, c->stream), "sigma");
-    CK(cudaMemsetAsync(c->ba.p, 0, (size_t)L.box.nbox * 4, c->stream), "p");
+    CK(cudaMemsetAsync(c->ba.u, 0, (size_t)L.box.nbox * 16, c->stream), "u");
+    CK(cudaMemsetAsync(c->ba.s, 0, (size_t)L.box.nbox * 32, c->stream), "sigma");
     // rigid-body state at t: r(t), d = I, v(t-1/2) = v0, w(t-1/2) = w0, L = J w0
     CK(cudaMemcpyAsync(&c->host_state, c->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream), "state");
     CK(cudaStreamSynchronize(c->stream), "load sync");

@@ -170,8 +170,9 @@ struct MarkerArrays {
     float *n;          // [3][nm] lab-frame normal
     float *arm;        // [3][nm] X_k - C_m
     float *hl;         // [3][nm] Lagrangian IBM force (the last cycle's result)
-    float *r0;         // [3][nm] U_k - I[u*](X_k): the force of step l = 0
-    float *hb;         // [3][nm] second buffer of the cycles
+    // vectors that the cycles gather by column: one 16-byte load per entry
+    float4 *r0;        // [nm] U_k - I[u*](X_k): the force of step l = 0
+    float4 *ha, *hb;   // [nm] buffers of the cycles
     float *aval;       // [nm][ROWCAP] A_kj = dS_j sum_x W(x - X_k) W(x - X_j)
     int *aidx;         // [nm][ROWCAP] column j of each entry, in marker order
     int *alen;         // [nm] entries per row
@@ -183,9 +184,10 @@ struct MarkerArrays {
 };
 
 struct BoxArrays {
-    float *u;   // [3][nbox] u*
-    float *s;   // [6][nbox] sigma xx yy zz xy xz yz
-    float *p;   // [nbox] pressure c_s^2 (rho - 1)
+    // per cell, so that a stencil row of four cells is whole sectors and a cell
+    // of the interpolation is three 16-byte loads
+    float4 *u;  // [nbox] u*, 0
+    float4 *s;  // [nbox][2] sigma xx yy zz xy | xz yz, pressure c_s^2 (rho - 1), 0
     float *h;   // [3][nbox] spread force (h_imm after the last cycle)
 };
 
@@ -263,7 +265,7 @@ struct CollideDesc {
     int storage, split, tx, tx16;  // tx16: tile width of the 16-bit x-pair bulk launch (bulk16)
 };
 // h arrays of the IBM cycles, selected per run in batched launches
-enum { HSEL_R0 = 0, HSEL_HL = 1, HSEL_HB = 2 };
+enum { HSEL_R0 = 0, HSEL_HA = 1, HSEL_HB = 2 };
 
 // ---------------------------------------------------------------------------
 // D3Q27 index i = ex + 3 ey + 9 ez with e = xi + 1 in {0,1,2}; opposite 26 - i.
@@ -447,6 +449,7 @@ cudaError_t launch_interp0(const BoxGeom &box, int nm, const MarkerArrays &m, co
 // The C IBM cycles of a step, one launch each, h <- h + r0 - A h (= steps l =
 // 1..4), from r0 (warm 0) or from the previous h, adaptively (warm 1); the
 // result in m.hl.
+// (The initial h of the warm form is in m.ha, put there by the interpolation.)
 cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, bool overlap,
                           cudaStream_t s);
 // F = sum_k f_k, T = sum_k t_k in FP64, fixed order, into the device state.
@@ -461,7 +464,7 @@ cudaError_t launch_batch_particle_markers(const RunDesc *runs, const int *prefix
 cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int warm,
                                  cudaStream_t s);
 cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int sel_in,
-                               int sel_out, int sel_final, int last, int cyc, int adaptive, cudaStream_t s);
+                               int sel_out, int last, int cyc, int adaptive, cudaStream_t s);
 cudaError_t launch_batch_reduce_ft(const RunDesc *runs, int nruns, int slot, cudaStream_t s);
 cudaError_t launch_batch_predict(const RunDesc *runs, int nruns, int slot, cudaStream_t s);
 cudaError_t launch_batch_spread(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s);
