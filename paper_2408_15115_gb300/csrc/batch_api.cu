@@ -9,10 +9,10 @@
 //
 //   batch stream: --fork--> bulk collide+stream (far cells: FP32 runs, then
 //                           16-bit runs on x-pairs) --------------------------> join
-//   side stream :       \-> near collide+stream -> particle + markers
-//                           -> support moments + tile lists -> interpolation
-//                           + rows of A -> cycles -> spread ---------------^
-//   aux stream  :                         \-> F, T of every run (FP64) ---^
+//   aux stream  :       \-> [predictions] -> particle + markers -> tile lists
+//                           -> rows of A          ... -> F, T of every run (FP64) ^
+//   side stream :       \-> near collide+stream -> support moments
+//                           -> interpolation -> cycles -> spread ----------------^
 #include <cuda_runtime.h>
 #include <string.h>
 
@@ -29,7 +29,7 @@ using namespace turret;
 
 namespace {
 
-enum { T_BULK = 0, T_NEAR, T_PM, T_MB, T_IP, T_CYC, T_SP, T_BULK16, T_COUNT };
+enum { T_BULK = 0, T_NEAR, T_WHOLE, T_PM, T_MOM, T_BIN, T_ROWS, T_INT, T_CYC, T_SP, T_BULK16, T_COUNT };
 
 std::string g_batch_init_err;
 
@@ -39,7 +39,7 @@ struct turret_batch {
     int n;
     std::vector<turret_ctx *> ctx;
     cudaStream_t stream, side, aux;
-    cudaEvent_t ev_fork, ev_join, ev_red, ev_red_done, ev_done, ev_pred;
+    cudaEvent_t ev_fork, ev_join, ev_red, ev_red_done, ev_done, ev_pred, ev_rows;
     std::vector<cudaEvent_t> ev_ctx;  // one per run: the work already on its context's stream
     RunDesc *d_runs;
     CollideDesc *d_cdesc;             // the collide+stream part of each descriptor
@@ -93,10 +93,13 @@ static bool build_tables(turret_batch *b) {
             int k = 0;
             switch (t) {
                 case T_BULK: k = blocks_bulk(R, b->threads); break;
-                case T_NEAR: k = blocks_near(R, b->threads); break;
+                case T_NEAR: k = blocks_near(R); break;
+                case T_WHOLE: k = blocks_whole(R, b->threads); break;
                 case T_PM: k = blocks_particle_markers(R); break;
-                case T_MB: k = blocks_box_moments_bin(R); break;
-                case T_IP: k = blocks_interp0(R); break;
+                case T_MOM: k = blocks_box_moments(R); break;
+                case T_BIN: k = blocks_bin(R); break;
+                case T_ROWS: k = blocks_rows(R); break;
+                case T_INT: k = blocks_interp(R); break;
                 case T_CYC: k = blocks_cycle(R); break;
                 case T_SP: k = blocks_spread(R); break;
                 default: k = blocks_bulk16(R); break;
@@ -150,7 +153,7 @@ static void release_batch(turret_batch *b) {
     drop_batch_graphs(b);
     if (b->side) cudaStreamDestroy(b->side);
     if (b->aux) cudaStreamDestroy(b->aux);
-    cudaEvent_t evs[6] = {b->ev_fork, b->ev_join, b->ev_red, b->ev_red_done, b->ev_done, b->ev_pred};
+    cudaEvent_t evs[7] = {b->ev_fork, b->ev_join, b->ev_red, b->ev_red_done, b->ev_done, b->ev_pred, b->ev_rows};
     for (cudaEvent_t e : evs)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : b->ev_ctx)
@@ -186,7 +189,7 @@ extern "C" turret_status turret_batch_init(turret_batch **out, turret_ctx *const
     b->ctx.assign(ctxs, ctxs + n);
     b->stream = (cudaStream_t)stream;
     b->side = b->aux = nullptr;
-    b->ev_fork = b->ev_join = b->ev_red = b->ev_red_done = b->ev_done = b->ev_pred = nullptr;
+    b->ev_fork = b->ev_join = b->ev_red = b->ev_red_done = b->ev_done = b->ev_pred = b->ev_rows = nullptr;
     b->graph_ready[0] = b->graph_ready[1] = false;
     b->d_runs = (RunDesc *)ws;
     b->d_prefix = (int *)((char *)ws + prefix_offset(n));
@@ -227,9 +230,10 @@ extern "C" turret_status turret_batch_init(turret_batch **out, turret_ctx *const
     }
     int lo = 0, hi = 0;
     cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
+    if (e == cudaSuccess) e = prepare_batch_kernels();
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, hi);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->aux, cudaStreamNonBlocking, hi);
-    cudaEvent_t *evs[6] = {&b->ev_fork, &b->ev_join, &b->ev_red, &b->ev_red_done, &b->ev_done, &b->ev_pred};
+    cudaEvent_t *evs[7] = {&b->ev_fork, &b->ev_join, &b->ev_red, &b->ev_red_done, &b->ev_done, &b->ev_pred, &b->ev_rows};
     for (cudaEvent_t *ev : evs)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     b->ev_ctx.assign(n, nullptr);
@@ -285,17 +289,22 @@ static cudaError_t batch_enqueue(turret_batch *b, int p) {
     if (b->predictor) CE(launch_batch_predict(R, n, p, b->aux));
     CE(launch_batch_particle_markers(R, tab(T_PM), n, p, b->total[T_PM], b->aux));
     CE(cudaEventRecord(b->ev_pred, b->aux));
+    CE(launch_batch_bin(R, tab(T_BIN), n, p, b->total[T_BIN], b->aux));
+    CE(launch_batch_rows(R, tab(T_ROWS), n, p, b->total[T_ROWS], b->aux));
+    CE(cudaEventRecord(b->ev_rows, b->aux));
     CE(launch_batch_collide(PHASE_BULK, b->d_cdesc, tab(T_BULK), n, p, b->total[T_BULK], b->threads, b->minb,
                             b->stream));
     CE(launch_batch_collide(PHASE_BULK16, b->d_cdesc, tab(T_BULK16), n, p, b->total[T_BULK16], 128, 5, b->stream));
-    CE(launch_batch_collide(PHASE_NEAR, b->d_cdesc, tab(T_NEAR), n, p, b->total[T_NEAR], b->threads, 1, b->side));
+    CE(launch_batch_collide(PHASE_NEAR, b->d_cdesc, tab(T_NEAR), n, p, b->total[T_NEAR], NEAR_THREADS, 6, b->side));
+    CE(launch_batch_collide(PHASE_WHOLE, b->d_cdesc, tab(T_WHOLE), n, p, b->total[T_WHOLE], b->threads, 2, b->side));
     CE(cudaStreamWaitEvent(b->side, b->ev_pred, 0));
-    CE(launch_batch_box_moments_bin(R, tab(T_MB), n, p, b->total[T_MB], b->side));
-    CE(launch_batch_interp0(R, tab(T_IP), n, p, b->total[T_IP], b->warm, b->side));
+    CE(launch_batch_box_moments(R, tab(T_MOM), n, p, b->total[T_MOM], b->side));
+    CE(launch_batch_interp(R, tab(T_INT), n, p, b->total[T_INT], b->warm, b->side));
     CE(cudaEventRecord(b->ev_red, b->side));
     CE(cudaStreamWaitEvent(b->aux, b->ev_red, 0));
     CE(launch_batch_reduce_ft(R, n, p ^ 1, b->aux));
     CE(cudaEventRecord(b->ev_red_done, b->aux));
+    CE(cudaStreamWaitEvent(b->side, b->ev_rows, 0));
     // the cycles as in a single run (launch_cycles)
     const int C = b->cycles - (b->warm ? 0 : 1);
     int src = b->warm ? HSEL_HA : HSEL_R0;

@@ -10,8 +10,7 @@
 //                and each marker's 4x4x4 Peskin stencil (Sec. 2.2) in
 //                support-box coordinates.
 //   k_rows     : row k of the interaction matrix A of the IBM cycles, one block
-//                per marker (k_interp0_tiles: rows and interpolation by tiles,
-//                for batches).
+//                per marker (k_batch_rows: by tiles, for batches).
 //   k_interp   : I[u](X_k) = sum_x u(x) W(x - X_k) for u* and sigma, one warp per
 //                marker, two stencil cells per lane, xor-shuffle sums
 //                (deterministic); forms dS sigma.n and its moment about C_m for
@@ -534,21 +533,17 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(BoxGeom box, int nm, 
     interp_marker_warp(box, nm, m, ba, k, rk, threadIdx.x & 31, warm);
 }
 
-// The same step l = 0 and rows of A with one block per TILE^3 tile of the
-// support box, for batched launches (many markers, throughput-bound): the
-// block finds the markers whose stencil base lies in the tile (from the
-// tile's list 0, in marker order), interpolates each with one warp (the code
-// above), and builds their rows from the tile's list 1 staged once in shared
-// memory in chunks, one warp per marker and one candidate per lane with warp
-// ordered compaction.  Entries and their order equal those of interp0_block.
+// The rows of A with one block per TILE^3 tile of the support box, for batched
+// launches (many markers, throughput-bound): the block finds the markers whose
+// stencil base lies in the tile (from the tile's list 0, in marker order) and
+// builds their rows from the tile's list 1 staged once in shared memory in
+// chunks, one warp per marker and one candidate per lane with warp ordered
+// compaction.  Entries and their order equal those of rows_block.
 constexpr int IT_MAXB = 256;   // markers based in one tile
 constexpr int IT_STAGE = 256;  // candidates staged per chunk
 
-__device__ __forceinline__ void interp0_tile_block(const BoxGeom &box, int nm, const MarkerArrays &m,
-                                                   const BoxArrays &ba, const int *__restrict__ tile_list,
-                                                   const int *__restrict__ tile_count, int cap, DevState *st,
-                                                   int tile, int warm) {
-    if (tile == 0 && threadIdx.x < 8) st->pr.slip[threadIdx.x] = 0u;  // as k_interp
+__device__ __forceinline__ void rows_tile_block(const BoxGeom &box, const MarkerArrays &m, int cap, DevState *st, int tile) {
+    const int *__restrict__ tile_list = m.tile_list, *__restrict__ tile_count = m.tile_count;
     __shared__ int kb[IT_MAXB], klen[IT_MAXB];
     __shared__ int wc[ROWS_WARPS];
     __shared__ int nbased;
@@ -596,11 +591,6 @@ __device__ __forceinline__ void interp0_tile_block(const BoxGeom &box, int nm, c
     const int nb = nbased < IT_MAXB ? nbased : IT_MAXB;
     if (tid == 0 && nbased > IT_MAXB) atomicCAS(&st->status, 0, STAT_OVERFLOW);
     if (nb == 0) return;
-    for (int q = warp; q < nb; q += ROWS_WARPS) {
-        const int k = kb[q];
-        const MRec rk = m.rec[k];
-        interp_marker_warp(box, nm, m, ba, k, rk, lane, warm);
-    }
     for (int q = tid; q < nb; q += ROWS_THREADS) klen[q] = 0;
     for (int q = tid; q < 3 * 6 * IT_STAGE; q += ROWS_THREADS) {
         const int a = q / (6 * IT_STAGE), r = (q / IT_STAGE) % 6, j = q % IT_STAGE;
@@ -887,62 +877,86 @@ __global__ void __launch_bounds__(288) k_reduce_ft(int nm, const float *__restri
 }
 
 constexpr int SPREAD_SLICES = 8;                               // candidate slices per tile
-constexpr int SPREAD_THREADS = TILE * TILE * TILE * SPREAD_SLICES;  // 64 cells x 8 slices
+constexpr int SPREAD_CELLS = TILE * TILE * TILE;
 constexpr int SPREAD_STAGE = 256;
 
 // h_imm(x) = S[h](x) = sum_k W(x - X_k) h_k dS_k on the support box.  One block
 // per 4^3 tile: the tile's candidate records are staged in shared memory as
-// structure of arrays; thread (cell c, slice q) sums slice q of each staged
+// structure of arrays; thread (cell c, slices q) sums its slices of each staged
 // chunk for cell c; the 8 slice sums are added in slice order (reproducible).
+// PER slices per thread: 1 (512 threads, the shortest chain of additions) for a
+// single run, where the launch is latency; 4 (128 threads) for batches, where
+// most of the tens of thousands of tiles are empty and cost a block's start
+// (32 runs, 18,444 tiles: 91 us with 512 threads, 60 with 128).
+template <int PER>
 __device__ __forceinline__ void spread_block(const BoxGeom &box, const MRec *rec, const BoxArrays &ba,
                                              const int *__restrict__ tile_list, const int *__restrict__ tile_count,
                                              int cap, int tile) {
-    constexpr int TC = TILE * TILE * TILE;
+    constexpr int TC = SPREAD_CELLS, NT = TC * SPREAD_SLICES / PER, STAGE = NT < SPREAD_STAGE ? NT : SPREAD_STAGE;
     __shared__ int sbase[SPREAD_STAGE];
     __shared__ float sw[12][SPREAD_STAGE];
     __shared__ float sh[3][SPREAD_STAGE];
     __shared__ float part[SPREAD_SLICES][3][TC];
     const int cnt = tile_count[tile];
     const int tx = tile % box.tx, ty = (tile / box.tx) % box.ty, tz = tile / (box.tx * box.ty);
-    const int tid = threadIdx.x, c = tid % TC, q = tid / TC;
+    const int tid = threadIdx.x, c = tid % TC, q0 = tid / TC * PER;
     const int cx = TILE * tx + c % TILE, cy = TILE * ty + (c / TILE) % TILE, cz = TILE * tz + c / (TILE * TILE);
     const int *list = tile_list + (size_t)tile * cap;
-    float ax = 0.0f, ay = 0.0f, az = 0.0f;
-    int k = tid < min(SPREAD_STAGE, cnt) ? __ldg(list + tid) : 0;
+    float ax[PER], ay[PER], az[PER];
+#pragma unroll
+    for (int s = 0; s < PER; ++s) ax[s] = ay[s] = az[s] = 0.0f;
+    int k = tid < min(STAGE, cnt) ? __ldg(list + tid) : 0;
     pdl_wait();  // the records' h dS come from the last cycle
+    if (PER > 1 && cnt == 0) {  // an empty tile: zeros
+        if (tid < TC && cx < box.Bx && cy < box.By && cz < box.Bz) {
+            const size_t b = ((size_t)cz * box.By + cy) * box.Bx + cx;
+            ba.h[b] = ba.h[box.nbox + b] = ba.h[2 * box.nbox + b] = 0.0f;
+        }
+        return;
+    }
     for (int base = 0; base < cnt; base += SPREAD_STAGE) {
         const int n = min(SPREAD_STAGE, cnt - base);
-        if (tid < n) {
-            if (base > 0) k = __ldg(list + base + tid);
-            const MRec r = rec[k];
-            sbase[tid] = r.base;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                sw[e][tid] = r.wx[e];
-                sw[4 + e][tid] = r.wy[e];
-                sw[8 + e][tid] = r.wz[e];
+        for (int o = 0; o < SPREAD_STAGE; o += STAGE) {
+            const int i = o + tid;
+            if (tid < STAGE && i < n) {
+                if (base > 0 || o > 0) k = __ldg(list + base + i);
+                const MRec r = rec[k];
+                sbase[i] = r.base;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    sw[e][i] = r.wx[e];
+                    sw[4 + e][i] = r.wy[e];
+                    sw[8 + e][i] = r.wz[e];
+                }
+                sh[0][i] = r.hdS[0];
+                sh[1][i] = r.hdS[1];
+                sh[2][i] = r.hdS[2];
             }
-            sh[0][tid] = r.hdS[0];
-            sh[1][tid] = r.hdS[1];
-            sh[2][tid] = r.hdS[2];
         }
         __syncthreads();
-        const int j0 = (n * q) / SPREAD_SLICES, j1 = (n * (q + 1)) / SPREAD_SLICES;
-        for (int jj = j0; jj < j1; ++jj) {
-            const int pb = sbase[jj];
-            const int dx = cx - (pb & 1023), dy = cy - ((pb >> 10) & 1023), dz = cz - ((pb >> 20) & 1023);
-            if ((unsigned)dx < 4u && (unsigned)dy < 4u && (unsigned)dz < 4u) {
-                const float wv = sw[dx][jj] * sw[4 + dy][jj] * sw[8 + dz][jj];
-                ax = fmaf(wv, sh[0][jj], ax);
-                ay = fmaf(wv, sh[1][jj], ay);
-                az = fmaf(wv, sh[2][jj], az);
+#pragma unroll
+        for (int s = 0; s < PER; ++s) {
+            const int j0 = (n * (q0 + s)) / SPREAD_SLICES, j1 = (n * (q0 + s + 1)) / SPREAD_SLICES;
+            for (int jj = j0; jj < j1; ++jj) {
+                const int pb = sbase[jj];
+                const int dx = cx - (pb & 1023), dy = cy - ((pb >> 10) & 1023), dz = cz - ((pb >> 20) & 1023);
+                if ((unsigned)dx < 4u && (unsigned)dy < 4u && (unsigned)dz < 4u) {
+                    const float wv = sw[dx][jj] * sw[4 + dy][jj] * sw[8 + dz][jj];
+                    ax[s] = fmaf(wv, sh[0][jj], ax[s]);
+                    ay[s] = fmaf(wv, sh[1][jj], ay[s]);
+                    az[s] = fmaf(wv, sh[2][jj], az[s]);
+                }
             }
         }
         __syncthreads();
     }
-    part[q][0][c] = ax;
-    part[q][1][c] = ay;
-    part[q][2][c] = az;
+#pragma unroll
+    for (int s = 0; s < PER; ++s) {
+        part[q0 + s][0][c] = ax[s];
+        part[q0 + s][1][c] = ay[s];
+        part[q0 + s][2][c] = az[s];
+    }
     __syncthreads();
     if (tid < TC) {
         float hx = 0.0f, hy = 0.0f, hz = 0.0f;
@@ -961,11 +975,14 @@ __device__ __forceinline__ void spread_block(const BoxGeom &box, const MRec *rec
     }
 }
 
+constexpr int SPREAD_THREADS = SPREAD_CELLS * SPREAD_SLICES;
+constexpr int SPREAD_BATCH_PER = 4, SPREAD_BATCH_THREADS = SPREAD_THREADS / SPREAD_BATCH_PER;
+
 __global__ void __launch_bounds__(SPREAD_THREADS) k_spread(BoxGeom box, const MRec *rec, BoxArrays ba,
                                                            const int *__restrict__ tile_list,
                                                            const int *__restrict__ tile_count, int cap) {
     pdl_trigger();
-    spread_block(box, rec, ba, tile_list, tile_count, cap, blockIdx.x);
+    spread_block<1>(box, rec, ba, tile_list, tile_count, cap, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -981,13 +998,24 @@ __global__ void __launch_bounds__(PM_THREADS) k_batch_particle_markers(const Run
     pm_block(R.g, R.bc, R.box, R.st, p, 1, R.m[p ^ 1], lb);
 }
 
-__global__ void __launch_bounds__(ROWS_THREADS) k_batch_interp0_tiles(const RunDesc *__restrict__ runs,
-                                                                      const int *__restrict__ prefix, int nruns,
-                                                                      int p, int warm) {
+__global__ void __launch_bounds__(ROWS_THREADS) k_batch_rows(const RunDesc *__restrict__ runs,
+                                                             const int *__restrict__ prefix, int nruns, int p) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
+    rows_tile_block(R.box, R.m[p ^ 1], R.cap, R.st, lb);
+}
+
+__global__ void __launch_bounds__(32 * INTERP_WARPS) k_batch_interp(const RunDesc *__restrict__ runs,
+                                                                    const int *__restrict__ prefix, int nruns, int p,
+                                                                    int warm) {
+    int lb;
+    const RunDesc &R = runs[block_run(prefix, nruns, lb)];
+    if (lb == 0 && threadIdx.x < 8) R.st->pr.slip[threadIdx.x] = 0u;  // as k_interp
+    const int k = lb * INTERP_WARPS + (threadIdx.x >> 5);
+    if (k >= R.nm) return;
     const MarkerArrays &m = R.m[p ^ 1];
-    interp0_tile_block(R.box, R.nm, m, R.ba, m.tile_list, m.tile_count, R.cap, R.st, lb, warm);
+    const MRec rk = m.rec[k];
+    interp_marker_warp(R.box, R.nm, m, R.ba, k, rk, threadIdx.x & 31, warm);
 }
 
 __device__ __forceinline__ float4 *hsel(const MarkerArrays &m, int sel) {
@@ -1009,12 +1037,12 @@ __global__ void __launch_bounds__(288) k_batch_reduce_ft(const RunDesc *__restri
     reduce_block(R.nm, R.m[slot].ft, R.st, slot, R.bc.predictor, R.bc.pred_opts, R.bc.resid_theta, R.bc.log, R.bc.log_cap);
 }
 
-__global__ void __launch_bounds__(SPREAD_THREADS) k_batch_spread(const RunDesc *__restrict__ runs,
+__global__ void __launch_bounds__(SPREAD_BATCH_THREADS) k_batch_spread(const RunDesc *__restrict__ runs,
                                                                  const int *__restrict__ prefix, int nruns, int p) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
     const MarkerArrays &m = R.m[p ^ 1];
-    spread_block(R.box, m.rec, R.ba, m.tile_list, m.tile_count, R.cap, lb);
+    spread_block<SPREAD_BATCH_PER>(R.box, m.rec, R.ba, m.tile_list, m.tile_count, R.cap, lb);
 }
 
 // ---------------------------------------------------------------------------
@@ -1083,7 +1111,8 @@ cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxAr
 }
 
 int blocks_particle_markers(const RunDesc &r) { return (r.nm + PM_THREADS - 1) / PM_THREADS; }
-int blocks_interp0(const RunDesc &r) { return r.box.tx * r.box.ty * r.box.tz; }
+int blocks_rows(const RunDesc &r) { return r.box.tx * r.box.ty * r.box.tz; }
+int blocks_interp(const RunDesc &r) { return (r.nm + INTERP_WARPS - 1) / INTERP_WARPS; }
 int blocks_cycle(const RunDesc &r) { return (r.nm + INTERP_WARPS - 1) / INTERP_WARPS; }
 int blocks_spread(const RunDesc &r) { return r.box.tx * r.box.ty * r.box.tz; }
 
@@ -1093,9 +1122,14 @@ cudaError_t launch_batch_particle_markers(const RunDesc *runs, const int *prefix
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int warm,
-                                 cudaStream_t s) {
-    k_batch_interp0_tiles<<<nblocks, ROWS_THREADS, 0, s>>>(runs, prefix, nruns, p, warm);
+cudaError_t launch_batch_rows(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s) {
+    k_batch_rows<<<nblocks, ROWS_THREADS, 0, s>>>(runs, prefix, nruns, p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_interp(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int warm,
+                                cudaStream_t s) {
+    k_batch_interp<<<nblocks, 32 * INTERP_WARPS, 0, s>>>(runs, prefix, nruns, p, warm);
     return cudaGetLastError();
 }
 
@@ -1112,8 +1146,21 @@ cudaError_t launch_batch_reduce_ft(const RunDesc *runs, int nruns, int slot, cud
 }
 
 cudaError_t launch_batch_spread(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s) {
-    k_batch_spread<<<nblocks, SPREAD_THREADS, 0, s>>>(runs, prefix, nruns, p);
+    k_batch_spread<<<nblocks, SPREAD_BATCH_THREADS, 0, s>>>(runs, prefix, nruns, p);
     return cudaGetLastError();
+}
+
+// Shared-memory share of an SM asked for by the two chain kernels that use
+// much of it.  An SM changes its split between shared memory and L1 only when
+// it is idle, and the bulk launch enters while these run: left to the default
+// (as many blocks as fit, 210 KB), it then streams with almost no L1 to the
+// end (32 mixed runs, us per step: 1855 with the default, 1883 / 1625 / 1602 at
+// 25 / 50 / 62 %; the far cells alone need a quarter of the SM as L1).
+cudaError_t prepare_batch_kernels() {
+    constexpr int pct = 62;
+    cudaError_t e = cudaFuncSetAttribute(k_batch_rows, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_batch_spread, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+    return e;
 }
 
 }  // namespace turret

@@ -29,8 +29,9 @@ __global__ void __launch_bounds__(256, MINB) k_collide_tiled(Geom g, const typen
 // keeps its own storage type, window, boundary conditions, relaxation times
 // and tile, read from its descriptor.  PHASE_BULK: the far cells of runs that
 // split (no blocks for the others; 16-bit runs have theirs in the
-// PHASE_BULK16 launch); PHASE_NEAR: the near region of runs that
-// split, the whole window (with forcing) of runs that do not.
+// PHASE_BULK16 launch); PHASE_WHOLE: the whole window (with forcing) of runs
+// that do not split; the near region of runs that do has a kernel of its own
+// (k_batch_near).
 template <int PHASE, int ST>
 __device__ __forceinline__ void batch_k1_run(const CollideDesc &R, int p, int lb) {
     using T = typename Codec<ST>::T;
@@ -43,24 +44,13 @@ __device__ __forceinline__ void batch_k1_run(const CollideDesc &R, int p, int lb
     if (PHASE == PHASE_BULK) {
         tile_coords(lb, R.tx, g.nx, g.ny, 2, cx, cy, cz);
         k1_pair<ST, K1_FAR>(g, src, dst, R.utop[1 - p], R.utop[p], S, R.hbox, box, cx, cy, cz);
-    } else if (R.split) {
-        // the near region (a box of some 20-40 cells a side) as one flat range
-        // of cells, x fastest: every thread has a cell but those of the last block
-        const int ex = box.Bx + 2 * NEAR_GROW, ey = box.By + 2 * NEAR_GROW, ez = box.Bz + 2 * NEAR_GROW;
-        const int i = lb * (int)blockDim.x + (int)threadIdx.x;
-        if (i >= ex * ey * ez) return;
-        cx = i % ex;
-        cy = (i / ex) % ey;
-        cz = i / (ex * ey);
-        k1_cell<ST, K1_NEAR>(g, src, dst, R.utop[1 - p], R.utop[p], S, R.hbox, box, cx, cy, cz);
     } else {
         tile_coords(lb, R.tx, g.nx, g.ny, 2, cx, cy, cz);
         k1_pair<ST, K1_ALLF>(g, src, dst, R.utop[1 - p], R.utop[p], S, R.hbox, box, cx, cy, cz);
     }
 }
 
-// MINB: resident blocks of 256 threads per SM the register budget is sized
-// for (the near phase of a large batch is thousands of blocks: 2).
+// MINB: resident blocks of 256 threads per SM the register budget is sized for.
 template <int PHASE, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_batch_collide(const CollideDesc *__restrict__ runs,
                                                        const int *__restrict__ prefix, int nruns, int p) {
@@ -79,6 +69,40 @@ __global__ void __launch_bounds__(256, MINB) k_batch_collide(const CollideDesc *
         case ST_F32: batch_k1_run<PHASE, ST_F32>(R, p, lb); break;
         case ST_F16: batch_k1_run<PHASE, ST_F16>(R, p, lb); break;
         default: batch_k1_run<PHASE, ST_BF16>(R, p, lb); break;
+    }
+}
+
+// The near regions (boxes of some 20-40 cells a side) of the runs that split,
+// each as one flat range of cells, x fastest, one cell per thread.  A kernel of
+// its own for its registers: as a branch of the window kernel it was held to
+// the cell pairs' 128 (16 warps per SM, 95 us for 32 runs); at 80 the one-cell
+// code keeps 24 warps' loads in flight (85 us).
+template <int ST>
+__device__ __forceinline__ void batch_near_run(const CollideDesc &R, int p, int lb) {
+    using T = typename Codec<ST>::T;
+    const Geom g = R.g;
+    const BoxGeom box = R.box;
+    const int ex = box.Bx + 2 * NEAR_GROW, ey = box.By + 2 * NEAR_GROW, ez = box.Bz + 2 * NEAR_GROW;
+    const int i = lb * (int)blockDim.x + (int)threadIdx.x;
+    if (i >= ex * ey * ez) return;
+    k1_cell<ST, K1_NEAR>(g, (const T *)R.f[p], (T *)R.f[1 - p], R.utop[1 - p], R.utop[p], R.st->s[p], R.hbox, box, i % ex,
+                         (i / ex) % ey, i / (ex * ey));
+}
+
+__global__ void __launch_bounds__(NEAR_THREADS, 6) k_batch_near(const CollideDesc *__restrict__ runs,
+                                                                const int *__restrict__ prefix, int nruns, int p) {
+    constexpr int NW = (int)(sizeof(CollideDesc) / 4);
+    static_assert(sizeof(CollideDesc) % 4 == 0 && NW <= NEAR_THREADS, "descriptor staged by one load per thread");
+    __shared__ CollideDesc R;
+    int lb;
+    const int r = block_run(prefix, nruns, lb);
+    if (threadIdx.x < NW)
+        reinterpret_cast<int *>(&R)[threadIdx.x] = __ldg(reinterpret_cast<const int *>(runs + r) + threadIdx.x);
+    __syncthreads();
+    switch (R.storage) {
+        case ST_F32: batch_near_run<ST_F32>(R, p, lb); break;
+        case ST_F16: batch_near_run<ST_F16>(R, p, lb); break;
+        default: batch_near_run<ST_BF16>(R, p, lb); break;
     }
 }
 
@@ -124,23 +148,14 @@ __global__ void __launch_bounds__(128, 5) k_batch_collide16(const CollideDesc *_
     else batch_bulk16_run<ST_BF16>(R, p, lb);
 }
 
-// Batched K2 + binning: per run nmom(r) moment blocks then its tiles, on
-// f(t+1) in buffer 1 - p and window slot 1 - p (the advanced body).
-__global__ void __launch_bounds__(MB_THREADS) k_batch_box_moments_bin(const RunDesc *__restrict__ runs,
-                                                                      const int *__restrict__ prefix, int nruns,
-                                                                      int p) {
+// Batched K2, on f(t+1) in buffer 1 - p and window slot 1 - p (the advanced body).
+__global__ void __launch_bounds__(MB_THREADS) k_batch_box_moments(const RunDesc *__restrict__ runs,
+                                                                  const int *__restrict__ prefix, int nruns, int p) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
     const Geom g = R.g;
     const BoxGeom box = R.box;
-    const int nmom = (int)((box.nbox + MB_THREADS - 1) / MB_THREADS);
     const int so = 1 - p;
-    if (lb >= nmom) {
-        const MarkerArrays &m = R.m[so];
-        bin_block(R.st, so, box, R.nm, m.base, m.seg, m.tile_list, m.tile_count, R.cap, R.st, R.bc.rmin, R.bc.rmax,
-                  lb - nmom);
-        return;
-    }
     switch (R.storage) {
         case ST_F32:
             moments_block<ST_F32>(g, (const float *)R.f[1 - p], R.utop[p], R.st, so, box, R.ba, R.bc.rmin, R.bc.rmax, lb);
@@ -153,6 +168,14 @@ __global__ void __launch_bounds__(MB_THREADS) k_batch_box_moments_bin(const RunD
                                    R.bc.rmax, lb);
             break;
     }
+}
+
+__global__ void __launch_bounds__(MB_THREADS) k_batch_bin(const RunDesc *__restrict__ runs,
+                                                          const int *__restrict__ prefix, int nruns, int p) {
+    int lb;
+    const RunDesc &R = runs[block_run(prefix, nruns, lb)];
+    bin_warp(R.st, 1 - p, R.box, R.nm, R.m[1 - p], R.cap, R.st, R.bc.rmin, R.bc.rmax, lb * BIN_TILES + (threadIdx.x >> 5),
+             threadIdx.x & 31);
 }
 
 template <int ST, int MINB>
@@ -212,16 +235,19 @@ int blocks_bulk16(const RunDesc &r) {
     return bulk16_run(r) ? tile_blocks(r.g.nx, r.g.ny, r.g.nz, 128, bulk16_tile(r), 2) : 0;
 }
 
-int blocks_near(const RunDesc &r, int threads) {
-    if (!r.split) return tile_blocks(r.g.nx, r.g.ny, r.g.nz, threads, r.tx, 2);
-    const long long cells = (long long)(r.box.Bx + 2 * NEAR_GROW) * (r.box.By + 2 * NEAR_GROW) *
-                            (r.box.Bz + 2 * NEAR_GROW);
-    return (int)((cells + threads - 1) / threads);
+int blocks_whole(const RunDesc &r, int threads) {
+    return r.split ? 0 : tile_blocks(r.g.nx, r.g.ny, r.g.nz, threads, r.tx, 2);
 }
 
-int blocks_box_moments_bin(const RunDesc &r) {
-    return (int)((r.box.nbox + MB_THREADS - 1) / MB_THREADS) + r.box.tx * r.box.ty * r.box.tz;
+int blocks_near(const RunDesc &r) {
+    if (!r.split) return 0;
+    const long long cells = (long long)(r.box.Bx + 2 * NEAR_GROW) * (r.box.By + 2 * NEAR_GROW) *
+                            (r.box.Bz + 2 * NEAR_GROW);
+    return (int)((cells + NEAR_THREADS - 1) / NEAR_THREADS);
 }
+
+int blocks_box_moments(const RunDesc &r) { return (int)((r.box.nbox + MB_THREADS - 1) / MB_THREADS); }
+int blocks_bin(const RunDesc &r) { return (r.box.tx * r.box.ty * r.box.tz + BIN_TILES - 1) / BIN_TILES; }
 
 cudaError_t launch_batch_collide(int phase, const CollideDesc *runs, const int *prefix, int nruns, int p,
                                  int nblocks, int threads, int minb, cudaStream_t s) {
@@ -229,7 +255,9 @@ cudaError_t launch_batch_collide(int phase, const CollideDesc *runs, const int *
     if (phase == PHASE_BULK16)
         k_batch_collide16<<<nblocks, 128, 0, s>>>(runs, prefix, nruns, p);
     else if (phase == PHASE_NEAR)
-        k_batch_collide<PHASE_NEAR, 2><<<nblocks, threads, 0, s>>>(runs, prefix, nruns, p);
+        k_batch_near<<<nblocks, NEAR_THREADS, 0, s>>>(runs, prefix, nruns, p);
+    else if (phase == PHASE_WHOLE)
+        k_batch_collide<PHASE_WHOLE, 2><<<nblocks, threads, 0, s>>>(runs, prefix, nruns, p);
     else if (minb == 2)
         k_batch_collide<PHASE_BULK, 2><<<nblocks, threads, 0, s>>>(runs, prefix, nruns, p);
     else
@@ -242,10 +270,14 @@ bool is_batch_bulk_kernel(const void *fn) {
            fn == (const void *)k_batch_collide16;
 }
 
-cudaError_t launch_batch_box_moments_bin(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
-                                         cudaStream_t s) {
-    if (nblocks <= 0) return cudaSuccess;
-    k_batch_box_moments_bin<<<nblocks, MB_THREADS, 0, s>>>(runs, prefix, nruns, p);
+cudaError_t launch_batch_box_moments(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
+                                     cudaStream_t s) {
+    k_batch_box_moments<<<nblocks, MB_THREADS, 0, s>>>(runs, prefix, nruns, p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_bin(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s) {
+    k_batch_bin<<<nblocks, MB_THREADS, 0, s>>>(runs, prefix, nruns, p);
     return cudaGetLastError();
 }
 

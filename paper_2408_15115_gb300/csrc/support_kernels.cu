@@ -15,12 +15,11 @@ __global__ void __launch_bounds__(MB_THREADS) k_box_moments(Geom g, const typena
     moments_block<ST>(g, src, utop_in, st, slot, box, ba, rmin, rmax, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(MB_THREADS) k_bin(const DevState *st, int slot, BoxGeom box, int nm, const int *mbase,
-                                                    const int *mseg, int *tile_list, int *tile_count, int cap,
-                                                    DevState *stw, float rmin, float rmax) {
+__global__ void __launch_bounds__(MB_THREADS) k_bin(DevState *st, int slot, BoxGeom box, int nm, MarkerArrays m, int cap,
+                                                    float rmin, float rmax) {
     pdl_trigger();
     pdl_wait();
-    bin_block(st, slot, box, nm, mbase, mseg, tile_list, tile_count, cap, stw, rmin, rmax, blockIdx.x);
+    bin_block(st, slot, box, nm, m.base, m.seg, m.tile_list, m.tile_count, cap, st, rmin, rmax, blockIdx.x);
 }
 
 cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
@@ -36,11 +35,9 @@ cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, cons
 
 cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const MarkerArrays &m, int cap, float rmin,
                        float rmax, bool overlap, cudaStream_t s) {
-    if (overlap)
-        return launch_pdl(k_bin, box.tx * box.ty * box.tz, MB_THREADS, s, st, slot, box, nm, m.base, m.seg, m.tile_list,
-                          m.tile_count, cap, st, rmin, rmax);
-    k_bin<<<box.tx * box.ty * box.tz, MB_THREADS, 0, s>>>(st, slot, box, nm, m.base, m.seg, m.tile_list, m.tile_count, cap,
-                                                          st, rmin, rmax);
+    const unsigned nb = (unsigned)(box.tx * box.ty * box.tz);
+    if (overlap) return launch_pdl(k_bin, nb, MB_THREADS, s, st, slot, box, nm, m, cap, rmin, rmax);
+    k_bin<<<nb, MB_THREADS, 0, s>>>(st, slot, box, nm, m, cap, rmin, rmax);
     return cudaGetLastError();
 }
 

@@ -217,7 +217,8 @@ struct RunDesc {
     int tx;              // collide+stream tile width (threads along x)
     MlpDev mlp;          // the force/torque network (predictor mode 2)
 };
-enum { PHASE_BULK = 0, PHASE_NEAR = 1, PHASE_BULK16 = 2 };
+enum { PHASE_BULK = 0, PHASE_NEAR = 1, PHASE_BULK16 = 2, PHASE_WHOLE = 3 };
+constexpr int NEAR_THREADS = 128;  // block of the batched near phase
 
 // Run r of block b of a batched launch (largest r < nruns with prefix[r] <=
 // b) by one warp: each pass reads 32 table entries at once and narrows the
@@ -416,14 +417,15 @@ bool valid_tile(int threads, int tx, int minb);
 cudaError_t launch_collide_tiled(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
                                  float *utop_out, const DevState *st, int slot, const float *hbox,
                                  const BoxGeom &box, bool has_box, int threads, int tx, int minb, cudaStream_t s);
-// Batched K1 of phase PHASE_BULK, PHASE_NEAR or PHASE_BULK16 over nblocks
+// Batched K1 of one phase over nblocks
 // blocks (PHASE_BULK16: the far cells of 16-bit runs on x-adjacent pairs,
 // 128-thread blocks; threads and minb are ignored).
 cudaError_t launch_batch_collide(int phase, const CollideDesc *runs, const int *prefix, int nruns, int p,
                                  int nblocks, int threads, int minb, cudaStream_t s);
 bool is_batch_bulk_kernel(const void *fn);
-cudaError_t launch_batch_box_moments_bin(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
-                                         cudaStream_t s);
+cudaError_t launch_batch_box_moments(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
+                                     cudaStream_t s);
+cudaError_t launch_batch_bin(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s);
 // Support-box moments (u*, sigma), and the tile candidate lists.  Tiles that
 // no marker can reach (outside the shell rmin <= |X - C_m| <= rmax grown by
 // the stencil reach) get empty lists without a scan.
@@ -461,8 +463,9 @@ cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxAr
 // (time level p -> p ^ 1; blocks per run from the per-phase prefix table).
 cudaError_t launch_batch_particle_markers(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks,
                                           cudaStream_t s);
-cudaError_t launch_batch_interp0(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int warm,
-                                 cudaStream_t s);
+cudaError_t launch_batch_rows(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, cudaStream_t s);
+cudaError_t launch_batch_interp(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int warm,
+                                cudaStream_t s);
 cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns, int p, int nblocks, int sel_in,
                                int sel_out, int last, int cyc, int adaptive, cudaStream_t s);
 cudaError_t launch_batch_reduce_ft(const RunDesc *runs, int nruns, int slot, cudaStream_t s);
@@ -473,10 +476,13 @@ int blocks_bulk(const RunDesc &r, int threads);
 bool bulk16_run(const RunDesc &r);  // far cells in the 16-bit x-pair bulk launch
 int bulk16_tile(const RunDesc &r);  // its tile width
 int blocks_bulk16(const RunDesc &r);
-int blocks_near(const RunDesc &r, int threads);
+int blocks_near(const RunDesc &r);
+int blocks_whole(const RunDesc &r, int threads);
 int blocks_particle_markers(const RunDesc &r);
-int blocks_box_moments_bin(const RunDesc &r);
-int blocks_interp0(const RunDesc &r);
+int blocks_box_moments(const RunDesc &r);
+int blocks_bin(const RunDesc &r);
+int blocks_rows(const RunDesc &r);
+int blocks_interp(const RunDesc &r);
 int blocks_cycle(const RunDesc &r);
 int blocks_spread(const RunDesc &r);
 
@@ -486,6 +492,7 @@ cudaError_t launch_mlp_infer(const MlpDev &w, const float *x, int n, float *y, c
 // (mode 1 linear, 2 network w; w may be null), single run or every run.
 cudaError_t launch_predict(const MlpDev *w, DevState *st, int slot, int mode, cudaStream_t s);
 
+cudaError_t prepare_batch_kernels();
 constexpr int TILE = 4;          // support-box tiles of TILE^3 cells (spreading)
 constexpr int INTERP_WARPS = 8;  // markers per interpolation block
 constexpr int MAX_CANDIDATES = 2048;  // markers listed per support tile
