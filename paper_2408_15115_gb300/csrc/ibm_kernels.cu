@@ -46,7 +46,7 @@ constexpr int PM_THREADS = MARKER_SEG;
 // in the other slot, so the marker work spreads over many SMs with no
 // grid-wide wait.
 __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, const BoxGeom &box, DevState *st,
-                                         int slot, int advance, const MarkerArrays &m, int blk) {
+                                         int slot, int advance, const MarkerArrays &m, BodySlot *fwd, int blk) {
     __shared__ BodySlot S;  // the body at the markers' time level
     __shared__ double s_F[3], s_T[3], s_src[3], s_sb[3], s_wb[3], s_mid[9];
     __shared__ float f_d[9], f_v[3], f_w[3], f_cf[3];
@@ -159,7 +159,10 @@ __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, con
             if (blk == 0) {
                 int *gdst = reinterpret_cast<int *>(&st->s[so]);
                 const int *ssrc = reinterpret_cast<const int *>(&S);
-                for (int q = lane; q < (int)(sizeof(BodySlot) / 4); q += 32) gdst[q] = ssrc[q];
+                for (int q = lane; q < (int)(sizeof(BodySlot) / 4); q += 32) {
+                    gdst[q] = ssrc[q];
+                    if (fwd) reinterpret_cast<int *>(fwd)[q] = ssrc[q];
+                }
             }
         }
         // marker velocities: v, w at t + 1/2 (the paper's step), or in the
@@ -305,9 +308,10 @@ __device__ __forceinline__ void pm_block(const Geom &g, const BodyConst &bc, con
 }
 
 __global__ void __launch_bounds__(PM_THREADS) k_particle_markers(Geom g, BodyConst bc, BoxGeom box, DevState *st,
-                                                                  int slot, int advance, MarkerArrays m) {
+                                                                  int slot, int advance, MarkerArrays m,
+                                                                  BodySlot *fwd) {
     pdl_trigger();
-    pm_block(g, bc, box, st, slot, advance, m, blockIdx.x);
+    pm_block(g, bc, box, st, slot, advance, m, fwd, blockIdx.x);
 }
 
 __device__ __forceinline__ float pick4(const float w[4], int i) {
@@ -767,16 +771,20 @@ __global__ void __launch_bounds__(32 * INTERP_WARPS) k_cycle(int nm, MarkerArray
 }
 
 // F = sum_k dS sigma.n, T = sum_k arm x (dS sigma.n) and the pressure part
-// Fp = sum_k -dS p n in FP64: warp c (of 9) sums component c, lane l the
-// markers l, l+32, ... in order, then an xor tree.
-// Then, in thread 0: the relative error of the prediction made for this time
-// level (predictor modes: a large one switches the next prediction to the
-// linear one), the force/torque history, and the trajectory record of time
-// level st->s[slot] (when a log is attached).
+// Fp = sum_k -dS p n in FP64: one warp and block per component (nine), lane l
+// the markers l, l+32, ... in order, then an xor tree.  An SM adds two FP64
+// values per clock, so nine warps on one SM took 41 us for 6762 markers and 15
+// us for 1000 beside the bulk launch, on the way to the next particle update;
+// on nine SMs 9 us beside it.
+// Then, in the last block to finish: the relative error of the prediction made
+// for this time level (predictor modes: a large one switches the next
+// prediction to the linear one), the force/torque history, and the trajectory
+// record of time level st->s[slot] (when a log is attached).
+constexpr int REDUCE_COMPONENTS = 9;
 __device__ __forceinline__ void reduce_block(int nm, const float *__restrict__ ft, DevState *st, int slot,
                                              int predictor, int opts, double theta, double *__restrict__ log,
-                                             long long log_cap) {
-    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                                             long long log_cap, int c) {
+    const int lane = threadIdx.x;
     // eight independent partial sums per lane, so that eight loads are in
     // flight at a time; combined in a fixed order (reproducible)
     double a8[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -795,19 +803,26 @@ __device__ __forceinline__ void reduce_block(int nm, const float *__restrict__ f
     double a = ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) {
-        if (c < 3) st->F[c] = a; else if (c < 6) st->T[c - 3] = a; else st->Fp[c - 6] = a;
-        if (!isfinite(a)) atomicCAS(&st->status, 0, STAT_DIVERGED);
+    if (lane != 0) return;
+    if (c < 3) st->F[c] = a; else if (c < 6) st->T[c - 3] = a; else st->Fp[c - 6] = a;
+    if (!isfinite(a)) atomicCAS(&st->status, 0, STAT_DIVERGED);
+    __threadfence();
+    if (atomicAdd(&st->counter, 1u) != REDUCE_COMPONENTS - 1) return;
+    __threadfence();
+    st->counter = 0u;  // every block has counted: ready for the next reduction
+    // F and T of the other blocks, from L2
+    double Fn[3], Tn[3];
+    for (int q = 0; q < 3; ++q) {
+        Fn[q] = __ldcg(&st->F[q]);
+        Tn[q] = __ldcg(&st->T[q]);
     }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
     Predictor &P = st->pr;
     double resid = -1.0, resid_net = -1.0, made = -1.0, fh[6] = {0, 0, 0, 0, 0, 0};
     auto rel_err = [&](const double *Fp) {
         double num = 0.0, den = 0.0;
         for (int q = 0; q < 3; ++q) {
-            num += (st->F[q] - Fp[q]) * (st->F[q] - Fp[q]);
-            den += st->F[q] * st->F[q];
+            num += (Fn[q] - Fp[q]) * (Fn[q] - Fp[q]);
+            den += Fn[q] * Fn[q];
         }
         return den > 0.0 ? sqrt(num / den) : (num > 0.0 ? INFINITY : 0.0);
     };
@@ -846,8 +861,8 @@ __device__ __forceinline__ void reduce_block(int nm, const float *__restrict__ f
             P.Th[h][q] = P.Th[h - 1][q];
         }
     for (int q = 0; q < 3; ++q) {
-        P.Fh[0][q] = st->F[q];
-        P.Th[0][q] = st->T[q];
+        P.Fh[0][q] = Fn[q];
+        P.Th[0][q] = Tn[q];
     }
     P.hist_n = P.hist_n < 4 ? P.hist_n + 1 : 4;
     if (log && log_cap > 0) {
@@ -857,8 +872,8 @@ __device__ __forceinline__ void reduce_block(int nm, const float *__restrict__ f
         for (int q = 0; q < 3; ++q) {
             r[9 + q] = S.v[q];
             r[12 + q] = S.w[q];
-            r[15 + q] = st->F[q];
-            r[18 + q] = st->T[q];
+            r[15 + q] = Fn[q];
+            r[18 + q] = Tn[q];
         }
         r[21] = (double)S.step;
         r[22] = resid;
@@ -870,10 +885,10 @@ __device__ __forceinline__ void reduce_block(int nm, const float *__restrict__ f
     P.logged += 1;
 }
 
-__global__ void __launch_bounds__(288) k_reduce_ft(int nm, const float *__restrict__ ft, DevState *st, int slot,
+__global__ void __launch_bounds__(32) k_reduce_ft(int nm, const float *__restrict__ ft, DevState *st, int slot,
                                                    int predictor, int opts, double theta,
                                                    double *__restrict__ log, long long log_cap) {
-    reduce_block(nm, ft, st, slot, predictor, opts, theta, log, log_cap);
+    reduce_block(nm, ft, st, slot, predictor, opts, theta, log, log_cap, blockIdx.x);
 }
 
 constexpr int SPREAD_SLICES = 8;                               // candidate slices per tile
@@ -887,7 +902,10 @@ constexpr int SPREAD_STAGE = 256;
 // PER slices per thread: 1 (512 threads, the shortest chain of additions) for a
 // single run, where the launch is latency; 4 (128 threads) for batches, where
 // most of the tens of thousands of tiles are empty and cost a block's start
-// (32 runs, 18,444 tiles: 91 us with 512 threads, 60 with 128).
+// (32 runs, 18,444 tiles: 91 us with 512 threads, 60 with 128).  (128 threads in
+// a single run: 96x96x192, 24 steps, 2171 us instead of 2066, and with the
+// default shared-memory split, which so many blocks draw to its largest, 256x256x512
+// 25.4 ms instead of 19.2: the far cells then stream without L1.)
 template <int PER>
 __device__ __forceinline__ void spread_block(const BoxGeom &box, const MRec *rec, const BoxArrays &ba,
                                              const int *__restrict__ tile_list, const int *__restrict__ tile_count,
@@ -995,7 +1013,7 @@ __global__ void __launch_bounds__(PM_THREADS) k_batch_particle_markers(const Run
                                                                         int p) {
     int lb;
     const RunDesc &R = runs[block_run(prefix, nruns, lb)];
-    pm_block(R.g, R.bc, R.box, R.st, p, 1, R.m[p ^ 1], lb);
+    pm_block(R.g, R.bc, R.box, R.st, p, 1, R.m[p ^ 1], nullptr, lb);
 }
 
 __global__ void __launch_bounds__(ROWS_THREADS) k_batch_rows(const RunDesc *__restrict__ runs,
@@ -1032,9 +1050,10 @@ __global__ void __launch_bounds__(32 * INTERP_WARPS) k_batch_cycle(const RunDesc
     cycle_block(R.nm, m, hsel(m, sel_in), hsel(m, sel_out), last, lb, R.st, cyc, adaptive, R.bc.slip_eps);
 }
 
-__global__ void __launch_bounds__(288) k_batch_reduce_ft(const RunDesc *__restrict__ runs, int slot) {
-    const RunDesc &R = runs[blockIdx.x];
-    reduce_block(R.nm, R.m[slot].ft, R.st, slot, R.bc.predictor, R.bc.pred_opts, R.bc.resid_theta, R.bc.log, R.bc.log_cap);
+__global__ void __launch_bounds__(32) k_batch_reduce_ft(const RunDesc *__restrict__ runs, int slot) {
+    const RunDesc &R = runs[blockIdx.x / REDUCE_COMPONENTS];
+    reduce_block(R.nm, R.m[slot].ft, R.st, slot, R.bc.predictor, R.bc.pred_opts, R.bc.resid_theta, R.bc.log, R.bc.log_cap,
+                 blockIdx.x % REDUCE_COMPONENTS);
 }
 
 __global__ void __launch_bounds__(SPREAD_BATCH_THREADS) k_batch_spread(const RunDesc *__restrict__ runs,
@@ -1047,8 +1066,8 @@ __global__ void __launch_bounds__(SPREAD_BATCH_THREADS) k_batch_spread(const Run
 
 // ---------------------------------------------------------------------------
 cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const BoxGeom &box, DevState *st, int slot,
-                                    int advance, MarkerArrays m, cudaStream_t s) {
-    k_particle_markers<<<(bc.nm + PM_THREADS - 1) / PM_THREADS, PM_THREADS, 0, s>>>(g, bc, box, st, slot, advance, m);
+                                    int advance, MarkerArrays m, BodySlot *fwd, cudaStream_t s) {
+    k_particle_markers<<<(bc.nm + PM_THREADS - 1) / PM_THREADS, PM_THREADS, 0, s>>>(g, bc, box, st, slot, advance, m, fwd);
     return cudaGetLastError();
 }
 
@@ -1097,7 +1116,7 @@ cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevSta
 }
 
 cudaError_t launch_reduce_ft(int nm, MarkerArrays m, DevState *st, int slot, const BodyConst &bc, cudaStream_t s) {
-    k_reduce_ft<<<1, 288, 0, s>>>(nm, m.ft, st, slot, bc.predictor, bc.pred_opts, bc.resid_theta, bc.log, bc.log_cap);
+    k_reduce_ft<<<REDUCE_COMPONENTS, 32, 0, s>>>(nm, m.ft, st, slot, bc.predictor, bc.pred_opts, bc.resid_theta, bc.log, bc.log_cap);
     return cudaGetLastError();
 }
 
@@ -1141,7 +1160,7 @@ cudaError_t launch_batch_cycle(const RunDesc *runs, const int *prefix, int nruns
 }
 
 cudaError_t launch_batch_reduce_ft(const RunDesc *runs, int nruns, int slot, cudaStream_t s) {
-    k_batch_reduce_ft<<<nruns, 288, 0, s>>>(runs, slot);
+    k_batch_reduce_ft<<<nruns * REDUCE_COMPONENTS, 32, 0, s>>>(runs, slot);
     return cudaGetLastError();
 }
 

@@ -4,6 +4,21 @@
 
 namespace turret {
 
+// The near region as one flat range of cells, x fastest: every thread but those
+// of the last block has a cell (rows of 26 to 46 cells leave 19 to 28 % of the
+// lanes of 32-wide rows idle, and the launch of a large body a second, nearly
+// empty wave: 46^3 cells 1152 blocks on 912 places, 761 flat).
+template <int ST>
+__device__ __forceinline__ void near_cell(const Geom &g, const typename Codec<ST>::T *__restrict__ src,
+                                          typename Codec<ST>::T *__restrict__ dst, const float *__restrict__ utop_in,
+                                          float *__restrict__ utop_out, const BodySlot &S,
+                                          const float *__restrict__ hbox, const BoxGeom &box) {
+    const int ex = box.Bx + 2 * NEAR_GROW, ey = box.By + 2 * NEAR_GROW, ez = box.Bz + 2 * NEAR_GROW;
+    const int i = blockIdx.x * 128 + threadIdx.y * 32 + threadIdx.x;
+    if (i < ex * ey * ez)
+        k1_cell<ST, K1_NEAR>(g, src, dst, utop_in, utop_out, S, hbox, box, i % ex, (i / ex) % ey, i / (ex * ey));
+}
+
 // Window launches with 16-bit storage: five blocks per SM (<= 102 registers, a
 // few spilled values in L1) measured faster than four; FP32 keeps four (128
 // registers, no spill); the small near-region launch is left unconstrained.
@@ -11,23 +26,22 @@ template <int ST, int MODE>
 __global__ void __launch_bounds__(128, MODE == K1_NEAR ? 1 : (ST == ST_F32 ? 4 : 5)) k_collide_stream(Geom g, const typename Codec<ST>::T *__restrict__ src,
                                                         typename Codec<ST>::T *__restrict__ dst,
                                                         const float *__restrict__ utop_in,
-                                                        float *__restrict__ utop_out, DevState *st, int slot,
-                                                        int slot_out, const float *__restrict__ hbox, BoxGeom box,
+                                                        float *__restrict__ utop_out, DevState *st,
+                                                        const BodySlot *win, int slot_out, const float *__restrict__ hbox, BoxGeom box,
                                                         int flat) {
     if (slot_out >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 &&
         threadIdx.y == 0) {
         // carry the body and window to the next time level (no entering plane there)
-        st->s[slot_out] = st->s[slot];
+        st->s[slot_out] = *win;
         st->s[slot_out].reseed = -1;
         st->s[slot_out].step += 1;
     }
     if (MODE == K1_NEAR)  // small, on the critical path: one cell per thread
-        k1_cell<ST, MODE>(g, src, dst, utop_in, utop_out, st->s[slot], hbox, box, blockIdx.x * 32 + threadIdx.x,
-                          blockIdx.y * 4 + threadIdx.y, blockIdx.z);
+        near_cell<ST>(g, src, dst, utop_in, utop_out, *win, hbox, box);
     else {  // the window: a pair of planes per thread
         int cx, cy;
         window_cell(g, flat, cx, cy);
-        k1_pair<ST, MODE>(g, src, dst, utop_in, utop_out, st->s[slot], hbox, box, cx, cy, 2 * blockIdx.z);
+        k1_pair<ST, MODE>(g, src, dst, utop_in, utop_out, *win, hbox, box, cx, cy, 2 * blockIdx.z);
     }
 }
 
@@ -90,38 +104,38 @@ __global__ void __launch_bounds__(128) k_macro(Geom g, const typename Codec<ST>:
 // Launchers.
 static dim3 near_grid(const BoxGeom &b) {
     const int ex = b.Bx + 2 * NEAR_GROW, ey = b.By + 2 * NEAR_GROW, ez = b.Bz + 2 * NEAR_GROW;
-    return dim3((ex + 31) / 32, (ey + 3) / 4, ez);
+    return dim3((unsigned)(((long long)ex * ey * ez + 127) / 128));
 }
 
 template <int ST>
 static cudaError_t collide_t(const Geom &g, const void *src, void *dst, const float *utop_in, float *utop_out,
-                             DevState *st, int slot, int slot_out, const float *hbox, const BoxGeom &box,
+                             DevState *st, const BodySlot *win, int slot_out, const float *hbox, const BoxGeom &box,
                              bool has_box, int region, cudaStream_t s, bool after_spread) {
     using T = typename Codec<ST>::T;
     const dim3 blk(32, 4);
     const T *fs = (const T *)src;
     T *fd = (T *)dst;
     if (region == REGION_NEAR && after_spread)
-        return launch_pdl(k_collide_stream<ST, K1_NEAR>, near_grid(box), blk, s, g, fs, fd, utop_in, utop_out, st, slot,
+        return launch_pdl(k_collide_stream<ST, K1_NEAR>, near_grid(box), blk, s, g, fs, fd, utop_in, utop_out, st, win,
                           slot_out, hbox, box, 0);
     if (region == REGION_NEAR)
-        k_collide_stream<ST, K1_NEAR><<<near_grid(box), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
+        k_collide_stream<ST, K1_NEAR><<<near_grid(box), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, win, slot_out, hbox, box, window_flat(g, ST));
     else if (region == REGION_FAR)
-        k_collide_stream<ST, K1_FAR><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
+        k_collide_stream<ST, K1_FAR><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, win, slot_out, hbox, box, window_flat(g, ST));
     else if (has_box)
-        k_collide_stream<ST, K1_ALLF><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
+        k_collide_stream<ST, K1_ALLF><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, win, slot_out, hbox, box, window_flat(g, ST));
     else
-        k_collide_stream<ST, K1_ALL><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, slot, slot_out, hbox, box, window_flat(g, ST));
+        k_collide_stream<ST, K1_ALL><<<window_grid(g, ST, (g.nz + 1) / 2), blk, 0, s>>>(g, fs, fd, utop_in, utop_out, st, win, slot_out, hbox, box, window_flat(g, ST));
     return cudaGetLastError();
 }
 
 cudaError_t launch_collide_stream(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
-                                  float *utop_out, DevState *st, int slot, int slot_out, const float *hbox,
+                                  float *utop_out, DevState *st, const BodySlot *win, int slot_out, const float *hbox,
                                   const BoxGeom &box, bool has_box, int region, cudaStream_t s, bool after_spread) {
     switch (storage) {
-        case ST_F32: return collide_t<ST_F32>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
-        case ST_F16: return collide_t<ST_F16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
-        default: return collide_t<ST_BF16>(g, src, dst, utop_in, utop_out, st, slot, slot_out, hbox, box, has_box, region, s, after_spread);
+        case ST_F32: return collide_t<ST_F32>(g, src, dst, utop_in, utop_out, st, win, slot_out, hbox, box, has_box, region, s, after_spread);
+        case ST_F16: return collide_t<ST_F16>(g, src, dst, utop_in, utop_out, st, win, slot_out, hbox, box, has_box, region, s, after_spread);
+        default: return collide_t<ST_BF16>(g, src, dst, utop_in, utop_out, st, win, slot_out, hbox, box, has_box, region, s, after_spread);
     }
 }
 

@@ -315,7 +315,7 @@ template <int ST, int MODE>
 __global__ void __launch_bounds__(STG_CONS + 32, 3)
     k_collide_staged(const __grid_constant__ CUtensorMap lmap, const __grid_constant__ CUtensorMap smap, Geom g,
                      const typename Codec<ST>::T *__restrict__ src, typename Codec<ST>::T *__restrict__ dst,
-                     const float *__restrict__ utop_in, float *__restrict__ utop_out, DevState *st, int slot,
+                     const float *__restrict__ utop_in, float *__restrict__ utop_out, DevState *st, const BodySlot *win,
                      int slot_out, const float *__restrict__ hbox, BoxGeom box) {
     extern __shared__ __align__(128) unsigned char stg_smem[];
     unsigned short *in = reinterpret_cast<unsigned short *>(stg_smem);  // [STG_NS][27][STG_BOX] sources
@@ -325,11 +325,11 @@ __global__ void __launch_bounds__(STG_CONS + 32, 3)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (MODE == K1_ALL && slot_out >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 &&
         threadIdx.x == 0) {
-        st->s[slot_out] = st->s[slot];
+        st->s[slot_out] = *win;
         st->s[slot_out].reseed = -1;
         st->s[slot_out].step += 1;
     }
-    const BodySlot &S = st->s[slot];
+    const BodySlot &S = *win;
     const int x0 = blockIdx.x * STG_TX, y0 = blockIdx.y * STG_TY, zb = blockIdx.z * (STG_TZ * STG_TPB);
     const int ntile = min(STG_TPB, (g.nz - zb + STG_TZ - 1) / STG_TZ);
     if (threadIdx.x == 0) {
@@ -461,7 +461,7 @@ bool is_staged_kernel(const void *fn) {
 
 cudaError_t launch_collide_staged(const Geom &g, int storage, const CUtensorMap &lmap, const CUtensorMap &smap,
                                   const void *src, void *dst, const float *utop_in, float *utop_out, DevState *st,
-                                  int slot, int slot_out, const float *hbox, const BoxGeom &box, int region,
+                                  const BodySlot *win, int slot_out, const float *hbox, const BoxGeom &box, int region,
                                   cudaStream_t s) {
     const dim3 grid(g.nx / STG_TX, g.ny / STG_TY, (g.nz + STG_TZ * STG_TPB - 1) / (STG_TZ * STG_TPB));
     const dim3 blk(STG_CONS + 32);
@@ -469,18 +469,18 @@ cudaError_t launch_collide_staged(const Geom &g, int storage, const CUtensorMap 
         using T = __half;
         if (region == REGION_FAR)
             k_collide_staged<ST_F16, K1_FAR><<<grid, blk, STG_SMEM, s>>>(lmap, smap, g, (const T *)src, (T *)dst, utop_in,
-                                                                         utop_out, st, slot, -1, hbox, box);
+                                                                         utop_out, st, win, -1, hbox, box);
         else
             k_collide_staged<ST_F16, K1_ALL><<<grid, blk, STG_SMEM, s>>>(lmap, smap, g, (const T *)src, (T *)dst, utop_in,
-                                                                         utop_out, st, slot, slot_out, hbox, box);
+                                                                         utop_out, st, win, slot_out, hbox, box);
     } else {
         using T = __nv_bfloat16;
         if (region == REGION_FAR)
             k_collide_staged<ST_BF16, K1_FAR><<<grid, blk, STG_SMEM, s>>>(lmap, smap, g, (const T *)src, (T *)dst,
-                                                                          utop_in, utop_out, st, slot, -1, hbox, box);
+                                                                          utop_in, utop_out, st, win, -1, hbox, box);
         else
             k_collide_staged<ST_BF16, K1_ALL><<<grid, blk, STG_SMEM, s>>>(
-                lmap, smap, g, (const T *)src, (T *)dst, utop_in, utop_out, st, slot, slot_out, hbox, box);
+                lmap, smap, g, (const T *)src, (T *)dst, utop_in, utop_out, st, win, slot_out, hbox, box);
     }
     return cudaGetLastError();
 }

@@ -26,16 +26,16 @@ constexpr int XP_TX = 64, XP_TY = 2, XP_TZ = 2;  // cells per tile: 32 x 4 threa
 template <int ST, int MODE>
 __global__ void __launch_bounds__(128, 5)
     k_collide_xpair(Geom g, const typename Codec<ST>::T *__restrict__ src, typename Codec<ST>::T *__restrict__ dst,
-                    const float *__restrict__ utop_in, float *__restrict__ utop_out, DevState *st, int slot,
+                    const float *__restrict__ utop_in, float *__restrict__ utop_out, DevState *st, const BodySlot *win,
                     int slot_out, const float *__restrict__ hbox, BoxGeom box) {
     const int tx = threadIdx.x, ty = threadIdx.y;
     if (MODE == K1_ALL && slot_out >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tx == 0 &&
         ty == 0) {
-        st->s[slot_out] = st->s[slot];
+        st->s[slot_out] = *win;
         st->s[slot_out].reseed = -1;
         st->s[slot_out].step += 1;
     }
-    const BodySlot &S = st->s[slot];
+    const BodySlot &S = *win;
     const int x0 = blockIdx.x * XP_TX, y0 = blockIdx.y * XP_TY, z0 = XP_TZ * blockIdx.z;
     if (!xpair_tile_ok<MODE, false>(g, S, box, x0, y0, z0, XP_TX, XP_TY)) {
         // the one-cell path: thread t takes column t of the tile, both planes.
@@ -59,25 +59,25 @@ bool xpair_eligible(const Geom &g, int storage) {
 }
 
 cudaError_t launch_collide_xpair(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
-                                 float *utop_out, DevState *st, int slot, int slot_out, const float *hbox,
+                                 float *utop_out, DevState *st, const BodySlot *win, int slot_out, const float *hbox,
                                  const BoxGeom &box, int region, cudaStream_t s) {
     const dim3 grid(g.nx / XP_TX, g.ny / XP_TY, g.nz / XP_TZ), blk(32, 4);
     if (storage == ST_F16) {
         using T = __half;
         if (region == REGION_FAR)
             k_collide_xpair<ST_F16, K1_FAR><<<grid, blk, 0, s>>>(g, (const T *)src, (T *)dst, utop_in, utop_out, st,
-                                                                 slot, -1, hbox, box);
+                                                                 win, -1, hbox, box);
         else
             k_collide_xpair<ST_F16, K1_ALL><<<grid, blk, 0, s>>>(g, (const T *)src, (T *)dst, utop_in, utop_out, st,
-                                                                 slot, slot_out, hbox, box);
+                                                                 win, slot_out, hbox, box);
     } else {
         using T = __nv_bfloat16;
         if (region == REGION_FAR)
             k_collide_xpair<ST_BF16, K1_FAR><<<grid, blk, 0, s>>>(g, (const T *)src, (T *)dst, utop_in, utop_out,
-                                                                  st, slot, -1, hbox, box);
+                                                                  st, win, -1, hbox, box);
         else
             k_collide_xpair<ST_BF16, K1_ALL><<<grid, blk, 0, s>>>(g, (const T *)src, (T *)dst, utop_in, utop_out,
-                                                                  st, slot, slot_out, hbox, box);
+                                                                  st, win, slot_out, hbox, box);
     }
     return cudaGetLastError();
 }

@@ -115,6 +115,7 @@ static void release(turret_ctx *c) {
     }
     if (c->side) cudaStreamDestroy(c->side);
     if (c->aux) cudaStreamDestroy(c->aux);
+    if (c->red) cudaStreamDestroy(c->red);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     cudaEvent_t *xs[7] = {c->ev_far, c->ev_near, c->ev_pm, c->ev_ired, c->ev_redd, c->ev_spread, c->ev_rowd};
@@ -143,7 +144,7 @@ extern "C" turret_status lbm_init(turret_ctx **out, const turret_window *win, tu
     if (((uintptr_t)ws & 255) != 0) return fail(c, TURRET_EINVAL, "workspace must be 256-byte aligned");
 
     c = new turret_ctx();
-    c->side = c->aux = nullptr;
+    c->side = c->aux = c->red = nullptr;
     c->ev_fork = c->ev_join = nullptr;
     for (int k = 0; k < 2; ++k) {
         c->ev_far[k] = c->ev_near[k] = c->ev_pm[k] = c->ev_ired[k] = c->ev_redd[k] = c->ev_spread[k] = c->ev_rowd[k] = nullptr;
@@ -210,6 +211,7 @@ extern "C" turret_status lbm_init(turret_ctx **out, const turret_window *win, tu
     cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo_prio, &hi_prio);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi_prio);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->aux, cudaStreamNonBlocking, hi_prio);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->red, cudaStreamNonBlocking, hi_prio);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
     {
@@ -461,6 +463,7 @@ static size_t carve_ibm(Carver &cv, const IbmLayout &L, turret_ctx *c) {
     ba.u = (float4 *)cv.take(nb * 16);
     ba.s = (float4 *)cv.take(nb * 32);
     ba.h = (float *)cv.take(3 * nb * 4);
+    BodySlot *fwd = (BodySlot *)cv.take(4 * sizeof(BodySlot));
     MarkerArrays m2 = m;
     const size_t before = cv.off;
     carve_level(cv, L, m);
@@ -471,6 +474,7 @@ static size_t carve_ibm(Carver &cv, const IbmLayout &L, turret_ctx *c) {
         c->mk[0] = m;
         c->mk[1] = m2;
         c->two_sets = two;
+        c->fwd = fwd;
         c->ba = ba;
     }
     return cv.off + 256;
@@ -549,13 +553,13 @@ static const CUtensorMap *dst_map(const turret_ctx *c, int p) {
 static cudaError_t collide_window(const turret_ctx *c, int p, cudaStream_t s) {
     if (src_map(c, p))
         return launch_collide_staged(c->geom, c->storage, *src_map(c, p), *dst_map(c, p), c->f[p], c->f[1 - p],
-                                     c->utop[1 - p], c->utop[p], c->dstate, p, 1 - p, nullptr, c->box, REGION_ALL,
+                                     c->utop[1 - p], c->utop[p], c->dstate, &c->dstate->s[p], 1 - p, nullptr, c->box, REGION_ALL,
                                      s);
     if (xpair_eligible(c->geom, c->storage))
         return launch_collide_xpair(c->geom, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate,
-                                    p, 1 - p, nullptr, c->box, REGION_ALL, s);
-    return launch_collide_stream(c->geom, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p,
-                                 1 - p, nullptr, c->box, false, REGION_ALL, s);
+                                    &c->dstate->s[p], 1 - p, nullptr, c->box, REGION_ALL, s);
+    return launch_collide_stream(c->geom, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, &c->dstate->s[p],
+                                  1 - p, nullptr, c->box, false, REGION_ALL, s);
 }
 
 static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K);
@@ -571,9 +575,9 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
         if (c->body.predictor != 0)
             CE(launch_predict(c->body.predictor == 2 ? mlp_device_view(c->net) : nullptr, c->dstate, p,
                               c->body.predictor, c->stream));
-        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p, -1,
+        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, &c->dstate->s[p], -1,
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
-        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], c->stream));
+        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], nullptr, c->stream));
         CE(launch_reinject(G, c->storage, c->f[1 - p], c->f[p], c->dstate, 1 - p, c->reinject, c->stream));
         CE(enqueue_lists(c, 1 - p, false, c->stream));
         return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
@@ -582,9 +586,9 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
     const MlpDev *net = (c->body.predictor == 2) ? mlp_device_view(c->net) : nullptr;
     if (!c->split) {
         if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->stream));
-        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p, -1,
+        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, &c->dstate->s[p], -1,
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
-        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], c->stream));
+        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], nullptr, c->stream));
         CE(enqueue_lists(c, 1 - p, true, c->stream));
         return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
@@ -592,19 +596,21 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
     return enqueue_steps_pipelined(c, p, 1);
 }
 
-// Steps t .. t+K-1 (parity p0 first) of a split window over three streams with
+// Steps t .. t+K-1 (parity p0 first) of a split window over four streams with
 // the exact dependencies, so the immersed-boundary chain of step t overlaps
 // the far-cell collide+stream of step t+1 and the markers, tile lists and rows
 // of A of t+1 are prepared beside the cycles and the spreading of t:
 //   caller  far(t)     after near(t-1) [its near-region cells of f*(t-1)] and
 //                      pm(t-1) [the window slot of t];
 //   aux     pm(t)      (prediction, particle update, markers of t+1) after
-//                      far(t-1) and near(t-1) [they read the slot pm(t) writes;
-//                      near(t-1) also follows the spreading of t-2, the last
-//                      reader of the marker set pm(t) writes] and reduce(t-1)
-//                      [F, T]; with a single marker set after spread(t-1);
+//                      near(t-1) [it reads the slot pm(t) writes and follows the
+//                      spreading of t-2, the last reader of the marker set pm(t)
+//                      writes] and reduce(t-1) [F, T]; with a single marker set
+//                      after spread(t-1); not after far(t-1), which reads a copy
+//                      of its slot (four in turn: pm(t) writes the copy of far(t+1),
+//                      last read by far(t-3));
 //           bin(t), rows(t)  tile lists and rows of A of those markers;
-//           reduce(t)  after interp(t);
+//   red     reduce(t)  after interp(t);
 //   side    near(t)    after far(t-1) [its far-cell sources, the buffer it writes;
 //                      on small windows cycles(t-1) wait for it already];
 //           moments(t) after near(t) and pm(t); interp(t);
@@ -632,22 +638,27 @@ static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K) {
             CE(cudaStreamWaitEvent(c->stream, c->ev_near[q], 0));
             CE(cudaStreamWaitEvent(c->stream, c->ev_pm[q], 0));
         }
-        CE(launch_collide_far(G, c->storage, c->f[p], c->f[q], c->utop[q], c->utop[p], c->dstate, p, c->ba.h, c->box,
-                              c->stream, src_map(c, p), dst_map(c, p)));
+        // (from its own copy of the window slot: the particle update of t+1 -> t+2
+        // may overwrite the slot while the far cells still run)
+        CE(launch_collide_far(G, c->storage, c->f[p], c->f[q], c->utop[q], c->utop[p], c->dstate,
+                              first ? &c->dstate->s[p] : &c->fwd[k % 4], c->ba.h, c->box, c->stream, src_map(c, p),
+                              dst_map(c, p)));
         CE(cudaEventRecord(c->ev_far[p], c->stream));
         // aux: prediction, particle/marker update, tile lists, rows of A
         if (!first) {
-            CE(cudaStreamWaitEvent(c->aux, c->ev_far[q], 0));
             CE(cudaStreamWaitEvent(c->aux, c->two_sets ? c->ev_near[q] : c->ev_spread[q], 0));
+            CE(cudaStreamWaitEvent(c->aux, c->ev_redd[q], 0));
+            // the first step's far cells read the context's slot itself
+            if (k == 1) CE(cudaStreamWaitEvent(c->aux, c->ev_far[q], 0));
         }
         if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->aux));
-        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[q], c->aux));
+        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[q], &c->fwd[(k + 1) % 4], c->aux));
         CE(cudaEventRecord(c->ev_pm[p], c->aux));
         CE(enqueue_lists(c, q, true, c->aux));
         CE(cudaEventRecord(c->ev_rowd[p], c->aux));
         // side: the near cells, then the immersed-boundary chain
         if (!first && !far_first) CE(cudaStreamWaitEvent(c->side, c->ev_far[q], 0));
-        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[q], c->utop[q], c->utop[p], c->dstate, p, -1, c->ba.h,
+        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[q], c->utop[q], c->utop[p], c->dstate, &c->dstate->s[p], -1, c->ba.h,
                                  c->box, true, REGION_NEAR, c->side, !first && far_first));
         CE(cudaEventRecord(c->ev_near[p], c->side));
         CE(cudaStreamWaitEvent(c->side, c->ev_pm[p], 0));
@@ -655,9 +666,9 @@ static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K) {
                               c->side));
         CE(launch_interp0(c->box, nm, c->mk[q], c->ba, c->dstate, warm, overlap, c->side));
         CE(cudaEventRecord(c->ev_ired[p], c->side));
-        CE(cudaStreamWaitEvent(c->aux, c->ev_ired[p], 0));
-        CE(launch_reduce_ft(nm, c->mk[q], c->dstate, q, c->body, c->aux));
-        CE(cudaEventRecord(c->ev_redd[p], c->aux));
+        CE(cudaStreamWaitEvent(c->red, c->ev_ired[p], 0));
+        CE(launch_reduce_ft(nm, c->mk[q], c->dstate, q, c->body, c->red));
+        CE(cudaEventRecord(c->ev_redd[p], c->red));
         CE(cudaStreamWaitEvent(c->side, c->ev_rowd[p], 0));
         if (far_first) CE(cudaStreamWaitEvent(c->side, c->ev_far[p], 0));
         CE(enqueue_cycles(c, q, warm, c->side));
@@ -801,7 +812,7 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     CK(cudaMemcpyAsync(c->dstate, &D, sizeof(DevState), cudaMemcpyHostToDevice, c->stream), "state upload");
     c->has_particle = true;
     drop_graphs(c);
-    CK(launch_particle_markers(c->geom, c->body, c->box, c->dstate, t, 0, c->mk[t], c->stream), "initial markers");
+    CK(launch_particle_markers(c->geom, c->body, c->box, c->dstate, t, 0, c->mk[t], nullptr, c->stream), "initial markers");
     CK(enqueue_lists(c, t, true, c->stream), "initial lists");
     CK(enqueue_coupling(c, c->f[t], c->utop[1 - t], t, 0, c->stream), "initial coupling");
     CK(cudaStreamSynchronize(c->stream), "initial coupling sync");
@@ -970,11 +981,11 @@ extern "C" turret_status lbm_fluid_step(turret_ctx *c, int64_t n) {
         if (split) {
             CK(cudaEventRecord(c->ev_fork, c->stream), "fluid step (fork)");
             CK(cudaStreamWaitEvent(c->side, c->ev_fork, 0), "fluid step (fork)");
-            CK(launch_collide_far(c->geom, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, p,
+            CK(launch_collide_far(c->geom, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, &c->dstate->s[p],
                                   c->ba.h, c->box, c->stream, src_map(c, p), dst_map(c, p)),
                "fluid step (far cells)");
             CK(launch_collide_stream(c->geom, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate,
-                                     p, 1 - p, c->ba.h, c->box, true, REGION_NEAR, c->side),
+                                     &c->dstate->s[p], 1 - p, c->ba.h, c->box, true, REGION_NEAR, c->side),
                "fluid step (near region)");
             CK(cudaEventRecord(c->ev_join, c->side), "fluid step (join)");
             CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0), "fluid step (join)");
@@ -982,7 +993,7 @@ extern "C" turret_status lbm_fluid_step(turret_ctx *c, int64_t n) {
             CK(collide_window(c, p, c->stream), "fluid step");
         } else {
             CK(launch_collide_stream(c->geom, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate,
-                                     p, 1 - p, c->ba.h, c->box, true, REGION_ALL, c->stream),
+                                     &c->dstate->s[p], 1 - p, c->ba.h, c->box, true, REGION_ALL, c->stream),
                "fluid step");
         }
         c->step++;
@@ -1176,6 +1187,7 @@ extern "C" turret_status lbm_destroy(turret_ctx *c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (c->side) cudaStreamSynchronize(c->side);
     if (c->aux) cudaStreamSynchronize(c->aux);
+    if (c->red) cudaStreamSynchronize(c->red);
     release(c);
     return TURRET_OK;
 }

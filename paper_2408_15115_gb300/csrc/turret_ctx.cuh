@@ -17,7 +17,8 @@ struct turret_ctx {
     double nu, tau0, kappa, g[3];
     cudaStream_t stream;  // caller's stream
     cudaStream_t side;    // internal high-priority stream of the immersed-boundary chain
-    cudaStream_t aux;     // internal stream of the FP64 force/torque reduction
+    cudaStream_t aux;     // internal stream of the markers, lists and rows of A
+    cudaStream_t red;     // internal stream of the FP64 force/torque reduction
     cudaEvent_t ev_fork, ev_join;
     // cross-step events of multi-step graphs, by step parity
     cudaEvent_t ev_far[2], ev_near[2], ev_pm[2], ev_ired[2], ev_redd[2], ev_spread[2], ev_rowd[2];
@@ -39,6 +40,7 @@ struct turret_ctx {
     turret::BoxGeom box;
     turret::MarkerArrays mk[2];  // by time-level parity (the same set twice unless two_sets)
     bool two_sets;
+    turret::BodySlot *fwd;  // [4] window slots of pipelined steps, for the far cells
     turret::BoxArrays ba;
     int cap;
     double vol, area;

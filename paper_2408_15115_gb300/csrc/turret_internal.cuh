@@ -345,6 +345,7 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t
 
 // ---------------------------------------------------------------------------
 // Launchers (lbm_kernels.cu).
+// win, here and below: the window slot of the time level pulled.
 // Collide+stream region: all cells, the cells outside the near region around
 // the particle, or the near region only.  The near region is the region of
 // the marker stencils (where h_imm can be nonzero) grown by NEAR_MARGIN cells;
@@ -362,7 +363,7 @@ static_assert(F_OFFSET == 2.0f, "the support box grows by F_OFFSET cells per sid
 // slot_out >= 0: the kernel also copies the window slot to slot_out (with no
 // entering plane) for a following step that has no particle update.
 cudaError_t launch_collide_stream(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
-                                  float *utop_out, DevState *st, int slot, int slot_out, const float *hbox,
+                                  float *utop_out, DevState *st, const BodySlot *win, int slot_out, const float *hbox,
                                   const BoxGeom &box, bool has_box, int region, cudaStream_t s,
                                   bool after_spread = false);
 // The far cells of a coupled step (lbm_far.cu): FP32 storage under a register
@@ -371,7 +372,7 @@ cudaError_t launch_collide_stream(const Geom &g, int storage, const void *src, v
 // dst are given (see encode_population_map), else on x-adjacent pairs where
 // xpair_eligible, else as launch_collide_stream(..., REGION_FAR).
 cudaError_t launch_collide_far(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
-                               float *utop_out, DevState *st, int slot, const float *hbox, const BoxGeom &box,
+                               float *utop_out, DevState *st, const BodySlot *win, const float *hbox, const BoxGeom &box,
                                cudaStream_t s, const CUtensorMap *lmap = nullptr, const CUtensorMap *smap = nullptr);
 // 16-bit collide+stream with sources and results staged in shared memory by
 // bulk tensor copies (lbm_staged.cu): REGION_FAR or REGION_ALL without
@@ -391,11 +392,11 @@ bool is_xpair_kernel(const void *fn);
 bool is_window_kernel(const void *fn);
 bool is_far_kernel(const void *fn);
 cudaError_t launch_collide_xpair(const Geom &g, int storage, const void *src, void *dst, const float *utop_in,
-                                 float *utop_out, DevState *st, int slot, int slot_out, const float *hbox,
+                                 float *utop_out, DevState *st, const BodySlot *win, int slot_out, const float *hbox,
                                  const BoxGeom &box, int region, cudaStream_t s);
 cudaError_t launch_collide_staged(const Geom &g, int storage, const CUtensorMap &lmap, const CUtensorMap &smap,
                                   const void *src, void *dst, const float *utop_in, float *utop_out, DevState *st,
-                                  int slot, int slot_out, const float *hbox, const BoxGeom &box, int region,
+                                  const BodySlot *win, int slot_out, const float *hbox, const BoxGeom &box, int region,
                                   cudaStream_t s);
 // Re-injection copy of Sec. 2.5 (windows without slide): once the centre's
 // window z in slot `slot` is below trigger, the post-collision planes
@@ -438,8 +439,9 @@ cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const
 // Rigid-body update t -> t+1 (advance = 1; reads window slot `slot`, writes
 // slot^1) and the marker kinematics for the resulting state, one launch; with
 // advance = 0 only the markers of the current state (window slot `slot`).
+// fwd: also receives the new slot (see launch_collide_far), or null.
 cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const BoxGeom &box, DevState *st, int slot,
-                                    int advance, MarkerArrays m, cudaStream_t s);
+                                    int advance, MarkerArrays m, BodySlot *fwd, cudaStream_t s);
 // (overlap, here and below: start beside the launch just before on the stream.)
 // Rows of the interaction matrix A from the tile lists (one block per marker).
 cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, bool overlap,
@@ -454,7 +456,8 @@ cudaError_t launch_interp0(const BoxGeom &box, int nm, const MarkerArrays &m, co
 // (The initial h of the warm form is in m.ha, put there by the interpolation.)
 cudaError_t launch_cycles(int nm, const MarkerArrays &m, int C, int warm, DevState *st, float eps, bool overlap,
                           cudaStream_t s);
-// F = sum_k f_k, T = sum_k t_k in FP64, fixed order, into the device state.
+// F = sum_k f_k, T = sum_k t_k in FP64, fixed order, into the device state: a
+// block per component, the last to finish records the time level.
 cudaError_t launch_reduce_ft(int nm, MarkerArrays m, DevState *st, int slot, const BodyConst &bc, cudaStream_t s);
 // h_imm on the support box (overlap only directly after a cycle).
 cudaError_t launch_spread(const BoxGeom &box, const MarkerArrays &m, const BoxArrays &ba, int cap, bool overlap,
