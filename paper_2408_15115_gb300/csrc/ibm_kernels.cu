@@ -520,6 +520,12 @@ __global__ void __launch_bounds__(NT) k_rows(BoxGeom box, MarkerArrays m, const 
     rows_block<NT, CU>(box, m, wlist, wcount, cap, st, blockIdx.x);
 }
 
+// LISTS_QUIET: the rows of the next level while the far cells of this one run.
+__global__ void __launch_bounds__(QUIET_THREADS, 16) k_rows_quiet(BoxGeom box, int nm, MarkerArrays m, const int *wlist,
+                                                                  const int *wcount, int cap, DevState *st) {
+    for (int k = blockIdx.x; k < nm; k += gridDim.x) rows_block<QUIET_THREADS, 4>(box, m, wlist, wcount, cap, st, k);
+}
+
 // One warp per marker, small blocks (as above).  It used to share a launch
 // with the rows of A: 10 us of a 41 us step of a 32x32x64 window, where the
 // rows now are built beside the near region's launch and the moments.
@@ -1071,10 +1077,15 @@ cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const Bo
     return cudaGetLastError();
 }
 
-cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, bool overlap,
+cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, int mode,
                         cudaStream_t s) {
     const int ntiles = box.tx * box.ty * box.tz;  // list 1 (rows of A) follows list 0
-    if (overlap)
+    if (mode == LISTS_QUIET) {
+        k_rows_quiet<<<QUIET_BLOCKS, QUIET_THREADS, 0, s>>>(box, nm, m, m.tile_list + (size_t)ntiles * cap,
+                                                            m.tile_count + ntiles, cap, st);
+        return cudaGetLastError();
+    }
+    if (mode == LISTS_OVERLAP)
         return launch_pdl(k_rows<ROWS_MARKER_THREADS_SMALL, 1>, nm, ROWS_MARKER_THREADS_SMALL, s, box, m, m.tile_list + (size_t)ntiles * cap,
                           m.tile_count + ntiles, cap, st);
     k_rows<ROWS_MARKER_THREADS, 4><<<nm, ROWS_MARKER_THREADS, 0, s>>>(box, m, m.tile_list + (size_t)ntiles * cap, m.tile_count + ntiles, cap, st);

@@ -22,6 +22,13 @@ __global__ void __launch_bounds__(MB_THREADS) k_bin(DevState *st, int slot, BoxG
     bin_block(st, slot, box, nm, m.base, m.seg, m.tile_list, m.tile_count, cap, st, rmin, rmax, blockIdx.x);
 }
 
+__global__ void __launch_bounds__(QUIET_THREADS, 16) k_bin_quiet(DevState *st, int slot, BoxGeom box, int nm,
+                                                                 MarkerArrays m, int cap, float rmin, float rmax) {
+    constexpr int W = QUIET_THREADS / 32;
+    for (int t = blockIdx.x * W + (threadIdx.x >> 5); t < box.tx * box.ty * box.tz; t += gridDim.x * W)
+        bin_warp(st, slot, box, nm, m, cap, st, rmin, rmax, t, threadIdx.x & 31);
+}
+
 cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
                                int slot, const BoxGeom &box, BoxArrays ba, float rmin, float rmax, cudaStream_t s) {
     const unsigned nb = (unsigned)((box.nbox + MB_THREADS - 1) / MB_THREADS);
@@ -34,9 +41,13 @@ cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, cons
 }
 
 cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const MarkerArrays &m, int cap, float rmin,
-                       float rmax, bool overlap, cudaStream_t s) {
+                       float rmax, int mode, cudaStream_t s) {
+    if (mode == LISTS_QUIET) {
+        k_bin_quiet<<<QUIET_BLOCKS, QUIET_THREADS, 0, s>>>(st, slot, box, nm, m, cap, rmin, rmax);
+        return cudaGetLastError();
+    }
     const unsigned nb = (unsigned)(box.tx * box.ty * box.tz);
-    if (overlap) return launch_pdl(k_bin, nb, MB_THREADS, s, st, slot, box, nm, m, cap, rmin, rmax);
+    if (mode == LISTS_OVERLAP) return launch_pdl(k_bin, nb, MB_THREADS, s, st, slot, box, nm, m, cap, rmin, rmax);
     k_bin<<<nb, MB_THREADS, 0, s>>>(st, slot, box, nm, m, cap, rmin, rmax);
     return cudaGetLastError();
 }

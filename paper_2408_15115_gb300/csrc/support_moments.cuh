@@ -129,7 +129,8 @@ __device__ __forceinline__ void bin_block(const DevState *st, int slot, const Bo
     }
 }
 
-// bin_warp, a warp per tile, for batches: its lanes test 32 marker segments at
+// bin_warp, a warp per tile, for batches and for lists built well ahead of their
+// use: its lanes test 32 marker segments at
 // once (the bounding boxes of their stencil bases), then the markers of the
 // segments that reach the tile go by in fours of 32.  Most tiles of a box reach
 // few segments or none, so a tile costs a block's start, not work; four tiles

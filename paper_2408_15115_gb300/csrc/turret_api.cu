@@ -502,15 +502,26 @@ constexpr long long OVERLAP_CELLS = 1 << 18;
 constexpr int OVERLAP_MARKERS = 152 * INTERP_WARPS;
 static bool overlap_chain(const turret_ctx *c) { return c->geom.ncell <= OVERLAP_CELLS && c->nm <= OVERLAP_MARKERS; }
 
+// Whether the lists and rows prepared ahead are built quietly (LISTS_QUIET):
+// the far cells must last as long (0.055 us per marker against 20 to 32 us per
+// million cells).  us per step, plain -> quiet: 256x256x512 FP32 (6762 markers)
+// 1161 -> 1148, 192x192x384 (4002) FP32 503 -> 497, FP16 337 -> 332, 160x160x320 FP16
+// (1962) 227 -> 225, even at 128x128x256 with 362 markers; at 1460 cells per
+// marker (96x96x192) the cycles wait for the rows: 85 -> 122.
+constexpr long long QUIET_CELLS_PER_MARKER = 3000;
+static bool quiet_lists(const turret_ctx *c) { return c->geom.ncell >= QUIET_CELLS_PER_MARKER * c->nm; }
+
 // Events (2)-(4) of Table 1 in two parts.  The markers' part: particle update
 // t -> t+1 from window slot `slot` (advance = 1; the markers land in slot^1,
 // and in that level's marker set) or the markers of the current level (advance
 // = 0, set-up of t = 0); then the tile lists and the rows of A, which depend
 // on the markers alone.
-// after_pm: the marker launch is the one just before on the stream.
-static cudaError_t enqueue_lists(turret_ctx *c, int so, bool after_pm, cudaStream_t s) {
-    CE(launch_bin(c->dstate, so, c->box, c->nm, c->mk[so], c->cap, c->body.rmin, c->body.rmax, after_pm && overlap_chain(c), s));
-    return launch_rows(c->box, c->nm, c->mk[so], c->cap, c->dstate, overlap_chain(c), s);
+// after_pm: the marker launch is the one just before on the stream; ahead: the
+// far cells of the step before still run.
+static cudaError_t enqueue_lists(turret_ctx *c, int so, bool after_pm, bool ahead, cudaStream_t s) {
+    const int mode = overlap_chain(c) ? LISTS_OVERLAP : (ahead && quiet_lists(c) ? LISTS_QUIET : LISTS_PLAIN);
+    CE(launch_bin(c->dstate, so, c->box, c->nm, c->mk[so], c->cap, c->body.rmin, c->body.rmax, mode == LISTS_OVERLAP && !after_pm ? LISTS_PLAIN : mode, s));
+    return launch_rows(c->box, c->nm, c->mk[so], c->cap, c->dstate, mode, s);
 }
 
 // The IBM cycles of one step (the paper's n - 1 cycles from r0, or the
@@ -579,7 +590,7 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
         CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], nullptr, c->stream));
         CE(launch_reinject(G, c->storage, c->f[1 - p], c->f[p], c->dstate, 1 - p, c->reinject, c->stream));
-        CE(enqueue_lists(c, 1 - p, false, c->stream));
+        CE(enqueue_lists(c, 1 - p, false, false, c->stream));
         return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
     const bool predict = c->body.predictor != 0;
@@ -589,7 +600,7 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
         CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, &c->dstate->s[p], -1,
                                  c->ba.h, c->box, true, REGION_ALL, c->stream));
         CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], nullptr, c->stream));
-        CE(enqueue_lists(c, 1 - p, true, c->stream));
+        CE(enqueue_lists(c, 1 - p, true, false, c->stream));
         return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
     // one step of the pipeline below
@@ -654,7 +665,7 @@ static cudaError_t enqueue_steps_pipelined(turret_ctx *c, int p0, int K) {
         if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->aux));
         CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[q], &c->fwd[(k + 1) % 4], c->aux));
         CE(cudaEventRecord(c->ev_pm[p], c->aux));
-        CE(enqueue_lists(c, q, true, c->aux));
+        CE(enqueue_lists(c, q, true, !first, c->aux));
         CE(cudaEventRecord(c->ev_rowd[p], c->aux));
         // side: the near cells, then the immersed-boundary chain
         if (!first && !far_first) CE(cudaStreamWaitEvent(c->side, c->ev_far[q], 0));
@@ -813,7 +824,7 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     c->has_particle = true;
     drop_graphs(c);
     CK(launch_particle_markers(c->geom, c->body, c->box, c->dstate, t, 0, c->mk[t], nullptr, c->stream), "initial markers");
-    CK(enqueue_lists(c, t, true, c->stream), "initial lists");
+    CK(enqueue_lists(c, t, true, false, c->stream), "initial lists");
     CK(enqueue_coupling(c, c->f[t], c->utop[1 - t], t, 0, c->stream), "initial coupling");
     CK(cudaStreamSynchronize(c->stream), "initial coupling sync");
     return TURRET_OK;

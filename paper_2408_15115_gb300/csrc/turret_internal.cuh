@@ -343,6 +343,17 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// How the tile lists and rows of A are launched:
+//   LISTS_PLAIN   ordinary launches
+//   LISTS_OVERLAP small windows: each starts beside the launch before it (launch_pdl)
+//   LISTS_QUIET   large windows: QUIET_BLOCKS blocks that stride over the work.
+//                 Four blocks of the FP32 far-cell kernel (120 registers) or five of
+//                 the 16-bit one (96) leave 4096 registers of an SM: room for one
+//                 block of 64 threads with 64 registers, which then runs beside
+//                 them instead of displacing them.
+enum { LISTS_PLAIN = 0, LISTS_OVERLAP = 1, LISTS_QUIET = 2 };
+constexpr int QUIET_BLOCKS = 152, QUIET_THREADS = 64;
+
 // ---------------------------------------------------------------------------
 // Launchers (lbm_kernels.cu).
 // win, here and below: the window slot of the time level pulled.
@@ -433,7 +444,7 @@ cudaError_t launch_batch_bin(const RunDesc *runs, const int *prefix, int nruns, 
 cudaError_t launch_box_moments(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
                                int slot, const BoxGeom &box, BoxArrays ba, float rmin, float rmax, cudaStream_t s);
 cudaError_t launch_bin(DevState *st, int slot, const BoxGeom &box, int nm, const MarkerArrays &m, int cap, float rmin,
-                       float rmax, bool overlap, cudaStream_t s);
+                       float rmax, int mode, cudaStream_t s);
 
 // Launchers (ibm_kernels.cu).
 // Rigid-body update t -> t+1 (advance = 1; reads window slot `slot`, writes
@@ -444,7 +455,7 @@ cudaError_t launch_particle_markers(const Geom &g, const BodyConst &bc, const Bo
                                     int advance, MarkerArrays m, BodySlot *fwd, cudaStream_t s);
 // (overlap, here and below: start beside the launch just before on the stream.)
 // Rows of the interaction matrix A from the tile lists (one block per marker).
-cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, bool overlap,
+cudaError_t launch_rows(const BoxGeom &box, int nm, const MarkerArrays &m, int cap, DevState *st, int mode,
                         cudaStream_t s);
 // l = 0 interpolation of u* and sigma and the surface traction (one warp per
 // marker); warm 0 also starts h there.  Clears the slips of the last step.
