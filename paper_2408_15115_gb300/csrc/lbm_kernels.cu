@@ -160,6 +160,10 @@ cudaError_t launch_init_equilibrium(const Geom &g, int storage, void *dst, const
 
 cudaError_t launch_macro(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
                          int slot, float *out, bool pops, cudaStream_t s) {
+    // the caller's array is only known to hold floats: pairs are stored where it
+    // is 8-byte aligned
+    if (xpair_eligible(g, storage) && reinterpret_cast<uintptr_t>(out) % sizeof(float2) == 0)
+        return launch_macro_xpair(g, storage, src, utop_in, st, slot, out, pops, s);
     switch (storage) {
         case ST_F32: k_macro<ST_F32><<<window_grid(g, storage, g.nz), dim3(32, 4), 0, s>>>(g, (const float *)src, utop_in, st, slot, out, pops, window_flat(g, storage)); break;
         case ST_F16: k_macro<ST_F16><<<window_grid(g, storage, g.nz), dim3(32, 4), 0, s>>>(g, (const __half *)src, utop_in, st, slot, out, pops, window_flat(g, storage)); break;

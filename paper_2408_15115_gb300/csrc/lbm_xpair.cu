@@ -50,6 +50,50 @@ __global__ void __launch_bounds__(128, 5)
     xpair_cells<ST, MODE>(g, src, dst, utop_out, S, hbox, box, x0 + 2 * tx, y0 + (ty & 1), z0 + (ty >> 1));
 }
 
+// rho, u (or the 27 pre-collision deviations) of f(t), as k_macro of
+// lbm_kernels.cu, on the tiles of k_collide_xpair: 4-byte loads of the
+// populations and 8-byte stores of the fields.  Bound by memory (70 bytes a cell
+// for rho and u).  192x192x384 FP16, call and synchronisation: 225 us with
+// 2-byte loads, 187 us so; 256x256x512: 501 and 418 us.  Six blocks
+// per SM: 214 / 193 / 187 / 190 us with 4 / 5 / 6 / 8; boundary tiles load all
+// sources of a cell together (pull27_edge): 64x64x64 24.3 us without, 20.1 with.
+template <int ST>
+__global__ void __launch_bounds__(128, 6) k_macro_xpair(Geom g, const typename Codec<ST>::T *__restrict__ src,
+                                                     const float *__restrict__ utop_in, const DevState *__restrict__ st,
+                                                     int slot, float *__restrict__ out, int pops) {
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const BodySlot &S = st->s[slot];
+    const int x0 = blockIdx.x * XP_TX, y0 = blockIdx.y * XP_TY, z0 = XP_TZ * blockIdx.z;
+    const int x = x0 + 2 * tx, y = y0 + (ty & 1), zl = z0 + (ty >> 1);
+    f2 q[27];
+    if (xpair_tile_ok<K1_ALL, false>(g, S, BoxGeom{}, x0, y0, z0, XP_TX, XP_TY))
+        xpair_pull<ST>(g, src, S.ring, x, y, zl, q);
+    else {
+        float a[27];
+        pull27<ST, true>(g, src, x, y, zl, S.ring, S.reseed, utop_in, a);
+#pragma unroll
+        for (int i = 0; i < 27; ++i) q[i].x = a[i];
+        pull27<ST, true>(g, src, x + 1, y, zl, S.ring, S.reseed, utop_in, a);
+#pragma unroll
+        for (int i = 0; i < 27; ++i) q[i].y = a[i];
+    }
+    f2 *o = reinterpret_cast<f2 *>(out + ((size_t)zl * g.ny + y) * g.nx + x);
+    const size_t n = (size_t)g.ncell / 2;
+    if (pops) {
+#pragma unroll
+        for (int i = 0; i < 27; ++i) {
+            const float k = (Codec<ST>::scaled ? Wq(i) / Codec<ST>::K : 1.0f) * INV_SCALE;
+            o[i * n] = make_float2(q[i].x * k, q[i].y * k);
+        }
+        return;
+    }
+    const MacroR<f2> M = macro_raw<ST>(moments_raw<ST>(q));
+    o[0] = M.rho;
+    o[n] = M.ux;
+    o[2 * n] = M.uy;
+    o[3 * n] = M.uz;
+}
+
 // ---------------------------------------------------------------------------
 // Host side.
 
@@ -79,6 +123,16 @@ cudaError_t launch_collide_xpair(const Geom &g, int storage, const void *src, vo
             k_collide_xpair<ST_BF16, K1_ALL><<<grid, blk, 0, s>>>(g, (const T *)src, (T *)dst, utop_in, utop_out,
                                                                   st, win, slot_out, hbox, box);
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_macro_xpair(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
+                               int slot, float *out, bool pops, cudaStream_t s) {
+    const dim3 grid(g.nx / XP_TX, g.ny / XP_TY, g.nz / XP_TZ), blk(32, 4);
+    if (storage == ST_F16)
+        k_macro_xpair<ST_F16><<<grid, blk, 0, s>>>(g, (const __half *)src, utop_in, st, slot, out, pops);
+    else
+        k_macro_xpair<ST_BF16><<<grid, blk, 0, s>>>(g, (const __nv_bfloat16 *)src, utop_in, st, slot, out, pops);
     return cudaGetLastError();
 }
 

@@ -78,13 +78,11 @@ __device__ __forceinline__ bool xpair_tile_ok(const Geom &g, const BodySlot &S, 
     return ok;
 }
 
-// Collide+stream of the cells (x, y, zl) and (x + 1, y, zl) of a tile that
-// xpair_tile_ok admits (x even; MODE K1_ALL or K1_FAR, no forcing).
-template <int ST, int MODE>
-__device__ __forceinline__ void xpair_cells(const Geom &g, const typename Codec<ST>::T *__restrict__ src,
-                                            typename Codec<ST>::T *__restrict__ dst, float *__restrict__ utop_out,
-                                            const BodySlot &S, const float *__restrict__ hbox, const BoxGeom &box,
-                                            int x, int y, int zl) {
+// The 27 populations streaming into the cells (x, y, zl) and (x + 1, y, zl) of a
+// tile that xpair_tile_ok admits (x even).
+template <int ST>
+__device__ __forceinline__ void xpair_pull(const Geom &g, const typename Codec<ST>::T *__restrict__ src, int ring, int x,
+                                           int y, int zl, f2 q[27]) {
     const int nx = g.nx, plane = (int)g.plane, ncell = (int)g.ncell;
     const int xm = x == 0 ? nx - 2 : x - 2, xp = x + 2 == nx ? 0 : x + 2;  // periodic here when at an edge
     int ys[3];
@@ -95,10 +93,9 @@ __device__ __forceinline__ void xpair_cells(const Geom &g, const typename Codec<
         yy -= yy >= g.ny ? g.ny : 0;
         ys[ey] = yy * nx;
     }
-    f2 q[27];
 #pragma unroll
     for (int ez = 0; ez < 3; ++ez) {
-        const int zrow = zphys(zl - (ez - 1), S.ring, g.nz) * plane;
+        const int zrow = zphys(zl - (ez - 1), ring, g.nz) * plane;
 #pragma unroll
         for (int ey = 0; ey < 3; ++ey) {
             const int row = zrow + ys[ey];
@@ -115,6 +112,18 @@ __device__ __forceinline__ void xpair_cells(const Geom &g, const typename Codec<
             }
         }
     }
+}
+
+// Collide+stream of the cells (x, y, zl) and (x + 1, y, zl) of a tile that
+// xpair_tile_ok admits (x even; MODE K1_ALL or K1_FAR, no forcing).
+template <int ST, int MODE>
+__device__ __forceinline__ void xpair_cells(const Geom &g, const typename Codec<ST>::T *__restrict__ src,
+                                            typename Codec<ST>::T *__restrict__ dst, float *__restrict__ utop_out,
+                                            const BodySlot &S, const float *__restrict__ hbox, const BoxGeom &box,
+                                            int x, int y, int zl) {
+    const int plane = (int)g.plane, nx = g.nx, ncell = (int)g.ncell;
+    f2 q[27];
+    xpair_pull<ST>(g, src, S.ring, x, y, zl, q);
     // the pair shares its plane: the plane's relaxation time for both lanes
     const int z[2] = {zl, zl};
     const bool on[2] = {true, true};

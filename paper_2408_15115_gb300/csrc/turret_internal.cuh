@@ -398,6 +398,9 @@ bool is_staged_kernel(const void *fn);
 // (lbm_xpair.cu): REGION_FAR or REGION_ALL without forcing; xpair_eligible:
 // FP16 or round-to-nearest BF16 on a window the 64 x 2 x 2 tiles cover.
 bool xpair_eligible(const Geom &g, int storage);
+// launch_macro where xpair_eligible and out is 8-byte aligned.
+cudaError_t launch_macro_xpair(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,
+                               int slot, float *out, bool pops, cudaStream_t s);
 bool is_xpair_kernel(const void *fn);
 // The other kernels that sweep the window (bulk nodes of a step graph).
 bool is_window_kernel(const void *fn);
