@@ -45,8 +45,14 @@ __device__ __forceinline__ unsigned pack2<ST_BF16>(f2 v) {
     return *reinterpret_cast<const unsigned *>(&h);
 }
 
-__device__ __forceinline__ unsigned ld_word(const void *base, int elem) {
-    return __ldg(reinterpret_cast<const unsigned *>(static_cast<const unsigned short *>(base) + elem));
+// The word `bytes` into the plane array of a population.  The array's address is
+// uniform over the grid and the offset has 32 bits, so the 45 loads of a pair
+// share 27 per-thread offsets; with a 64-bit address formed for each load the
+// kernel took 294 us on 192x192x384 FP16 (670 on 256x256x512), so 287 (650);
+// BF16 313 -> 303, with stochastic rounding 361 -> 355.  The stores keep one
+// thread pointer: in this form they cost what the loads gain.
+__device__ __forceinline__ unsigned ld_word(const void *base, unsigned bytes) {
+    return __ldg(reinterpret_cast<const unsigned *>(static_cast<const char *>(base) + bytes));
 }
 
 // Whether the cells [c0, c0 + len) of one axis meet the near region (relative
@@ -98,16 +104,17 @@ __device__ __forceinline__ void xpair_pull(const Geom &g, const typename Codec<S
         const int zrow = zphys(zl - (ez - 1), ring, g.nz) * plane;
 #pragma unroll
         for (int ey = 0; ey < 3; ++ey) {
-            const int row = zrow + ys[ey];
+            const unsigned row = 2 * (zrow + ys[ey]);
+            const unsigned ox = row + 2 * x, om = row + 2 * xm, op = row + 2 * xp;
 #pragma unroll
             for (int ex = 0; ex < 3; ++ex) {
                 const int i = ex + 3 * ey + 9 * ez;
-                const typename Codec<ST>::T *r = src + (size_t)i * ncell + row;
-                const unsigned a = ld_word(r, x);
+                const typename Codec<ST>::T *r = src + (size_t)i * ncell;
+                const unsigned a = ld_word(r, ox);
                 unsigned w;
                 if (ex == 1) w = a;
-                else if (ex == 2) w = __byte_perm(ld_word(r, xm), a, 0x5432);  // (x - 1, x)
-                else w = __byte_perm(a, ld_word(r, xp), 0x5432);                // (x + 1, x + 2)
+                else if (ex == 2) w = __byte_perm(ld_word(r, om), a, 0x5432);  // (x - 1, x)
+                else w = __byte_perm(a, ld_word(r, op), 0x5432);                // (x + 1, x + 2)
                 q[i] = unpack2<ST>(w);
             }
         }
