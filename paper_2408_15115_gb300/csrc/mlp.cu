@@ -260,12 +260,15 @@ __global__ void k_adamw(float *__restrict__ P, const float *__restrict__ G, floa
 // products take them, sums run in the k order of a 16-wide mma chain and
 // weight gradients over 256-row slices in order.
 constexpr int RT_ROWS = 32, RT_THREADS = 256;
+// outputs of many rows: ROWS / 16 x 4 warps per block (launch_rows)
+constexpr int RT_WIDE = 128;
 constexpr int LDK = MLP_H + 8, LDX = MLP_INP + 8, LDY = 24;  // row strides (BF16) free of bank conflicts for ldmatrix
 
+template <int ROWS>
 struct RowsSmem {
     __nv_bfloat16 w1[MLP_H][LDX], w2[MLP_H][LDK], w3[MLP_H][LDK], w4[MLP_OUTP][LDK];
-    __nv_bfloat16 x[RT_ROWS][LDX];
-    __nv_bfloat16 a[2][RT_ROWS][LDK];  // the operand of the current layer and the one being formed
+    __nv_bfloat16 x[ROWS][LDX];
+    __nv_bfloat16 a[2][ROWS][LDK];  // the operand of the current layer and the one being formed
     __nv_bfloat16 dy[RT_ROWS][LDY];
     double loss[RT_THREADS / 32];
 };
@@ -379,40 +382,42 @@ __device__ __forceinline__ void rows_dgelu(const float (&z)[4][4], float (&acc)[
 template <int LD>
 __device__ __forceinline__ void load_rows16(__nv_bfloat16 (*s)[LD], const __nv_bfloat16 *__restrict__ g, int rows, int cols) {
     const int per = cols / 8;
-    for (int e = threadIdx.x; e < rows * per; e += RT_THREADS)
+    for (int e = threadIdx.x; e < rows * per; e += blockDim.x)
         *reinterpret_cast<uint4 *>(&s[e / per][(e % per) * 8]) = __ldg(reinterpret_cast<const uint4 *>(g) + e);
 }
 template <int LD>
 __device__ __forceinline__ void store_rows16(__nv_bfloat16 *__restrict__ g, const __nv_bfloat16 (*s)[LD], int rows, int cols) {
     const int per = cols / 8;
-    for (int e = threadIdx.x; e < rows * per; e += RT_THREADS)
+    for (int e = threadIdx.x; e < rows * per; e += blockDim.x)
         reinterpret_cast<uint4 *>(g)[e] = *reinterpret_cast<const uint4 *>(&s[e / per][(e % per) * 8]);
 }
 
 // TRAIN: forward, loss and backward of rows 32 b .. (b = blockIdx.x), raw
 // inputs x and raw targets t.  Otherwise the outputs y, blocks striding over
 // the row groups so that the weights are staged once per block.
-template <bool TRAIN>
-__global__ void __launch_bounds__(RT_THREADS) k_rows(MlpDev w, const float *__restrict__ x, const float *__restrict__ t,
+template <bool TRAIN, int ROWS>
+__global__ void __launch_bounds__(8 * ROWS) k_rows(MlpDev w, const float *__restrict__ x, const float *__restrict__ t,
                                                      int n, float *__restrict__ y, TrainOut o) {
     extern __shared__ __align__(16) unsigned char rows_raw[];
-    RowsSmem &S = *reinterpret_cast<RowsSmem *>(rows_raw);
+    static_assert(!TRAIN || ROWS == 32, "the loss is the sum of two warps");
+    constexpr int NT = 8 * ROWS, MT = ROWS / 16;
+    RowsSmem<ROWS> &S = *reinterpret_cast<RowsSmem<ROWS> *>(rows_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = lane >> 2, tig = lane & 3;
-    const int m0 = 16 * (warp & 1), n0 = 32 * (warp >> 1);
+    const int m0 = 16 * (warp % MT), n0 = 32 * (warp / MT);
     load_rows16(S.w1, w.Wb + WB1, MLP_H, MLP_INP);
     load_rows16(S.w2, w.Wb + WB2, MLP_H, MLP_H);
     load_rows16(S.w3, w.Wb + WB3, MLP_H, MLP_H);
     load_rows16(S.w4, w.Wb + WB4, MLP_OUTP, MLP_H);
-    for (int row0 = blockIdx.x * RT_ROWS; row0 < n; row0 += gridDim.x * RT_ROWS) {
-        const int nrows = min(RT_ROWS, n - row0);
-        for (int e = tid; e < RT_ROWS * MLP_INP; e += RT_THREADS) {
+    for (int row0 = blockIdx.x * ROWS; row0 < n; row0 += gridDim.x * ROWS) {
+        const int nrows = min(ROWS, n - row0);
+        for (int e = tid; e < ROWS * MLP_INP; e += NT) {
             const int r = e / MLP_INP, c = e % MLP_INP;
             float v = 0.0f;
             if (r < nrows && c < MLP_IN) v = (x[(size_t)(row0 + r) * MLP_IN + c] - w.mean_x[c]) / w.std_x[c];
             S.x[r][c] = __float2bfloat16_rn(v);
         }
         if (TRAIN)
-            for (int e = tid; e < RT_ROWS * 16; e += RT_THREADS) S.dy[e / 16][e % 16] = __float2bfloat16_rn(0.0f);
+            for (int e = tid; e < ROWS * 16; e += NT) S.dy[e / 16][e % 16] = __float2bfloat16_rn(0.0f);
         __syncthreads();
         float z[3][4][4];
         rows_product(S.x, S.w1, MLP_INP, m0, n0, z[0]);
@@ -431,7 +436,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_rows(MlpDev w, const float *__re
         __syncthreads();
         if (TRAIN) store_rows16(o.a[2] + (size_t)row0 * MLP_H, S.a[0], nrows, MLP_H);
         double sq = 0.0;
-        if (warp < 2) {  // the six outputs: one 16 x 8 tile per warp
+        if (warp < MT) {  // the six outputs: one 16 x 8 tile per warp
             float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
             for (int k = 0; k < MLP_H; k += 16) {
@@ -921,10 +926,24 @@ __global__ void k_build_samples(const double *__restrict__ log, long long nsamp,
     }
 }
 
-// BF16 outputs of n rows: two blocks per SM at most, each striding over the row groups
+// BF16 outputs of n rows, blocks striding over the row groups: 32 rows per block
+// and two blocks per SM, or 128 rows in a block of 1024 threads per SM, which holds
+// twice the rows and does in one round what takes the narrow blocks two: us with
+// narrow / wide blocks, 9728 rows (one round) 14.4 / 18.5, 12000 20.5 / 18.5, 15967
+// 22.5 / 18.5, 19457 (three) 26.1 / 30.7, 30000 (four) 35.1 / 32.8, 40000 (five)
+// 43.1 / 47.1, 84000 (nine) 74.7 / 74.6, 90000 80.6 / 75.5.  Bound by latency and
+// the GELU (384 erff a row), not by the products (1.2 GFLOP at 15967 rows).
 static cudaError_t launch_rows(const MlpDev &w, const float *x, int n, float *y, cudaStream_t s) {
+    const int rounds = (n + 304 * RT_ROWS - 1) / (304 * RT_ROWS);  // of narrow blocks
+    if (rounds % 2 == 0 || rounds > 8) {
+        const int groups = (n + RT_WIDE - 1) / RT_WIDE;
+        k_rows<false, RT_WIDE><<<groups < 152 ? groups : 152, 8 * RT_WIDE, sizeof(RowsSmem<RT_WIDE>), s>>>(w, x, nullptr, n, y,
+                                                                                                   TrainOut{});
+        return cudaGetLastError();
+    }
     const int groups = (n + RT_ROWS - 1) / RT_ROWS;
-    k_rows<false><<<groups < 304 ? groups : 304, RT_THREADS, sizeof(RowsSmem), s>>>(w, x, nullptr, n, y, TrainOut{});
+    k_rows<false, RT_ROWS><<<groups < 304 ? groups : 304, RT_THREADS, sizeof(RowsSmem<RT_ROWS>), s>>>(w, x, nullptr, n, y,
+                                                                                                TrainOut{});
     return cudaGetLastError();
 }
 
@@ -1118,7 +1137,7 @@ cudaError_t train_bf16(turret_mlp *m, const float *x, const float *y, int n, con
     o.loss = (double *)m->T;
     const size_t need = (size_t)nsl * MLP_NPARAM, have = (size_t)MAX_SLICES * MLP_H * MLP_H;
     float *part = need <= have ? m->part : m->D[0];
-    k_rows<true><<<groups, RT_THREADS, sizeof(RowsSmem), m->stream>>>(m->dev, x, y, n, nullptr, o);
+    k_rows<true, RT_ROWS><<<groups, RT_THREADS, sizeof(RowsSmem<RT_ROWS>), m->stream>>>(m->dev, x, y, n, nullptr, o);
     k_wgrad<<<dim3(WG_TILES + WG_COLS, nsl), WG_THREADS, sizeof(WgradSmem), m->stream>>>(o, n, part);
     const turret_adamw a = opt ? *opt : turret_adamw{0.0f, 0.0f, 0.0f, 1.0f, 0.0f};
     k_update<<<(MLP_NPARAM + 255) / 256, 256, 0, m->stream>>>(part, nsl, m->G, opt != nullptr, m->P, m->Mm, m->Vv, m->Wb,
@@ -1183,9 +1202,10 @@ extern "C" turret_status mlp_init(turret_mlp **out, int32_t batch_cap, int32_t p
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->norm, norm.data(), norm.size() * 4, cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess) e = refresh(m);
     if (e == cudaSuccess && precision == 0) {
-        e = cudaFuncSetAttribute(k_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RowsSmem));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RowsSmem));
+        const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        e = cudaFuncSetAttribute(k_rows<true, RT_ROWS>, smem, (int)sizeof(RowsSmem<RT_ROWS>));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rows<false, RT_ROWS>, smem, (int)sizeof(RowsSmem<RT_ROWS>));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rows<false, RT_WIDE>, smem, (int)sizeof(RowsSmem<RT_WIDE>));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradSmem));
         if (cudaHostAlloc((void **)&m->host_loss, sizeof(double), cudaHostAllocDefault) != cudaSuccess) {

@@ -136,3 +136,17 @@ def test_bf16_gradients_at_block_and_slice_edges(n):
     assert abs(L - want_L) / want_L < 2e-2
     assert _per_tensor_err(g.cpu().numpy().astype(np.float64), want_g) < 2e-2
     net.close()
+
+
+@pytest.mark.parametrize("n", [9728, 9729, 9856, 9857, 19456, 19457, 39000, 78000])
+def test_many_rows_give_the_bits_of_few(n):
+    # above 304 x 32 rows a block may take 128 of them (an even number of rounds of
+    # narrow blocks, or more than eight): at the edges of the rule, of a block and of
+    # a round, and several rounds.  A row's products, sums
+    # and their order are the same in every block, so its outputs are too.
+    x, y = _data(n, 6)
+    net = _net("bf16", I.mlp_init_params(5), _norm(x, y))
+    whole = net.infer(x).cpu().numpy()
+    parts = np.concatenate([net.infer(x[i:i + 4001]).cpu().numpy() for i in range(0, n, 4001)])
+    assert np.array_equal(whole.view(np.uint32), parts.view(np.uint32))
+    net.close()
