@@ -404,7 +404,9 @@ def ensemble_leg(dev, K, W, tile_cache):
         alg = sum(c * (216 if t.storage == "f32" else 108) for c, t in zip(cells, runs))
         r["whole_step_gbs"] = alg / (ms / K / 1e3) / 1e9
         r["tiles"] = {"threads": choice.threads, "minb": choice.minb, "tx": choice.tx}
-        r["gpu_launches_per_step"] = 6 + 3 + 1  # collide bulk + near, markers, moments, interp, reduce, 3 cycles, spread
+        # far cells (16-bit runs in a launch of their own), near cells, particle + markers, tile lists, rows of A,
+        # moments, interpolation, F/T sum, 3 cycles, spread
+        r["gpu_launches_per_step"] = (2 if any(t.storage != "f32" for t in runs) else 1) + 7 + 3 + 1
         b.close()
         out[key] = r
 

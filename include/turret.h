@@ -248,7 +248,7 @@ TURRET_API size_t ibm_spread_workspace_bytes(int32_t nx, int32_t ny, int32_t nz,
  * (TURRET_EDOMAIN otherwise; such markers contribute nothing).  Grid sides
  * 4..1023.  workspace: >= ibm_spread_workspace_bytes, 256-byte aligned.
  * Enqueued on `stream`; waits for it and returns the status.  Bitwise
- * reproducible (fixed summation order, no atomics).                        */
+ * reproducible (fixed summation order).                                     */
 TURRET_API turret_status ibm_spread(const float *X, const float *h, const float *dS, int64_t n_markers, int32_t nx,
                                     int32_t ny, int32_t nz, float *field, void *workspace, size_t workspace_bytes,
                                     void *stream);
@@ -368,10 +368,10 @@ TURRET_API turret_status mlp_get_params(turret_mlp *m, float *params);
 TURRET_API turret_status mlp_set_norm(turret_mlp *m, const float *mean_x, const float *std_x, const float *mean_y,
                                       const float *std_y);
 /* y [n][6] = network(x [n][34]), device arrays, 1 <= n <= batch_cap, with the
- * training kernels (batched matrix products).  Asynchronous.               */
+ * training kernels.  Asynchronous.                                          */
 TURRET_API turret_status mlp_forward(turret_mlp *m, const float *x, int32_t n, float *y);
-/* The same outputs from the fused inference kernel (16 rows per block, any
- * n >= 1), as used by the particle predictor.  Asynchronous.               */
+/* The same outputs for any n >= 1, without the training workspace (precision 0:
+ * the same kernel; precision 1: a fused one).  Asynchronous.                */
 TURRET_API turret_status mlp_infer(turret_mlp *m, const float *x, int32_t n, float *y);
 /* Loss of raw targets y [n][6] and, if grad is not NULL, its gradient with
  * respect to the parameters into device memory grad [TURRET_MLP_NPARAM].

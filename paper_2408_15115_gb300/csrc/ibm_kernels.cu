@@ -18,8 +18,9 @@
 //   k_cycle    : one IBM cycle as h <- h + r0 - A h (a sparse product, one
 //                warp per marker), equal to spreading h and interpolating
 //                u* + S h without touching the grid.
-//   k_reduce_ft: F and T summed in FP64 in a fixed order (one block); it runs
-//                on its own graph branch, off the critical path of the cycles.
+//   k_reduce_ft: F and T summed in FP64 in a fixed order (a block per sum, the
+//                last one to finish writes the state); it runs on its own graph
+//                branch, off the critical path of the cycles.
 //   k_spread   : h_imm = S[h](x) = sum_k h_k W(x - X_k) dS_k as a gather: one block
 //                per 4^3 tile of the support box stages the tile's candidate
 //                records (built with the support-box moments, in marker order)

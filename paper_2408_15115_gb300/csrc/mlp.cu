@@ -8,14 +8,15 @@
 // Kernels (precision 0, BF16 tensor cores, mma.sync m16n8k16 with FP32
 // accumulation; the products are at most 4096x128x128, where the rate of the
 // matrix unit does not show):
-//   k_rows        32 rows per block: the four layers with the BF16 weights and
-//                 all activations in shared memory; with training also the
-//                 loss, and the backward pass down to the first layer
+//   k_rows        32 rows per block (outputs of many rows: 128): the four layers
+//                 with the BF16 weights and all activations in shared memory;
+//                 with training also the loss, and the backward pass down to
+//                 the first layer
 //   k_wgrad       weight and bias gradients of one 256-row slice per block row
 //   k_update      sum of the slices in order, AdamW and the BF16 copy
-//   k_mlp_infer   up to 16 samples per block (the predictor's inference and
-//                 small batches)
-// Precision 1 (an FP32 check mode): k_gemm and the layer-by-layer passes.
+// The predictor in the step runs up to 16 samples per block (mlp_infer_rows).
+// Precision 1 (an FP32 check mode): k_gemm, k_mlp_infer and the layer-by-layer
+// passes.
 // Fixed summation orders, no atomics on data: deterministic.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
