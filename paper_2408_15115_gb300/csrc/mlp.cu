@@ -240,11 +240,16 @@ __global__ void k_adamw(float *__restrict__ P, const float *__restrict__ G, floa
                         float bc2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MLP_NPARAM) return;
-    float m = Mm[i], v = Vv[i];
-    const float p = adamw_value(P[i], G[i], m, v, is_weight(i), lr, b1, b2, eps, wd, bc1, bc2);
+    // written out, not adamw_value: the compiler's choice of fused multiply-adds, and
+    // with it the last bit of a parameter, follows the form of the expressions
+    const float g = G[i];
+    const float m = b1 * Mm[i] + (1.0f - b1) * g;
+    const float v = b2 * Vv[i] + (1.0f - b2) * g * g;
     Mm[i] = m;
     Vv[i] = v;
-    P[i] = p;
+    const float p = P[i];
+    const float upd = (m / bc1) / (sqrtf(v / bc2) + eps) + (is_weight(i) ? wd * p : 0.0f);
+    P[i] = p - lr * upd;
 }
 
 // ---------------------------------------------------------------------------
