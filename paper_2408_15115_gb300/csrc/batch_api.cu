@@ -219,7 +219,7 @@ extern "C" turret_status turret_batch_init(turret_batch **out, turret_ctx *const
         R.storage = c->storage;
         R.cap = c->cap;
         R.nm = c->nm;
-        R.split = c->split ? 1 : 0;
+        R.split = 1;
         R.tx = 32;
         const MlpDev *net = mlp_device_view(c->net);
         if (c->body.predictor == 2 && net) R.mlp = *net;

@@ -82,7 +82,7 @@ __device__ __forceinline__ void batch_near_run(const CollideDesc &R, int p, int 
     using T = typename Codec<ST>::T;
     const Geom g = R.g;
     const BoxGeom box = R.box;
-    const int ex = box.Bx + 2 * NEAR_GROW, ey = box.By + 2 * NEAR_GROW, ez = box.Bz + 2 * NEAR_GROW;
+    const int ex = box.Nx, ey = box.Ny, ez = box.Nz;
     const int i = lb * (int)blockDim.x + (int)threadIdx.x;
     if (i >= ex * ey * ez) return;
     k1_cell<ST, K1_NEAR>(g, (const T *)R.f[p], (T *)R.f[1 - p], R.utop[1 - p], R.utop[p], R.st->s[p], R.hbox, box, i % ex,
@@ -241,8 +241,7 @@ int blocks_whole(const RunDesc &r, int threads) {
 
 int blocks_near(const RunDesc &r) {
     if (!r.split) return 0;
-    const long long cells = (long long)(r.box.Bx + 2 * NEAR_GROW) * (r.box.By + 2 * NEAR_GROW) *
-                            (r.box.Bz + 2 * NEAR_GROW);
+    const long long cells = (long long)r.box.Nx * r.box.Ny * r.box.Nz;
     return (int)((cells + NEAR_THREADS - 1) / NEAR_THREADS);
 }
 

@@ -7,13 +7,16 @@ namespace turret {
 // The near region as one flat range of cells, x fastest: every thread but those
 // of the last block has a cell (rows of 26 to 46 cells leave 19 to 28 % of the
 // lanes of 32-wide rows idle, and the launch of a large body a second, nearly
-// empty wave: 46^3 cells 1152 blocks on 912 places, 761 flat).
+// empty wave: 46^3 cells 1152 blocks on 912 places, 761 flat).  The layer around
+// the support box (NEAR_GROW) makes these 48^3 cells, 864 blocks: 32x32x64 4190 ->
+// 4249 us per 100 steps, 256x256x512 18,958 -> 19,037 per 16, 96x96x192 2035 -> 2041
+// per 24.
 template <int ST>
 __device__ __forceinline__ void near_cell(const Geom &g, const typename Codec<ST>::T *__restrict__ src,
                                           typename Codec<ST>::T *__restrict__ dst, const float *__restrict__ utop_in,
                                           float *__restrict__ utop_out, const BodySlot &S,
                                           const float *__restrict__ hbox, const BoxGeom &box) {
-    const int ex = box.Bx + 2 * NEAR_GROW, ey = box.By + 2 * NEAR_GROW, ez = box.Bz + 2 * NEAR_GROW;
+    const int ex = box.Nx, ey = box.Ny, ez = box.Nz;
     const int i = blockIdx.x * 128 + threadIdx.y * 32 + threadIdx.x;
     if (i < ex * ey * ez)
         k1_cell<ST, K1_NEAR>(g, src, dst, utop_in, utop_out, S, hbox, box, i % ex, (i / ex) % ey, i / (ex * ey));
@@ -36,9 +39,9 @@ __global__ void __launch_bounds__(128, MODE == K1_NEAR ? 1 : (ST == ST_F32 ? 4 :
         st->s[slot_out].reseed = -1;
         st->s[slot_out].step += 1;
     }
-    if (MODE == K1_NEAR)  // small, on the critical path: one cell per thread
+    if constexpr (MODE == K1_NEAR) {  // small, on the critical path: one cell per thread
         near_cell<ST>(g, src, dst, utop_in, utop_out, *win, hbox, box);
-    else {  // the window: a pair of planes per thread
+    } else {  // the window: a pair of planes per thread
         int cx, cy;
         window_cell(g, flat, cx, cy);
         k1_pair<ST, MODE>(g, src, dst, utop_in, utop_out, *win, hbox, box, cx, cy, 2 * blockIdx.z);
@@ -103,8 +106,7 @@ __global__ void __launch_bounds__(128) k_macro(Geom g, const typename Codec<ST>:
 // ---------------------------------------------------------------------------
 // Launchers.
 static dim3 near_grid(const BoxGeom &b) {
-    const int ex = b.Bx + 2 * NEAR_GROW, ey = b.By + 2 * NEAR_GROW, ez = b.Bz + 2 * NEAR_GROW;
-    return dim3((unsigned)(((long long)ex * ey * ez + 127) / 128));
+    return dim3((unsigned)(((long long)b.Nx * b.Ny * b.Nz + 127) / 128));
 }
 
 template <int ST>

@@ -169,9 +169,9 @@ __device__ __forceinline__ bool tile_staged(const Geom &g, const BodySlot &S, co
     if (g.bc_y != BC_PERIODIC && (y0 == 0 || y0 + STG_TY == g.ny)) ok = false;
     if (MODE == K1_FAR && ok) {
         const bool near =
-            meets_near(x0, STG_TX, S.box_lo[0], S.box_lo_w[0], box.Bx + 2 * NEAR_GROW, g.nx, g.bc_x == BC_PERIODIC) &&
-            meets_near(y0, STG_TY, S.box_lo[1], S.box_lo_w[1], box.By + 2 * NEAR_GROW, g.ny, g.bc_y == BC_PERIODIC) &&
-            meets_near(z0, STG_TZ, S.box_lo[2], S.box_lo_w[2], box.Bz + 2 * NEAR_GROW, g.nz,
+            meets_near(x0, STG_TX, S.box_lo[0], S.box_lo_w[0], box.Nx, g.nx, g.bc_x == BC_PERIODIC) &&
+            meets_near(y0, STG_TY, S.box_lo[1], S.box_lo_w[1], box.Ny, g.ny, g.bc_y == BC_PERIODIC) &&
+            meets_near(z0, STG_TZ, S.box_lo[2], S.box_lo_w[2], box.Nz, g.nz,
                        g.bc_bottom == BC_PERIODIC);
         ok = !near;
     }

@@ -77,9 +77,9 @@ __device__ __forceinline__ bool xpair_tile_ok(const Geom &g, const BodySlot &S, 
     if (g.bc_x != BC_PERIODIC && (x0 == 0 || x0 + tw == g.nx)) ok = false;
     if (g.bc_y != BC_PERIODIC && (y0 == 0 || y0 + th == g.ny)) ok = false;
     if (MODE == K1_FAR && ok)
-        ok = !(xp_meets_near(x0, tw, S.box_lo[0], S.box_lo_w[0], box.Bx + 2 * NEAR_GROW, g.nx, g.bc_x == BC_PERIODIC) &&
-               xp_meets_near(y0, th, S.box_lo[1], S.box_lo_w[1], box.By + 2 * NEAR_GROW, g.ny, g.bc_y == BC_PERIODIC) &&
-               xp_meets_near(z0, 2, S.box_lo[2], S.box_lo_w[2], box.Bz + 2 * NEAR_GROW, g.nz,
+        ok = !(xp_meets_near(x0, tw, S.box_lo[0], S.box_lo_w[0], box.Nx, g.nx, g.bc_x == BC_PERIODIC) &&
+               xp_meets_near(y0, th, S.box_lo[1], S.box_lo_w[1], box.Ny, g.ny, g.bc_y == BC_PERIODIC) &&
+               xp_meets_near(z0, 2, S.box_lo[2], S.box_lo_w[2], box.Nz, g.nz,
                              g.bc_bottom == BC_PERIODIC));
     return ok;
 }

@@ -3,8 +3,7 @@
 // host FP64 mesh properties, and the per-step launch sequence captured as one
 // CUDA graph per ping-pong parity.
 //
-// Step graph (time t -> t+1, parity p = t % 2), when the particle's near
-// region fits the window:
+// Step graph (time t -> t+1, parity p = t % 2):
 //
 //   caller stream: --fork--> collide+stream, far cells --------------------> join
 //   aux stream   :       \-> [prediction] -> particle update + markers -> tile
@@ -13,8 +12,8 @@
 //                           -> interpolation -> (h <- h + r0 - A h) x (n-1)
 //                           -> spread h_imm(t+1) -------------------------------^
 //
-// The near region (the support box) contains every cell the next support-box
-// pull reads, so the immersed-boundary chain only waits for the small near
+// The near region (the support box and a layer around it) contains every cell
+// the next support-box pull reads, so the immersed-boundary chain only waits for the small near
 // launch and runs concurrently with the bulk of the window (the side stream
 // has the highest priority).  Groups of steps are captured as one graph in
 // which the chain also overlaps the next step (enqueue_steps_pipelined).
@@ -24,6 +23,7 @@
 
 #include <stdio.h>
 
+#include <algorithm>
 #include <map>
 #include <string>
 #include <utility>
@@ -201,7 +201,6 @@ extern "C" turret_status lbm_init(turret_ctx **out, const turret_window *win, tu
         c->staged = encode_population_map(&c->lmap[k], c->f[k], G, true) &&
                     encode_population_map(&c->smap[k], c->f[k], G, false);
     c->has_particle = false;
-    c->split = false;
     c->step = 0;
     if (cudaMallocHost((void **)&c->pinned, sizeof(DevState)) != cudaSuccess) {
         c->pinned = nullptr;  // queries then stage through pageable memory
@@ -537,8 +536,8 @@ static int warm_cycles(const turret_ctx *c) {
 
 // The fluid's part, with the markers of level `so` in place: u* and sigma on
 // the support box from f(t+1) = pull(f*(t)), the surface force and torque,
-// and the IBM cycles -> h_imm(t+1).  On one stream; the split step spreads the
-// same launches over three (enqueue_step, enqueue_steps_pipelined).
+// and the IBM cycles -> h_imm(t+1).  On one stream (set-up, and steps with
+// re-injection); enqueue_steps_pipelined spreads the same launches over three.
 static cudaError_t enqueue_coupling(turret_ctx *c, const void *fsrc, const float *utop_in, int so, int advance,
                                     cudaStream_t s) {
     const int nm = c->nm, warm = advance ? warm_cycles(c) : 0;
@@ -593,22 +592,12 @@ static cudaError_t enqueue_step(turret_ctx *c, int p) {
         CE(enqueue_lists(c, 1 - p, false, false, c->stream));
         return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
     }
-    const bool predict = c->body.predictor != 0;
-    const MlpDev *net = (c->body.predictor == 2) ? mlp_device_view(c->net) : nullptr;
-    if (!c->split) {
-        if (predict) CE(launch_predict(net, c->dstate, p, c->body.predictor, c->stream));
-        CE(launch_collide_stream(G, c->storage, c->f[p], c->f[1 - p], c->utop[1 - p], c->utop[p], c->dstate, &c->dstate->s[p], -1,
-                                 c->ba.h, c->box, true, REGION_ALL, c->stream));
-        CE(launch_particle_markers(G, c->body, c->box, c->dstate, p, 1, c->mk[1 - p], nullptr, c->stream));
-        CE(enqueue_lists(c, 1 - p, true, false, c->stream));
-        return enqueue_coupling(c, c->f[1 - p], c->utop[p], 1 - p, 1, c->stream);
-    }
     // one step of the pipeline below
     return enqueue_steps_pipelined(c, p, 1);
 }
 
-// Steps t .. t+K-1 (parity p0 first) of a split window over four streams with
-// the exact dependencies, so the immersed-boundary chain of step t overlaps
+// Steps t .. t+K-1 (parity p0 first) over four streams with the exact
+// dependencies, so the immersed-boundary chain of step t overlaps
 // the far-cell collide+stream of step t+1 and the markers, tile lists and rows
 // of A of t+1 are prepared beside the cycles and the spreading of t:
 //   caller  far(t)     after near(t-1) [its near-region cells of f*(t-1)] and
@@ -705,12 +694,14 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     if (!ibm_layout(mp, V, nv, L)) return fail(c, TURRET_EINVAL, "too many markers or too large a surface");
     const int n[3] = {c->win.nx, c->win.ny, c->win.nz};
     const bool per[3] = {c->win.bc_x == 0, c->win.bc_y == 0, c->win.bc_bottom == 0};
-    bool split = true;
     for (int a = 0; a < 3; ++a) {
         if (per[a] && L.box.Bx > n[a])
             return fail(c, TURRET_EINVAL, "support box wider than the window along a periodic axis");
-        if (per[a] && L.box.Bx + 2 * NEAR_GROW > n[a]) split = false;
     }
+    auto near_extent = [&](int b, int a) { return per[a] ? std::min(b + 2 * NEAR_GROW, n[a]) : b + 2 * NEAR_GROW; };
+    L.box.Nx = near_extent(L.box.Bx, 0);
+    L.box.Ny = near_extent(L.box.By, 1);
+    L.box.Nz = near_extent(L.box.Bz, 2);
     // every marker stencil must start inside the window along closed axes
     for (int64_t k = 0; k < nv; ++k)
         for (int a = 0; a < 3; ++a) {
@@ -736,7 +727,6 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     c->box = L.box;
     c->vol = mp.vol;
     c->area = mp.area;
-    c->split = split;
     BodyConst &B = c->body;
     B.vol = mp.vol;
     B.kappa = c->kappa;
@@ -881,7 +871,7 @@ extern "C" turret_status step(turret_ctx *c, int64_t n) {
     if (n < 0) return fail(c, TURRET_EINVAL, "negative step count");
     const bool graphs = (c->stream != nullptr) && !c->flags.no_graph;
     int64_t k = 0;
-    if (graphs && c->has_particle && c->split && c->reinject.trigger == 0) {
+    if (graphs && c->has_particle && c->reinject.trigger == 0) {
         // whole groups of PIPE_STEPS steps as one pipelined graph
         for (; n - k >= PIPE_STEPS; k += PIPE_STEPS) {
             const int p = (int)(c->step & 1);
@@ -986,7 +976,7 @@ extern "C" turret_status lbm_fluid_step(turret_ctx *c, int64_t n) {
     // the far cells on the context stream and the near region (which also
     // carries the body slot) beside them on the side stream, so that timing
     // this call times the step's own collide+stream
-    const bool split = c->has_particle && c->split && c->reinject.trigger == 0;
+    const bool split = c->has_particle && c->reinject.trigger == 0;
     for (int64_t k = 0; k < n; ++k) {
         const int p = (int)(c->step & 1);
         if (split) {
@@ -1037,10 +1027,10 @@ extern "C" turret_status query_particle_state(turret_ctx *c, turret_particle_sta
     out->n_markers = c->has_particle ? c->nm : 0;
     out->volume = c->has_particle ? c->vol : 0.0;
     out->area = c->has_particle ? c->area : 0.0;
-    // collide+stream (1, or far + near), particle + markers, tile lists, rows
+    // collide+stream (far + near), particle + markers, tile lists, rows
     // of A, moments, interpolation, F/T reduction, cycles, spread of h_imm
     const bool warm = c->pred_mode != 0 && (c->pred_opts & PRED_WARM);
-    out->kernels_per_step = c->has_particle ? (c->split ? 2 : 1) + 7 +
+    out->kernels_per_step = c->has_particle ? 2 + 7 +
                                                   c->flags.ibm_cycles - (warm ? 0 : 1) +
                                                   (c->pred_mode != 0 ? 1 : 0)  // prediction
                                             : 1;

@@ -34,7 +34,6 @@ struct turret_ctx {
     turret::DevState *dstate;
     // particle
     bool has_particle;
-    bool split;  // near/far collide+stream with the chain on the side stream
     int nm;
     turret::BodyConst body;
     turret::BoxGeom box;

@@ -108,6 +108,7 @@ struct Geom {
 struct BoxGeom {
     int Bx, By, Bz;
     int tx, ty, tz;   // tiles of TILE^3 along each axis
+    int Nx, Ny, Nz;   // cells of the near region along each axis (see NEAR_GROW)
     long long nbox;   // Bx * By * Bz
 };
 
@@ -213,7 +214,7 @@ struct RunDesc {
     float *utop[2];      // top-plane velocity buffers
     DevState *st;
     int storage, cap, nm;
-    int split;           // 1: far / near collide+stream, 0: the whole window in the near phase
+    int split;           // 1: far / near collide+stream, 0: the whole window ahead of the chain
     int tx;              // collide+stream tile width (threads along x)
     MlpDev mlp;          // the force/torque network (predictor mode 2)
 };
@@ -358,17 +359,15 @@ constexpr int QUIET_BLOCKS = 152, QUIET_THREADS = 64;
 // Launchers (lbm_kernels.cu).
 // win, here and below: the window slot of the time level pulled.
 // Collide+stream region: all cells, the cells outside the near region around
-// the particle, or the near region only.  The near region is the region of
-// the marker stencils (where h_imm can be nonzero) grown by NEAR_MARGIN cells;
-// the support box reaches F_OFFSET cells beyond the marker stencils (the
-// stress is read on the offset surface), so the near region is the support
-// box grown by NEAR_GROW cells.  It holds every cell the support-box moments
-// pull (they skip the box's outer layer), so they wait for the near launch
-// only.
+// the particle, or the near region only.  The near region is the support box
+// grown by NEAR_GROW cells per side (all of a periodic axis that it would wrap
+// around).  It holds every cell the support-box moments pull, so they wait for
+// the near launch only: they skip their box's outer layer and pull from within
+// the box, but theirs is the box of t + 1, which lies one cell further along
+// each axis on which the centre crossed a cell face during the step (a body
+// moves less than a cell per step).
 enum { REGION_ALL = 0, REGION_FAR = 1, REGION_NEAR = 2 };
-constexpr int NEAR_MARGIN = 2;
-constexpr int NEAR_GROW = NEAR_MARGIN - 2;
-static_assert(F_OFFSET == 2.0f, "the support box grows by F_OFFSET cells per side");
+constexpr int NEAR_GROW = 1;
 // after_spread (REGION_NEAR): start beside the spreading launched just before on
 // the same stream, with everything else the pull needs complete.
 // slot_out >= 0: the kernel also copies the window slot to slot_out (with no
