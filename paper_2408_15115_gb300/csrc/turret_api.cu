@@ -779,6 +779,9 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
     CK(cudaMemcpyAsync((void *)c->mk[0].dSo, c->staging.data() + 7 * nm, nm * 4, cudaMemcpyHostToDevice, c->stream),
        "dSo");
     CK(cudaMemsetAsync(c->ba.h, 0, 3 * (size_t)L.box.nbox * 4, c->stream), "h");
+    // a batched step leaves the row of a marker that its tile's lists cannot hold
+    // as it was (and latches the overflow), and its cycles read every row's length
+    for (int k = 0; k < 2; ++k) CK(cudaMemsetAsync(c->mk[k].alen, 0, nm * 4, c->stream), "row lengths");
     // the moments kernel skips the box cells no stencil reads: they keep
     // finite values (zeros, or an earlier step's moments)
     CK(cudaMemsetAsync(c->ba.u, 0, (size_t)L.box.nbox * 16, c->stream), "u");

@@ -223,3 +223,24 @@ def test_batched_16bit_xpair_launch_equals_runs_alone_bitwise():
         _assert_same(_snapshot(t), r)
     assert abs(runs[0].state()["origin"][2]) >= 1 and abs(runs[1].state()["origin"][2]) >= 1  # both slid
     b.close()
+
+
+def test_crowded_tiles_end_a_batched_step_with_overflow(monkeypatch):
+    # more markers per support tile than a batched step lists: their rows of A are
+    # skipped and the overflow latched; rows never built have length zero, whatever
+    # the workspace held before (here 0x3f3f3f3f, a length of a billion entries)
+    import torch
+    from paper_2408_15115_gb300 import turret as T
+    empty = torch.empty
+    monkeypatch.setattr(torch, "empty", lambda *a, **k: empty(*a, **k).fill_(0x3f)
+                        if k.get("dtype") is torch.uint8 else empty(*a, **k))
+    V, Tr = I.icosphere(14, 3.5)
+    t = T.Turret(24, 24, 32, 0.05, 2.0, (0, 0, 0), 1, 1, 1, 1)
+    t.load_surface(V, Tr, (11.5, 11.5, 16.0))
+    b = T.Batch([t])
+    b.step(2)
+    b.close()
+    with pytest.raises(T.TurretError) as e:
+        t.state()
+    assert e.value.status == 8
+    t.close()
