@@ -282,7 +282,8 @@ TURRET_API turret_status ibm_spread_noalloc(const float *X, const float *h, cons
  * IBM cycles, spreading, F/T reduction) ONCE for all runs, over a table of
  * (run, block) pairs, and replays it as one CUDA graph per step parity.  The
  * per-cell and per-marker arithmetic is the single-run arithmetic, so every
- * run of a batch evolves bit for bit as it does alone under step().          */
+ * run of a batch evolves bit for bit as it does alone under step(), with the
+ * settings its context has when a call steps it.                             */
 typedef struct turret_batch turret_batch;
 
 /* Bytes of device workspace a batch of n_runs runs needs (descriptors and
@@ -312,7 +313,8 @@ TURRET_API turret_status turret_batch_set_tiles(turret_batch *b, int32_t threads
 
 /* Advances every run of the batch by n coupled steps (the order of step()).
  * Runs may be stepped alone between calls; every run must then still be at a
- * time level of the same parity (TURRET_ESTATE otherwise).                  */
+ * time level of the same parity, and their settings as turret_batch_init
+ * wants them (TURRET_ESTATE otherwise).                                     */
 TURRET_API turret_status turret_batch_step(turret_batch *b, int64_t n);
 
 /* Releases the batch (not the contexts or the workspace); waits for it.     */

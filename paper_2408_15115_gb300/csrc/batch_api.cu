@@ -13,6 +13,9 @@
 //                           -> rows of A          ... -> F, T of every run (FP64) ^
 //   side stream :       \-> near collide+stream -> support moments
 //                           -> interpolation -> cycles -> spread ----------------^
+//
+// (With runs that re-inject: their whole windows behind the near cells, then the
+// copies, and the tile lists and rows behind those.)
 #include <cuda_runtime.h>
 #include <string.h>
 
@@ -49,6 +52,8 @@ struct turret_batch {
     std::vector<int> h_prefix;
     int total[T_COUNT];
     int threads, minb, cycles, predictor, warm;
+    bool reinject;                    // some run re-injects
+    std::vector<long long> settings;  // turret_ctx::settings behind each descriptor
     long long step;
     cudaGraphExec_t graph[2];
     bool graph_ready[2];
@@ -161,49 +166,35 @@ static void release_batch(turret_batch *b) {
     delete b;
 }
 
-extern "C" turret_status turret_batch_init(turret_batch **out, turret_ctx *const *ctxs, int32_t n, void *ws,
-                                           size_t ws_bytes, void *stream) {
-    turret_batch *b = nullptr;
-    if (!out) return bfail(b, TURRET_EINVAL, "out is NULL");
-    *out = nullptr;
-    if (!ctxs || n < 1) return bfail(b, TURRET_EINVAL, "no runs");
-    std::set<const turret_ctx *> seen;
+// Whether the runs can be stepped together with their present settings.
+static turret_status check_settings(turret_ctx *const *ctxs, int n, std::string &why) {
     for (int r = 0; r < n; ++r) {
         const turret_ctx *c = ctxs[r];
-        if (!c) return bfail(b, TURRET_EINVAL, "NULL context in the run list");
-        if (!seen.insert(c).second) return bfail(b, TURRET_EINVAL, "a context appears twice");
-        if (!c->has_particle) return bfail(b, TURRET_ESTATE, "every run needs a loaded surface");
-        if ((c->step & 1) != (ctxs[0]->step & 1)) return bfail(b, TURRET_ESTATE, "runs at time levels of different parity");
-        if (c->flags.ibm_cycles != ctxs[0]->flags.ibm_cycles)
-            return bfail(b, TURRET_EINVAL, "runs with different ibm_cycles");
-        if ((c->body.predictor != 0) != (ctxs[0]->body.predictor != 0))
-            return bfail(b, TURRET_EINVAL, "runs with and without a force predictor");
-        if (c->body.predictor != 0 && ((c->body.pred_opts ^ ctxs[0]->body.pred_opts) & PRED_WARM))
-            return bfail(b, TURRET_EINVAL, "runs with and without warm-started IBM cycles");
+        if (c->flags.ibm_cycles != ctxs[0]->flags.ibm_cycles) why = "runs with different ibm_cycles";
+        else if ((c->body.predictor != 0) != (ctxs[0]->body.predictor != 0)) why = "runs with and without a force predictor";
+        else if (c->body.predictor != 0 && ((c->body.pred_opts ^ ctxs[0]->body.pred_opts) & PRED_WARM))
+            why = "runs with and without warm-started IBM cycles";
+        else continue;
+        return TURRET_EINVAL;
     }
-    if (!ws || ws_bytes < turret_batch_workspace_bytes(n)) return bfail(b, TURRET_ENOMEM, "batch workspace too small");
-    if (((uintptr_t)ws & 255) != 0) return bfail(b, TURRET_EINVAL, "workspace must be 256-byte aligned");
+    return TURRET_OK;
+}
 
-    b = new turret_batch();
-    b->n = n;
-    b->ctx.assign(ctxs, ctxs + n);
-    b->stream = (cudaStream_t)stream;
-    b->side = b->aux = nullptr;
-    b->ev_fork = b->ev_join = b->ev_red = b->ev_red_done = b->ev_done = b->ev_pred = b->ev_rows = nullptr;
-    b->graph_ready[0] = b->graph_ready[1] = false;
-    b->d_runs = (RunDesc *)ws;
-    b->d_prefix = (int *)((char *)ws + prefix_offset(n));
-    b->d_cdesc = (CollideDesc *)((char *)ws + cdesc_offset(n));
-    b->threads = 128;
-    b->minb = 2;
-    b->cycles = ctxs[0]->flags.ibm_cycles;
-    b->predictor = ctxs[0]->body.predictor != 0 ? 1 : 0;
-    b->warm = (b->predictor && (ctxs[0]->body.pred_opts & PRED_WARM)) ? 1 : 0;
-    b->step = ctxs[0]->step;
-    b->h_runs.resize(n);
-    for (int r = 0; r < n; ++r) {
-        const turret_ctx *c = ctxs[r];
+// The descriptors of the runs with their present settings (tile widths stay).
+// A run that re-injects is stepped as it is alone: the whole window ahead of
+// the chain, with the copy between.
+static void describe_runs(turret_batch *b) {
+    const turret_ctx *c0 = b->ctx[0];
+    b->cycles = c0->flags.ibm_cycles;
+    b->predictor = c0->body.predictor != 0 ? 1 : 0;
+    b->warm = (b->predictor && (c0->body.pred_opts & PRED_WARM)) ? 1 : 0;
+    b->reinject = false;
+    b->h_runs.resize(b->n);
+    b->settings.resize(b->n);
+    for (int r = 0; r < b->n; ++r) {
+        const turret_ctx *c = b->ctx[r];
         RunDesc &R = b->h_runs[r];
+        const int tx = R.tx;
         memset(&R, 0, sizeof R);
         R.g = c->geom;
         R.bc = c->body;
@@ -219,11 +210,49 @@ extern "C" turret_status turret_batch_init(turret_batch **out, turret_ctx *const
         R.storage = c->storage;
         R.cap = c->cap;
         R.nm = c->nm;
-        R.split = 1;
-        R.tx = 32;
+        R.split = c->reinject.trigger == 0;
+        R.tx = tx;
         const MlpDev *net = mlp_device_view(c->net);
         if (c->body.predictor == 2 && net) R.mlp = *net;
+        b->reinject = b->reinject || !R.split;
+        b->settings[r] = c->settings;
     }
+}
+
+extern "C" turret_status turret_batch_init(turret_batch **out, turret_ctx *const *ctxs, int32_t n, void *ws,
+                                           size_t ws_bytes, void *stream) {
+    turret_batch *b = nullptr;
+    if (!out) return bfail(b, TURRET_EINVAL, "out is NULL");
+    *out = nullptr;
+    if (!ctxs || n < 1) return bfail(b, TURRET_EINVAL, "no runs");
+    std::set<const turret_ctx *> seen;
+    for (int r = 0; r < n; ++r) {
+        const turret_ctx *c = ctxs[r];
+        if (!c) return bfail(b, TURRET_EINVAL, "NULL context in the run list");
+        if (!seen.insert(c).second) return bfail(b, TURRET_EINVAL, "a context appears twice");
+        if (!c->has_particle) return bfail(b, TURRET_ESTATE, "every run needs a loaded surface");
+        if ((c->step & 1) != (ctxs[0]->step & 1)) return bfail(b, TURRET_ESTATE, "runs at time levels of different parity");
+    }
+    std::string why;
+    if (check_settings(ctxs, n, why) != TURRET_OK) return bfail(b, TURRET_EINVAL, why);
+    if (!ws || ws_bytes < turret_batch_workspace_bytes(n)) return bfail(b, TURRET_ENOMEM, "batch workspace too small");
+    if (((uintptr_t)ws & 255) != 0) return bfail(b, TURRET_EINVAL, "workspace must be 256-byte aligned");
+
+    b = new turret_batch();
+    b->n = n;
+    b->ctx.assign(ctxs, ctxs + n);
+    b->stream = (cudaStream_t)stream;
+    b->side = b->aux = nullptr;
+    b->ev_fork = b->ev_join = b->ev_red = b->ev_red_done = b->ev_done = b->ev_pred = b->ev_rows = nullptr;
+    b->graph_ready[0] = b->graph_ready[1] = false;
+    b->d_runs = (RunDesc *)ws;
+    b->d_prefix = (int *)((char *)ws + prefix_offset(n));
+    b->d_cdesc = (CollideDesc *)((char *)ws + cdesc_offset(n));
+    b->threads = 128;
+    b->minb = 2;
+    b->step = ctxs[0]->step;
+    describe_runs(b);
+    for (RunDesc &R : b->h_runs) R.tx = 32;
     if (!build_tables(b)) {
         release_batch(b);
         return bfail(nullptr, TURRET_EINVAL, "too many blocks in one batched launch");
@@ -289,15 +318,28 @@ static cudaError_t batch_enqueue(turret_batch *b, int p) {
     if (b->predictor) CE(launch_batch_predict(R, n, p, b->aux));
     CE(launch_batch_particle_markers(R, tab(T_PM), n, p, b->total[T_PM], b->aux));
     CE(cudaEventRecord(b->ev_pred, b->aux));
-    CE(launch_batch_bin(R, tab(T_BIN), n, p, b->total[T_BIN], b->aux));
-    CE(launch_batch_rows(R, tab(T_ROWS), n, p, b->total[T_ROWS], b->aux));
-    CE(cudaEventRecord(b->ev_rows, b->aux));
+    auto lists = [&]() -> cudaError_t {
+        CE(launch_batch_bin(R, tab(T_BIN), n, p, b->total[T_BIN], b->aux));
+        CE(launch_batch_rows(R, tab(T_ROWS), n, p, b->total[T_ROWS], b->aux));
+        return cudaEventRecord(b->ev_rows, b->aux);
+    };
+    if (!b->reinject) CE(lists());
     CE(launch_batch_collide(PHASE_BULK, b->d_cdesc, tab(T_BULK), n, p, b->total[T_BULK], b->threads, b->minb,
                             b->stream));
     CE(launch_batch_collide(PHASE_BULK16, b->d_cdesc, tab(T_BULK16), n, p, b->total[T_BULK16], 128, 5, b->stream));
     CE(launch_batch_collide(PHASE_NEAR, b->d_cdesc, tab(T_NEAR), n, p, b->total[T_NEAR], NEAR_THREADS, 6, b->side));
     CE(launch_batch_collide(PHASE_WHOLE, b->d_cdesc, tab(T_WHOLE), n, p, b->total[T_WHOLE], b->threads, 2, b->side));
     CE(cudaStreamWaitEvent(b->side, b->ev_pred, 0));
+    if (b->reinject) {
+        // the copies of the runs that re-inject, which also move their window
+        // slots: the lists read those
+        for (const turret_ctx *c : b->ctx)
+            if (c->reinject.trigger > 0)
+                CE(launch_reinject(c->geom, c->storage, c->f[1 - p], c->f[p], c->dstate, 1 - p, c->reinject, b->side));
+        CE(cudaEventRecord(b->ev_red, b->side));
+        CE(cudaStreamWaitEvent(b->aux, b->ev_red, 0));
+        CE(lists());
+    }
     CE(launch_batch_box_moments(R, tab(T_MOM), n, p, b->total[T_MOM], b->side));
     CE(launch_batch_interp(R, tab(T_INT), n, p, b->total[T_INT], b->warm, b->side));
     CE(cudaEventRecord(b->ev_red, b->side));
@@ -354,6 +396,21 @@ extern "C" turret_status turret_batch_step(turret_batch *b, int64_t nsteps) {
     for (int r = 0; r < b->n; ++r) {
         BK(cudaEventRecord(b->ev_ctx[r], b->ctx[r]->stream), "order after run streams");
         BK(cudaStreamWaitEvent(b->stream, b->ev_ctx[r], 0), "order after run streams");
+    }
+    // the descriptors hold the runs' settings: a predictor, log, wall velocity or
+    // re-injection set since they were made
+    bool changed = false;
+    for (int r = 0; r < b->n; ++r) changed = changed || b->settings[r] != b->ctx[r]->settings;
+    if (changed) {
+        std::string why;
+        if (check_settings(b->ctx.data(), b->n, why) != TURRET_OK) return bfail(b, TURRET_ESTATE, why);
+        describe_runs(b);
+        drop_batch_graphs(b);
+        const bool fits = build_tables(b);
+        const cudaError_t e = fits ? upload(b) : cudaSuccess;
+        if (!fits || e != cudaSuccess) b->settings[0] = -1;  // described anew by the next call
+        if (!fits) return bfail(b, TURRET_EINVAL, "too many blocks in one batched launch");
+        BK(e, "settings upload");
     }
     const bool graphs = b->stream != nullptr;
     for (int64_t k = 0; k < nsteps; ++k) {

@@ -163,6 +163,7 @@ extern "C" turret_status lbm_init(turret_ctx **out, const turret_window *win, tu
     memset(&c->flags, 0, sizeof c->flags);
     c->flags.ibm_cycles = 4;
     c->reinject = Reinject{0, 0, 0, 0};
+    c->settings = 0;
     c->storage = (int)st;
     c->nu = nu;
     c->tau0 = tau;
@@ -243,7 +244,9 @@ extern "C" turret_status lbm_init(turret_ctx **out, const turret_window *win, tu
     return TURRET_OK;
 }
 
+// A setting that the step graphs hold has changed.
 static void drop_graphs(turret_ctx *c) {
+    c->settings++;
     for (int k = 0; k < 2; ++k) {
         if (c->graph_ready[k]) cudaGraphExecDestroy(c->graph[k]);
         if (c->multi_ready[k]) cudaGraphExecDestroy(c->graph_multi[k]);

@@ -56,6 +56,7 @@ struct turret_ctx {
     long long log_cap;
     // re-injection copy (Sec. 2.5) instead of the ring window; trigger 0 = off
     turret::Reinject reinject;
+    long long settings;  // counts changes of settings that steps depend on (batches copy them)
     // stepping
     long long step;
     cudaGraphExec_t graph[2];

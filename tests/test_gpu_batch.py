@@ -244,3 +244,60 @@ def test_crowded_tiles_end_a_batched_step_with_overflow(monkeypatch):
         t.state()
     assert e.value.status == 8
     t.close()
+
+
+def _falling(storage, reinject=True):
+    # as test_reinjection_copy_vs_oracle: crosses the trigger plane within 60 steps
+    from paper_2408_15115_gb300 import turret as T
+    V, Tr = I.icosphere(3, 3.0)
+    t = T.Turret(20, 20, 64, 0.1, 2.0, (0, 0, -1e-4), 0, 0, 1, 2, sponge=4, storage=storage)
+    if reinject:
+        t.set_reinjection(22, 40, 12, 14)
+    t.load_surface(V, Tr, (9.8, 10.1, 22.5), (0, 0, -0.05))
+    return t
+
+
+@pytest.mark.parametrize("when", ["before", "after"])
+def test_batched_runs_re_inject(when):
+    # re-injection set before the batch is made or after; beside a run without
+    from paper_2408_15115_gb300 import turret as T
+    forms = [("f32", True), ("f16", True), ("f32", False)]
+    alone = [_falling(*f) for f in forms]
+    runs = [_falling(s, r and when == "before") for s, r in forms]
+    b = T.Batch(runs)
+    if when == "after":
+        for t, (_, r) in zip(runs, forms):
+            if r:
+                t.set_reinjection(22, 40, 12, 14)
+    b.step(41)
+    b.step(19)
+    for t, a in zip(runs, alone):
+        a.step(60)
+        _assert_same(_snapshot(t), _snapshot(a))
+    assert [t.state()["origin"][2] < 0 for t in runs] == [True, True, False]
+    b.close()
+
+
+def test_batch_follows_its_runs_settings():
+    from paper_2408_15115_gb300 import turret as T
+    runs, alone = ([_falling("f32", False) for _ in range(2)] for _ in range(2))
+    b = T.Batch(runs)
+    b.step(5)
+    for t in runs:
+        t.set_predictor("linear", warm=True)
+        t.set_log(64)
+    b.step(11)
+    for t, a in zip(runs, alone):
+        a.step(5)
+        a.set_predictor("linear", warm=True)
+        a.set_log(64)
+        a.step(11)
+        _assert_same(_snapshot(t), _snapshot(a))
+        assert np.array_equal(t.log_records().cpu().numpy(), a.log_records().cpu().numpy())
+    runs[0].set_predictor("paper")  # one of two: the runs no longer step together
+    with pytest.raises(T.TurretError) as e:
+        b.step(1)
+    assert e.value.status == 4
+    runs[1].set_predictor("paper")
+    b.step(2)
+    b.close()
