@@ -505,17 +505,24 @@ class MLP:
     def train_step(self, x, y, lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, want_loss=True):
         """One AdamW step; x, y float32 CUDA tensors [n][34], [n][6] (n <= batch_cap).
 
-        Ordered after the work enqueued on the current stream (x and y may still be in the making)."""
+        Ordered after the work enqueued on the current stream (x and y may still be in the making), unless
+        that stream is being captured: the step is not part of the capture.  x and y may be dropped once
+        the call returns, also without want_loss, when the step still runs."""
         n = x.shape[0]
         cur = self.torch.cuda.current_stream(self.device)
-        if cur != self.stream:
+        if cur != self.stream and not self.torch.cuda.is_current_stream_capturing():
             self._inputs.record(cur)
             self.stream.wait_event(self._inputs)
         opt = AdamW(lr, beta1, beta2, eps, weight_decay)
         L = C.c_float()
         self._check(self._L.mlp_train_step(self.m, C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()), n,
                                            C.byref(opt), C.byref(L) if want_loss else None))
-        return float(L.value) if want_loss else None
+        if want_loss:
+            return float(L.value)
+        for t in (x, y):  # their memory is not handed out again before the step has read it
+            if t.is_cuda:
+                t.record_stream(self.stream)
+        return None
 
     def close(self):
         if getattr(self, "m", None) is not None:

@@ -150,3 +150,54 @@ def test_many_rows_give_the_bits_of_few(n):
     parts = np.concatenate([net.infer(x[i:i + 4001]).cpu().numpy() for i in range(0, n, 4001)])
     assert np.array_equal(whole.view(np.uint32), parts.view(np.uint32))
     net.close()
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp32"])
+def test_training_step_outlives_its_inputs(precision):
+    # the network's stream is busy when the steps are enqueued; their inputs are
+    # dropped at once and the next allocations of that size overwritten
+    import torch
+    x, y = _data(256, 3)
+    norm, p = _norm(x, y), I.mlp_init_params(2)
+    xs = torch.tensor(x, dtype=torch.float32, device="cuda:0")
+    ys = torch.tensor(y, dtype=torch.float32, device="cuda:0")
+    want, got = _net(precision, p, norm), _net(precision, p, norm)
+    torch.cuda.synchronize()
+    for k in range(3):
+        want.train_step(xs * (k + 1), ys + k)
+    for _ in range(2):
+        with torch.cuda.stream(got.stream):
+            torch.cuda._sleep(20_000_000)  # about 10 ms
+        for k in range(3):
+            a, b = xs * (k + 1), ys + k
+            assert got.train_step(a, b, want_loss=False) is None
+            del a, b
+            junk = [torch.full_like(xs, 7.0), torch.full_like(ys, -7.0)]  # noqa: F841
+        torch.cuda.synchronize()
+        assert np.array_equal(got.params().view(np.uint32), want.params().view(np.uint32))
+        got.close()
+        got = _net(precision, p, norm)
+    want.close()
+    got.close()
+
+
+def test_training_step_beside_a_capture():
+    # a capture of the caller's stream neither takes the step in nor refuses it
+    import torch
+    x, y = _data(64, 3)
+    norm, p = _norm(x, y), I.mlp_init_params(2)
+    xs = torch.tensor(x, dtype=torch.float32, device="cuda:0")
+    ys = torch.tensor(y, dtype=torch.float32, device="cuda:0")
+    want, got = _net("bf16", p, norm), _net("bf16", p, norm)
+    torch.cuda.synchronize()
+    want.train_step(xs, ys)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        z = xs + 1.0
+        got.train_step(xs, ys, want_loss=False)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(z, xs + 1.0)
+    assert np.array_equal(got.params().view(np.uint32), want.params().view(np.uint32))
+    want.close()
+    got.close()
