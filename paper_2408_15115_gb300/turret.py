@@ -168,6 +168,16 @@ def _aligned_workspace(torch, nbytes, device):
     return buf, buf.data_ptr() + off
 
 
+def _follow_current(torch, device, stream, event):
+    """`stream`, which is about to use memory that the current stream allocated, follows the current
+    stream's work: an earlier owner of that memory may still be in use there.  (A capture has no work
+    to follow.)"""
+    cur = torch.cuda.current_stream(device)
+    if cur != stream and not torch.cuda.is_current_stream_capturing():
+        event.record(cur)
+        stream.wait_event(event)
+
+
 def ibm_spread(X, h, dS, shape, stream=None):
     """S[h](x) = sum_k h_k W(x - X_k) dS_k on a (nz, ny, nx) grid (Sec. 2.2, step l = 1).
 
@@ -183,6 +193,8 @@ def ibm_spread(X, h, dS, shape, stream=None):
         raise TurretError(1, "invalid spread sizes")
     ws, ptr = _aligned_workspace(torch, nb, dev)
     st = stream if stream is not None else torch.cuda.current_stream(dev)
+    if stream is not None:
+        _follow_current(torch, dev, st, torch.cuda.Event())
     rc = L.ibm_spread(C.c_void_p(X.data_ptr()), C.c_void_p(h.data_ptr()), C.c_void_p(dS.data_ptr()), n, nx, ny, nz,
                       C.c_void_p(out.data_ptr()), C.c_void_p(ptr), C.c_size_t(nb), C.c_void_p(st.cuda_stream))
     if rc != 0:
@@ -210,7 +222,8 @@ class Turret:
         nb = self._L.lbm_workspace_bytes(C.byref(self.win), st)
         if nb == 0:
             raise TurretError(1, "invalid window")
-        self._ws, ptr = _aligned_workspace(torch, nb, self.device)
+        self._order = torch.cuda.Event()
+        self._ws, ptr = self._buffer(nb)
         self._ibm_ws = None
         g3 = (C.c_double * 3)(*g)
         ctx = C.c_void_p()
@@ -228,6 +241,16 @@ class Turret:
     def _check(self, rc):
         if rc != 0:
             raise TurretError(rc, self._L.turret_last_error(self.ctx).decode())
+
+    def _buffer(self, nbytes):
+        buf, ptr = _aligned_workspace(self.torch, nbytes, self.device)
+        _follow_current(self.torch, self.device, self.stream, self._order)
+        return buf, ptr
+
+    def _output(self, n):
+        out = self.torch.empty((n,) + self.shape, dtype=self.torch.float32, device=self.device)
+        _follow_current(self.torch, self.device, self.stream, self._order)
+        return out
 
     def set_wall_velocity(self, u_bottom=(0.0, 0.0, 0.0), u_top=(0.0, 0.0, 0.0)):
         """Velocities of moving bottom / top walls (window bc 3), in their plane."""
@@ -248,7 +271,7 @@ class Turret:
         nb = self._L.ibm_workspace_bytes(self.ctx, vp, V.shape[0], tp, T.shape[0])
         if nb == 0:
             raise TurretError(1, "invalid surface mesh")
-        self._ibm_ws, ptr = _aligned_workspace(self.torch, nb, self.device)
+        self._ibm_ws, ptr = self._buffer(nb)
         r0 = (C.c_double * 3)(*r0)
         v0 = (C.c_double * 3)(*v0)
         w0 = (C.c_double * 3)(*w0)
@@ -273,13 +296,13 @@ class Turret:
 
     def macro(self):
         """(4, nz, ny, nx) float32 tensor: rho, u_x, u_y, u_z of f(t)."""
-        out = self.torch.empty((4,) + self.shape, dtype=self.torch.float32, device=self.device)
+        out = self._output(4)
         self._check(self._L.lbm_copy_macro(self.ctx, C.c_void_p(out.data_ptr())))
         return out
 
     def populations(self):
         """(27, nz, ny, nx) float32 tensor: deviations f_i(t) - w_i."""
-        out = self.torch.empty((27,) + self.shape, dtype=self.torch.float32, device=self.device)
+        out = self._output(27)
         self._check(self._L.lbm_copy_populations(self.ctx, C.c_void_p(out.data_ptr())))
         return out
 
@@ -318,21 +341,23 @@ class Turret:
 
     def set_log(self, capacity):
         """Attach a device trajectory log of `capacity` records (0 detaches)."""
+        log = None
         if capacity > 0:
-            self._log = self.torch.zeros((int(capacity), self.LOG_REC), dtype=self.torch.float64, device=self.device)
-            self._check(self._L.turret_set_log(self.ctx, C.c_void_p(self._log.data_ptr()), int(capacity)))
-        else:
-            self._check(self._L.turret_set_log(self.ctx, None, 0))
-            self._log = None
+            log = self.torch.zeros((int(capacity), self.LOG_REC), dtype=self.torch.float64, device=self.device)
+            _follow_current(self.torch, self.device, self.stream, self._order)
+        self._check(self._L.turret_set_log(self.ctx, None if log is None else C.c_void_p(log.data_ptr()),
+                                           0 if log is None else int(capacity)))
+        self.stream.synchronize()  # steps still running write to the log before
+        self._log = log
 
     def log_records(self):
         """The logged records in time order (float64 CUDA tensor [n][32])."""
         n = self.predictor_stats()["logged"]
         cap = self._log.shape[0]
-        if n <= cap:
-            return self._log[:n].clone()
         k = n % cap
-        return self.torch.cat([self._log[k:], self._log[:k]]).clone()
+        out = self._log[:n].clone() if n <= cap else self.torch.cat([self._log[k:], self._log[:k]])
+        _follow_current(self.torch, self.device, self.stream, self._order)  # later steps write where this reads
+        return out
 
     def predictor_stats(self):
         s = PredictorStats()
@@ -375,6 +400,7 @@ class Batch:
         if nb == 0:
             raise TurretError(1, "empty batch")
         self._ws, ptr = _aligned_workspace(torch, nb, self.device)
+        _follow_current(torch, self.device, self.stream, torch.cuda.Event())
         arr = (C.c_void_p * n)(*[t.ctx.value for t in self.runs])
         b = C.c_void_p()
         rc = self._L.turret_batch_init(C.byref(b), arr, n, C.c_void_p(ptr), C.c_size_t(nb),
@@ -440,7 +466,9 @@ class MLP:
         nb = self._L.mlp_workspace_bytes(self.cap)
         if nb == 0:
             raise TurretError(1, "invalid batch capacity")
+        self._inputs = torch.cuda.Event()  # orders the network's stream after the caller's
         self._ws, ptr = _aligned_workspace(torch, nb, self.device)
+        _follow_current(torch, self.device, self.stream, self._inputs)
         p = _arr(params, np.float32)
         m = C.c_void_p()
         rc = self._L.mlp_init(C.byref(m), self.cap, {"bf16": 0, "fp32": 1}[precision], p.ctypes.data_as(_fp),
@@ -449,7 +477,6 @@ class MLP:
             raise TurretError(rc, self._L.mlp_last_error(None).decode())
         self.m = m
         self.precision = precision
-        self._inputs = torch.cuda.Event()  # orders a training step after its inputs' stream
 
     def _check(self, rc):
         if rc != 0:
@@ -509,10 +536,7 @@ class MLP:
         that stream is being captured: the step is not part of the capture.  x and y may be dropped once
         the call returns, also without want_loss, when the step still runs."""
         n = x.shape[0]
-        cur = self.torch.cuda.current_stream(self.device)
-        if cur != self.stream and not self.torch.cuda.is_current_stream_capturing():
-            self._inputs.record(cur)
-            self.stream.wait_event(self._inputs)
+        _follow_current(self.torch, self.device, self.stream, self._inputs)
         opt = AdamW(lr, beta1, beta2, eps, weight_decay)
         L = C.c_float()
         self._check(self._L.mlp_train_step(self.m, C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()), n,
