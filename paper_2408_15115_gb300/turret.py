@@ -330,10 +330,12 @@ class Turret:
         or 'mlp' (with the MLP object `net`); warm: warm-started adaptive IBM
         cycles; velocity: marker velocities at t + 1; relative: resid_theta is
         a ratio to linear extrapolation's running error.  See turret_set_predictor."""
-        self._net = net
         opts = (1 if warm else 0) | (2 if velocity else 0) | (4 if relative else 0)
         self._check(self._L.turret_set_predictor(self.ctx, self.PREDICTORS[mode], net.m if net is not None else None,
                                                  opts, float(slip_eps), float(resid_theta)))
+        if net is not getattr(self, "_net", None):
+            self.stream.synchronize()  # steps still running read the network before
+        self._net = net  # (only now: a refused call leaves the context with the one before)
 
     def set_reinjection(self, trigger, target, below, above):
         """The re-injection copy of Sec. 2.5 (see turret_set_reinjection); trigger 0 = off."""

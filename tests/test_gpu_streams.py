@@ -69,3 +69,38 @@ def test_workspaces_and_logs_follow_the_writers_of_their_memory():
     want = run(False)
     for a, b in zip(run(True), want):
         assert np.array_equal(a, b, equal_nan=True)
+
+
+def test_networks_in_use_are_kept():
+    # a refused change of the predictor leaves the context with its network, and
+    # the network keeps its memory; a replaced one outlives the steps that read it
+    import torch
+    from paper_2408_15115_gb300 import turret as T
+    V, Tr = I.sphere(3, 5.0)
+
+    def net(seed):
+        n = T.MLP(I.mlp_init_params(seed).astype(np.float32), batch_cap=64)
+        n.set_norm(np.zeros(T.MLP_IN), np.ones(T.MLP_IN), np.zeros(T.MLP_OUT), np.full(T.MLP_OUT, 1e-3))
+        return n
+
+    def run(spoil):
+        t = _small(4)
+        t.load_surface(V, Tr, (9.6, 10.2, 16.3))
+        keep = [net(1), net(2)]
+        t.set_predictor("mlp", keep[0], resid_theta=1e30)
+        if spoil:
+            with pytest.raises(T.TurretError):
+                t.set_predictor("mlp", net(9), slip_eps=-1.0)
+            assert t._net is keep[0]
+            keep[0] = None
+        t.step(9)
+        t.set_predictor("mlp", keep[1], resid_theta=1e30)
+        junk = torch.full((1 << 20,), -1, dtype=torch.int32, device="cuda:0")  # noqa: F841
+        t.step(3)
+        assert t.predictor_stats()["net_steps"] > 0
+        out = t.populations().cpu().numpy()
+        t.close()
+        return out
+
+    want = run(False)
+    assert np.array_equal(run(True), want)
