@@ -201,3 +201,31 @@ def test_training_step_beside_a_capture():
     assert np.array_equal(got.params().view(np.uint32), want.params().view(np.uint32))
     want.close()
     got.close()
+
+
+def test_epochs_are_gathered_in_parts(monkeypatch):
+    # the parts change neither the minibatches nor their order, and bound the
+    # memory an epoch takes beside a large set (its own size is 671 MB here)
+    import torch
+    from paper_2408_15115_gb300 import surrogate as S
+    x, y = (torch.tensor(a, dtype=torch.float32, device="cuda:0") for a in _data(1000, 3))
+    runs = []
+    for rows in (S.GATHER_ROWS, 100, 1):
+        monkeypatch.setattr(S, "GATHER_ROWS", rows)
+        net, hist = S.train(x, y, epochs=2, batch=64, seed=4)
+        runs.append((hist, net.params()))
+        net.close()
+    monkeypatch.undo()
+    for hist, p in runs[1:]:
+        assert hist == runs[0][0]
+        assert np.array_equal(p.view(np.uint32), runs[0][1].view(np.uint32))
+    n = 1 << 22
+    x, y = x.repeat(-(-n // 1000), 1)[:n].clone(), y.repeat(-(-n // 1000), 1)[:n].clone()
+    net = _net("bf16", I.mlp_init_params(2), _norm(*(a[:1000].cpu().numpy().astype(np.float64) for a in (x, y))),
+               cap=1 << 14)
+    torch.cuda.synchronize()
+    torch.cuda.reset_peak_memory_stats()
+    before = torch.cuda.memory_allocated()
+    S.train(x, y, epochs=1, batch=1 << 14, net=net)
+    assert torch.cuda.max_memory_allocated() - before < 8 * n + 2 * 160 * S.GATHER_ROWS + (1 << 24)
+    net.close()
