@@ -649,9 +649,10 @@ __device__ __forceinline__ void k1_cell(const Geom &g, const typename Codec<ST>:
     typename Codec<ST>::T *d = dst + (y * g.nx + x);
     if (ST == ST_BF16 && g.sround) {
         const int own = oz + y * g.nx + x;
+        const long long step = S.step;  // (as in k1_pair_collide_store)
 #pragma unroll
         for (int i = 0; i < 27; ++i)
-            store_bf16_sr(reinterpret_cast<__nv_bfloat16 *>(d + (i * ncell + oz)), q[i], sr_bits(i * ncell + own, S.step));
+            store_bf16_sr(reinterpret_cast<__nv_bfloat16 *>(d + (i * ncell + oz)), q[i], sr_bits(i * ncell + own, step));
         return;
     }
 #pragma unroll
@@ -832,12 +833,15 @@ __device__ __forceinline__ void k1_pair_collide_store(const Geom &g, typename Co
     typename Codec<ST>::T *d = dst + (y * g.nx + x);
     if (ST == ST_BF16 && g.sround) {
         const int own_a = oa + y * g.nx + x, own_b = ob + y * g.nx + x;
+        // held in a register: read through S the step would be loaded again after
+        // each of the 54 stores (96x96x192 periodic, us: 78.1, so 74.1; 160^3 172 / 163)
+        const long long step = S.step;
 #pragma unroll
         for (int i = 0; i < 27; ++i) {
             if (on[0])
-                store_bf16_sr(reinterpret_cast<__nv_bfloat16 *>(d + (i * ncell + oa)), q[i].x, sr_bits(i * ncell + own_a, S.step));
+                store_bf16_sr(reinterpret_cast<__nv_bfloat16 *>(d + (i * ncell + oa)), q[i].x, sr_bits(i * ncell + own_a, step));
             if (on[1])
-                store_bf16_sr(reinterpret_cast<__nv_bfloat16 *>(d + (i * ncell + ob)), q[i].y, sr_bits(i * ncell + own_b, S.step));
+                store_bf16_sr(reinterpret_cast<__nv_bfloat16 *>(d + (i * ncell + ob)), q[i].y, sr_bits(i * ncell + own_b, step));
         }
         return;
     }
