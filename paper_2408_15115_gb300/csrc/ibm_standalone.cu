@@ -15,7 +15,7 @@
 // Work is proportional to the markers plus one write of the field.  Before, a
 // block per tile scanned every marker (6252 markers on 96x80x72, 8640 tiles:
 // 158 us of scans and 25 us of gathering by 512 threads per mostly empty
-// tile; the whole call 227 us, now 64 us).
+// tile; the whole call 227 us, now 61 us).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -75,15 +75,21 @@ __global__ void __launch_bounds__(128) k_records(int nm, const float *__restrict
         r.hdS[2] = h[2 * nm + k] * d;
         rec[k] = r;
         if (bad) atomicMax(err, 1);
-        const int x1 = (bv[0] + 3) / TILE, y1 = (bv[1] + 3) / TILE, z1 = (bv[2] + 3) / TILE;
-        for (int z = bv[2] / TILE; z <= z1; ++z)
-            for (int y = bv[1] / TILE; y <= y1; ++y)
-                for (int x = bv[0] / TILE; x <= x1; ++x) {
-                    const int tile = x + box.tx * (y + box.ty * z);
-                    const int pos = atomicAdd(tile_count + tile, 1);
-                    if (pos < cap) tile_list[(size_t)tile * cap + pos] = k;
-                    else atomicMax(err, 2);
-                }
+        // one or two tiles per axis; the positions of all are fetched together
+        int tile[8], pos[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int x = bv[0] / TILE + (q & 1), y = bv[1] / TILE + (q >> 1 & 1), z = bv[2] / TILE + (q >> 2);
+            const bool in = x <= (bv[0] + 3) / TILE && y <= (bv[1] + 3) / TILE && z <= (bv[2] + 3) / TILE;
+            tile[q] = in ? x + box.tx * (y + box.ty * z) : -1;
+            pos[q] = in ? atomicAdd(tile_count + tile[q], 1) : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (tile[q] >= 0) {
+                if (pos[q] < cap) tile_list[(size_t)tile[q] * cap + pos[q]] = k;
+                else atomicMax(err, 2);
+            }
     }
     const long long total = 3 * box.nbox, step = (long long)gridDim.x * blockDim.x;
     if ((reinterpret_cast<uintptr_t>(field) & 15) == 0) {
@@ -97,21 +103,63 @@ __global__ void __launch_bounds__(128) k_records(int nm, const float *__restrict
 
 // Gather of the non-empty tiles.  Block b looks at tiles b, b + gridDim.x, ...
 // (the tiles of a surface are neighbours: the stride spreads them), ST_LOOK at
-// a time, and gathers each that has candidates: its list is ranked into marker
-// order (every thread counts the smaller indices of its entries; a list holds
-// some tens of markers, 2048 at most), then summed as in the time step's
-// spreading: thread (cell c, slice q) sums slice q of each staged chunk, the
+// a time, and gathers each that has candidates: its list is put into marker
+// order (a thread per entry counts the smaller ones; a list holds some tens of
+// markers, and beyond ST_THREADS, 2048 at most, it is sorted), then summed as in
+// the time step's spreading: thread (cell c, slice q) sums slice q of each staged chunk, the
 // slice sums are added in slice order.
 constexpr int ST_SLICES = 8, ST_CELLS = TILE * TILE * TILE, ST_THREADS = ST_CELLS * ST_SLICES;
 constexpr int ST_STAGE = 256, ST_LOOK = ST_THREADS;
 constexpr int ST_BLOCKS = 152 * 4;  // four resident blocks per SM
 
-__global__ void __launch_bounds__(ST_THREADS) k_spread_tiles(BoxGeom box, const MRec *__restrict__ rec,
+// The cnt > ST_THREADS indices of a long list into ord in ascending order, by
+// the whole block: bitonic sort, padded to a power of two; exchanges over less
+// than a warp's width are shuffles.  (Ranked like a short list, 2000 markers in
+// one cell of an 8^3 grid took 170 us a call, so 93; 1000 84 and 69.)
+static_assert((MAX_CANDIDATES & (MAX_CANDIDATES - 1)) == 0, "the longest list fits its padding");
+__device__ __forceinline__ void sort_list(const int *__restrict__ list, int cnt, int *ord) {
+    const int tid = threadIdx.x;
+    int n = 2 * ST_THREADS;
+    while (n < cnt) n *= 2;
+    // element i of a sequence sorted upwards where (i & run) is 0
+    auto exchange = [](int i, int v, int run, int d) {
+        const int o = __shfl_xor_sync(0xffffffffu, v, d);
+        return ((i & run) == 0) == ((i & d) == 0) ? min(v, o) : max(v, o);
+    };
+    for (int i = tid; i < n; i += ST_THREADS) {
+        int v = i < cnt ? __ldg(list + i) : 0x7fffffff;
+        for (int run = 2; run <= 32; run *= 2)
+            for (int d = run / 2; d > 0; d /= 2) v = exchange(i, v, run, d);
+        ord[i] = v;
+    }
+    for (int run = 64; run <= n; run *= 2) {
+        for (int d = run / 2; d >= 32; d /= 2) {
+            __syncthreads();
+            for (int i = tid; i < n / 2; i += ST_THREADS) {
+                const int a = 2 * i - (i & (d - 1)), b = a + d;
+                const int u = ord[a], v = ord[b];
+                if ((u > v) == ((a & run) == 0)) {
+                    ord[a] = v;
+                    ord[b] = u;
+                }
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < n; i += ST_THREADS) {
+            int v = ord[i];
+            for (int d = 16; d > 0; d /= 2) v = exchange(i, v, run, d);
+            ord[i] = v;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(ST_THREADS, 4) k_spread_tiles(BoxGeom box, const MRec *__restrict__ rec,
                                                              const int *__restrict__ tile_list,
                                                              const int *__restrict__ tile_count, int cap, int ntiles,
                                                              float *__restrict__ field) {
     __shared__ int s_tile[ST_LOOK], s_cnt[ST_LOOK], s_work;
-    __shared__ int raw[MAX_CANDIDATES], ord[MAX_CANDIDATES];
+    __shared__ __align__(16) int raw[MAX_CANDIDATES];
+    __shared__ int ord[MAX_CANDIDATES];
     __shared__ int sbase[ST_STAGE];
     __shared__ float sw[12][ST_STAGE], sh[3][ST_STAGE];
     float *part = reinterpret_cast<float *>(raw);  // [ST_SLICES][3][ST_CELLS] once the list is ranked
@@ -132,13 +180,20 @@ __global__ void __launch_bounds__(ST_THREADS) k_spread_tiles(BoxGeom box, const 
         for (int it = 0; it < work; ++it) {
             const int tile = s_tile[it], cnt = s_cnt[it];
             const int *list = tile_list + (size_t)tile * cap;
-            for (int i = tid; i < cnt; i += ST_THREADS) raw[i] = __ldg(list + i);
-            __syncthreads();
-            for (int i = tid; i < cnt; i += ST_THREADS) {
-                const int k = raw[i];
-                int r = 0;
-                for (int j = 0; j < cnt; ++j) r += raw[j] < k;
-                ord[r] = k;
+            if (cnt <= ST_THREADS) {
+                const int k = tid < cnt ? __ldg(list + tid) : 0x7fffffff;
+                raw[tid] = k;
+                __syncthreads();
+                if (tid < cnt) {
+                    int r = 0;
+                    for (int j = 0; j < cnt; j += 4) {
+                        const int4 v = *reinterpret_cast<const int4 *>(raw + j);
+                        r += (v.x < k) + (v.y < k) + (v.z < k) + (v.w < k);
+                    }
+                    ord[r] = k;
+                }
+            } else {
+                sort_list(list, cnt, ord);
             }
             const int tx = tile % box.tx, ty = (tile / box.tx) % box.ty, tz = tile / (box.tx * box.ty);
             const int cx = TILE * tx + c % TILE, cy = TILE * ty + (c / TILE) % TILE, cz = TILE * tz + c / (TILE * TILE);
@@ -305,7 +360,7 @@ extern "C" turret_status ibm_spread_noalloc(const float *X, const float *h, cons
         }
         scratch = g_noalloc_ptr[dev];
     }
-    // run_spread clears the error word first; records, lists and counts are
-    // fully rewritten by every call
+    // run_spread clears the counts and the error word first; records and listed
+    // entries are rewritten by every call
     return run_spread(X, h, dS, n_markers, nx, ny, nz, field, (char *)scratch, L, (cudaStream_t)stream);
 }
