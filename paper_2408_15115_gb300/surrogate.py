@@ -93,11 +93,13 @@ def train(x, y, epochs=30, batch=4096, lr=1e-3, weight_decay=1e-4, seed=0, preci
     for _ in range(epochs):
         # the epoch's minibatches in order, gathered many at a time (a gather and
         # its launches per minibatch cost as much as the training step)
-        perm = torch.as_tensor(rng.permutation(n)[:n - n % bsz], device=x.device)
+        used, rows = n - n % bsz, max(1, GATHER_ROWS // bsz) * bsz
+        perm = torch.as_tensor(rng.permutation(n)[:used], device=x.device)
         tot, cnt = 0.0, 0
-        for part in perm.split(max(1, GATHER_ROWS // bsz) * bsz):
+        for first in range(0, used, rows):
+            part = perm if used <= rows else perm[first:first + rows]
             xe, ye = x.index_select(0, part), y.index_select(0, part)
-            for s in range(0, part.shape[0], bsz):
+            for s in range(0, min(rows, used - first), bsz):
                 tot += net.train_step(xe[s:s + bsz], ye[s:s + bsz], lr=lr, weight_decay=weight_decay)
                 cnt += 1
         if val is None:

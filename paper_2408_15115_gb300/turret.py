@@ -469,6 +469,7 @@ class MLP:
         if nb == 0:
             raise TurretError(1, "invalid batch capacity")
         self._inputs = torch.cuda.Event()  # orders the network's stream after the caller's
+        self._capturing = torch.cuda.is_current_stream_capturing
         self._ws, ptr = _aligned_workspace(torch, nb, self.device)
         _follow_current(torch, self.device, self.stream, self._inputs)
         p = _arr(params, np.float32)
@@ -538,7 +539,10 @@ class MLP:
         that stream is being captured: the step is not part of the capture.  x and y may be dropped once
         the call returns, also without want_loss, when the step still runs."""
         n = x.shape[0]
-        _follow_current(self.torch, self.device, self.stream, self._inputs)
+        cur = self.torch.cuda.current_stream(self.device)
+        if cur != self.stream and not self._capturing():
+            self._inputs.record(cur)
+            self.stream.wait_event(self._inputs)
         opt = AdamW(lr, beta1, beta2, eps, weight_decay)
         L = C.c_float()
         self._check(self._L.mlp_train_step(self.m, C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()), n,
