@@ -90,3 +90,56 @@ def test_lists_built_ahead(window, storage, steps):
                     t.populations().cpu().numpy()))
     assert np.array_equal(out[0][0], out[1][0])
     assert np.array_equal(out[0][1], out[1][1])
+
+
+def _alone_and_batched(make, steps):
+    # a batch launches every kernel after the one before it, from plain lists: no
+    # launch of a step starts beside another of its stream, or is built quietly
+    from paper_2408_15115_gb300 import turret as T
+    out = []
+    for batched in (False, True):
+        t = make()
+        if batched:
+            b = T.Batch([t])
+            b.step(steps)
+            b.close()
+        else:
+            t.step(steps)
+        s = t.state()
+        out.append((np.concatenate([np.ravel(s[k]) for k in ("r", "v", "w", "F", "T")]),
+                    t.populations().cpu().numpy()))
+        t.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("window", [(32, 32, 64), (96, 96, 96)])
+@pytest.mark.parametrize("warm", [False, True])
+@pytest.mark.parametrize("cycles", [1, 4])
+def test_overlapped_and_quiet_steps_equal_plain_ones(window, warm, cycles):
+    # windows as above, also with cycles started from the previous force and with a
+    # single cycle (none but the first force in the paper's form)
+    nx, ny, nz = window
+    V, T = sphere_case()
+
+    def make():
+        return make_pair(nx, ny, nz, 0.05, (0, 0, 1, 2), kappa=2.5, g=(0, 0, -1e-4), sponge=8, slide=1, anchor=0.5,
+                         flags={"ibm_cycles": cycles}, predictor=(True, 1e-4) if warm else None,
+                         particle=(V, T, (nx / 2 - 0.5, ny / 2 - 0.5, nz / 2.0), (0, 0, -0.02), (0, 0, 0)))[0]
+
+    _alone_and_batched(make, 29)
+
+
+def test_a_surface_with_one_marker_set():
+    # 77,442 markers: a second set of the arrays of a time level would take more than
+    # 1 GiB, so the levels share one and the particle update waits for the spreading
+    from paper_2408_15115_gb300 import turret as T
+    V, Tr = I.icosphere(88, 66.0)
+
+    def make():
+        t = T.Turret(160, 160, 176, 0.05, 2.5, (0, 0, -1e-5), 0, 0, 1, 2, sponge=8)
+        t.load_surface(V, Tr, (79.6, 79.4, 80.3), (0.001, 0, -0.01), (0, 1e-4, 0))
+        assert 1 << 30 < t._ibm_ws.numel() < 2 << 30
+        return t
+
+    _alone_and_batched(make, 19)
