@@ -495,13 +495,16 @@ extern "C" size_t ibm_workspace_bytes(const turret_ctx *c, const double *V, int6
 
 // Whether the launches of the chain start beside the ones before them
 // (programmatic dependent launch): windows whose far cells take no longer than
-// the launches before the cycles (64^3: 9 of 12 us), with a cycle of at most
-// one block per SM.  There the chain is the step: 32x32x64, 362 markers, 100
-// steps 4797 us without, 4420 us with it.  On a larger window the bulk
-// collide+stream fills the SMs and blocks that wait take its slots: 96x96x192
-// (1212 markers, 24 steps) 2148 us without, 2489 us with it.
+// the launches before the cycles (64^3: 9 of 12 us), with few enough markers that
+// the waiting blocks of the rows (256 threads a marker) and of the cycles find
+// room beside the running ones.  There the chain is the step.  us per step, plain /
+// overlapped, FP32: 32x32x64 with 362, 812 and 1002 markers 27.3 / 22.7, 29.5 / 27.1 and
+// 31.2 / 34.7; 64^3 with 642, 812, 1002 and 1692 32.0 / 28.4, 32.7 / 31.3, 34.2 / 36.8 and
+// 38.5 / 45.2.  By cells, 492 markers: 64^3 30.9 / 27.1, 48x48x128 31.4 / 28.1, 64x64x96
+// 35.3 / 35.4, 64x64x128 39.9 / 43.4, 96x96x192 78.4 / 83.3: on larger windows the bulk
+// collide+stream fills the SMs and blocks that wait take its slots.
 constexpr long long OVERLAP_CELLS = 1 << 18;
-constexpr int OVERLAP_MARKERS = 152 * INTERP_WARPS;
+constexpr int OVERLAP_MARKERS = 900;
 static bool overlap_chain(const turret_ctx *c) { return c->geom.ncell <= OVERLAP_CELLS && c->nm <= OVERLAP_MARKERS; }
 
 // Whether the lists and rows prepared ahead are built quietly (LISTS_QUIET):
