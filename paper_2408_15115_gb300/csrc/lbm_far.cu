@@ -4,9 +4,9 @@
 // In the step graph this launch shares the SMs with the immersed-boundary
 // chain.  At 128 registers its four resident blocks of 128 threads fill the
 // 65,536-register file, so any chain block resident on an SM displaces one of
-// them (a quarter of that SM's streaming).  At 120 registers (no spill) four
-// blocks leave 4,096 registers free, room for a small chain block (the
-// 64-thread interpolation blocks) beside them.  The cell code is the same
+// them (a quarter of that SM's streaming).  At 120 registers (four values of the
+// boundary path spilled, 16 bytes) four blocks leave 4,096 registers free, room
+// for a small chain block (the 64-thread interpolation blocks) beside them.  The cell code is the same
 // device function as every other collide+stream launch (lbm_cell.cuh), so
 // results are identical.
 #include "lbm_cell.cuh"

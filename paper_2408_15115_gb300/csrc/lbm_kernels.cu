@@ -22,9 +22,13 @@ __device__ __forceinline__ void near_cell(const Geom &g, const typename Codec<ST
         k1_cell<ST, K1_NEAR>(g, src, dst, utop_in, utop_out, S, hbox, box, i % ex, (i / ex) % ey, i / (ex * ey));
 }
 
-// Window launches with 16-bit storage: five blocks per SM (<= 102 registers, a
-// few spilled values in L1) measured faster than four; FP32 keeps four (128
-// registers, no spill); the small near-region launch is left unconstrained.
+// Window launches with 16-bit storage: five blocks per SM (96 registers; 88 to
+// 104 bytes of spills in L1, 456 loaded with forcing) measured faster than four;
+// FP32 keeps four (128 registers; 28 bytes with forcing); the small near-region
+// launch is left unconstrained.  The spills are those of the boundary path
+// (pull27_edge), which pays wherever a window has closed faces (130x131x160
+// between walls FP16 256 -> 134 us) and costs where it has none at most 1.6 %
+// (160^3 periodic FP16 94.6 -> 96.1; BF16 96.4 -> 95.4, FP32 134.9 -> 134.7).
 template <int ST, int MODE>
 __global__ void __launch_bounds__(128, MODE == K1_NEAR ? 1 : (ST == ST_F32 ? 4 : 5)) k_collide_stream(Geom g, const typename Codec<ST>::T *__restrict__ src,
                                                         typename Codec<ST>::T *__restrict__ dst,

@@ -54,8 +54,9 @@ __global__ void __launch_bounds__(128, 5)
 // lbm_kernels.cu, on the tiles of k_collide_xpair: 4-byte loads of the
 // populations and 8-byte stores of the fields.  Bound by memory (70 bytes a cell
 // for rho and u).  192x192x384 FP16, call and synchronisation: 225 us with
-// 2-byte loads, 187 us so; 256x256x512: 501 and 418 us.  Six blocks
-// per SM: 214 / 193 / 187 / 190 us with 4 / 5 / 6 / 8; boundary tiles load all
+// 2-byte loads, 187 us so; 256x256x512: 501 and 418 us.  Six blocks per SM (80
+// registers, 160 bytes of spills): 214 / 193 / 187 / 190 us with 4 / 5 / 6 / 8,
+// forms without spills among them; boundary tiles load all
 // sources of a cell together (pull27_edge): 64x64x64 24.3 us without, 20.1 with.
 template <int ST>
 __global__ void __launch_bounds__(128, 6) k_macro_xpair(Geom g, const typename Codec<ST>::T *__restrict__ src,

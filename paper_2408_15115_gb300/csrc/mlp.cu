@@ -608,8 +608,8 @@ __device__ __forceinline__ int wb_index(int i) {
 }
 
 // Gradient of every parameter as the slice sums in slice order, and (step)
-// its AdamW update with the BF16 copy.  Block 0 also adds the blocks' losses
-// in block order: to *loss and, when given, to host-visible memory.
+// its AdamW update with the BF16 copy.  Block 0 also adds the blocks' losses (a
+// lane every 32nd in order, then an xor tree): to *loss and, when given, to host-visible memory.
 __global__ void __launch_bounds__(256) k_update(const float *__restrict__ part, int nsl, float *__restrict__ G, int step,
                                                 float *__restrict__ P, float *__restrict__ Mm, float *__restrict__ Vv,
                                                 __nv_bfloat16 *__restrict__ wb, float lr, float b1, float b2, float eps,
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(256) k_update(const float *__restrict__ part, 
 // Inference of up to 16 samples per block (the predictor): features
 // standardised, four layers with activations in shared memory, outputs
 // de-standardised.  TC: BF16 tensor cores with the padded BF16 weights (the
-// same operands and k order as k_gemm, hence the same results); otherwise
+// same operands and k order as k_rows, hence the same results); otherwise
 // FP32 on the CUDA cores with the FP32 weights.
 constexpr int INF_ROWS = 16, INF_THREADS = 128, ACT_LD = MLP_H + 8;
 
@@ -936,8 +936,9 @@ __global__ void k_build_samples(const double *__restrict__ log, long long nsamp,
 // and two blocks per SM, or 128 rows in a block of 1024 threads per SM, which holds
 // twice the rows and does in one round what takes the narrow blocks two: us with
 // narrow / wide blocks, 9728 rows (one round) 14.4 / 18.5, 12000 20.5 / 18.5, 15967
-// 22.5 / 18.5, 19457 (three) 26.1 / 30.7, 30000 (four) 35.1 / 32.8, 40000 (five)
-// 43.1 / 47.1, 84000 (nine) 74.7 / 74.6, 90000 80.6 / 75.5.  Bound by latency and
+// 22.5 / 18.5, 29184 (three) 30.4 / 32.8, 38912 (four) 37.1 / 32.8, 48640 (five) 45.1 /
+// 47.2, 58368 (six) 52.9 / 47.1, 68096 (seven) 60.1 / 61.5, 77824 (eight) 67.8 / 61.5,
+// 87552 (nine) 75.5 / 75.3, 97280 (ten) 82.7 / 75.4.  Bound by latency and
 // the GELU (384 erff a row), not by the products (1.2 GFLOP at 15967 rows).
 static cudaError_t launch_rows(const MlpDev &w, const float *x, int n, float *y, cudaStream_t s) {
     const int rounds = (n + 304 * RT_ROWS - 1) / (304 * RT_ROWS);  // of narrow blocks

@@ -427,8 +427,10 @@ static bool ibm_layout(const MeshProps &mp, const double *V, int64_t nv, IbmLayo
 }
 
 // Two sets of the level's own marker arrays while the second costs at most
-// this much; a surface beyond it (some 200,000 markers) shares one set, and a
-// step's particle update then waits for the previous spreading.
+// this much; a surface beyond it shares one set, and a step's particle update
+// then waits for the previous spreading.  A set is 4.3 KB per marker and up to
+// 16 KB of lists per support tile: a sphere with a marker per 0.6 to 0.8 cells
+// reaches the limit at 70,000 to 97,000 of them (radius 63 to 67).
 constexpr size_t SECOND_SET_MAX = (size_t)1 << 30;
 
 // The arrays a time level owns (see MarkerArrays).

@@ -155,7 +155,7 @@ struct __align__(16) MRec {
 };
 
 // Markers of one time level.  A context has two sets, by the level's parity:
-// Xb, nb, dS, dSo, ft, hl, r0 and hb are shared, the others (what the particle
+// Xb, nb, dS, dSo, ft, hl, r0, ha and hb are shared, the others (what the particle
 // update, the tile lists and the rows of A write) are the level's own, so those
 // of t + 1 are prepared while the cycles and the spreading of t still run.
 struct MarkerArrays {
@@ -395,7 +395,7 @@ bool prepare_staged();
 bool is_staged_kernel(const void *fn);
 // 16-bit collide+stream on x-adjacent cell pairs with 4-byte accesses
 // (lbm_xpair.cu): REGION_FAR or REGION_ALL without forcing; xpair_eligible:
-// FP16 or round-to-nearest BF16 on a window the 64 x 2 x 2 tiles cover.
+// FP16 or BF16 (either rounding) on a window the 64 x 2 x 2 tiles cover.
 bool xpair_eligible(const Geom &g, int storage);
 // launch_macro where xpair_eligible and out is 8-byte aligned.
 cudaError_t launch_macro_xpair(const Geom &g, int storage, const void *src, const float *utop_in, const DevState *st,

@@ -519,7 +519,7 @@ class MLP:
         return self._run(self._L.mlp_forward, x)
 
     def infer(self, x):
-        """Outputs [n][6] through the fused inference kernel of the predictor."""
+        """Outputs [n][6] for any number of rows, without the training workspace."""
         return self._run(self._L.mlp_infer, x)
 
     def loss_grad(self, x, y):
