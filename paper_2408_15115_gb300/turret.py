@@ -168,12 +168,24 @@ def _aligned_workspace(torch, nbytes, device):
     return buf, buf.data_ptr() + off
 
 
+_default_streams = {}  # by device, as Stream objects (making one takes longer than asking it)
+
+
 def _follow_current(torch, device, stream, event):
     """`stream`, which is about to use memory that the current stream allocated, follows the current
     stream's work: an earlier owner of that memory may still be in use there.  (A capture has no work
-    to follow.)"""
-    cur = torch.cuda.current_stream(device)
-    if cur != stream and not torch.cuda.is_current_stream_capturing():
+    to follow, and an idle stream none either: asking costs less than the event.)"""
+    index = device.index if device.index is not None else torch.cuda.current_device()
+    raw = torch._C._cuda_getCurrentRawStream(index)
+    if raw == stream.cuda_stream:
+        return
+    if raw:
+        cur = torch.cuda.current_stream(index)
+    else:
+        cur = _default_streams.get(index)
+        if cur is None:
+            cur = _default_streams[index] = torch.cuda.default_stream(index)
+    if not (raw and torch.cuda.is_current_stream_capturing()) and not cur.query():
         event.record(cur)
         stream.wait_event(event)
 
@@ -539,8 +551,8 @@ class MLP:
         that stream is being captured: the step is not part of the capture.  x and y may be dropped once
         the call returns, also without want_loss, when the step still runs."""
         n = x.shape[0]
-        cur = self.torch.cuda.current_stream(self.device)
-        if cur != self.stream and not self._capturing():
+        cur = self.torch.cuda.current_stream(self.device.index)
+        if cur != self.stream and not (cur.cuda_stream and self._capturing()):
             self._inputs.record(cur)
             self.stream.wait_event(self._inputs)
         opt = AdamW(lr, beta1, beta2, eps, weight_decay)
