@@ -583,9 +583,9 @@ __device__ __forceinline__ void k1_cell(const Geom &g, const typename Codec<ST>:
     const bool perx = g.bc_x == BC_PERIODIC, pery = g.bc_y == BC_PERIODIC, perz = g.bc_bottom == BC_PERIODIC;
     if (MODE == K1_NEAR) {
         // grid over the near region; map to window cells, skip cells outside closed faces
-        x = (perx ? S.box_lo_w[0] : S.box_lo[0]) - NEAR_GROW + cx;
-        y = (pery ? S.box_lo_w[1] : S.box_lo[1]) - NEAR_GROW + cy;
-        zl = (perz ? S.box_lo_w[2] : S.box_lo[2]) - NEAR_GROW + cz;
+        x = (perx ? S.box_lo_w[0] : S.box_lo[0]) - box.grow + cx;
+        y = (pery ? S.box_lo_w[1] : S.box_lo[1]) - box.grow + cy;
+        zl = (perz ? S.box_lo_w[2] : S.box_lo[2]) - box.grow + cz;
         if (perx) { x += (x < 0) ? g.nx : 0; x -= (x >= g.nx) ? g.nx : 0; } else if (x < 0 || x >= g.nx) return;
         if (pery) { y += (y < 0) ? g.ny : 0; y -= (y >= g.ny) ? g.ny : 0; } else if (y < 0 || y >= g.ny) return;
         if (perz) { zl += (zl < 0) ? g.nz : 0; zl -= (zl >= g.nz) ? g.nz : 0; } else if (zl < 0 || zl >= g.nz) return;
@@ -596,10 +596,10 @@ __device__ __forceinline__ void k1_cell(const Geom &g, const typename Codec<ST>:
         if (x >= g.nx || y >= g.ny) return;
         if (MODE == K1_FAR) {
             // the z test first: zl is the same for a whole block (plane)
-            const int rz = rel_axis(zl, S.box_lo[2], S.box_lo_w[2], NEAR_GROW, g.nz, perz);
+            const int rz = rel_axis(zl, S.box_lo[2], S.box_lo_w[2], box.grow, g.nz, perz);
             if ((unsigned)rz < (unsigned)box.Nz) {
-                const int rx = rel_axis(x, S.box_lo[0], S.box_lo_w[0], NEAR_GROW, g.nx, perx);
-                const int ry = rel_axis(y, S.box_lo[1], S.box_lo_w[1], NEAR_GROW, g.ny, pery);
+                const int rx = rel_axis(x, S.box_lo[0], S.box_lo_w[0], box.grow, g.nx, perx);
+                const int ry = rel_axis(y, S.box_lo[1], S.box_lo_w[1], box.grow, g.ny, pery);
                 if ((unsigned)rx < (unsigned)box.Nx && (unsigned)ry < (unsigned)box.Ny) return;
             }
         }
@@ -760,11 +760,11 @@ __device__ __forceinline__ void k1_pair(const Geom &g, const typename Codec<ST>:
         bool xy_checked = false, in_xy = false;
 #pragma unroll
         for (int l = 0; l < 2; ++l) {
-            const int rz = rel_axis(z[l], S.box_lo[2], S.box_lo_w[2], NEAR_GROW, g.nz, perz);
+            const int rz = rel_axis(z[l], S.box_lo[2], S.box_lo_w[2], box.grow, g.nz, perz);
             if (on[l] && (unsigned)rz < (unsigned)box.Nz) {
                 if (!xy_checked) {
-                    const int rx = rel_axis(x, S.box_lo[0], S.box_lo_w[0], NEAR_GROW, g.nx, perx);
-                    const int ry = rel_axis(y, S.box_lo[1], S.box_lo_w[1], NEAR_GROW, g.ny, pery);
+                    const int rx = rel_axis(x, S.box_lo[0], S.box_lo_w[0], box.grow, g.nx, perx);
+                    const int ry = rel_axis(y, S.box_lo[1], S.box_lo_w[1], box.grow, g.ny, pery);
                     in_xy = (unsigned)rx < (unsigned)box.Nx && (unsigned)ry < (unsigned)box.Ny;
                     xy_checked = true;
                 }

@@ -7,10 +7,9 @@ namespace turret {
 // The near region as one flat range of cells, x fastest: every thread but those
 // of the last block has a cell (rows of 26 to 46 cells leave 19 to 28 % of the
 // lanes of 32-wide rows idle, and the launch of a large body a second, nearly
-// empty wave: 46^3 cells 1152 blocks on 912 places, 761 flat).  The layer around
-// the support box (NEAR_GROW) makes these 48^3 cells, 864 blocks: 32x32x64 4190 ->
-// 4249 us per 100 steps, 256x256x512 18,958 -> 19,037 per 16, 96x96x192 2035 -> 2041
-// per 24.
+// empty wave: 46^3 cells 1152 blocks on 912 places, 761 flat; 864 where a body
+// needs a layer around the box, 256x256x512 18,958 -> 19,037 us per 16 steps,
+// 32x32x64 4190 -> 4249 per 100: the reason for NEAR_SLACK).
 template <int ST>
 __device__ __forceinline__ void near_cell(const Geom &g, const typename Codec<ST>::T *__restrict__ src,
                                           typename Codec<ST>::T *__restrict__ dst, const float *__restrict__ utop_in,

@@ -147,9 +147,9 @@ __device__ __forceinline__ int wrap(int c, int n) { return c < 0 ? c + n : (c >=
 
 // Whether the cells [c0, c0 + len) of one axis meet the near region (its
 // relative coordinates 0 .. ext - 1 from the support box origin lo / lo_w
-// less NEAR_GROW), as the per-cell test of k1_pair does cell by cell.
-__device__ __forceinline__ bool meets_near(int c0, int len, int lo, int lo_w, int ext, int n, bool periodic) {
-    const int r0 = rel_axis(c0, lo, lo_w, NEAR_GROW, n, periodic);
+// less the layers around it), as the per-cell test of k1_pair does cell by cell.
+__device__ __forceinline__ bool meets_near(int c0, int len, int lo, int lo_w, int ext, int grow, int n, bool periodic) {
+    const int r0 = rel_axis(c0, lo, lo_w, grow, n, periodic);
     return periodic ? (r0 < ext || r0 + len > n) : (r0 < ext && r0 + len > 0);
 }
 
@@ -169,9 +169,9 @@ __device__ __forceinline__ bool tile_staged(const Geom &g, const BodySlot &S, co
     if (g.bc_y != BC_PERIODIC && (y0 == 0 || y0 + STG_TY == g.ny)) ok = false;
     if (MODE == K1_FAR && ok) {
         const bool near =
-            meets_near(x0, STG_TX, S.box_lo[0], S.box_lo_w[0], box.Nx, g.nx, g.bc_x == BC_PERIODIC) &&
-            meets_near(y0, STG_TY, S.box_lo[1], S.box_lo_w[1], box.Ny, g.ny, g.bc_y == BC_PERIODIC) &&
-            meets_near(z0, STG_TZ, S.box_lo[2], S.box_lo_w[2], box.Nz, g.nz,
+            meets_near(x0, STG_TX, S.box_lo[0], S.box_lo_w[0], box.Nx, box.grow, g.nx, g.bc_x == BC_PERIODIC) &&
+            meets_near(y0, STG_TY, S.box_lo[1], S.box_lo_w[1], box.Ny, box.grow, g.ny, g.bc_y == BC_PERIODIC) &&
+            meets_near(z0, STG_TZ, S.box_lo[2], S.box_lo_w[2], box.Nz, box.grow, g.nz,
                        g.bc_bottom == BC_PERIODIC);
         ok = !near;
     }

@@ -56,9 +56,9 @@ __device__ __forceinline__ unsigned ld_word(const void *base, unsigned bytes) {
 }
 
 // Whether the cells [c0, c0 + len) of one axis meet the near region (relative
-// coordinates 0 .. ext - 1 from the support box origin less NEAR_GROW).
-__device__ __forceinline__ bool xp_meets_near(int c0, int len, int lo, int lo_w, int ext, int n, bool periodic) {
-    const int r0 = rel_axis(c0, lo, lo_w, NEAR_GROW, n, periodic);
+// coordinates 0 .. ext - 1 from the support box origin less the layers around it).
+__device__ __forceinline__ bool xp_meets_near(int c0, int len, int lo, int lo_w, int ext, int grow, int n, bool periodic) {
+    const int r0 = rel_axis(c0, lo, lo_w, grow, n, periodic);
     return periodic ? (r0 < ext || r0 + len > n) : (r0 < ext && r0 + len > 0);
 }
 
@@ -77,9 +77,9 @@ __device__ __forceinline__ bool xpair_tile_ok(const Geom &g, const BodySlot &S, 
     if (g.bc_x != BC_PERIODIC && (x0 == 0 || x0 + tw == g.nx)) ok = false;
     if (g.bc_y != BC_PERIODIC && (y0 == 0 || y0 + th == g.ny)) ok = false;
     if (MODE == K1_FAR && ok)
-        ok = !(xp_meets_near(x0, tw, S.box_lo[0], S.box_lo_w[0], box.Nx, g.nx, g.bc_x == BC_PERIODIC) &&
-               xp_meets_near(y0, th, S.box_lo[1], S.box_lo_w[1], box.Ny, g.ny, g.bc_y == BC_PERIODIC) &&
-               xp_meets_near(z0, 2, S.box_lo[2], S.box_lo_w[2], box.Nz, g.nz,
+        ok = !(xp_meets_near(x0, tw, S.box_lo[0], S.box_lo_w[0], box.Nx, box.grow, g.nx, g.bc_x == BC_PERIODIC) &&
+               xp_meets_near(y0, th, S.box_lo[1], S.box_lo_w[1], box.Ny, box.grow, g.ny, g.bc_y == BC_PERIODIC) &&
+               xp_meets_near(z0, 2, S.box_lo[2], S.box_lo_w[2], box.Nz, box.grow, g.nz,
                              g.bc_bottom == BC_PERIODIC));
     return ok;
 }

@@ -12,8 +12,8 @@
 //                           -> interpolation -> (h <- h + r0 - A h) x (n-1)
 //                           -> spread h_imm(t+1) -------------------------------^
 //
-// The near region (the support box and a layer around it) contains every cell
-// the next support-box pull reads, so the immersed-boundary chain only waits for the small near
+// The near region (around the support box) contains every cell the next
+// support-box pull reads, so the immersed-boundary chain only waits for the small near
 // launch and runs concurrently with the bulk of the window (the side stream
 // has the highest priority).  Groups of steps are captured as one graph in
 // which the chain also overlaps the next step (enqueue_steps_pipelined).
@@ -400,6 +400,10 @@ struct IbmLayout {
     double rmin, rmax;
 };
 
+// Margin for the FP32 rounding of the marker positions on the GPU (their
+// stencils must stay off the box's outer layer).
+constexpr double POSITION_MARGIN = 1e-3;
+
 // Support box: every marker lies within rc = ceil(bounding radius) of C_m,
 // so all 4x4x4 stencils fit a cube of 2 rc + 6 cells placed at floor(C) - rc - 2;
 // rc includes the offset F_OFFSET of the stress surface (its stencils too).
@@ -414,9 +418,7 @@ static bool ibm_layout(const MeshProps &mp, const double *V, int64_t nv, IbmLayo
     }
     L.rmin = rs;
     L.rmax = rb;
-    // 1e-3: margin for the FP32 rounding of the marker positions on the GPU
-    // (their stencils must stay off the box's outer layer)
-    L.rc = (int)ceil(rb + F_OFFSET + 1e-3);
+    L.rc = (int)ceil(rb + F_OFFSET + POSITION_MARGIN);
     const int B = 2 * L.rc + 6;
     L.box.Bx = L.box.By = L.box.Bz = B;
     L.box.tx = L.box.ty = L.box.tz = (B + TILE - 1) / TILE;
@@ -706,7 +708,9 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
         if (per[a] && L.box.Bx > n[a])
             return fail(c, TURRET_EINVAL, "support box wider than the window along a periodic axis");
     }
-    auto near_extent = [&](int b, int a) { return per[a] ? std::min(b + 2 * NEAR_GROW, n[a]) : b + 2 * NEAR_GROW; };
+    // (with the stress at the markers no stencil comes near the box's edge)
+    L.box.grow = near_grow(L.rc, L.rmax + (c->flags.force_eval == 0 ? F_OFFSET : 0.0) + POSITION_MARGIN);
+    auto near_extent = [&](int b, int a) { return per[a] ? std::min(b + 2 * L.box.grow, n[a]) : b + 2 * L.box.grow; };
     L.box.Nx = near_extent(L.box.Bx, 0);
     L.box.Ny = near_extent(L.box.By, 1);
     L.box.Nz = near_extent(L.box.Bz, 2);
@@ -788,8 +792,9 @@ extern "C" turret_status ibm_load_surface(turret_ctx *c, const double *V, int64_
        "dSo");
     CK(cudaMemsetAsync(c->ba.h, 0, 3 * (size_t)L.box.nbox * 4, c->stream), "h");
     // a batched step leaves the row of a marker that its tile's lists cannot hold
-    // as it was (and latches the overflow), and its cycles read every row's length
-    for (int k = 0; k < 2; ++k) CK(cudaMemsetAsync(c->mk[k].alen, 0, nm * 4, c->stream), "row lengths");
+    // as it was (and latches the overflow), and its cycles read every row's length:
+    // those of the set whose rows are not built here
+    CK(cudaMemsetAsync(c->mk[1 - (c->step & 1)].alen, 0, nm * 4, c->stream), "row lengths");
     // the moments kernel skips the box cells no stencil reads: they keep
     // finite values (zeros, or an earlier step's moments)
     CK(cudaMemsetAsync(c->ba.u, 0, (size_t)L.box.nbox * 16, c->stream), "u");

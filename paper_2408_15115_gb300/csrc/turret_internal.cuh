@@ -108,7 +108,8 @@ struct Geom {
 struct BoxGeom {
     int Bx, By, Bz;
     int tx, ty, tz;   // tiles of TILE^3 along each axis
-    int Nx, Ny, Nz;   // cells of the near region along each axis (see NEAR_GROW)
+    int Nx, Ny, Nz;   // cells of the near region along each axis
+    int grow;         // layers of it around the support box (see near_grow)
     long long nbox;   // Bx * By * Bz
 };
 
@@ -359,15 +360,20 @@ constexpr int QUIET_BLOCKS = 152, QUIET_THREADS = 64;
 // Launchers (lbm_kernels.cu).
 // win, here and below: the window slot of the time level pulled.
 // Collide+stream region: all cells, the cells outside the near region around
-// the particle, or the near region only.  The near region is the support box
-// grown by NEAR_GROW cells per side (all of a periodic axis that it would wrap
-// around).  It holds every cell the support-box moments pull, so they wait for
-// the near launch only: they skip their box's outer layer and pull from within
-// the box, but theirs is the box of t + 1, which lies one cell further along
-// each axis on which the centre crossed a cell face during the step (a body
-// moves less than a cell per step).
+// the particle, or the near region only.  The near region holds every cell the
+// support-box moments pull, so they wait for the near launch only.  They skip
+// their box's outer layer and pull from within the box, but theirs is the box of
+// t + 1, which lies one cell further along each axis on which the centre crossed
+// a cell face during the step.  Then a stencil reaches the cells next to the
+// outer layer, and the pull a cell outside the box of t, if the body's reach is
+// less than the step's motion below a whole number of cells: the near region is
+// the support box with a layer around it (all of a periodic axis that it would
+// wrap around), or the box itself where the reach leaves NEAR_SLACK cells, more
+// than a body moves in a step (wall speeds are held below 0.3; at 0.5 a body is
+// close to the lattice's speed of sound, 0.577).
 enum { REGION_ALL = 0, REGION_FAR = 1, REGION_NEAR = 2 };
-constexpr int NEAR_GROW = 1;
+constexpr double NEAR_SLACK = 0.5;
+inline int near_grow(int rc, double reach) { return rc - reach >= NEAR_SLACK ? 0 : 1; }
 // after_spread (REGION_NEAR): start beside the spreading launched just before on
 // the same stream, with everything else the pull needs complete.
 // slot_out >= 0: the kernel also copies the window slot to slot_out (with no
