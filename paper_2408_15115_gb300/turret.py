@@ -168,26 +168,35 @@ def _aligned_workspace(torch, nbytes, device):
     return buf, buf.data_ptr() + off
 
 
-_default_streams = {}  # by device, as Stream objects (making one takes longer than asking it)
+class _Follow:
+    """Call it before `stream` uses memory that the current stream allocated: it then follows the current
+    stream's work, where an earlier owner of that memory may still be in use.  (A capture has no work to
+    follow, and an idle stream none either: asking costs less than an event.)"""
 
+    _default = {}  # by device: Stream objects take longer to make than to ask
 
-def _follow_current(torch, device, stream, event):
-    """`stream`, which is about to use memory that the current stream allocated, follows the current
-    stream's work: an earlier owner of that memory may still be in use there.  (A capture has no work
-    to follow, and an idle stream none either: asking costs less than the event.)"""
-    index = device.index if device.index is not None else torch.cuda.current_device()
-    raw = torch._C._cuda_getCurrentRawStream(index)
-    if raw == stream.cuda_stream:
-        return
-    if raw:
-        cur = torch.cuda.current_stream(index)
-    else:
-        cur = _default_streams.get(index)
-        if cur is None:
-            cur = _default_streams[index] = torch.cuda.default_stream(index)
-    if not (raw and torch.cuda.is_current_stream_capturing()) and not cur.query():
-        event.record(cur)
-        stream.wait_event(event)
+    def __init__(self, torch, device, stream):
+        self.torch, self.stream = torch, stream
+        self.index = device.index if device.index is not None else torch.cuda.current_device()
+        self.own = stream.cuda_stream
+        self.current = torch._C._cuda_getCurrentRawStream
+        self.default = _Follow._default.get(self.index)
+        if self.default is None:
+            self.default = _Follow._default[self.index] = torch.cuda.default_stream(self.index)
+        self.event = torch.cuda.Event()
+
+    def __call__(self):
+        raw = self.current(self.index)
+        if raw == self.own:
+            return
+        cur = self.default
+        if raw:
+            if self.torch.cuda.is_current_stream_capturing():
+                return
+            cur = self.torch.cuda.current_stream(self.index)
+        if not cur.query():
+            self.event.record(cur)
+            self.stream.wait_event(self.event)
 
 
 def ibm_spread(X, h, dS, shape, stream=None):
@@ -206,7 +215,7 @@ def ibm_spread(X, h, dS, shape, stream=None):
     ws, ptr = _aligned_workspace(torch, nb, dev)
     st = stream if stream is not None else torch.cuda.current_stream(dev)
     if stream is not None:
-        _follow_current(torch, dev, st, torch.cuda.Event())
+        _Follow(torch, dev, st)()
     rc = L.ibm_spread(C.c_void_p(X.data_ptr()), C.c_void_p(h.data_ptr()), C.c_void_p(dS.data_ptr()), n, nx, ny, nz,
                       C.c_void_p(out.data_ptr()), C.c_void_p(ptr), C.c_size_t(nb), C.c_void_p(st.cuda_stream))
     if rc != 0:
@@ -234,7 +243,7 @@ class Turret:
         nb = self._L.lbm_workspace_bytes(C.byref(self.win), st)
         if nb == 0:
             raise TurretError(1, "invalid window")
-        self._order = torch.cuda.Event()
+        self._follow = _Follow(torch, self.device, self.stream)
         self._ws, ptr = self._buffer(nb)
         self._ibm_ws = None
         g3 = (C.c_double * 3)(*g)
@@ -256,12 +265,12 @@ class Turret:
 
     def _buffer(self, nbytes):
         buf, ptr = _aligned_workspace(self.torch, nbytes, self.device)
-        _follow_current(self.torch, self.device, self.stream, self._order)
+        self._follow()
         return buf, ptr
 
     def _output(self, n):
         out = self.torch.empty((n,) + self.shape, dtype=self.torch.float32, device=self.device)
-        _follow_current(self.torch, self.device, self.stream, self._order)
+        self._follow()
         return out
 
     def set_wall_velocity(self, u_bottom=(0.0, 0.0, 0.0), u_top=(0.0, 0.0, 0.0)):
@@ -358,7 +367,7 @@ class Turret:
         log = None
         if capacity > 0:
             log = self.torch.zeros((int(capacity), self.LOG_REC), dtype=self.torch.float64, device=self.device)
-            _follow_current(self.torch, self.device, self.stream, self._order)
+            self._follow()
         self._check(self._L.turret_set_log(self.ctx, None if log is None else C.c_void_p(log.data_ptr()),
                                            0 if log is None else int(capacity)))
         self.stream.synchronize()  # steps still running write to the log before
@@ -370,7 +379,7 @@ class Turret:
         cap = self._log.shape[0]
         k = n % cap
         out = self._log[:n].clone() if n <= cap else self.torch.cat([self._log[k:], self._log[:k]])
-        _follow_current(self.torch, self.device, self.stream, self._order)  # later steps write where this reads
+        self._follow()  # later steps write where this reads
         return out
 
     def predictor_stats(self):
@@ -414,7 +423,7 @@ class Batch:
         if nb == 0:
             raise TurretError(1, "empty batch")
         self._ws, ptr = _aligned_workspace(torch, nb, self.device)
-        _follow_current(torch, self.device, self.stream, torch.cuda.Event())
+        _Follow(torch, self.device, self.stream)()
         arr = (C.c_void_p * n)(*[t.ctx.value for t in self.runs])
         b = C.c_void_p()
         rc = self._L.turret_batch_init(C.byref(b), arr, n, C.c_void_p(ptr), C.c_size_t(nb),
@@ -480,10 +489,10 @@ class MLP:
         nb = self._L.mlp_workspace_bytes(self.cap)
         if nb == 0:
             raise TurretError(1, "invalid batch capacity")
-        self._inputs = torch.cuda.Event()  # orders the network's stream after the caller's
+        self._inputs = torch.cuda.Event()  # orders a training step after its inputs' stream
         self._capturing = torch.cuda.is_current_stream_capturing
         self._ws, ptr = _aligned_workspace(torch, nb, self.device)
-        _follow_current(torch, self.device, self.stream, self._inputs)
+        _Follow(torch, self.device, self.stream)()
         p = _arr(params, np.float32)
         m = C.c_void_p()
         rc = self._L.mlp_init(C.byref(m), self.cap, {"bf16": 0, "fp32": 1}[precision], p.ctypes.data_as(_fp),
